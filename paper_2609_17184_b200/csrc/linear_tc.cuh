@@ -24,6 +24,7 @@ constexpr int TC_THREADS = 128;
 constexpr int TC_BM = 128;         // weight rows per CTA = rows of one MMA
 constexpr int TC_BK = 64;          // k per stage: 64 bf16 = one 128-byte swizzled row
 constexpr int TC_MAX_STAGES = 8;
+constexpr int TC_SMEM_MAX = 101 * 1024;  // most dynamic shared memory any launch of linear_tc_kernel asks for
 constexpr long long TC_WAIT_CYCLES = 400000000LL;  // ~0.2 s: a wait that runs this long gives up and raises the flag
 
 struct LinearTcParams {

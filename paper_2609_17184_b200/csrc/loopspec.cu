@@ -1101,6 +1101,8 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
   c->m = *m, c->s = *s, c->d = d, c->L = L, c->n_sm = n_sm;
   c->s.d1 = d.d1, c->s.d2 = d.d2;
   if (c->s.top_p <= 0.f || c->s.top_p > 1.f) c->s.top_p = 1.f;  // 0 and anything above 1: no nucleus cut
+  // (A kernel's shared-memory limit is the process's, not the context's: every context asks for the same ceiling, so that none
+  // lowers it below what another one launches with.)
   c->filters = c->s.temperature > 0.f && ((c->s.top_k > 0 && c->s.top_k < m->vocab) || c->s.top_p < 1.f);
   {  // selection kernel, sampling: every CTA stages its slice of up to three logits rows in shared memory, plus the
      // slice of exp(z/T - max) when C filters; rows too long for that are read from global memory in every pass
@@ -1109,7 +1111,7 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
     c->sel_smem = (c->sel_staged ? 3 * slice : 0) + (c->filters ? slice : 0);
     if (c->sel_smem > 200 * 1024 ||
         (c->sel_smem > 48 * 1024 &&
-         cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->sel_smem) != cudaSuccess)) {
+         cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)) {
       (void)cudaGetLastError();
       delete c;
       return LOOPSPEC_EUNSUPPORTED;
@@ -1229,7 +1231,6 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
     const int x_k[4] = {m->hidden, dd.Hq, m->ffn, 2 * m->hidden};
     const bool want[2] = {!s->prefill_skinny, c->ng_dec > 1};
     const int rows[2] = {dd.max_rows_pf, std::min(dd.max_rows_dec, (int)GROUP_ROWS)};  // (wider decode passes: groups of 64 columns)
-    size_t smem_max = 0;
     for (int k = 0; k < 2 && ok; ++k) {
       if (!want[k]) continue;
       loopspec_ctx::TcCfg& tc = c->tc[k];
@@ -1237,11 +1238,10 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
       const int sb = tc_stage_bytes(tc.cols);
       tc.stages = std::max(2, std::min(TC_MAX_STAGES, (100 * 1024) / sb));
       tc.smem = (size_t)tc.stages * sb + 1024;
-      smem_max = std::max(smem_max, tc.smem);
       for (int i = 0; i < (dd.raven ? 4 : 3) && ok; ++i)
         ok = make_map_planes3d(&tc.xmaps[i], c->ws + x_off[i], x_k[i], x_k[i], dd.max_rows, tc.cols);
     }
-    if (smem_max) ok = ok && cudaFuncSetAttribute(linear_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max) == cudaSuccess;
+    ok = ok && cudaFuncSetAttribute(linear_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MAX) == cudaSuccess;
     if (!ok) (void)cudaGetLastError();
     for (int k = 0; k < 2; ++k) c->tc[k].on = ok && want[k];
   }
@@ -1864,7 +1864,7 @@ int loopspec_op_linear_tc(const void* W, const float* x, float* y, int32_t M, in
   p.out = t.n_split > 1 ? reinterpret_cast<float*>(sc + t.part_off) : y;
   p.M = M, p.MP = t.MP, p.N = N, p.K = K, p.kb_per_split = t.kb_per_split, p.stages = t.stages;
   p.err = reinterpret_cast<int*>(sc), p.err_code = 1;
-  if (cudaFuncSetAttribute(linear_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t.smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(linear_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MAX) != cudaSuccess)
     return LOOPSPEC_ECUDA;
   linear_tc_kernel<<<dim3(t.n_rb, t.n_split), TC_THREADS, t.smem, st>>>(map_w, map_x, p);
   if (t.n_split > 1) tc_sum_splits_kernel<<<296, 256, 0, st>>>(p.out, y, (size_t)M * N, t.n_split);
@@ -1892,7 +1892,7 @@ int loopspec_time_linear_tc(const void* const* Ws, int32_t n_w, const float* x, 
   p.out = reinterpret_cast<float*>(sc + t.part_off);
   p.M = M, p.MP = t.MP, p.N = N, p.K = K, p.kb_per_split = t.kb_per_split, p.stages = t.stages;
   p.err = reinterpret_cast<int*>(sc), p.err_code = 1;
-  if (cudaFuncSetAttribute(linear_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t.smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(linear_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MAX) != cudaSuccess)
     return LOOPSPEC_ECUDA;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);

@@ -609,3 +609,17 @@ def test_longer_context_spans_many_attention_chunks():
     ctx.decode(24)
     U.assert_same_run(ctx, ref, 24)
     ctx.close()
+
+
+def test_contexts_of_different_widths_coexist():
+    """A kernel's shared-memory limit belongs to the process: a context (or a stand-alone call) that needs less of it must
+    not lower the limit under one that was created before."""
+    import paper_2609_17184_b200 as ls
+    ref = U.oracle_run("tiny_bf16", 20, 12, 1, 2, T=1.0, seed=2)
+    a = U.make_ctx("tiny_bf16", 1, 2, T=1.0, seed=2, max_ctx=64, max_prefill_rows=32)
+    b = U.make_ctx("tiny_bf16", 1, 2, T=1.0, seed=2, max_ctx=64, max_prefill_rows=64)
+    ls.linear_tc(torch.zeros(128, 64, dtype=torch.bfloat16, device="cuda"), torch.zeros(1, 64, device="cuda"))
+    for ctx in (a, b):
+        assert ctx.prefill(ref["prompt"]) == ref["first"]
+        assert ctx.decode(12)[0].tolist() == ref["tokens"]
+        ctx.close()
