@@ -216,7 +216,7 @@ def run_profile_pass(args):
     shape = W.CONFIGS[wl.model]
     weights = ls.upload_weights(shape, W.make_weights(shape, seed=wl.weight_seed))
     ctx = ls.LoopSpec(shape, weights, d1=wl.d1, d2=wl.d2, temperature=wl.temperature, seed=wl.sample_seed, gate=wl.gate,
-                      max_seqs=1, max_ctx=wl.prompt_len + wl.decode_len + 16, max_prefill_rows=64)
+                      max_seqs=1, max_ctx=wl.prompt_len + wl.decode_len + 16)
     ctx.prefill(W.make_prompt(shape.vocab, wl.prompt_len, seed=wl.prompt_seed))
     ctx.decode(args.profile_pass)
     st = ctx.stats()
@@ -233,7 +233,7 @@ def select_depths(ls, shape, weights, prompt, wl, n_tokens=96):
     tv = {}
     for r in range(2, R):
         ctx = ls.LoopSpec(shape, weights, d1=1, d2=r, temperature=wl.temperature, seed=wl.sample_seed, gate=False, max_seqs=1,
-                          max_ctx=len(prompt) + n_tokens + 16, max_prefill_rows=64, top_k=wl.top_k, top_p=wl.top_p,
+                          max_ctx=len(prompt) + n_tokens + 16, top_k=wl.top_k, top_p=wl.top_p,
                           measure_tv=True)
         ctx.prefill(prompt)
         ctx.decode(n_tokens)
@@ -277,7 +277,7 @@ def run_ours(args):
     if args.closed_form and wl.temperature > 0:
         d1, d2, depth_sel = select_depths(ls, shape, weights, prompt, wl)
     ctx = ls.LoopSpec(shape, weights, d1=d1, d2=d2, temperature=wl.temperature, seed=wl.sample_seed, gate=wl.gate,
-                      max_seqs=batch, max_ctx=n_prompt + n_decode + 16, max_prefill_rows=64, top_k=wl.top_k, top_p=wl.top_p)
+                      max_seqs=batch, max_ctx=n_prompt + n_decode + 16, top_k=wl.top_k, top_p=wl.top_p)
     stream = ctx.stream
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
 
@@ -452,7 +452,7 @@ def run_calibrated(ls, shape, wl, prompt, n_prompt, n_decode, args):
     for scale in (0.0001, 0.0003, 0.001, 0.00003):
         w = ls.upload_weights(shape, W.make_weights(shape, seed=wl.weight_seed, out_scale=scale))
         ctx = ls.LoopSpec(shape, w, d1=wl.d1, d2=wl.d2, temperature=wl.temperature, seed=wl.sample_seed, gate=wl.gate,
-                          max_seqs=1, max_ctx=n_prompt + n_decode + 16, max_prefill_rows=64)
+                          max_seqs=1, max_ctx=n_prompt + n_decode + 16)
         ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         times = {}
         for name, fn in (("loopspec", ctx.decode), ("vanilla", ctx.vanilla_decode)):

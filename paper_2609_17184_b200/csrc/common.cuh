@@ -134,6 +134,26 @@ __device__ __forceinline__ void store_split(__nv_bfloat16* row_planes, int ld, i
   row_planes[2 * ld + k] = __ushort_as_bfloat16(l);
 }
 
+// the same for two / four neighbouring values (k even / a multiple of 4): 4- and 8-byte stores
+__device__ __forceinline__ void store_split2(__nv_bfloat16* row_planes, int ld, int k, float a, float b) {
+  unsigned short h0, m0, l0, h1, m1, l1;
+  split3(a, h0, m0, l0);
+  split3(b, h1, m1, l1);
+  *reinterpret_cast<unsigned*>(row_planes + k) = h0 | ((unsigned)h1 << 16);
+  *reinterpret_cast<unsigned*>(row_planes + ld + k) = m0 | ((unsigned)m1 << 16);
+  *reinterpret_cast<unsigned*>(row_planes + 2 * ld + k) = l0 | ((unsigned)l1 << 16);
+}
+__device__ __forceinline__ void store_split4(__nv_bfloat16* row_planes, int ld, int k, float4 v) {
+  unsigned short h[4], m[4], l[4];
+  split3(v.x, h[0], m[0], l[0]);
+  split3(v.y, h[1], m[1], l[1]);
+  split3(v.z, h[2], m[2], l[2]);
+  split3(v.w, h[3], m[3], l[3]);
+  *reinterpret_cast<uint2*>(row_planes + k) = make_uint2(h[0] | ((unsigned)h[1] << 16), h[2] | ((unsigned)h[3] << 16));
+  *reinterpret_cast<uint2*>(row_planes + ld + k) = make_uint2(m[0] | ((unsigned)m[1] << 16), m[2] | ((unsigned)m[3] << 16));
+  *reinterpret_cast<uint2*>(row_planes + 2 * ld + k) = make_uint2(l[0] | ((unsigned)l[1] << 16), l[2] | ((unsigned)l[3] << 16));
+}
+
 // tuning aid: earliest CTA start / latest CTA end of kernel `id` on the global nanosecond timer
 __device__ __forceinline__ void timeline_mark(unsigned long long* tl, int id, bool end) {
   if (!kTune || tl == nullptr || threadIdx.x != 0) return;

@@ -23,6 +23,7 @@
 #include "select.cuh"
 #include "linear_tc.cuh"
 #include "gemm_dec.cuh"
+#include "prefill.cuh"
 
 using namespace ls;
 
@@ -170,6 +171,30 @@ bool make_map_planes_all(CUtensorMap* map, const void* ptr, int K, int x_ld, int
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+// gate/up weights [2F][K] as a (k, feature, gate | up) tensor; box = 64 k x 64 features of both
+bool make_map_gateup(CUtensorMap* map, const void* ptr, int F, int K) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)F, 2};
+  cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)F * K * 2};
+  cuuint32_t box[3] = {(cuuint32_t)TC_BK, 64, 2};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+// the planes of a prompt pass, [row][3][K] bf16, as a (k, row, plane) tensor; box = 64 k x box_rows rows of one plane
+bool make_map_pf_planes(CUtensorMap* map, const void* ptr, int K, int n_rows, int box_rows) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)n_rows, 3};
+  cuuint64_t strides[2] = {(cuuint64_t)K * 6, (cuuint64_t)K * 2};
+  cuuint32_t box[3] = {(cuuint32_t)TC_BK, (cuuint32_t)box_rows, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 // k-split of a prefill GEMM on the tcgen05 kernel: a function of the matrix alone, so that a prompt position's sums
 // do not depend on how many positions share the pass
 struct TcPfPlan {
@@ -195,7 +220,7 @@ int tc_pf_cols(int max_rows_pf) { return (max_rows_pf + 15) / 16 * 16; }
 
 struct Layout {  // byte offsets into the workspace
   size_t wpack, rope, kv, hid, qbuf, xplanes, aplanes, splanes, sumsq, logits, argpart, tcpart, flt, sel_flt, tv, tune, tune_bytes, apart, acnt, nodes, seqs, ctr, tab_dec, tab_pf,
-      estore, cplanes, tab_pre, tab_coda, tab_pfc, tab_vanc, tab_van, sel_tok, sel_aux, sel_lse, sel_z2, kvcopy, out_ids, commits, trace, trace_n, prompt, total;
+      estore, cplanes, pf_hid, pf_hid2, pf_e, pf_x, pf_a, pf_s, pf_c, pf_q, pf_part, pf_sumsq, tab_pre, tab_coda, tab_pfc, tab_vanc, tab_van, sel_tok, sel_aux, sel_lse, sel_z2, kvcopy, out_ids, commits, trace, trace_n, prompt, total;
 };
 
 struct Derived {
@@ -205,6 +230,7 @@ struct Derived {
       trace_cap, Hq, Hkv, d1, d2;
   // Raven-style layout (P and C hold transformer blocks): all layers in one list - prelude, recurrent, coda
   int raven, n_pre, n_coda, NL, n_classes, class_depth[3], hid_coda_base;
+  int pf_rows;    // positions a prompt pass of the wide kernels carries (0: the prompt runs the kernels of the narrow passes)
 };
 
 int max_branches(int R, int d1, int d2) {
@@ -281,6 +307,9 @@ bool resolve_sched(const loopspec_model* m, const loopspec_sched* s, Derived* d,
   d->max_rows_dec = d->S * d->B;
   d->max_rows_pf = s->max_prefill_rows ? s->max_prefill_rows : 32;
   if (d->max_rows_pf > GROUP_ROWS) return false;
+  // prompts run the wide kernels unless the caller bounds the pass (max_prefill_rows) or asks for the decode kernels
+  d->pf_rows = (m->weight_dtype == 1 && s->max_prefill_rows == 0 && !s->prefill_skinny) ? std::min(PF_MAX_ROWS, (s->max_ctx + 127) / 128 * 128) : 0;
+  if (d->pf_rows) d->max_rows_pf = GROUP_ROWS;  // (the narrow passes are left with the prompts that fit one of them)
   {  // rows of the pass buffers: one group of 8 / 16 / 32 / 64 token columns, or whole groups of 64
     const int need = std::max(d->max_rows_dec, d->max_rows_pf);
     d->max_rows = need <= GROUP_ROWS ? 8 * ng_for_rows(need) : (need + GROUP_ROWS - 1) / GROUP_ROWS * GROUP_ROWS;
@@ -349,6 +378,19 @@ Layout make_layout(const loopspec_model* m, const loopspec_sched* s, const Deriv
     }
     L.tcpart = take(need);
   }
+  {  // buffers of a prompt pass of the wide kernels
+    const size_t P = d.pf_rows;
+    L.pf_hid = take(P * m->hidden * 4);
+    L.pf_hid2 = take(d.raven ? P * m->hidden * 4 : 0);
+    L.pf_e = take(d.raven ? P * m->hidden * 4 : 0);
+    L.pf_x = take(P * 3 * m->hidden * 2);
+    L.pf_a = take(P * 3 * d.Hq * 2);
+    L.pf_s = take(P * 3 * m->ffn * 2);
+    L.pf_c = take(d.raven ? P * 6 * m->hidden * 2 : 0);
+    L.pf_q = take(P * d.Hq * 4);
+    L.pf_part = take(P * PF_MAX_SPLIT * m->hidden * 4);
+    L.pf_sumsq = take(P * 4);
+  }
   L.tune_bytes = kTune ? (size_t)1 << 20 : 0;  // kernel timeline of tuning builds
   L.tune = take(L.tune_bytes);
   int G = m->n_q_heads / m->n_kv_heads;
@@ -414,6 +456,10 @@ struct loopspec_ctx {
   TcCfg tc[2];                  // 0: prefill passes, 1: decode passes
   std::vector<CUtensorMap> tc_wmaps;  // 4 per block, then the adapter
   TcPfPlan tc_plan[5];          // qkv, o, gate/up, down, adapter
+  // prompt passes of the wide kernels: tensor maps of the weights (4 per block, then the adapter) and of the four plane buffers
+  bool pf = false;
+  std::vector<CUtensorMap> pf_wmaps;
+  CUtensorMap pf_x1[4], pf_x2[4];     // planes read by QKV and gate/up, by O, by down, by the adapter: boxes of 128 / 64 rows
   // readout GEMM of the decode passes on the tcgen05 kernel (bf16 weights): plan, tensor maps of the row-major lm_head
   // (one box per 128-row tile) and of the hidden-state planes (all three planes of dg_mp rows in one box)
   bool dg = false;
@@ -664,6 +710,11 @@ GemmParams gemm_params(loopspec_ctx* c, int which, int layer, const RowTable* ta
   return p;
 }
 
+// most rows a pass over `tab` can carry (grids with one CTA or cluster per row)
+int table_rows(loopspec_ctx* c, const RowTable* tab) {
+  return (tab == c->at<RowTable>(c->L.tab_pf) || tab == c->at<RowTable>(c->L.tab_pfc)) ? c->d.max_rows_pf : c->d.max_rows_dec;
+}
+
 // planes and sums of squares for the first block of a stack (`first_layer`); use_src: on copies of the rows' states
 cudaError_t launch_prep(loopspec_ctx* c, const RowTable* tab, int first_layer = 0, bool use_src = false) {
   PrepParams q;
@@ -671,7 +722,7 @@ cudaError_t launch_prep(loopspec_ctx* c, const RowTable* tab, int first_layer = 
   q.tab = tab, q.hid = c->at<float>(c->L.hid), q.K = c->m.hidden, q.planes = c->at<__nv_bfloat16>(c->L.xplanes);
   q.gain = static_cast<const float*>(c->layers[6 * first_layer]), q.sumsq = c->at<float>(c->L.sumsq), q.sq_stride = c->d.sq_stride;
   q.use_src = use_src ? 1 : 0;
-  return launch_k(prep_planes_kernel, dim3(c->d.max_rows), dim3(256), 0, c->stream, q, c->use_pdl);
+  return launch_k(prep_planes_kernel, dim3(table_rows(c, tab)), dim3(256), 0, c->stream, q, c->use_pdl);
 }
 
 
@@ -741,17 +792,19 @@ cudaError_t launch_dg_raw(int epi, const DgPlan& g, const CUtensorMap& mw, const
   return cudaLaunchKernelEx(&cfg, dg_fn(epi), mw, mx, q);
 }
 // the readout GEMM of a decode pass on the tcgen05 kernel
-cudaError_t launch_dg_lm(loopspec_ctx* c, const RowTable* tab) {
+cudaError_t launch_dg_lm(loopspec_ctx* c, const RowTable* tab, bool one_sum = false) {
   const DgPlan& g = c->dgp;
   DgParams q;
   memset(&q, 0, sizeof q);
   q.g = gemm_params(c, G_LM, 0, tab);
   q.g.cluster_size = g.cs, q.g.n_clusters = g.n_clusters, q.g.n_rb = g.n_rb;
+  if (one_sum) q.g.n_sq = 1;
   q.g.err = c->host_flags_dev + HF_ERROR, q.g.tl_id = 120;
   q.MP = c->dg_mp, q.stages = g.stages, q.acc_bufs = g.acc_bufs, q.recv_bufs = g.recv_bufs, q.err_code = ERR_WAIT;
   q.wait_cycles = c->dg_wait_cycles;
   q.drop_unit = c->dg_drop_unit;
-  return launch_dg_raw(EPI_LOGITS, g, c->dg_wmap, c->dg_xmap, q, c->stream, c->use_pdl);
+  // (one_sum: the row table was written by the launch before, and this kernel reads it ahead of its dependency wait)
+  return launch_dg_raw(EPI_LOGITS, g, c->dg_wmap, c->dg_xmap, q, c->stream, c->use_pdl && !one_sum);
 }
 
 // launches a GEMM of a pass over `tab` takes: decode passes that can carry more than 64 rows run every GEMM once per group of
@@ -795,8 +848,6 @@ cudaError_t launch_attention(loopspec_ctx* c, const RowTable* tab, int l, unsign
 // the blocks [l0, l0 + count) of the layer list on the rows of `tab`
 cudaError_t launch_stack(loopspec_ctx* c, const RowTable* tab, int ng, int l0, int count, int* n_launch, int tc) {
   const loopspec_model& m = c->m;
-  const Derived& d = c->d;
-  const int G = m.n_q_heads / m.n_kv_heads;
   const bool pdl = c->use_pdl;
   cudaError_t e;
   const int groups = col_groups(c, tab);
@@ -843,7 +894,7 @@ cudaError_t launch_layers(loopspec_ctx* c, const RowTable* tab, int ng, int* n_l
   ConcatParams cp;
   cp.tab = tab, cp.hid = c->at<float>(c->L.hid), cp.e_store = c->at<float>(c->L.estore), cp.H = m.hidden;
   cp.planes = c->at<__nv_bfloat16>(c->L.cplanes);
-  if ((e = launch_k(raven_concat_kernel, dim3(d.max_rows), dim3(256), 0, c->stream, cp, c->use_pdl))) return e;
+  if ((e = launch_k(raven_concat_kernel, dim3(table_rows(c, tab)), dim3(256), 0, c->stream, cp, c->use_pdl))) return e;
   const int groups = col_groups(c, tab);
   if (tc >= 0) {
     if ((e = launch_tc_gemm(c, G_ADAPT, 0, tab, tc))) return e;
@@ -865,13 +916,15 @@ cudaError_t launch_coda(loopspec_ctx* c, const RowTable* tab_coda, int ng, int* 
   return launch_stack(c, tab_coda, ng, d.n_pre + c->m.n_recurrent, d.n_coda, n_launch, tc);
 }
 
-cudaError_t launch_lm_head(loopspec_ctx* c, const RowTable* tab, int ng) {
-  if (c->dg && tab != c->at<RowTable>(c->L.tab_pf) && tab != c->at<RowTable>(c->L.tab_pfc)) return launch_dg_lm(c, tab);
+// one_sum: the readout of a prompt - the row's sum of squares is a complete sum, not the partials of a down projection
+cudaError_t launch_lm_head(loopspec_ctx* c, const RowTable* tab, int ng, bool one_sum = false) {
+  if (c->dg && (one_sum || (tab != c->at<RowTable>(c->L.tab_pf) && tab != c->at<RowTable>(c->L.tab_pfc)))) return launch_dg_lm(c, tab, one_sum);
   const int groups = col_groups(c, tab);
   for (int g = 0; g < groups; ++g) {
     GemmParams gl = gemm_params(c, G_LM, 0, tab, g * GROUP_ROWS);
     gl.tl = tune_timeline(c), gl.tl_id = 120;
-    cudaError_t e = launch_gemm(c->m.weight_dtype, ng, EPI_LOGITS, gl, c->stream, c->use_pdl);
+    if (one_sum) gl.n_sq = 1;
+    cudaError_t e = launch_gemm(c->m.weight_dtype, ng, EPI_LOGITS, gl, c->stream, c->use_pdl && !one_sum);
     if (e) return e;
   }
   return cudaSuccess;
@@ -889,7 +942,9 @@ cudaError_t launch_select(loopspec_ctx* c, const RowTable* tab, int kinds_mask) 
   sp.top_k = c->filters ? c->s.top_k : 0, sp.top_p = c->filters ? c->s.top_p : 1.0f, sp.sel_flt = c->at<float4>(c->L.sel_flt);
   sp.staged = c->sel_staged;
   sp.tv_acc = (c->s.measure_tv && c->s.temperature > 0.f) ? c->at<double>(c->L.tv) : nullptr;
-  return launch_k(select_kernel, dim3(c->d.max_rows * SEL_CS), dim3(SEL_THREADS), c->sel_smem, c->stream, sp, c->use_pdl, SEL_CS);
+  // (a pass whose rows are drawn from p_R itself - a prompt's last position, vanilla decoding - reads out one row per sequence)
+  const int readouts = kinds_mask == 1 << RO_TARGET ? c->d.S : table_rows(c, tab);
+  return launch_k(select_kernel, dim3(readouts * SEL_CS), dim3(SEL_THREADS), c->sel_smem, c->stream, sp, c->use_pdl, SEL_CS);
 }
 
 ControlParams control_params(loopspec_ctx* c, int phases) {
@@ -984,6 +1039,152 @@ int check_device_error(loopspec_ctx* c) {
     return fail(c, LOOPSPEC_ETIMEOUT, "a bounded device-side wait ran out (%s)", e == ERR_WAIT ? "decode-pass GEMM" : "prefill GEMM or grid barrier");
   return fail(c, LOOPSPEC_ECAPACITY, "device scheduler reported %s",
               e == ERR_NODES ? "node/row table overflow" : e == ERR_CTX ? "max_ctx exceeded" : "speculative chain too deep");
+}
+
+// ---- a prompt on the wide kernels (prefill.cuh) --------------------------------------------------------------------
+template <int EPI>
+cudaError_t launch_pf_gemm_epi(loopspec_ctx* c, const CUtensorMap& w, int xi, const PfGemmParams& p) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  const int items = p.n_rp * p.n_tt * p.n_split;
+  cfg.gridDim = dim3(2 * std::min(c->n_sm / 2, items)), cfg.blockDim = dim3(PG_THREADS), cfg.dynamicSmemBytes = PG_SMEM, cfg.stream = c->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at, cfg.numAttrs = c->use_pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, pf_gemm_kernel<EPI>, w, c->pf_x1[xi], c->pf_x2[xi], p);
+}
+struct PfPass {  // rows of a pass: positions p0 .. p0 + n - 1 of sequence seq
+  int seq, p0, n;
+};
+// one GEMM of block `layer`; plane: KV plane the QKV projection writes
+cudaError_t launch_pf_gemm(loopspec_ctx* c, int which, int layer, const PfPass& ps, int plane) {
+  const loopspec_model& m = c->m;
+  const Derived& d = c->d;
+  PfGemmParams p;
+  memset(&p, 0, sizeof p);
+  const int Ns[6] = {d.Hq + 2 * d.Hkv, m.hidden, 2 * m.ffn, m.hidden, 0, m.hidden}, Ks[6] = {m.hidden, d.Hq, m.hidden, m.ffn, 0, 2 * m.hidden};
+  p.N = Ns[which], p.n_kb = (Ks[which] + TC_BK - 1) / TC_BK, p.n_tok = ps.n, p.n_tt = (ps.n + PG_TOK - 1) / PG_TOK;
+  p.n_rp = which == G_GU ? (m.ffn + 127) / 128 : (p.N + 255) / 256;
+  p.n_split = (which == G_QKV || which == G_GU) ? 1 : pf_splits(Ks[which]);
+  p.err = const_cast<int*>(c->host_flags_dev + HF_ERROR), p.err_code = ERR_WAIT_PF;
+  p.sumsq = c->at<float>(c->L.pf_sumsq), p.H = m.hidden, p.eps = m.rms_eps;
+  const CUtensorMap& w = which == G_ADAPT ? c->pf_wmaps[4 * d.NL] : c->pf_wmaps[4 * layer + which];
+  switch (which) {
+    case G_QKV:
+      p.qbuf = c->at<float>(c->L.pf_q);
+      p.kv = c->at<__nv_bfloat16>(c->L.kv) + (size_t)layer * c->kv_layer_stride() + (size_t)plane * c->kv_plane_stride();
+      p.kv_sel_stride = c->kv_sel_stride(), p.slots = d.slots, p.n_kv_heads = m.n_kv_heads, p.n_q_heads = m.n_q_heads, p.head_dim = m.head_dim;
+      p.seq = ps.seq, p.p0 = ps.p0, p.rope = c->at<float2>(c->L.rope);
+      return launch_pf_gemm_epi<PG_QKV>(c, w, 0, p);
+    case G_GU:
+      p.planes = c->at<__nv_bfloat16>(c->L.pf_s), p.F = m.ffn;
+      return launch_pf_gemm_epi<PG_SWIGLU>(c, w, 0, p);
+    default:
+      p.part = c->at<float>(c->L.pf_part), p.split_stride = (long long)ps.n * m.hidden;
+      return launch_pf_gemm_epi<PG_PART>(c, w, which == G_O ? 1 : which == G_DOWN ? 2 : 3, p);
+  }
+}
+cudaError_t launch_pf_reduce(loopspec_ctx* c, const PfPass& ps, int K, const float* hid_in, float* hid_out, const float* gain) {
+  PfReduceParams r;
+  memset(&r, 0, sizeof r);
+  r.part = c->at<float>(c->L.pf_part), r.n_split = pf_splits(K), r.split_stride = (long long)ps.n * c->m.hidden;
+  r.hid_in = hid_in, r.hid_out = hid_out, r.H = c->m.hidden, r.gain = gain;
+  r.planes = c->at<__nv_bfloat16>(c->L.pf_x), r.sumsq = c->at<float>(c->L.pf_sumsq);
+  return launch_k(pf_reduce_kernel, dim3(ps.n), dim3(256), 0, c->stream, r, c->use_pdl);
+}
+// the blocks [l0, l0 + count) on KV plane `plane`: the stream is read from `in` by the first residual and kept in `hid`;
+// next_gain: of the norm that reads the stream after the last block (null: nobody reads planes)
+cudaError_t launch_pf_stack(loopspec_ctx* c, const PfPass& ps, int l0, int count, int plane, const float* in, float* hid, const float* next_gain) {
+  const loopspec_model& m = c->m;
+  const Derived& d = c->d;
+  cudaError_t e;
+  PfAttnParams a;
+  memset(&a, 0, sizeof a);
+  a.qbuf = c->at<float>(c->L.pf_q), a.aplanes = c->at<__nv_bfloat16>(c->L.pf_a);
+  a.n_rows = ps.n, a.p0 = ps.p0, a.slots = d.slots, a.n_kv_heads = m.n_kv_heads, a.n_q_heads = m.n_q_heads, a.scale = 1.0f / sqrtf((float)m.head_dim);
+  const dim3 agrid(m.n_q_heads * ((ps.n + PFA_ROWS - 1) / PFA_ROWS));
+  for (int l = l0; l < l0 + count; ++l) {
+    const void* const* lp = &c->layers[6 * l];
+    if ((e = launch_pf_gemm(c, G_QKV, l, ps, plane))) return e;
+    a.k = c->at<__nv_bfloat16>(c->L.kv) + (size_t)l * c->kv_layer_stride() + (size_t)plane * c->kv_plane_stride() +
+          (size_t)ps.seq * m.n_kv_heads * d.slots * m.head_dim;
+    a.v = a.k + c->kv_sel_stride();
+    e = m.head_dim == 128 ? launch_k(pf_attn_kernel<128>, agrid, dim3(PFA_THREADS), (size_t)PfaCfg<128>::SMEM_BYTES, c->stream, a, c->use_pdl)
+                          : launch_k(pf_attn_kernel<64>, agrid, dim3(PFA_THREADS), (size_t)PfaCfg<64>::SMEM_BYTES, c->stream, a, c->use_pdl);
+    if (e) return e;
+    if ((e = launch_pf_gemm(c, G_O, l, ps, plane))) return e;
+    if ((e = launch_pf_reduce(c, ps, d.Hq, l == l0 ? in : hid, hid, static_cast<const float*>(lp[3])))) return e;
+    if ((e = launch_pf_gemm(c, G_GU, l, ps, plane))) return e;
+    if ((e = launch_pf_gemm(c, G_DOWN, l, ps, plane))) return e;
+    const float* gain = l + 1 < l0 + count ? static_cast<const float*>(c->layers[6 * (l + 1)]) : next_gain;
+    if ((e = launch_pf_reduce(c, ps, m.ffn, hid, hid, gain))) return e;
+  }
+  return cudaSuccess;
+}
+cudaError_t launch_pf_prep(loopspec_ctx* c, const PfPass& ps, bool embed, const float* gain) {
+  PfPrepParams q;
+  memset(&q, 0, sizeof q);
+  if (embed) q.prompt = c->at<int>(c->L.prompt) + ps.p0, q.embed = static_cast<const __nv_bfloat16*>(c->embed);
+  q.src = q.hid = c->at<float>(c->L.pf_hid), q.H = c->m.hidden, q.gain = gain;
+  q.planes = c->at<__nv_bfloat16>(c->L.pf_x), q.sumsq = c->at<float>(c->L.pf_sumsq);
+  return launch_k(pf_prep_kernel, dim3(ps.n), dim3(256), 0, c->stream, q, c->use_pdl);
+}
+// all recurrences of one pass; *last: the state the readout of the pass's rows starts from
+cudaError_t launch_pf_pass(loopspec_ctx* c, const PfPass& ps, const float** last) {
+  const loopspec_model& m = c->m;
+  const Derived& d = c->d;
+  float* hid = c->at<float>(c->L.pf_hid);
+  auto norm1 = [&](int l) { return static_cast<const float*>(c->layers[6 * l]); };
+  cudaError_t e;
+  *last = hid;
+  if (!d.raven) {
+    if ((e = launch_pf_prep(c, ps, true, norm1(0)))) return e;
+    for (int r = 1; r <= m.R; ++r)
+      if ((e = launch_pf_stack(c, ps, 0, m.n_recurrent, r - 1, hid, hid, r < m.R ? norm1(0) : nullptr))) return e;
+    return cudaSuccess;
+  }
+  if ((e = launch_pf_prep(c, ps, true, d.n_pre ? norm1(0) : nullptr))) return e;
+  if (d.n_pre && (e = launch_pf_stack(c, ps, 0, d.n_pre, 0, hid, hid, nullptr))) return e;
+  for (int r = 1; r <= m.R; ++r) {
+    PfConcatParams cp;
+    cp.hid = hid, cp.e = c->at<float>(c->L.pf_e), cp.H = m.hidden, cp.first = r == 1, cp.planes = c->at<__nv_bfloat16>(c->L.pf_c);
+    if ((e = launch_k(pf_concat_kernel, dim3(ps.n), dim3(256), 0, c->stream, cp, c->use_pdl))) return e;
+    if ((e = launch_pf_gemm(c, G_ADAPT, 0, ps, 0))) return e;
+    if ((e = launch_pf_reduce(c, ps, 2 * m.hidden, nullptr, hid, norm1(d.n_pre)))) return e;
+    if ((e = launch_pf_stack(c, ps, d.n_pre, m.n_recurrent, r - 1, hid, hid, nullptr))) return e;
+    int cls = 0;  // the prompt fills the coda cache of every readout depth (App. B)
+    for (int k = 0; k < d.n_classes; ++k)
+      if (d.class_depth[k] == r && cls == 0) cls = k + 1;
+    if (r == m.R) cls = d.n_classes;
+    if (d.n_coda > 0 && cls > 0) {  // on a copy of the states
+      float* hid2 = c->at<float>(c->L.pf_hid2);
+      const int l0 = d.n_pre + m.n_recurrent;
+      if ((e = launch_pf_prep(c, ps, false, norm1(l0)))) return e;
+      if ((e = launch_pf_stack(c, ps, l0, d.n_coda, cls - 1, hid, hid2, nullptr))) return e;
+      *last = hid2;
+    }
+  }
+  return cudaSuccess;
+}
+// every pass of a prompt (of about equal sizes, whole token tiles), then the row table and planes of its last position for
+// the readout
+cudaError_t launch_pf_prompt(loopspec_ctx* c, int seq, int n) {
+  const int P = c->d.pf_rows, n_pass = (n + P - 1) / P;
+  const int per = std::min(P, ((n + n_pass - 1) / n_pass + PG_TOK - 1) / PG_TOK * PG_TOK);
+  cudaError_t e;
+  const float* last = nullptr;
+  int cnt = 0;
+  for (int p0 = 0; p0 < n; p0 += cnt) {
+    cnt = std::min(per, n - p0);
+    if ((e = launch_pf_pass(c, PfPass{seq, p0, cnt}, &last))) return e;
+  }
+  PfReadoutParams q;
+  memset(&q, 0, sizeof q);
+  q.tab = c->at<RowTable>(c->L.tab_pf), q.row = last + (size_t)(cnt - 1) * c->m.hidden, q.H = c->m.hidden, q.seq = seq, q.pos = n - 1, q.R = c->m.R;
+  q.hid_idx = c->d.S * c->d.NB, q.logit_idx = c->d.p_logit_base + seq, q.gain = c->final_norm;
+  q.planes = c->at<__nv_bfloat16>(c->L.xplanes), q.sumsq = c->at<float>(c->L.sumsq);
+  return launch_k(pf_readout_kernel, dim3(1), dim3(256), 0, c->stream, q, c->use_pdl);
 }
 
 int capture(loopspec_ctx* c, cudaGraphExec_t* out, bool vanilla) {
@@ -1245,6 +1446,29 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
     if (!ok) (void)cudaGetLastError();
     for (int k = 0; k < 2; ++k) c->tc[k].on = ok && want[k];
   }
+  if (d.pf_rows > 0 && encode_tiled_fn()) {  // prompts on the wide kernels
+    const int Ns[4] = {d.Hq + 2 * d.Hkv, m->hidden, 2 * m->ffn, m->hidden}, Kw[4] = {m->hidden, d.Hq, m->hidden, m->ffn}, w_idx[4] = {1, 2, 4, 5};
+    bool ok = true;
+    c->pf_wmaps.resize((size_t)4 * d.NL + 1);
+    for (int l = 0; l < d.NL && ok; ++l)
+      for (int i = 0; i < 4 && ok; ++i)
+        ok = i == 2 ? make_map_gateup(&c->pf_wmaps[4 * l + i], c->layers[6 * l + w_idx[i]], m->ffn, Kw[i])
+                    : make_map_bf16(&c->pf_wmaps[4 * l + i], c->layers[6 * l + w_idx[i]], Ns[i], Kw[i], TC_BM);
+    if (d.raven) ok = ok && make_map_bf16(&c->pf_wmaps[4 * d.NL], c->adapter, m->hidden, 2 * m->hidden, TC_BM);
+    const size_t x_off[4] = {L.pf_x, L.pf_a, L.pf_s, L.pf_c};
+    const int x_k[4] = {m->hidden, d.Hq, m->ffn, 2 * m->hidden};
+    for (int i = 0; i < (d.raven ? 4 : 3) && ok; ++i)
+      ok = make_map_pf_planes(&c->pf_x1[i], c->ws + x_off[i], x_k[i], d.pf_rows, PG_TOK) &&
+           make_map_pf_planes(&c->pf_x2[i], c->ws + x_off[i], x_k[i], d.pf_rows, PG_TOK / 2);
+    ok = ok && cudaFuncSetAttribute(pf_gemm_kernel<PG_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, PG_SMEM) == cudaSuccess &&
+         cudaFuncSetAttribute(pf_gemm_kernel<PG_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, PG_SMEM) == cudaSuccess &&
+         cudaFuncSetAttribute(pf_gemm_kernel<PG_PART>, cudaFuncAttributeMaxDynamicSharedMemorySize, PG_SMEM) == cudaSuccess &&
+         (m->head_dim == 128
+              ? cudaFuncSetAttribute(pf_attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, PfaCfg<128>::SMEM_BYTES)
+              : cudaFuncSetAttribute(pf_attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, PfaCfg<64>::SMEM_BYTES)) == cudaSuccess;
+    if (!ok) (void)cudaGetLastError();
+    c->pf = ok;
+  }
   // readout GEMM of the decode passes on the tcgen05 kernel: bf16 weights whose rows are 16-byte multiples (TMA strides)
   if (m->weight_dtype == 1 && encode_tiled_fn() && m->hidden % 8 == 0) {
     const Derived& dd = c->d;
@@ -1378,7 +1602,11 @@ int loopspec_prefill(loopspec_ctx* c, int32_t seq, const int32_t* prompt_ids, in
   CU(c, cudaMemcpyAsync(c->ws + c->L.prompt, c->pin_ids, (size_t)n * 4, cudaMemcpyHostToDevice, c->stream));
   RowTable* tab = c->at<RowTable>(c->L.tab_pf);
   const int chunk = c->d.max_rows_pf;
-  for (int p0 = 0; p0 < n; p0 += chunk) {
+  // A prompt that fits one narrow pass of 64 columns streams the weights faster there (more CTAs per GEMM; 1.4B shape: 16 / 33
+  // tokens 6.5 / 7.2 ms against 8.4 / 9.1 ms on the wide kernels; from 65 tokens on it would take two: 77 tokens 13.9 ms against 11.3)
+  const bool wide = c->pf && n > chunk;
+  if (wide) CU(c, launch_pf_prompt(c, seq, n));
+  for (int p0 = 0; p0 < n && !wide; p0 += chunk) {
     int cnt = std::min(chunk, n - p0);
     for (int r = 1; r <= c->m.R; ++r) {
       PrefillParams pp;
@@ -1399,8 +1627,8 @@ int loopspec_prefill(loopspec_ctx* c, int32_t seq, const int32_t* prompt_ids, in
       if (pp.coda_class > 0) CU(c, launch_coda(c, pp.tab_coda, c->ng_pf, nullptr, c->tc[0].on ? 0 : -1));
     }
   }
-  if (c->d.raven && c->d.n_coda > 0) tab = c->at<RowTable>(c->L.tab_pfc);  // its last state: last chunk, depth R
-  CU(c, launch_lm_head(c, tab, c->ng_pf));
+  if (!wide && c->d.raven && c->d.n_coda > 0) tab = c->at<RowTable>(c->L.tab_pfc);  // its last state: last chunk, depth R
+  CU(c, launch_lm_head(c, tab, c->ng_pf, wide));
   CU(c, launch_select(c, tab, 1 << RO_TARGET));
   PrefillFinishParams fp;
   fp.tab = c->at<RowTable>(c->L.tab_pf), fp.nodes = c->nodes(), fp.seqs = c->seqs(), fp.seq = seq, fp.NB = c->d.NB, fp.n_prompt = n, fp.n_target = 0;

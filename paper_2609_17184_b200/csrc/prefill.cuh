@@ -1,0 +1,680 @@
+// Prompt passes of hundreds of positions (Algorithm 1, lines before the main loop): the prompt is the one place where the
+// shared blocks see many token columns at once, so its GEMMs are bound by the tensor cores (three exact bf16 planes per
+// fp32 activation) and not by the weight stream.  A pass carries up to PF_MAX_ROWS consecutive positions of one sequence at
+// one recurrence; its rows need no row table (row i = position p0 + i, KV slot = position).
+//
+//   pf_prep_kernel     embedding rows (or states) -> fp32 stream, planes of x * gain, sum of squares
+//   pf_concat_kernel   planes of [H; e] for the adapter of a Raven-style model
+//   pf_gemm_kernel     QKV (+ 1/rms, RoPE, KV write), gate/up (+ 1/rms, SwiGLU, planes), O / down / adapter (k-split sums)
+//   pf_reduce_kernel   k-split sums in split order + residual + planes of x * next gain + sum of squares
+//   pf_attn_kernel     causal attention of the pass's rows over the cached keys and values
+//
+// A row's arithmetic is a function of its own operands and of the model's shapes: k-splits depend on the matrix alone, every
+// accumulation chain runs over the whole k-range of its split, so results do not depend on how the prompt is cut into passes.
+//
+// Prompt of the 1.4B shape, wall clock of loopspec_prefill: 512 tokens 100 ms (passes of 32 rows; 61 ms with 64) -> 21.5 ms, 1024
+// tokens 132 -> 35 ms, 3001 tokens 716 -> 128 ms; three-plane products at the measured GEMM peak would take 9 / 19 / 56 ms.
+#pragma once
+#include <cuda.h>
+
+#include "attention.cuh"
+#include "common.cuh"
+#include "gemm.cuh"
+#include "gemm_dec.cuh"
+#include "linear_tc.cuh"
+
+namespace ls {
+
+constexpr int PF_MAX_ROWS = 1024;  // positions of one pass: at 1024 the persistent grid's last wave costs 5 to 14 % of a GEMM of
+                                   // the 1.4B shape (21 to 35 % at 512), and a pass's activations still fit the L2
+constexpr int PF_MAX_SPLIT = 4;
+// k-splits of O, down and the adapter (few row blocks: 8 pairs at 2048 rows, on 74 pairs of CTAs): a function of K alone, at
+// least eight 64-wide k-blocks each
+__host__ __device__ inline int pf_splits(int K) {
+  const int n = (K + 63) / 64 / 8;
+  return n < 1 ? 1 : n > PF_MAX_SPLIT ? PF_MAX_SPLIT : n;
+}
+
+// ---- states -> planes ----------------------------------------------------------------------------------------------
+struct PfPrepParams {
+  const int* prompt;          // ids of the pass's positions (null: the rows' states are read from src)
+  const __nv_bfloat16* embed; // [V][H]
+  const float* src;           // [row][H]
+  float* hid;                 // [row][H] written when the rows come from the embedding
+  int H;
+  const float* gain;          // null: no planes (the rows are only embedded)
+  __nv_bfloat16* planes;      // [row][3][H]
+  float* sumsq;               // [row]
+};
+// sum over the CTA (warp partials added in warp order), valid in thread 0
+__device__ __forceinline__ float pf_block_sum(float v, float (&s_part)[8]) {
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = v;
+  __syncthreads();
+  float t = 0.f;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < 8; ++w) t += s_part[w];
+  return t;
+}
+__device__ __forceinline__ float pf_square_sum(float4 v) { return (v.x * v.x + v.y * v.y) + (v.z * v.z + v.w * v.w); }
+__device__ __forceinline__ void pf_store_planes(__nv_bfloat16* row_planes, int H, int k, float4 v, const float* gain) {
+  const float4 g = *reinterpret_cast<const float4*>(gain + k);
+  store_split4(row_planes, H, k, make_float4(v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w));
+}
+// one CTA per row, four elements per thread and step (H is a multiple of 128)
+__global__ void __launch_bounds__(256) pf_prep_kernel(const __grid_constant__ PfPrepParams p) {
+  __shared__ float s_part[8];
+  pdl_launch_dependents();
+  pdl_wait();
+  const int row = blockIdx.x;
+  float ss = 0.f;
+  for (int k = threadIdx.x * 4; k < p.H; k += 1024) {
+    float4 v;
+    if (p.prompt) {
+      const uint2 w = *reinterpret_cast<const uint2*>(p.embed + (size_t)p.prompt[row] * p.H + k);
+      v = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
+      *reinterpret_cast<float4*>(p.hid + (size_t)row * p.H + k) = v;
+    } else {
+      v = *reinterpret_cast<const float4*>(p.src + (size_t)row * p.H + k);
+    }
+    if (!p.gain) continue;
+    ss += pf_square_sum(v);
+    pf_store_planes(p.planes + (size_t)row * 3 * p.H, p.H, k, v, p.gain);
+  }
+  if (!p.gain) return;
+  ss = pf_block_sum(ss, s_part);
+  if (threadIdx.x == 0) p.sumsq[row] = ss;
+}
+
+struct PfConcatParams {
+  const float* hid;        // [row][H]
+  float* e;                // [row][H] prelude outputs (written when first)
+  int H, first;
+  __nv_bfloat16* planes;   // [row][3][2 H]
+};
+__global__ void __launch_bounds__(256) pf_concat_kernel(const __grid_constant__ PfConcatParams p) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int row = blockIdx.x;
+  __nv_bfloat16* dst = p.planes + (size_t)row * 6 * p.H;
+  for (int k = threadIdx.x * 4; k < p.H; k += 1024) {
+    const float4 h = *reinterpret_cast<const float4*>(p.hid + (size_t)row * p.H + k);
+    float4* ep = reinterpret_cast<float4*>(p.e + (size_t)row * p.H + k);
+    const float4 ev = p.first ? h : *ep;
+    if (p.first) *ep = h;
+    store_split4(dst, 2 * p.H, k, h);
+    store_split4(dst, 2 * p.H, p.H + k, ev);
+  }
+}
+
+// ---- the GEMM ------------------------------------------------------------------------------------------------------
+// y[token][n] = sum_k x[token][k] W[n][k] for a whole pass.  Bound by the tensor cores: 3 x 2 x rows x N x K operations, so
+// everything here serves to keep tcgen05 fed.  A pair of CTAs (cluster of two, cta_group::2) owns 256 weight rows x 128 token
+// columns: each CTA holds its 128 weight rows and half of the columns' operand, so a k-block of 64 costs an SM 40 KB of L2
+// reads for 768 cycles of MMA (52 B per cycle; one CTA alone with 128 x 128 would need 83).  Per 16-wide k-step two MMAs:
+// [hi | mid] as 256 columns (CTA 0 holds the hi rows, CTA 1 the mid rows of all 128 tokens) and lo as 128 columns that
+// accumulate onto mid's - two chains, hi and (mid + lo), folded when the accumulator is read.  256 TMEM columns per
+// accumulator, two accumulators: the epilogue of a tile runs under the main loop of the next (persistent CTAs, tiles dealt
+// round robin, the token tiles of one weight block next to each other so that its weights come from HBM once).
+constexpr int PG_THREADS = 256;
+constexpr int PG_TOK = 128;                        // token columns of a tile
+constexpr int PG_A_BYTES = 128 * TC_BK * 2;        // a CTA's weight rows of a stage
+constexpr int PG_B1_BYTES = PG_TOK * TC_BK * 2;    // hi (rank 0) or mid (rank 1) of all tokens
+constexpr int PG_B2_BYTES = PG_TOK / 2 * TC_BK * 2;  // lo of half the tokens
+constexpr int PG_STAGE_BYTES = PG_A_BYTES + PG_B1_BYTES + PG_B2_BYTES;
+constexpr int PG_STAGES = 5;
+constexpr int PG_ST_LD = 132;                      // floats per token of the epilogue's exchange buffer
+constexpr int PG_ST_TOK = 16;                      // tokens exchanged at a time
+constexpr int PG_SMEM = 1024 + PG_STAGES * PG_STAGE_BYTES + 2 * PG_ST_TOK * PG_ST_LD * 4;
+enum { PG_QKV = 0, PG_SWIGLU = 1, PG_PART = 2 };
+
+struct PfGemmParams {
+  int n_rp, n_tt, n_split;  // pairs of 128-row weight blocks, token tiles, k-splits
+  int n_kb;                 // 64-wide k-blocks of the matrix
+  int n_tok, N;             // live rows of the pass, weight rows
+  int* err;
+  int err_code;
+  const float* sumsq;       // [token]: columns are scaled by 1/sqrt(sumsq / H + eps)
+  int H;
+  float eps;
+  float* part;              // PART: [split][token][N]
+  long long split_stride;
+  float* qbuf;              // QKV: [token][Hq]
+  __nv_bfloat16* kv;        // QKV: this layer's and recurrence's plane [2][S][n_kv][slots][d]
+  long long kv_sel_stride;
+  int slots, n_kv_heads, n_q_heads, head_dim, seq, p0;
+  const float2* rope;
+  __nv_bfloat16* planes;    // SWIGLU: [token][3][F]
+  int F;
+};
+
+__device__ __forceinline__ void pg_tma_2d(unsigned dst, const CUtensorMap* map, unsigned bar, int x, int y) {
+  asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
+               "l"(reinterpret_cast<unsigned long long>(map)), "r"(bar), "r"(x), "r"(y)
+               : "memory");
+}
+__device__ __forceinline__ void pg_tma_3d(unsigned dst, const CUtensorMap* map, unsigned bar, int x, int y, int z) {
+  asm volatile("cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
+               "l"(reinterpret_cast<unsigned long long>(map)), "r"(bar), "r"(x), "r"(y), "r"(z)
+               : "memory");
+}
+__device__ __forceinline__ void pg_mma(unsigned d_tmem, unsigned long long adesc, unsigned long long bdesc, unsigned idesc, unsigned accumulate) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+               "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+               : "memory");
+}
+// arrives on the barrier at this offset in both CTAs of the pair once the MMAs issued so far are done
+__device__ __forceinline__ void pg_commit(unsigned bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"((unsigned short)3)
+               : "memory");
+}
+__device__ __forceinline__ void pg_cluster_sync() { asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory"); }
+__device__ __forceinline__ void pg_team_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }  // the epilogue's four warps
+__device__ __forceinline__ void pg_ld16(unsigned (&w)[16], unsigned taddr) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+               : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]), "=r"(w[8]), "=r"(w[9]),
+                 "=r"(w[10]), "=r"(w[11]), "=r"(w[12]), "=r"(w[13]), "=r"(w[14]), "=r"(w[15])
+               : "r"(taddr)
+               : "memory");
+}
+
+template <int EPI>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
+    pf_gemm_kernel(const __grid_constant__ CUtensorMap map_w,   // weights: box 64 k x 128 rows; gate/up: (k, f, gate | up), box 64 x 64 x 2
+                   const __grid_constant__ CUtensorMap map_x1,  // planes as (k, token, plane): box 64 x 128 x 1
+                   const __grid_constant__ CUtensorMap map_x2,  // ... box 64 x 64 x 1
+                   const __grid_constant__ PfGemmParams p) {
+  extern __shared__ unsigned char pg_smem_raw[];
+  __shared__ __align__(8) unsigned long long s_full[PG_STAGES], s_empty[PG_STAGES], s_accf[2], s_acce[2];
+  __shared__ unsigned s_tmem;
+  __shared__ int s_fail;
+  __shared__ float s_rstd[PG_TOK];
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const unsigned rank = blockIdx.x & 1u;  // the pair's leader (rank 0) issues the MMAs and owns the full barriers
+  const int cid = blockIdx.x >> 1, n_cl = gridDim.x >> 1;
+  const unsigned base = (tc_smem_u32(pg_smem_raw) + 1023u) & ~1023u;
+  float* st = reinterpret_cast<float*>(pg_smem_raw + (base - tc_smem_u32(pg_smem_raw)) + PG_STAGES * PG_STAGE_BYTES);
+  const int n_items = p.n_rp * p.n_tt * p.n_split;
+
+  pdl_launch_dependents();
+  if (tid == 0) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<unsigned long long>(&map_w)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<unsigned long long>(&map_x1)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<unsigned long long>(&map_x2)) : "memory");
+    for (int s = 0; s < PG_STAGES; ++s) tc_mbar_init(tc_smem_u32(&s_full[s]), 1), tc_mbar_init(tc_smem_u32(&s_empty[s]), 1);
+    for (int b = 0; b < 2; ++b) tc_mbar_init(tc_smem_u32(&s_accf[b]), 1), tc_mbar_init(tc_smem_u32(&s_acce[b]), 8);  // four warps of each CTA
+    s_fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  __syncthreads();
+  // Both CTAs run and their barriers exist.  The allocation below is collective over the pair, so neither CTA may ask for it
+  // before the other is known to be there (asked for at once, it was seen - rarely - never to return).
+  pg_cluster_sync();
+  if (warp == 2)
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem_u32(&s_tmem)), "r"(512u) : "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const unsigned tmem = s_tmem;
+
+  // item -> (weight block pair, token tile, split): token tiles vary fastest
+  struct Item {
+    int rp, tt, sp, kb_lo, n_kb, cols;  // cols: MMA columns of the tile (its live tokens rounded up to 32)
+  };
+  auto item_of = [&](int it) {
+    Item r;
+    r.tt = it % p.n_tt;
+    const int q = it / p.n_tt;
+    r.rp = q % p.n_rp, r.sp = q / p.n_rp;
+    r.kb_lo = (int)((long long)p.n_kb * r.sp / p.n_split);
+    r.n_kb = (int)((long long)p.n_kb * (r.sp + 1) / p.n_split) - r.kb_lo;
+    const int live = min(PG_TOK, p.n_tok - r.tt * PG_TOK);
+    r.cols = (live + 31) & ~31;
+    return r;
+  };
+  bool ok = true;
+  auto wait = [&](unsigned long long* bar, unsigned parity) {  // bounded; after the first failure every later wait gives up at once
+    if (!dg_wait(tc_smem_u32(bar), parity, ok ? TC_WAIT_CYCLES : 2000LL)) ok = false;
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---- producer: this CTA's weight rows and its share of the planes; both CTAs complete on the leader's barrier --------
+      auto load_w = [&](const Item& r, int kb, int s) {
+        const unsigned bar = tc_smem_u32(&s_full[s]) & 0xFEFFFFFFu, a = base + s * PG_STAGE_BYTES;
+        if (rank == 0) tc_mbar_expect_tx(tc_smem_u32(&s_full[s]), 2u * PG_STAGE_BYTES);
+        if (EPI == PG_SWIGLU) pg_tma_3d(a, &map_w, bar, kb * TC_BK, (2 * r.rp + (int)rank) * 64, 0);
+        else pg_tma_2d(a, &map_w, bar, kb * TC_BK, (2 * r.rp + (int)rank) * 128);
+      };
+      auto load_x = [&](const Item& r, int kb, int s) {
+        const unsigned bar = tc_smem_u32(&s_full[s]) & 0xFEFFFFFFu, b = base + s * PG_STAGE_BYTES + PG_A_BYTES;
+        const int row = r.tt * PG_TOK;
+        pg_tma_3d(b, &map_x1, bar, kb * TC_BK, row, (int)rank);
+        pg_tma_3d(b + PG_B1_BYTES, &map_x2, bar, kb * TC_BK, row + (int)rank * (r.cols >> 1), 2);
+      };
+      // the first ring-full of weights is requested ahead of the predecessor's completion
+      int pre = 0;
+      if (cid < n_items) {
+        const Item r = item_of(cid);
+        for (; pre < min(PG_STAGES, r.n_kb); ++pre) load_w(r, r.kb_lo + pre, pre);
+      }
+      pdl_wait();
+      int s = 0, u = 0;
+      unsigned par = 1;  // (the first use of a stage finds it free)
+      for (int it = cid; it < n_items; it += n_cl) {
+        const Item r = item_of(it);
+        for (int kb = 0; kb < r.n_kb; ++kb, ++u) {
+          if (u >= PG_STAGES) wait(&s_empty[s], par);
+          if (u >= pre) load_w(r, r.kb_lo + kb, s);
+          load_x(r, r.kb_lo + kb, s);
+          if (++s == PG_STAGES) s = 0, par ^= 1u;
+        }
+      }
+      for (int i = 0; i < min(u, PG_STAGES); ++i) {  // the leader's last arrivals on this CTA's barriers have landed before it may exit
+        if (u < PG_STAGES) wait(&s_empty[i], 0);
+        else {
+          wait(&s_empty[s], par);
+          if (++s == PG_STAGES) s = 0, par ^= 1u;
+        }
+      }
+      if (!ok) s_fail = 1, *p.err = p.err_code;
+    }
+  } else if (warp == 1) {
+    if (lane == 0 && rank == 0) {
+      // ---- MMA issuer of the pair --------------------------------------------------------------------------------------
+      const unsigned long long desc0 = tc_smem_desc(0);
+      int s = 0, n = 0;
+      unsigned par = 0;
+      for (int it = cid; it < n_items; it += n_cl, ++n) {
+        const Item r = item_of(it);
+        const int buf = n & 1, uses = n >> 1;
+        if (uses > 0) wait(&s_acce[buf], (uses - 1) & 1);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const unsigned d = tmem + buf * 256;
+        const unsigned idesc1 = tc_idesc(256, 2 * r.cols), idesc2 = tc_idesc(256, r.cols);
+        for (int kb = 0; kb < r.n_kb; ++kb) {
+          wait(&s_full[s], par);
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const unsigned a = base + s * PG_STAGE_BYTES, b1 = a + PG_A_BYTES, b2 = b1 + PG_B1_BYTES;
+          const unsigned long long ad = desc0 | ((a >> 4) & 0x3FFF), bd1 = desc0 | ((b1 >> 4) & 0x3FFF), bd2 = desc0 | ((b2 >> 4) & 0x3FFF);
+#pragma unroll
+          for (int ks = 0; ks < TC_BK / 16; ++ks) {
+            pg_mma(d, ad + 2 * ks, bd1 + 2 * ks, idesc1, (kb | ks) != 0);
+            pg_mma(d + r.cols, ad + 2 * ks, bd2 + 2 * ks, idesc2, 1);
+          }
+          pg_commit(tc_smem_u32(&s_empty[s]));
+          if (++s == PG_STAGES) s = 0, par ^= 1u;
+        }
+        pg_commit(tc_smem_u32(&s_accf[buf]));
+      }
+      if (!ok) s_fail = 1, *p.err = p.err_code;
+    }
+  } else if (warp >= 4) {
+    // ---- epilogue: thread = weight row of this CTA's block --------------------------------------------------------------
+    pdl_wait();
+    const int j = tid - 128, ew = warp - 4;
+    const unsigned lane_off = (unsigned)(ew * 32) << 16;
+    int n = 0, sb = 0;
+    for (int it = cid; it < n_items; it += n_cl, ++n) {
+      const Item r = item_of(it);
+      const int buf = n & 1, uses = n >> 1;
+      const int t0 = r.tt * PG_TOK, live = min(PG_TOK, p.n_tok - t0);
+      const int n0 = (2 * r.rp + (int)rank) * (EPI == PG_SWIGLU ? 64 : 128);
+      if (EPI != PG_PART) {
+        pg_team_sync();  // the previous tile's readers of s_rstd are done
+        if (j < live) s_rstd[j] = 1.0f / sqrtf(p.sumsq[t0 + j] / (float)p.H + p.eps);
+      }
+      wait(&s_accf[buf], uses & 1);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      for (int c0 = 0; c0 < live; c0 += PG_ST_TOK) {
+        unsigned hi[16], ml[16];
+        pg_ld16(hi, tmem + lane_off + buf * 256 + c0);
+        pg_ld16(ml, tmem + lane_off + buf * 256 + r.cols + c0);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (EPI == PG_PART) {
+          if (n0 + j < p.N) {
+            float* out = p.part + (size_t)r.sp * p.split_stride + (size_t)(t0 + c0) * p.N + n0 + j;
+#pragma unroll
+            for (int c = 0; c < 16; ++c)
+              if (c0 + c < live) out[(size_t)c * p.N] = __uint_as_float(hi[c]) + __uint_as_float(ml[c]);
+          }
+          continue;
+        }
+        float* sx = st + sb * (PG_ST_TOK * PG_ST_LD);
+        sb ^= 1;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) sx[c * PG_ST_LD + j] = __uint_as_float(hi[c]) + __uint_as_float(ml[c]);
+        pg_team_sync();  // (two buffers: the readers of the one before are past their own barrier by the time it is written again)
+        if (EPI == PG_SWIGLU) {  // two neighbouring features, four tokens per thread
+          const int f2 = 2 * lane, f = n0 + f2;
+          if (f < p.F) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const int c = ew * 4 + q;
+              if (c0 + c >= live) break;
+              const float rs = s_rstd[c0 + c];
+              const float2 gt = *reinterpret_cast<const float2*>(sx + c * PG_ST_LD + f2), up = *reinterpret_cast<const float2*>(sx + c * PG_ST_LD + 64 + f2);
+              const float g0 = gt.x * rs, g1 = gt.y * rs;
+              store_split2(p.planes + (size_t)(t0 + c0 + c) * 3 * p.F, p.F, f, g0 / (1.0f + expf(-g0)) * (up.x * rs), g1 / (1.0f + expf(-g1)) * (up.y * rs));
+            }
+          }
+        } else {  // QKV: rotary pairs, eight tokens per thread
+          const int d = p.head_dim, hd2 = d >> 1, Hq = p.n_q_heads * d, Hk = p.n_kv_heads * d;
+          const int region = n0 < Hq ? 0 : (n0 < Hq + Hk ? 1 : 2);
+          const int rbase = region == 0 ? 0 : (region == 1 ? Hq : Hq + Hk);
+          const int pj = j & 63, hh = pj / hd2, i = pj - hh * hd2, head = (n0 - rbase) / d + hh;
+          if (n0 < p.N) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const int c = (j >> 6) * 8 + q;
+              if (c0 + c >= live) break;
+              const float rs = s_rstd[c0 + c];
+              const float x1 = sx[c * PG_ST_LD + hh * d + i] * rs, x2 = sx[c * PG_ST_LD + hh * d + i + hd2] * rs;
+              float y1 = x1, y2 = x2;
+              const int pos = p.p0 + t0 + c0 + c;
+              if (region < 2) {
+                const float2 cs = p.rope[(size_t)pos * hd2 + i];
+                y1 = x1 * cs.x - x2 * cs.y;
+                y2 = x2 * cs.x + x1 * cs.y;
+              }
+              if (region == 0) {
+                float* qd = p.qbuf + (size_t)(t0 + c0 + c) * Hq + head * d + i;
+                qd[0] = y1, qd[hd2] = y2;
+              } else {
+                __nv_bfloat16* dst = p.kv + (size_t)(region - 1) * p.kv_sel_stride + ((size_t)(p.seq * p.n_kv_heads + head) * p.slots + pos) * d + i;
+                dst[0] = __float2bfloat16_rn(y1), dst[hd2] = __float2bfloat16_rn(y2);
+              }
+            }
+          }
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) dg_arrive_cluster(dg_mapa(tc_smem_u32(&s_acce[buf]), 0));  // the accumulator may be overwritten
+    }
+    if (!ok && lane == 0) s_fail = 1, *p.err = p.err_code;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (tid == 0 && s_fail) {  // a wait gave up: copies may still be in flight; give them a bounded time before the memory goes
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000LL) {
+    }
+  }
+  __syncthreads();
+  pg_cluster_sync();  // the partner still reads this CTA's memory until here
+  if (warp == 2) {
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+  }
+}
+
+// ---- k-split sums + residual + planes of the next consumer's input ------------------------------------------------------
+struct PfReduceParams {
+  const float* part;       // [split][token][H]
+  int n_split;
+  long long split_stride;
+  const float* hid_in;     // null: the sums replace the stream (the adapter of a Raven-style model)
+  float* hid_out;          // [token][H]
+  int H;
+  const float* gain;       // of the norm that reads the stream next (null: nobody reads planes)
+  __nv_bfloat16* planes;
+  float* sumsq;            // [token]
+};
+// Bound by its bytes (per row: n_split + 2 fp32 rows and three bf16 planes, mostly in the L2): one CTA per row, 16-byte
+// accesses, every load of a step in flight at once.
+__global__ void __launch_bounds__(256) pf_reduce_kernel(const __grid_constant__ PfReduceParams p) {
+  __shared__ float s_part[8];
+  pdl_launch_dependents();
+  pdl_wait();
+  const int row = blockIdx.x;
+  float ss = 0.f;
+  for (int k = threadIdx.x * 4; k < p.H; k += 1024) {
+    const size_t at = (size_t)row * p.H + k;
+    float4 t[PF_MAX_SPLIT];
+#pragma unroll
+    for (int s = 0; s < PF_MAX_SPLIT; ++s)
+      if (s < p.n_split) t[s] = __ldcg(reinterpret_cast<const float4*>(p.part + (size_t)s * p.split_stride + at));
+    float4 v = p.hid_in ? *reinterpret_cast<const float4*>(p.hid_in + at) : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 y = t[0];
+#pragma unroll
+    for (int s = 1; s < PF_MAX_SPLIT; ++s)
+      if (s < p.n_split) y.x += t[s].x, y.y += t[s].y, y.z += t[s].z, y.w += t[s].w;
+    v.x += y.x, v.y += y.y, v.z += y.z, v.w += y.w;
+    *reinterpret_cast<float4*>(p.hid_out + at) = v;
+    if (!p.gain) continue;
+    ss += pf_square_sum(v);
+    pf_store_planes(p.planes + (size_t)row * 3 * p.H, p.H, k, v, p.gain);
+  }
+  if (!p.gain) return;
+  ss = pf_block_sum(ss, s_part);
+  if (threadIdx.x == 0) p.sumsq[row] = ss;
+}
+
+// ---- attention ---------------------------------------------------------------------------------------------------------
+// A CTA owns 64 rows of the pass (16 per warp) and one query head and walks the keys 64 at a time; every row keeps a running
+// softmax.  Both contractions are mma.sync on exact three-plane splits, chains hi and (mid + lo) of one chunk folded in fp32
+// (a row's result depends on its own prefix only).  The softmax weights never leave registers: an accumulator fragment of the
+// scores is the A fragment of the second contraction.  Keys and values are double-buffered (cp.async); rows of shared memory
+// are swizzled in 16-byte pieces so that ldmatrix is free of bank conflicts.  Blocks with the longest prefixes start first.
+constexpr int PFA_ROWS = 64, PFA_KEYS = 64, PFA_THREADS = 128;
+template <int D>
+struct PfaCfg {
+  static constexpr int ROWB = D * 2;                                // bytes of a row of Q, K, V
+  static constexpr int Q_BYTES = 3 * PFA_ROWS * ROWB, KV_BYTES = PFA_KEYS * ROWB;
+  static constexpr int SMEM_BYTES = Q_BYTES + 4 * KV_BYTES;         // Q planes, two buffers of K and V
+};
+struct PfAttnParams {
+  const float* qbuf;         // [row][n_q_heads * D], rotary applied, unscaled
+  __nv_bfloat16* aplanes;    // [row][3][n_q_heads * D]
+  const __nv_bfloat16* k;    // the sequence's keys of this layer and recurrence [n_kv][slots][D]
+  const __nv_bfloat16* v;
+  int n_rows, p0, slots, n_kv_heads, n_q_heads;
+  float scale;
+};
+__device__ __forceinline__ void pfa_ldsm4(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void pfa_ldsm4_t(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ unsigned pfa_pack(unsigned short a, unsigned short b) { return a | ((unsigned)b << 16); }
+
+template <int D>
+__global__ void __launch_bounds__(PFA_THREADS, 2) pf_attn_kernel(const __grid_constant__ PfAttnParams p) {
+  using C = PfaCfg<D>;
+  constexpr int PCS = D / 8;  // 16-byte pieces per row
+  extern __shared__ __align__(128) unsigned char pfa_smem[];
+  const unsigned sq = (unsigned)__cvta_generic_to_shared(pfa_smem), sk = sq + C::Q_BYTES, sv = sk + 2 * C::KV_BYTES;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  pdl_launch_dependents();
+  const int h = blockIdx.x % p.n_q_heads, n_blocks = (p.n_rows + PFA_ROWS - 1) / PFA_ROWS;
+  const int blk = n_blocks - 1 - blockIdx.x / p.n_q_heads;
+  const int row0 = blk * PFA_ROWS, rows_here = min(PFA_ROWS, p.n_rows - row0);
+  const int HQ = p.n_q_heads * D, kvh = h / (p.n_q_heads / p.n_kv_heads);
+  const int n_keys = p.p0 + row0 + rows_here;            // keys the block's last row sees
+  const int n_chunks = (n_keys + PFA_KEYS - 1) / PFA_KEYS;
+  const __nv_bfloat16* Kb = p.k + (size_t)kvh * p.slots * D;
+  const __nv_bfloat16* Vb = p.v + (size_t)kvh * p.slots * D;
+  auto piece = [](int row, int c) { return (unsigned)(row * C::ROWB + ((c ^ (row & 7)) << 4)); };
+  auto load_chunk = [&](int chunk, int b) {
+    const int k0 = chunk * PFA_KEYS;
+#pragma unroll
+    for (int i = 0; i < PFA_KEYS * PCS / PFA_THREADS; ++i) {
+      const int idx = tid + i * PFA_THREADS, key = idx / PCS, c = idx % PCS;
+      const bool live = k0 + key < n_keys;
+      const size_t off = (size_t)(live ? k0 + key : 0) * D + c * 8;
+      const int n = live ? 16 : 0;  // keys beyond the block's last position: zeros
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sk + b * C::KV_BYTES + piece(key, c)), "l"(Kb + off), "r"(n) : "memory");
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sv + b * C::KV_BYTES + piece(key, c)), "l"(Vb + off), "r"(n) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  pdl_wait();
+  load_chunk(0, 0);
+  // the block's queries, split into three planes (rows the pass does not have: zeros)
+  for (int idx = tid; idx < PFA_ROWS * PCS; idx += PFA_THREADS) {
+    const int lr = idx / PCS, c = idx % PCS;
+    float x[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (lr < rows_here) {
+      const float4* src = reinterpret_cast<const float4*>(p.qbuf + (size_t)(row0 + lr) * HQ + (size_t)h * D + c * 8);
+      const float4 a = src[0], b = src[1];
+      x[0] = a.x, x[1] = a.y, x[2] = a.z, x[3] = a.w, x[4] = b.x, x[5] = b.y, x[6] = b.z, x[7] = b.w;
+    }
+    unsigned short s[3][8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) split3(x[i], s[0][i], s[1][i], s[2][i]);
+#pragma unroll
+    for (int pl = 0; pl < 3; ++pl)
+      *reinterpret_cast<uint4*>(pfa_smem + pl * PFA_ROWS * C::ROWB + piece(lr, c)) =
+          make_uint4(pfa_pack(s[pl][0], s[pl][1]), pfa_pack(s[pl][2], s[pl][3]), pfa_pack(s[pl][4], s[pl][5]), pfa_pack(s[pl][6], s[pl][7]));
+  }
+  float o[D / 8][4], m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
+#pragma unroll
+  for (int j = 0; j < D / 8; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) o[j][i] = 0.f;
+  const int wr = warp * 16;                 // this warp's first row of the block
+  const int last_pos = p.p0 + row0 + wr + 15;  // ... and the last position any of them has
+  // ldmatrix lane addresses: A tiles (16 x 16): rows lane & 15, piece half lane >> 4; B tiles of K (two 8-key tiles x 16 dims):
+  // keys (lane & 7) + 8 (lane >> 4), piece half (lane >> 3) & 1; V, transposed: keys lane & 15, piece half lane >> 4
+  for (int chunk = 0; chunk < n_chunks; ++chunk) {
+    const int b = chunk & 1, k0 = chunk * PFA_KEYS;
+    if (chunk + 1 < n_chunks) {
+      load_chunk(chunk + 1, b ^ 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    if (k0 <= last_pos) {  // (uniform over the warp) some row of the warp sees this chunk
+      float s0[8][4], s1[8][4];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s0[j][i] = s1[j][i] = 0.f;
+#pragma unroll 2
+      for (int ks = 0; ks < D / 16; ++ks) {
+        unsigned a[3][4];
+#pragma unroll
+        for (int pl = 0; pl < 3; ++pl) pfa_ldsm4(a[pl], sq + pl * PFA_ROWS * C::ROWB + piece(wr + (lane & 15), 2 * ks + (lane >> 4)));
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {  // two tiles of eight keys
+          unsigned kb[4];
+          pfa_ldsm4(kb, sk + b * C::KV_BYTES + piece(16 * jj + (lane & 7) + 8 * (lane >> 4), 2 * ks + ((lane >> 3) & 1)));
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            att_mma(s0[2 * jj + e], a[0], kb[2 * e], kb[2 * e + 1]);
+            att_mma(s1[2 * jj + e], a[1], kb[2 * e], kb[2 * e + 1]);
+            att_mma(s1[2 * jj + e], a[2], kb[2 * e], kb[2 * e + 1]);
+          }
+        }
+      }
+      // scores, causal mask, running maximum of rows g and g + 8
+      const bool edge = k0 + PFA_KEYS - 1 > p.p0 + row0 + wr;  // some key of the chunk lies beyond some row of the warp
+      float mn[2] = {m[0], m[1]};
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int hf = i >> 1;
+          float sv_ = (s0[j][i] + s1[j][i]) * p.scale;
+          if (edge && k0 + 8 * j + 2 * t + (i & 1) > p.p0 + row0 + wr + g + 8 * hf) sv_ = -INFINITY;
+          s0[j][i] = sv_;
+          mn[hf] = fmaxf(mn[hf], sv_);
+        }
+      float wa[2], lc[2] = {0.f, 0.f};
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        mn[hf] = fmaxf(mn[hf], __shfl_xor_sync(0xffffffffu, mn[hf], 1));
+        mn[hf] = fmaxf(mn[hf], __shfl_xor_sync(0xffffffffu, mn[hf], 2));
+        wa[hf] = m[hf] == -INFINITY ? 0.f : expf(m[hf] - mn[hf]);
+        m[hf] = mn[hf];
+      }
+      // weights, split into three planes as A fragments: keys 16 kk + 2 t (+ 1) from tile 2 kk, + 8 from tile 2 kk + 1
+      unsigned pa[PFA_KEYS / 16][3][4];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          const float e0 = expf(s0[j][2 * hf] - m[hf]), e1 = expf(s0[j][2 * hf + 1] - m[hf]);  // (key 0 is visible to every row: m is finite)
+          lc[hf] += e0 + e1;
+          unsigned short h0, m0, l0, h1, m1, l1;
+          split3(e0, h0, m0, l0);
+          split3(e1, h1, m1, l1);
+          const int r = hf + 2 * (j & 1);
+          pa[j >> 1][0][r] = pfa_pack(h0, h1), pa[j >> 1][1][r] = pfa_pack(m0, m1), pa[j >> 1][2][r] = pfa_pack(l0, l1);
+        }
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        lc[hf] += __shfl_xor_sync(0xffffffffu, lc[hf], 1);
+        lc[hf] += __shfl_xor_sync(0xffffffffu, lc[hf], 2);
+        l[hf] = fmaf(l[hf], wa[hf], lc[hf]);
+      }
+      // weighted values: 16 dims at a time (two tiles of eight)
+#pragma unroll
+      for (int dt = 0; dt < D / 16; ++dt) {
+        float a0[2][4], a1[2][4];
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) a0[e][i] = a1[e][i] = 0.f;
+#pragma unroll
+        for (int kk = 0; kk < PFA_KEYS / 16; ++kk) {
+          unsigned vb[4];
+          pfa_ldsm4_t(vb, sv + b * C::KV_BYTES + piece(16 * kk + (lane & 15), 2 * dt + (lane >> 4)));
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            att_mma(a0[e], pa[kk][0], vb[2 * e], vb[2 * e + 1]);
+            att_mma(a1[e], pa[kk][1], vb[2 * e], vb[2 * e + 1]);
+            att_mma(a1[e], pa[kk][2], vb[2 * e], vb[2 * e + 1]);
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) o[2 * dt + e][i] = fmaf(o[2 * dt + e][i], wa[i >> 1], a0[e][i] + a1[e][i]);
+      }
+    }
+    __syncthreads();  // the buffer may be refilled
+  }
+#pragma unroll
+  for (int hf = 0; hf < 2; ++hf) {
+    const int lr = wr + g + 8 * hf;
+    if (lr >= rows_here) continue;
+    __nv_bfloat16* dst = p.aplanes + (size_t)(row0 + lr) * 3 * HQ;
+#pragma unroll
+    for (int j = 0; j < D / 8; ++j) store_split2(dst, HQ, h * D + 8 * j + 2 * t, o[j][2 * hf] / l[hf], o[j][2 * hf + 1] / l[hf]);
+  }
+}
+
+// ---- the prompt's last row, ready for the readout: one table row, its planes of x * final gain, its sum of squares ----------
+struct PfReadoutParams {
+  RowTable* tab;
+  const float* row;        // [H] the last position's state after R recurrences (and the post-layers' blocks)
+  int H, seq, pos, R, hid_idx, logit_idx;
+  const float* gain;
+  __nv_bfloat16* planes;   // [3][H]: column 0 of the decode passes' planes
+  float* sumsq;
+};
+__global__ void __launch_bounds__(256) pf_readout_kernel(const __grid_constant__ PfReadoutParams p) {
+  __shared__ float s_part[8];
+  pdl_wait();
+  float ss = 0.f;
+  for (int k = threadIdx.x * 4; k < p.H; k += 1024) {
+    const float4 v = *reinterpret_cast<const float4*>(p.row + k);
+    ss += pf_square_sum(v);
+    pf_store_planes(p.planes, p.H, k, v, p.gain);
+  }
+  ss = pf_block_sum(ss, s_part);
+  if (threadIdx.x != 0) return;
+  p.sumsq[0] = ss;
+  RowTable& t = *p.tab;
+  t.n_rows = 1, t.n_readout = 1, t.attn_items = 0, t.chunk_start[0] = t.chunk_start[1] = 0;
+  t.seq[0] = p.seq, t.r[0] = p.R, t.pos[0] = p.pos, t.kv_slot[0] = p.pos, t.n_canon[0] = p.pos + 1, t.n_spec[0] = 0, t.n_safe[0] = p.pos;
+  t.hid_idx[0] = p.hid_idx, t.node[0] = -1, t.src_hid[0] = -1, t.readout[0] = RO_TARGET, t.logit_idx[0] = p.logit_idx, t.ro_rows[0] = 0;
+}
+
+}  // namespace ls

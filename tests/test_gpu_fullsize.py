@@ -94,6 +94,19 @@ def test_full_run_properties(setup):
     ctx.close()
 
 
+def test_the_wide_prompt_path_matches_the_oracle(setup):
+    """The same golden with the prompt on the wide kernels (no bound on the prefill passes, the default)."""
+    ls, wl, shape, weights, prompt, gold = setup
+    g = gold["runs"]["greedy"]
+    ctx = ls.LoopSpec(shape, weights, d1=wl.d1, d2=wl.d2, max_ctx=wl.prompt_len + wl.decode_len + 16)
+    assert ctx.prefill(prompt) == g["first_token"]
+    z = ctx.debug_logits(0, 0)
+    for i, v in g["first_logits_probe"].items():
+        assert abs(z[int(i)] - v) < 5e-3
+    assert ctx.decode(gold["n_tokens"])[0].tolist() == g["tokens"]
+    ctx.close()
+
+
 # ---- Ouro-2.6B shape: temperature 1 with rejection verification, depths from the closed form (Theorem 2) ---------------
 GOLD_2P6B = os.path.join(os.path.dirname(__file__), "golden", "ouro_2p6b_oracle.json")
 

@@ -623,3 +623,18 @@ def test_contexts_of_different_widths_coexist():
         assert ctx.prefill(ref["prompt"]) == ref["first"]
         assert ctx.decode(12)[0].tolist() == ref["tokens"]
         ctx.close()
+
+
+@pytest.mark.parametrize("name,n_prompt,T", [("tiny_bf16", 64, 0.0), ("tiny_bf16", 65, 1.0), ("tiny_bf16", 128, 0.0), ("tiny_bf16", 129, 1.0),
+                                             ("tiny_bf16", 1025, 0.0), ("tiny_gqa", 300, 1.0), ("small_bf16", 97, 1.0),
+                                             ("small_bf16", 260, 0.0), ("tiny_raven_r4", 161, 1.0)])
+def test_wide_prompt_passes_match_oracle(name, n_prompt, T):
+    """Prompts without a bound on the pass (the default) run the wide kernels from 65 tokens on: the edges of a 128-token
+    tile, two passes, ragged feature and row blocks, grouped-query heads, both layouts."""
+    ref = U.oracle_run(name, n_prompt, 12, 1, 2, T=T, seed=9)
+    ctx = U.make_ctx(name, 1, 2, T=T, seed=9, max_ctx=n_prompt + 40)
+    assert ctx.prefill(ref["prompt"]) == ref["first"]
+    np.testing.assert_allclose(ctx.debug_logits(0, 0), ref["dec"].first_logits, atol=2e-3, rtol=0)
+    ctx.decode(12)
+    U.assert_same_run(ctx, ref, 12)
+    ctx.close()
