@@ -224,7 +224,8 @@ int loopspec_time_kernel(loopspec_ctx*, int32_t which, int32_t rows, int32_t ite
 /* Stand-alone linear map y[M][N] = x[M][K] * W[N][K]^T through the same weight-streaming kernel (token
  * activations split into three bf16 terms, fp32 accumulation; fp32 weights use the CUDA-core path).
  * All pointers device; x, y fp32; scratch: device, 16-byte aligned, loopspec_linear_scratch_bytes(M, N, K)
- * bytes (it receives the bf16 planes of x and, for bf16 weights, a tile-major copy of W; contents on entry are
+ * bytes (it receives the bf16 planes of x where x is split by a launch of its own - more than 16 rows, fp32 weights; W is read
+ * in place; contents on entry are
  * irrelevant).  M <= 64, N % 16 == 0, K % 8 == 0. */
 size_t loopspec_linear_scratch_bytes(int32_t M, int32_t N, int32_t K);
 int loopspec_op_linear(const void* W, int32_t weight_dtype, const float* x, float* y, int32_t M, int32_t N,

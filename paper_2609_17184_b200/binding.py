@@ -142,21 +142,23 @@ def linear_scratch_bytes(M, N, K):
     return lib.loopspec_linear_scratch_bytes(M, N, K)
 
 
+def _raw_stream(torch):
+    """The current stream's handle (the call torch's own generated code makes: no Stream object per call)."""
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
 def linear(W, x, scratch=None):
     """y = x @ W.T through the weight-streaming kernel.  W [N,K] bf16 or fp32, x [M,K] fp32 (cuda tensors)."""
     import torch
     M, K = x.shape
     N = W.shape[0]
-    need = linear_scratch_bytes(M, N, K)
-    if need == 0:
-        raise LoopSpecError(-1, "unsupported linear shape")
     if scratch is None:
-        scratch = torch.zeros(need, dtype=torch.uint8, device=x.device)
-    y = torch.empty(M, N, dtype=torch.float32, device=x.device)
+        scratch = torch.zeros(linear_scratch_bytes(M, N, K), dtype=torch.uint8, device=x.device)
+    y = torch.empty((M, N), dtype=torch.float32, device=x.device)
     rc = lib.loopspec_op_linear(W.data_ptr(), 1 if W.dtype == torch.bfloat16 else 0, x.data_ptr(), y.data_ptr(), M, N, K,
-                                scratch.data_ptr(), scratch.numel(), torch.cuda.current_stream().cuda_stream)
+                                scratch.data_ptr(), scratch.numel(), _raw_stream(torch))
     if rc:
-        raise LoopSpecError(rc)
+        raise LoopSpecError(rc, "unsupported linear shape" if rc == -1 else "")
     return y
 
 
@@ -166,17 +168,19 @@ def linear_tc(W, x, scratch=None, check=True):
     import torch
     M, K = x.shape
     N = W.shape[0]
-    need = lib.loopspec_linear_tc_scratch_bytes(M, N, K)
-    if need == 0 or W.dtype != torch.bfloat16:
+    if W.dtype != torch.bfloat16:
         raise LoopSpecError(-1, "unsupported linear_tc shape or dtype")
     if scratch is None:
+        need = lib.loopspec_linear_tc_scratch_bytes(M, N, K)
+        if need == 0:
+            raise LoopSpecError(-1, "unsupported linear_tc shape or dtype")
         scratch = torch.empty(need + 256, dtype=torch.uint8, device=x.device)
-    off = (-scratch.data_ptr()) % 256
-    y = torch.empty(M, N, dtype=torch.float32, device=x.device)
-    rc = lib.loopspec_op_linear_tc(W.data_ptr(), x.data_ptr(), y.data_ptr(), M, N, K, scratch.data_ptr() + off,
-                                   scratch.numel() - off, torch.cuda.current_stream().cuda_stream)
+    base = scratch.data_ptr()
+    off = (-base) % 256
+    y = torch.empty((M, N), dtype=torch.float32, device=x.device)
+    rc = lib.loopspec_op_linear_tc(W.data_ptr(), x.data_ptr(), y.data_ptr(), M, N, K, base + off, scratch.numel() - off, _raw_stream(torch))
     if rc:
-        raise LoopSpecError(rc, "op_linear_tc")
+        raise LoopSpecError(rc, "op_linear_tc" if rc != -1 else "unsupported linear_tc shape or dtype")
     if check:
         torch.cuda.current_stream().synchronize()
         if int(scratch[off:off + 4].view(torch.int32).item()) != 0:
@@ -211,9 +215,9 @@ def linear_static(W, x):
     import torch
     M, K = x.shape
     N = W.shape[0]
-    y = torch.empty(M, N, dtype=torch.float32, device=x.device)
+    y = torch.empty((M, N), dtype=torch.float32, device=x.device)
     rc = lib.loopspec_op_linear_static(W.data_ptr(), 1 if W.dtype == torch.bfloat16 else 0, x.data_ptr(), y.data_ptr(), M, N, K,
-                                       torch.cuda.current_stream().cuda_stream)
+                                       _raw_stream(torch))
     if rc:
         raise LoopSpecError(rc, "op_linear_static")
     return y

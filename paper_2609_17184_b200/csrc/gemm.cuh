@@ -374,6 +374,9 @@ __global__ void __launch_bounds__(GEMM_THREADS) __maxnreg__(NG == 1 ? LS_MAXREG 
   const unsigned ring_s = (unsigned)__cvta_generic_to_shared(ring) + tid * 16;
   const __nv_bfloat16* const Wb = static_cast<const __nv_bfloat16*>(p.W);
   const char* i_ptr = reinterpret_cast<const char*>(Wb);
+  // EPI_PLAIN (stand-alone calls) reads row-major weights in place: a unit is 64 bytes of 16 rows; k beyond the row is zero-filled
+  const size_t i_hi = EPI == EPI_PLAIN ? (size_t)16 * p.K : 512;  // bytes from a lane's low piece to its high piece
+  int i_k = 0;
   unsigned i_slot = 0;
   int i_rb = cid, i_left = my_upt, i_tasks = my_upt > 0 ? n_tasks : 0, i_size = 0;
   auto i_setup = [&]() {
@@ -381,14 +384,21 @@ __global__ void __launch_bounds__(GEMM_THREADS) __maxnreg__(NG == 1 ? LS_MAXREG 
     i_size = r0 >= 0 ? 16 : 0;  // rows beyond the matrix: zero-fill, nothing is read
     const int pt = r0 >= 0 ? packed_tile(p.perm, p.perm_a, p.perm_d, r0) : 0;
     i_ptr = reinterpret_cast<const char*>(Wb + ((size_t)pt * kpr + kb_lo + khalf) * 512 + lane * 8);
+    if (EPI == EPI_PLAIN) {
+      i_k = kb_lo * 32 + t * 8;
+      i_ptr = reinterpret_cast<const char*>(Wb + (size_t)((r0 >= 0 ? r0 : 0) + g) * p.K + i_k);
+    }
   };
   i_setup();
   auto issue_unit = [&]() {
     if (i_tasks > 0) {
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ring_s + i_slot), "l"(i_ptr), "r"(i_size) : "memory");
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ring_s + i_slot + HI_OFF), "l"(i_ptr + 512), "r"(i_size)
+      const int size = EPI == EPI_PLAIN && i_k >= p.K ? 0 : i_size;
+      const char* src = EPI == EPI_PLAIN && i_k >= p.K ? reinterpret_cast<const char*>(Wb) : i_ptr;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ring_s + i_slot), "l"(src), "r"(size) : "memory");
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ring_s + i_slot + HI_OFF), "l"(src + (size ? i_hi : 0)), "r"(size)
                    : "memory");
-      i_ptr += 1024 * KH;
+      i_ptr += EPI == EPI_PLAIN ? 64 : 1024 * KH;
+      i_k += 32;
       i_slot += SLOT_BYTES;
       if (i_slot == RING_BYTES) i_slot = 0;
       if (--i_left == 0) {

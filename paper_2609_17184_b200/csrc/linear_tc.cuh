@@ -252,24 +252,45 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
   }
 }
 
-// x fp32 [M][K] -> planes bf16 [3][MP][K] (rows M..MP-1 zero)
-__global__ void tc_split_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ planes, int M, int MP, int K) {
-  const int m = blockIdx.x;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    unsigned short h = 0, mi = 0, l = 0;
-    if (m < M) split3(x[(size_t)m * K + k], h, mi, l);
-    planes[((size_t)0 * MP + m) * K + k] = __ushort_as_bfloat16(h);
-    planes[((size_t)1 * MP + m) * K + k] = __ushort_as_bfloat16(mi);
-    planes[((size_t)2 * MP + m) * K + k] = __ushort_as_bfloat16(l);
+// x fp32 [M][K] -> planes bf16 [3][MP][K] (rows M..MP-1 zero); clears the flag of the kernel that follows.  Eight values a
+// thread (K is a multiple of 64), one CTA per row and 2048 of k.
+inline int tc_split_blocks(int K) { return (K + 2047) / 2048; }
+__global__ void __launch_bounds__(256) tc_split_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ planes, int M, int MP, int K, int* err) {
+  pdl_launch_dependents();
+  const int m = blockIdx.x, k = (blockIdx.y * 256 + threadIdx.x) * 8;
+  if (m == 0 && k == 0) *err = 0;
+  if (k >= K) return;
+  unsigned short s[3][8];
+  float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  if (m < M) {
+    const float* src = x + (size_t)m * K + k;
+    if ((reinterpret_cast<unsigned long long>(x) & 15) == 0) {
+      const float4 a = *reinterpret_cast<const float4*>(src), b = *reinterpret_cast<const float4*>(src + 4);
+      v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+    } else {
+      for (int i = 0; i < 8; ++i) v[i] = src[i];
+    }
   }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) split3(v[i], s[0][i], s[1][i], s[2][i]);
+#pragma unroll
+  for (int p = 0; p < 3; ++p)
+    *reinterpret_cast<uint4*>(planes + ((size_t)p * MP + m) * K + k) =
+        make_uint4(s[p][0] | ((unsigned)s[p][1] << 16), s[p][2] | ((unsigned)s[p][3] << 16), s[p][4] | ((unsigned)s[p][5] << 16), s[p][6] | ((unsigned)s[p][7] << 16));
 }
 
-// y = sum over the k-splits, in split order
-__global__ void tc_sum_splits_kernel(const float* __restrict__ part, float* __restrict__ y, size_t MN, int n_split) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < MN; i += (size_t)gridDim.x * blockDim.x) {
-    float v = part[i];
-    for (int s = 1; s < n_split; ++s) v += part[(size_t)s * MN + i];
-    y[i] = v;
+// y = sum over the k-splits, in split order (MN is a multiple of 8: four values a thread and step where y is 16-byte aligned)
+__global__ void __launch_bounds__(256) tc_sum_splits_kernel(const float* __restrict__ part, float* __restrict__ y, size_t MN, int n_split) {
+  pdl_wait();
+  const size_t step = (size_t)gridDim.x * blockDim.x * 4;
+  for (size_t i = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) * 4; i < MN; i += step) {
+    float4 v = __ldcg(reinterpret_cast<const float4*>(part + i));
+    for (int s = 1; s < n_split; ++s) {
+      const float4 t = __ldcg(reinterpret_cast<const float4*>(part + (size_t)s * MN + i));
+      v.x += t.x, v.y += t.y, v.z += t.z, v.w += t.w;
+    }
+    if ((reinterpret_cast<unsigned long long>(y) & 15) == 0) *reinterpret_cast<float4*>(y + i) = v;
+    else y[i] = v.x, y[i + 1] = v.y, y[i + 2] = v.z, y[i + 3] = v.w;
   }
 }
 

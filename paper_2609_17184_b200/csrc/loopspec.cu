@@ -24,6 +24,7 @@
 #include "linear_tc.cuh"
 #include "gemm_dec.cuh"
 #include "prefill.cuh"
+#include "linear_direct.cuh"
 
 using namespace ls;
 
@@ -217,6 +218,17 @@ bool tc_prefill_shapes_ok(const loopspec_model* m) {
   return m->weight_dtype == 1 && m->hidden % TC_BK == 0 && (m->n_q_heads * m->head_dim) % TC_BK == 0 && m->ffn % TC_BK == 0;
 }
 int tc_pf_cols(int max_rows_pf) { return (max_rows_pf + 15) / 16 * 16; }
+
+// linear_tc_kernel's shared-memory ceiling, asked for once per device (two threads racing on a first call set the same value)
+bool tc_allow_smem() {
+  static std::atomic<bool> done[64];
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  if (done[dev].load(std::memory_order_acquire)) return true;
+  if (cudaFuncSetAttribute(linear_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MAX) != cudaSuccess) return false;
+  done[dev].store(true, std::memory_order_release);
+  return true;
+}
 
 struct Layout {  // byte offsets into the workspace
   size_t wpack, rope, kv, hid, qbuf, xplanes, aplanes, splanes, sumsq, logits, argpart, tcpart, flt, sel_flt, tv, tune, tune_bytes, apart, acnt, nodes, seqs, ctr, tab_dec, tab_pf,
@@ -1442,7 +1454,7 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
       for (int i = 0; i < (dd.raven ? 4 : 3) && ok; ++i)
         ok = make_map_planes3d(&tc.xmaps[i], c->ws + x_off[i], x_k[i], x_k[i], dd.max_rows, tc.cols);
     }
-    ok = ok && cudaFuncSetAttribute(linear_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MAX) == cudaSuccess;
+    ok = ok && tc_allow_smem();
     if (!ok) (void)cudaGetLastError();
     for (int k = 0; k < 2; ++k) c->tc[k].on = ok && want[k];
   }
@@ -1984,19 +1996,22 @@ int loopspec_op_linear(const void* W, int32_t weight_dtype, const float* x, floa
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const int ng = ng_for_rows(M);
   GemmPlan g = plan_gemm((N + 127) / 128, K, 148 * kCtasPerSm, true);
+  // Up to 16 rows: one launch that splits x itself.  Beyond, every warp would read and split more of x than it reads of W, and
+  // the cluster GEMM on planes made once is the faster one.
+  if (weight_dtype == 1 && ng <= 2 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(W)) & 15) == 0) {
+    LinearDirectParams q = {static_cast<const __nv_bfloat16*>(W), x, y, M, N, K, g.cs};
+    const int tpc = 8 / g.cs, tiles = N / 16;
+    // two tiles per warp share the split of x; below two CTAs per SM the parallelism is worth more [2048 x 2048, 4 rows: 5.0 us
+    // with one, 5.6 with two; 12288 x 5632: 44 / 40 us with 4 rows, 96 / 59 us with 12]
+    const int T = tiles / tpc >= 296 ? 2 : 1;
+    const auto fn = ng == 1 ? (T == 2 ? linear_direct_kernel<1, 2> : linear_direct_kernel<1, 1>) : (T == 2 ? linear_direct_kernel<2, 2> : linear_direct_kernel<2, 1>);
+    cudaError_t e = launch_k(fn, dim3((tiles + tpc * T - 1) / (tpc * T)), dim3(256), 0, st, q, false);
+    return e == cudaSuccess ? LOOPSPEC_OK : LOOPSPEC_ECUDA;
+  }
   PrepParams q;
   memset(&q, 0, sizeof q);
   q.m_fixed = M, q.x = x, q.K = K, q.planes = static_cast<__nv_bfloat16*>(scratch);
   if (launch_k(prep_planes_kernel, dim3(M), dim3(256), 0, st, q, false) != cudaSuccess) return LOOPSPEC_ECUDA;
-  if (weight_dtype == 1) {  // stream from a tile-major copy, as the decode path does
-    PackParams pp;
-    memset(&pp, 0, sizeof pp);
-    pp.src = static_cast<const __nv_bfloat16*>(W), pp.N = N, pp.K = K, pp.kpr = (K + 31) / 32;
-    pp.dst = reinterpret_cast<__nv_bfloat16*>(static_cast<unsigned char*>(scratch) + align_up((size_t)M * 3 * K * 2));
-    pack_weights_kernel<<<296, 256, 0, st>>>(pp);
-    if (cudaGetLastError() != cudaSuccess) return LOOPSPEC_ECUDA;
-    W = pp.dst;
-  }
   GemmParams p;
   memset(&p, 0, sizeof p);
   p.W = W, p.N = N, p.K = K, p.n_rb = g.n_rb, p.kb_per_rb = g.kpr, p.cluster_size = g.cs, p.n_clusters = g.n_clusters;
@@ -2006,7 +2021,7 @@ int loopspec_op_linear(const void* W, int32_t weight_dtype, const float* x, floa
   if (gemm_smem(weight_dtype, ng) > 48 * 1024 &&
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(weight_dtype, ng)) != cudaSuccess)
     return LOOPSPEC_ECUDA;
-  cudaError_t e = launch_gemm(weight_dtype, ng, EPI_PLAIN, p, st, false);
+  cudaError_t e = launch_gemm(weight_dtype, ng, EPI_PLAIN, p, st, true);  // (its first weights are requested while x is split)
   return e == cudaSuccess ? LOOPSPEC_OK : LOOPSPEC_ECUDA;
 }
 
@@ -2085,18 +2100,27 @@ int loopspec_op_linear_tc(const void* W, const float* x, float* y, int32_t M, in
   __nv_bfloat16* planes = reinterpret_cast<__nv_bfloat16*>(sc + t.planes_off);
   CUtensorMap map_w, map_x;
   if (!make_map_bf16(&map_w, W, N, K, TC_BM) || !make_map_bf16(&map_x, planes, 3 * t.MP, K, 3 * t.MP)) return LOOPSPEC_ECUDA;
-  if (cudaMemsetAsync(sc, 0, 256, st) != cudaSuccess) return LOOPSPEC_ECUDA;
-  tc_split_kernel<<<t.MP, 256, 0, st>>>(x, planes, M, t.MP, K);
+  tc_split_kernel<<<dim3(t.MP, tc_split_blocks(K)), 256, 0, st>>>(x, planes, M, t.MP, K, reinterpret_cast<int*>(sc));
   LinearTcParams p;
   memset(&p, 0, sizeof p);
   p.out = t.n_split > 1 ? reinterpret_cast<float*>(sc + t.part_off) : y;
   p.M = M, p.MP = t.MP, p.N = N, p.K = K, p.kb_per_split = t.kb_per_split, p.stages = t.stages;
   p.err = reinterpret_cast<int*>(sc), p.err_code = 1;
-  if (cudaFuncSetAttribute(linear_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MAX) != cudaSuccess)
-    return LOOPSPEC_ECUDA;
-  linear_tc_kernel<<<dim3(t.n_rb, t.n_split), TC_THREADS, t.smem, st>>>(map_w, map_x, p);
-  if (t.n_split > 1) tc_sum_splits_kernel<<<296, 256, 0, st>>>(p.out, y, (size_t)M * N, t.n_split);
-  return cudaGetLastError() == cudaSuccess ? LOOPSPEC_OK : LOOPSPEC_ECUDA;
+  if (!tc_allow_smem()) return LOOPSPEC_ECUDA;
+  // programmatic dependent launches: the weights are requested while x is split, the sums start as the last tile ends
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  cfg.gridDim = dim3(t.n_rb, t.n_split), cfg.blockDim = dim3(TC_THREADS), cfg.dynamicSmemBytes = t.smem, cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at, cfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, linear_tc_kernel, map_w, map_x, p);
+  if (e == cudaSuccess && t.n_split > 1) {
+    cfg.gridDim = dim3((unsigned)std::min<size_t>(296, ((size_t)M * N / 4 + 255) / 256)), cfg.blockDim = dim3(256), cfg.dynamicSmemBytes = 0;
+    e = cudaLaunchKernelEx(&cfg, tc_sum_splits_kernel, static_cast<const float*>(p.out), y, (size_t)M * N, t.n_split);
+  }
+  return e == cudaSuccess ? LOOPSPEC_OK : LOOPSPEC_ECUDA;
 }
 
 int loopspec_time_linear_tc(const void* const* Ws, int32_t n_w, const float* x, int32_t M, int32_t N, int32_t K,
@@ -2113,15 +2137,13 @@ int loopspec_time_linear_tc(const void* const* Ws, int32_t n_w, const float* x, 
   for (int i = 0; i < n_w; ++i)
     if (!Ws[i] || (reinterpret_cast<uintptr_t>(Ws[i]) & 15) || !make_map_bf16(&maps[i], Ws[i], N, K, TC_BM)) return LOOPSPEC_EINVAL;
   if (!make_map_bf16(&map_x, planes, 3 * t.MP, K, 3 * t.MP)) return LOOPSPEC_ECUDA;
-  if (cudaMemsetAsync(sc, 0, 256, st) != cudaSuccess) return LOOPSPEC_ECUDA;
-  tc_split_kernel<<<t.MP, 256, 0, st>>>(x, planes, M, t.MP, K);
+  tc_split_kernel<<<dim3(t.MP, tc_split_blocks(K)), 256, 0, st>>>(x, planes, M, t.MP, K, reinterpret_cast<int*>(sc));
   LinearTcParams p;
   memset(&p, 0, sizeof p);
   p.out = reinterpret_cast<float*>(sc + t.part_off);
   p.M = M, p.MP = t.MP, p.N = N, p.K = K, p.kb_per_split = t.kb_per_split, p.stages = t.stages;
   p.err = reinterpret_cast<int*>(sc), p.err_code = 1;
-  if (cudaFuncSetAttribute(linear_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MAX) != cudaSuccess)
-    return LOOPSPEC_ECUDA;
+  if (!tc_allow_smem()) return LOOPSPEC_ECUDA;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = dim3(t.n_rb, t.n_split), cfg.blockDim = dim3(TC_THREADS), cfg.dynamicSmemBytes = t.smem, cfg.stream = st;

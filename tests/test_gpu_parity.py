@@ -65,6 +65,24 @@ def test_linear_tc_matches_definition(M, N, K):
     assert (np.abs(y - y2) <= 4e-6 * scale + 1e-30).all()
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 16, 8), (3, 16, 40), (8, 9488, 520), (9, 12304, 1032), (16, 304, 72), (17, 304, 72), (40, 2064, 1000)])
+def test_linear_reads_row_major_weights_at_the_edges(M, N, K):
+    """Weights read in place (one launch up to 16 rows, the cluster GEMM beyond): rows that end inside a 32-wide k-block,
+    odd tile counts, one and two tiles per warp; an x that is not 16-byte aligned gives the same bits."""
+    import paper_2609_17184_b200 as ls
+    rng = np.random.default_rng(N + K + M)
+    Wn = W.bf16_round((rng.standard_normal((N, K)) * 0.05).astype(np.float32))
+    x = rng.standard_normal((M, K)).astype(np.float32)
+    Wt, buf = torch.from_numpy(Wn).cuda().to(torch.bfloat16), torch.zeros(M * K + 1, device="cuda")
+    y = ls.linear(Wt, torch.from_numpy(x).cuda()).cpu().numpy()
+    ref = x.astype(np.float64) @ Wn.astype(np.float64).T
+    scale = np.abs(x).astype(np.float64) @ np.abs(Wn).astype(np.float64).T
+    assert (np.abs(y - ref) <= 2e-6 * scale + 1e-30).all()
+    xo = buf[1:].view(M, K)
+    xo.copy_(torch.from_numpy(x))
+    assert np.array_equal(ls.linear(Wt, xo).cpu().numpy().view(np.uint32), y.view(np.uint32))
+
+
 def test_linear_tc_rejects_unsupported_shapes():
     import paper_2609_17184_b200 as ls
     assert ls.lib.loopspec_linear_tc_scratch_bytes(4, 256, 256) > 0
