@@ -561,12 +561,17 @@ __global__ void __launch_bounds__(GEMM_THREADS) __maxnreg__(NG == 1 ? LS_MAXREG 
 }
 
 // ======================================= fp32 weights: CUDA cores ==========================================
-// Same decomposition and epilogues; the activation is rebuilt exactly from its three planes.  Used by the
-// small fp32 configuration only, so it is written for clarity, not speed.
+// Same decomposition and epilogues; the activation is rebuilt exactly from its three planes.  The fp32 models are small (a block
+// of the 256-wide one is 3 MB, in the L2), so a launch is bound by its chain of latencies: the weights of the first k-blocks are
+// requested ahead of the predecessor, the whole k-range of activations is staged at once, and K is split over clusters of up
+// to 8 CTAs (see plan_gemm_f32).  A decode step of the 256-wide model (4 rows, 10 of these launches, each 17 to 23 us serialised
+// before) went from 148 to 66 us, some 10 us of that by the control kernel.
+__host__ __device__ constexpr int f32_xch(int NG) { return NG == 1 ? 32 : NG == 2 ? 16 : 8; }  // k-blocks staged at a time
 template <int NG, int EPI>
 __global__ void __launch_bounds__(GEMM_THREADS) gemm_f32_kernel(const __grid_constant__ GemmParams p) {
   constexpr int NTOK = 8 * NG;
-  constexpr int XCH = 4;
+  constexpr int XCH = f32_xch(NG);
+  constexpr int DEPTH = NG <= 2 ? 4 : 2;  // k-blocks of weights in flight per warp
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* xf = reinterpret_cast<float*>(smem_raw);              // [XCH][NTOK][32]
   float* recv = xf + XCH * NTOK * 32;                          // [cs][own_max][128]
@@ -584,18 +589,36 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_f32_kernel(const __grid_con
   const int n_tasks = (p.n_rb - cid + p.n_clusters - 1) / p.n_clusters;
   const int own_max = (NTOK + cs - 1) / cs;
   pdl_launch_dependents();
-  pdl_wait();
+  float4 w[DEPTH][4];  // rows g and g + 8, eight k each
+  int row0 = gemm_row0<EPI>(p, cid, warp);
+  auto fetch = [&](int u, int kb) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[u][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int k = kb * 32 + t * 8;
+    if (row0 >= 0 && kb < kb_hi && k < p.K) {
+      const float4* wl = reinterpret_cast<const float4*>(static_cast<const float*>(p.W) + (size_t)(row0 + g) * p.K + k);
+      const float4* wh = reinterpret_cast<const float4*>(static_cast<const float*>(p.W) + (size_t)(row0 + g + 8) * p.K + k);
+      w[u][0] = __ldg(wl), w[u][1] = __ldg(wl + 1), w[u][2] = __ldg(wh), w[u][3] = __ldg(wh + 1);
+    }
+  };
+#pragma unroll
+  for (int u = 0; u < DEPTH; ++u) fetch(u, kb_lo + u);
+  // the row table was written before this pass started
   const RowTable* tab = p.tab;
   int n_cols = (tab ? (p.cols_from_readout ? tab->n_readout : tab->n_rows) : p.m_fixed) - p.col0;
   if (n_cols > NTOK) n_cols = NTOK;
-  if (n_cols <= 0) return;
   gemm_load_cols(p, n_cols, NTOK, s_ct);
+  pdl_wait();
+  if (n_cols <= 0) return;
   __syncthreads();
-  gemm_rstd(p, n_cols, s_rstd, s_ct, NTOK);
 
   for (int task = 0; task < n_tasks; ++task) {
     const int rb = cid + task * p.n_clusters;
-    const int row0 = gemm_row0<EPI>(p, rb, warp);
+    if (task > 0) {
+      row0 = gemm_row0<EPI>(p, rb, warp);
+#pragma unroll
+      for (int u = 0; u < DEPTH; ++u) fetch(u, kb_lo + u);
+    }
     float accf[NG][8][2];
 #pragma unroll
     for (int n = 0; n < NG; ++n)
@@ -603,40 +626,56 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_f32_kernel(const __grid_con
       for (int c = 0; c < 8; ++c) accf[n][c][0] = accf[n][c][1] = 0.f;
     for (int ck = 0; ck < upt; ck += XCH) {
       const int nkb = min(XCH, upt - ck);
-      __syncthreads();
-      for (int idx = tid; idx < nkb * NTOK * 32; idx += GEMM_THREADS) {
-        int e = idx & 31, c = (idx >> 5) % NTOK, kbl = idx / (32 * NTOK);
-        int k = (kb_lo + ck + kbl) * 32 + e;
-        float v = 0.f;
-        if (c < n_cols && k < p.K) {
-          const int xr = p.cols_from_readout ? s_ct[CT_XROW * NTOK + c] : c;
-          const __nv_bfloat16* pl = p.xplanes + (size_t)xr * 3 * p.x_ld + k;
-          v = (__bfloat162float(pl[0]) + __bfloat162float(pl[p.x_ld])) + __bfloat162float(pl[2 * p.x_ld]);
-        }
-        xf[idx] = v;
-      }
-      __syncthreads();
-      if (row0 >= 0) {
-        for (int kbl = 0; kbl < nkb; ++kbl) {
-          const int k = (kb_lo + ck + kbl) * 32 + t * 8;
+      if (task == 0 || upt > XCH) {
+        if (task > 0 || ck > 0) __syncthreads();
+        // eight values a thread: quarter q of k-block kbl of column c
+        for (int idx = tid; idx < nkb * n_cols * 4; idx += GEMM_THREADS) {
+          const int q = idx & 3, rest = idx >> 2, c = rest % n_cols, kbl = rest / n_cols;
+          const int k = (kb_lo + ck + kbl) * 32 + q * 8;
+          float* dst = xf + (kbl * NTOK + c) * 32 + q * 8;
+          uint4 pl[3] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
           if (k < p.K) {
-            const float* wl = static_cast<const float*>(p.W) + (size_t)(row0 + g) * p.K + k;
-            const float* wh = wl + (size_t)8 * p.K;
-            float4 l0 = *reinterpret_cast<const float4*>(wl), l1 = *reinterpret_cast<const float4*>(wl + 4);
-            float4 h0 = *reinterpret_cast<const float4*>(wh), h1 = *reinterpret_cast<const float4*>(wh + 4);
-            const float wlo[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
-            const float whi[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+            const int xr = p.cols_from_readout ? s_ct[CT_XROW * NTOK + c] : c;
+            const __nv_bfloat16* src = p.xplanes + (size_t)xr * 3 * p.x_ld + k;
+#pragma unroll
+            for (int s = 0; s < 3; ++s) pl[s] = *reinterpret_cast<const uint4*>(src + (size_t)s * p.x_ld);
+          }
+          const unsigned a[3][4] = {{pl[0].x, pl[0].y, pl[0].z, pl[0].w}, {pl[1].x, pl[1].y, pl[1].z, pl[1].w}, {pl[2].x, pl[2].y, pl[2].z, pl[2].w}};
+          float v[8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            v[2 * i] = (__uint_as_float(a[0][i] << 16) + __uint_as_float(a[1][i] << 16)) + __uint_as_float(a[2][i] << 16);
+            v[2 * i + 1] = (__uint_as_float(a[0][i] & 0xffff0000u) + __uint_as_float(a[1][i] & 0xffff0000u)) + __uint_as_float(a[2][i] & 0xffff0000u);
+          }
+          *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+          *reinterpret_cast<float4*>(dst + 4) = make_float4(v[4], v[5], v[6], v[7]);
+        }
+        if (task == 0 && ck == 0) gemm_rstd(p, n_cols, s_rstd, s_ct, NTOK);
+        __syncthreads();
+      }
+      for (int kb0 = 0; kb0 < nkb; kb0 += DEPTH) {
+#pragma unroll
+        for (int u = 0; u < DEPTH; ++u) {
+          const int kbl = kb0 + u;
+          if (kbl < nkb) {
+            const float wlo[8] = {w[u][0].x, w[u][0].y, w[u][0].z, w[u][0].w, w[u][1].x, w[u][1].y, w[u][1].z, w[u][1].w};
+            const float whi[8] = {w[u][2].x, w[u][2].y, w[u][2].z, w[u][2].w, w[u][3].x, w[u][3].y, w[u][3].z, w[u][3].w};
+            // (XCH is a multiple of DEPTH: slot u of the next chunk's first k-blocks is refilled here too)
+            fetch(u, kb_lo + ck + kbl + DEPTH);
 #pragma unroll
             for (int n = 0; n < NG; ++n)
 #pragma unroll
-              for (int c = 0; c < 8; ++c) {
-                const float* xv = xf + (kbl * NTOK + n * 8 + c) * 32 + t * 8;
+              for (int c = 0; c < 8; ++c)
+                if (n * 8 + c < n_cols) {  // (uniform)
+                  const float4* xv = reinterpret_cast<const float4*>(xf + (kbl * NTOK + n * 8 + c) * 32 + t * 8);
+                  const float4 x0 = xv[0], x1 = xv[1];
+                  const float xe[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                  accf[n][c][0] = fmaf(wlo[e], xv[e], accf[n][c][0]);
-                  accf[n][c][1] = fmaf(whi[e], xv[e], accf[n][c][1]);
+                  for (int e = 0; e < 8; ++e) {
+                    accf[n][c][0] = fmaf(wlo[e], xe[e], accf[n][c][0]);
+                    accf[n][c][1] = fmaf(whi[e], xe[e], accf[n][c][1]);
+                  }
                 }
-              }
           }
         }
       }
@@ -662,7 +701,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_f32_kernel(const __grid_con
   }
 }
 __host__ __device__ constexpr int gemm_f32_smem_bytes(int NG) {
-  return 4 * 8 * NG * 32 * 4 + recv_floats(NG) * 4 + 2 * RB_ROWS * 4 + 8 * NG * 4 * (1 + CT_FIELDS) + 64;
+  return f32_xch(NG) * 8 * NG * 32 * 4 + recv_floats(NG) * 4 + 2 * RB_ROWS * 4 + 8 * NG * 4 * (1 + CT_FIELDS) + 64;
 }
 
 // ---- one-time repacking of a bf16 weight matrix [N][K] into the tile-major streaming layout ----------------
@@ -724,13 +763,13 @@ __global__ void __launch_bounds__(256) raven_concat_kernel(const __grid_constant
   float* e = p.e_store + (size_t)idx * p.H;
   const bool first = p.tab->r[c] == 1;
   __nv_bfloat16* dst = p.planes + (size_t)c * 3 * 2 * p.H;
-  for (int k = threadIdx.x; k < p.H; k += blockDim.x) {
-    const float hv = h[k];
-    float ev = hv;
-    if (first) e[k] = hv;
-    else ev = e[k];
-    store_split(dst, 2 * p.H, k, hv);
-    store_split(dst, 2 * p.H, p.H + k, ev);
+  for (int k = threadIdx.x * 4; k < p.H; k += 1024) {  // (H is a multiple of 128)
+    const float4 hv = *reinterpret_cast<const float4*>(h + k);
+    float4 ev = hv;
+    if (first) *reinterpret_cast<float4*>(e + k) = hv;
+    else ev = *reinterpret_cast<const float4*>(e + k);
+    store_split4(dst, 2 * p.H, k, hv);
+    store_split4(dst, 2 * p.H, p.H + k, ev);
   }
 }
 
@@ -752,11 +791,23 @@ __global__ void __launch_bounds__(256) prep_planes_kernel(const __grid_constant_
   }
   __nv_bfloat16* dst = p.planes + (size_t)c * 3 * p.K;
   float ss = 0.f;
-  for (int k = threadIdx.x; k < p.K; k += blockDim.x) {
-    float v = src[k];
-    if (copy) copy[k] = v;
-    ss += v * v;
-    store_split(dst, p.K, k, p.gain ? v * p.gain[k] : v);
+  if (p.tab) {  // a pass's rows: K = hidden, a multiple of 128; four values a thread
+    for (int k = threadIdx.x * 4; k < p.K; k += 1024) {
+      float4 v = *reinterpret_cast<const float4*>(src + k);
+      if (copy) *reinterpret_cast<float4*>(copy + k) = v;
+      ss += (v.x * v.x + v.y * v.y) + (v.z * v.z + v.w * v.w);
+      if (p.gain) {
+        const float4 g = *reinterpret_cast<const float4*>(p.gain + k);
+        v.x *= g.x, v.y *= g.y, v.z *= g.z, v.w *= g.w;
+      }
+      store_split4(dst, p.K, k, v);
+    }
+  } else {
+    for (int k = threadIdx.x; k < p.K; k += blockDim.x) {
+      const float v = src[k];
+      ss += v * v;
+      store_split(dst, p.K, k, p.gain ? v * p.gain[k] : v);
+    }
   }
   ss = warp_sum(ss);
   if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = ss;

@@ -82,6 +82,17 @@ GemmPlan plan_gemm(int n_rb, int K, int slots, bool pow2_only, int kh = 1, int c
   return g;
 }
 
+// fp32 weights (CUDA cores): clusters of up to 8 as long as every CTA keeps a k-block and the grid fits the resident slots -
+// what counts is a short chain per CTA (one rank per block of 128 rows before: 17 to 23 us a launch at K = 256 .. 688)
+GemmPlan plan_gemm_f32(int n_rb, int K, int slots) {
+  GemmPlan g;
+  g.n_rb = n_rb, g.kpr = (K + 31) / 32, g.cs = 1;
+  while (2 * g.cs <= std::min(8, g.kpr) && 2 * g.cs * n_rb <= slots) g.cs *= 2;
+  const int max_clusters = std::max(1, slots / g.cs), rounds = (n_rb + max_clusters - 1) / max_clusters;
+  g.n_clusters = (n_rb + rounds - 1) / rounds, g.grid = g.n_clusters * g.cs;
+  return g;
+}
+
 size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 
 // ---- plan of a decode-pass GEMM on the tcgen05 kernel (dgemm_kernel) ----
@@ -1347,8 +1358,8 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
   // buffer holds one column then): the down projection's 176 k-blocks over 11 ranks instead of 8 [measured: pass 1.122 ->
   // 1.099 ms; 12 ranks 1.110 ms, 16 ranks 1.21 ms - they no longer fit at once]
   const int cs_cap = c->ng_dec == 1 ? 11 : 8;
-  for (int i = 0; i < 6; ++i) c->plan[i] = plan_gemm(n_rbs[i], Ks[i], slots, false, 1, cs_cap);
-  for (int i = 0; i < 6; ++i) c->plan_pf[i] = plan_gemm(n_rbs[i], Ks[i], slots, false);
+  for (int i = 0; i < 6; ++i) c->plan[i] = m->weight_dtype ? plan_gemm(n_rbs[i], Ks[i], slots, false, 1, cs_cap) : plan_gemm_f32(n_rbs[i], Ks[i], slots);
+  for (int i = 0; i < 6; ++i) c->plan_pf[i] = m->weight_dtype ? plan_gemm(n_rbs[i], Ks[i], slots, false) : c->plan[i];
   if (kTune) {  // tuning aid: cluster size of GEMM i from LOOPSPEC_CS_i
     for (int i = 0; i < 6; ++i) {
       char name[32];
@@ -1995,7 +2006,7 @@ int loopspec_op_linear(const void* W, int32_t weight_dtype, const float* x, floa
   if (!scratch || scratch_bytes < need || (reinterpret_cast<uintptr_t>(scratch) & 15)) return LOOPSPEC_ECAPACITY;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const int ng = ng_for_rows(M);
-  GemmPlan g = plan_gemm((N + 127) / 128, K, 148 * kCtasPerSm, true);
+  GemmPlan g = weight_dtype ? plan_gemm((N + 127) / 128, K, 148 * kCtasPerSm, true) : plan_gemm_f32((N + 127) / 128, K, 148 * kCtasPerSm);
   // Up to 16 rows: one launch that splits x itself.  Beyond, every warp would read and split more of x than it reads of W, and
   // the cluster GEMM on planes made once is the faster one.
   if (weight_dtype == 1 && ng <= 2 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(W)) & 15) == 0) {
