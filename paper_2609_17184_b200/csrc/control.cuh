@@ -10,7 +10,7 @@ namespace ls {
 constexpr int CTRL_THREADS = 256;
 constexpr int MAX_NODES = 512;   // max_seqs * nodes-per-sequence
 enum { PH_ADVANCE = 1, PH_VERIFY = 2, PH_BUILD = 4 };
-enum { HF_ERROR = 0, HF_MIN_DEC = 1, HF_N_ROWS = 2, HF_NEED_VERIFY = 3, HF_FIRST_TOKEN = 4, HF_COUNT = 8 };
+enum { HF_ERROR = 0, HF_N_ROWS = 2, HF_NEED_VERIFY = 3, HF_FIRST_TOKEN = 4, HF_COUNT = 8 };
 enum { ERR_NODES = 1, ERR_CTX = 2, ERR_SPEC = 3, ERR_WAIT = 4 /* bounded wait, decode GEMM */, ERR_WAIT_PF = 5 /* prefill GEMM, grid barrier */ };
 
 struct ControlParams {
@@ -46,43 +46,21 @@ struct ControlParams {
   int hid_coda_base;   // first hidden-state index of the coda pass's copies
 };
 
-// Sub-pass tables of the Raven-style layout, derived from the pass's rows (thread 0, straight to global memory).
-// class_of_readout: RO_D1 -> coda cache 1, RO_D2 -> 2, RO_VERIFY / RO_TARGET -> the last one (its plane index + 1 is `r`).
-__device__ void derive_raven_tables(const RowTable& t, RowTable* pre, RowTable* coda, int hid_coda_base, int n_classes) {
-  auto copy_row = [&](RowTable* dst, int j, int i) {
-    dst->seq[j] = t.seq[i], dst->pos[j] = t.pos[i], dst->kv_slot[j] = t.kv_slot[i], dst->n_canon[j] = t.n_canon[i];
-    dst->n_spec[j] = t.n_spec[i], dst->n_safe[j] = t.n_safe[i], dst->node[j] = t.node[i], dst->logit_idx[j] = t.logit_idx[i];
-    for (int k = 0; k < MAX_SPEC; ++k) dst->spec_slot[j][k] = t.spec_slot[i][k];
-  };
+// Post-layers table of a vanilla token in the Raven-style layout, derived from the last recurrence's rows (thread 0): every row reads
+// out from the last cache (its plane index + 1 is `r`) on a copy of its state.
+__device__ void derive_coda_table(const RowTable& t, RowTable* coda, int hid_coda_base, int n_classes) {
   int items = 0;
-  if (pre) {
-    int np = 0;
-    for (int i = 0; i < t.n_rows; ++i) {
-      if (t.r[i] != 1) continue;  // P runs once per branch, before its first recurrence
-      copy_row(pre, np, i);
-      pre->r[np] = 1, pre->hid_idx[np] = t.hid_idx[i], pre->src_hid[np] = -1, pre->readout[np] = RO_NONE;
-      pre->chunk_start[np] = items;
-      items += att_items(t.n_canon[i], t.att_mode);
-      ++np;
-    }
-    pre->chunk_start[np] = items;
-    pre->n_rows = np, pre->n_readout = 0, pre->attn_items = items, pre->att_mode = t.att_mode;
-  }
-  int nc = 0;
-  items = 0;
   for (int j = 0; j < t.n_readout; ++j) {
     const int i = t.ro_rows[j];
-    copy_row(coda, nc, i);
-    const int ro = t.readout[i];
-    coda->r[nc] = ro == RO_D1 ? 1 : (ro == RO_D2 ? 2 : n_classes);
-    coda->hid_idx[nc] = hid_coda_base + nc, coda->src_hid[nc] = t.hid_idx[i];
-    coda->readout[nc] = ro, coda->ro_rows[nc] = nc;
-    coda->chunk_start[nc] = items;
+    coda->seq[j] = t.seq[i], coda->pos[j] = t.pos[i], coda->kv_slot[j] = t.kv_slot[i], coda->n_canon[j] = t.n_canon[i];
+    coda->n_spec[j] = 0, coda->n_safe[j] = t.n_safe[i], coda->node[j] = t.node[i], coda->logit_idx[j] = t.logit_idx[i];
+    coda->r[j] = n_classes, coda->hid_idx[j] = hid_coda_base + j, coda->src_hid[j] = t.hid_idx[i];
+    coda->readout[j] = t.readout[i], coda->ro_rows[j] = j;
+    coda->chunk_start[j] = items;
     items += att_items(t.n_canon[i], t.att_mode);
-    ++nc;
   }
-  coda->chunk_start[nc] = items;
-  coda->n_rows = nc, coda->n_readout = nc, coda->attn_items = items, coda->att_mode = t.att_mode;
+  coda->chunk_start[t.n_readout] = items;
+  coda->n_rows = t.n_readout, coda->n_readout = t.n_readout, coda->attn_items = items, coda->att_mode = t.att_mode;
 }
 
 struct NodeSmem {
@@ -130,161 +108,218 @@ __device__ __forceinline__ void embed_rows(const int (*list)[2], int n, float* h
   }
 }
 
-__device__ __forceinline__ int alloc_node(int* state, int NB) {
-  for (int i = 0; i < NB; ++i)
+__device__ __forceinline__ int alloc_node(const int* state, int NB, int from = 0) {  // lowest free node at or beyond `from`
+  for (int i = from; i < NB; ++i)
     if (!state[i]) return i;
   return -1;
 }
 
-// Fill the row table from the active branches (thread 0; tables live in shared memory).
-__device__ void build_rows(RowTable& t, const NodeSmem& nd, const int* root, const int* n_dec, const int* n_target,
-                           const ControlParams& p, int* err) {
-  int n_rows = 0, n_ro = 0, items = 0;
-  for (int s = 0; s < p.S; ++s) {
-    if (root[s] < 0 || n_dec[s] >= n_target[s]) continue;
-    const int o = s * p.NB;
-    const int rt = root[s];
-    for (int n = 0; n < p.NB; ++n) {
-      if (!nd.state[o + n]) continue;
-      if (n_rows >= MAX_ROWS) { *err = ERR_NODES; break; }
-      // a position outside the KV pool is never scheduled (the host refuses such a decode before it starts; this is
-      // the second line of defence): the branch stays where it is and the flag tells the host
-      if (nd.pos[o + n] + 2 >= p.ctx_cap) { *err = ERR_CTX; continue; }
-      const int i = n_rows++;
-      const int r = nd.depth[o + n] + 1;
-      const bool is_root = nd.parent[o + n] < 0;
-      t.seq[i] = s, t.r[i] = r, t.pos[i] = nd.pos[o + n], t.node[i] = o + n, t.hid_idx[i] = o + n;
-      t.kv_slot[i] = is_root ? nd.pos[o + n] : p.ctx_cap + n;
-      t.src_hid[i] = -1;
-      t.n_canon[i] = nd.pos[o + rt] + 1;
-      t.n_safe[i] = is_root ? nd.pos[o + n] : t.n_canon[i];
-      int chain[MAX_SPEC], len = 0;
-      for (int a = n; a >= 0 && nd.parent[o + a] >= 0; a = nd.parent[o + a]) {
-        if (len >= MAX_SPEC) { *err = ERR_SPEC; break; }
-        chain[len++] = a;
-      }
-      t.n_spec[i] = len;
-      for (int j = 0; j < len; ++j) t.spec_slot[i][j] = p.ctx_cap + chain[len - 1 - j];
-      int ro = RO_NONE, li = 0;
-      if (r == p.d1) ro = RO_D1, li = (o + n) * 2;
-      else if (p.d2 > 0 && r == p.d2) ro = RO_D2, li = (o + n) * 2 + 1;
-      else if (r == p.R) ro = RO_VERIFY, li = p.p_logit_base + s;
-      t.readout[i] = ro, t.logit_idx[i] = li;
-      if (ro) t.ro_rows[n_ro++] = i;
-      t.chunk_start[i] = items;
-      items += att_items(t.n_canon[i], p.att_mode);
-    }
+// inclusive sum over the CTA of one value per thread, packed fields in 64 bits; s_part: [8] of the warps
+__device__ __forceinline__ unsigned long long ctrl_scan(unsigned long long v, unsigned long long* s_part) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long u = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += u;
   }
-  t.chunk_start[n_rows] = items;
-  t.n_rows = n_rows, t.n_readout = n_ro, t.attn_items = items, t.att_mode = p.att_mode;
+  __syncthreads();  // the previous scan's partials have been read
+  if (lane == 31) s_part[warp] = v;
+  __syncthreads();
+  for (int w = 0; w < warp; ++w) v += s_part[w];
+  return v;
 }
 
-// dynamic shared memory of control_kernel: the branch table, the row table and the per-row selection results
+// Fill the row table from the active branches: one thread per node, in node order (256 nodes at a time); row numbers, readout
+// columns and attention work items are prefix sums.  For the Raven-style layout the same threads write the sub-pass tables: the rows
+// entering their first recurrence (prelude) and the reading-out rows on copies of their states (post-layers).
+__device__ void build_rows(const ControlParams& p, const NodeSmem& nd, const int* root, const int* n_dec, const int* n_target,
+                           unsigned long long* s_part, int* s_err, int* s_n_rows) {
+  RowTable* const t = p.tab;
+  RowTable *const pre = p.tab_pre, *const coda = p.tab_coda;
+  const int n_nodes = p.S * p.NB, n_classes = p.d2 > 0 ? 3 : 2;
+  int rows0 = 0, ros0 = 0, items0 = 0, pres0 = 0, pitems0 = 0, citems0 = 0;
+  __shared__ unsigned long long s_tot[2];
+  for (int base = 0; base < n_nodes; base += CTRL_THREADS) {
+    const int gn = base + threadIdx.x, s = gn / p.NB, n = gn - s * p.NB, o = s * p.NB;
+    bool live = gn < n_nodes && nd.state[gn] && root[s] >= 0 && n_dec[s] < n_target[s];
+    // a position outside the KV pool is never scheduled (the host refuses such a decode before it starts; this is
+    // the second line of defence): the branch stays where it is and the flag tells the host
+    if (live && nd.pos[gn] + 2 >= p.ctx_cap) live = false, *s_err = ERR_CTX;
+    int r = 0, n_canon = 0, items = 0, ro = RO_NONE, li = 0;
+    bool is_root = false;
+    if (live) {
+      r = nd.depth[gn] + 1, is_root = nd.parent[gn] < 0, n_canon = nd.pos[o + root[s]] + 1, items = att_items(n_canon, p.att_mode);
+      if (r == p.d1) ro = RO_D1, li = gn * 2;
+      else if (p.d2 > 0 && r == p.d2) ro = RO_D2, li = gn * 2 + 1;
+      else if (r == p.R) ro = RO_VERIFY, li = p.p_logit_base + s;
+    }
+    const unsigned long long mine = live ? 1ull | (ro ? 1ull << 16 : 0) | ((unsigned long long)items << 32) : 0ull;
+    const unsigned long long sum = ctrl_scan(mine, s_part);
+    if (threadIdx.x == CTRL_THREADS - 1) s_tot[0] = sum;
+    unsigned long long mine2 = 0, sum2 = 0;
+    if (pre) {
+      mine2 = (live && r == 1 ? 1ull | ((unsigned long long)items << 16) : 0ull) | (ro ? (unsigned long long)items << 40 : 0ull);
+      sum2 = ctrl_scan(mine2, s_part);
+      if (threadIdx.x == CTRL_THREADS - 1) s_tot[1] = sum2;
+    }
+    const unsigned long long ex = sum - mine, ex2 = sum2 - mine2;
+    const int i = rows0 + (int)(ex & 0xffff), iro = ros0 + (int)((ex >> 16) & 0xffff), start = items0 + (int)(ex >> 32);
+    if (live && i >= MAX_ROWS) *s_err = ERR_NODES;
+    if (live && i < MAX_ROWS) {
+      int chain[MAX_SPEC], len = 0;
+      for (int a = n; a >= 0 && nd.parent[o + a] >= 0; a = nd.parent[o + a]) {
+        if (len >= MAX_SPEC) { *s_err = ERR_SPEC; break; }
+        chain[len++] = a;
+      }
+      const int kv_slot = is_root ? nd.pos[gn] : p.ctx_cap + n, n_safe = is_root ? nd.pos[gn] : n_canon;
+      auto put = [&](RowTable* d, int k, int plane, int hid, int src, int readout, int at) {
+        d->seq[k] = s, d->r[k] = plane, d->pos[k] = nd.pos[gn], d->node[k] = gn, d->kv_slot[k] = kv_slot, d->n_canon[k] = n_canon;
+        d->n_safe[k] = n_safe, d->n_spec[k] = len, d->hid_idx[k] = hid, d->src_hid[k] = src, d->readout[k] = readout, d->logit_idx[k] = li;
+        d->chunk_start[k] = at;
+        for (int q = 0; q < len; ++q) d->spec_slot[k][q] = p.ctx_cap + chain[len - 1 - q];
+      };
+      put(t, i, r, gn, -1, ro, start);
+      if (ro) t->ro_rows[iro] = i;
+      if (pre && r == 1) put(pre, pres0 + (int)(ex2 & 0xffff), 1, gn, -1, RO_NONE, pitems0 + (int)((ex2 >> 16) & 0xffffff));
+      if (pre && ro) {
+        put(coda, iro, ro == RO_D1 ? 1 : (ro == RO_D2 ? 2 : n_classes), p.hid_coda_base + iro, gn, ro, citems0 + (int)(ex2 >> 40));
+        coda->ro_rows[iro] = iro;
+      }
+    }
+    __syncthreads();
+    rows0 += (int)(s_tot[0] & 0xffff), ros0 += (int)((s_tot[0] >> 16) & 0xffff), items0 += (int)(s_tot[0] >> 32);
+    if (pre) pres0 += (int)(s_tot[1] & 0xffff), pitems0 += (int)((s_tot[1] >> 16) & 0xffffff), citems0 += (int)(s_tot[1] >> 40);
+  }
+  rows0 = min(rows0, MAX_ROWS), ros0 = min(ros0, MAX_ROWS);  // (more: the error flag is up)
+  if (threadIdx.x == 0) {
+    t->n_rows = rows0, t->n_readout = ros0, t->attn_items = items0, t->chunk_start[rows0] = items0, t->att_mode = p.att_mode;
+    if (pre) {
+      pre->n_rows = pres0, pre->n_readout = 0, pre->attn_items = pitems0, pre->chunk_start[pres0] = pitems0, pre->att_mode = p.att_mode;
+      coda->n_rows = coda->n_readout = ros0, coda->attn_items = citems0, coda->chunk_start[ros0] = citems0, coda->att_mode = p.att_mode;
+    }
+    *s_n_rows = rows0;
+  }
+}
+
+// dynamic shared memory of control_kernel: the branch table, what the bookkeeping reads of the row table and of the selection
 struct ControlSmem {
   NodeSmem nd;
-  RowTable t;
   int emb[2 * MAX_ROWS][2];
+  int seq[MAX_ROWS], r[MAX_ROWS], node[MAX_ROWS], readout[MAX_ROWS];
   int sel_tok[MAX_ROWS], sel_aux[MAX_ROWS];
   float sel_lse[MAX_ROWS], sel_z2[MAX_ROWS];
 };
 
+// One CTA, bound by its chains of dependent loads and steps; a thread per sequence takes the decisions, a thread per node prunes
+// and builds rows.  (With thread 0 building all rows and the whole row table - 30 KB - copied in and out: 20 us at one sequence of four rows,
+// 76 us at eight sequences of ~45 rows, serialised.)
 __global__ void __launch_bounds__(CTRL_THREADS) control_kernel(const __grid_constant__ ControlParams p) {
   extern __shared__ __align__(16) unsigned char ctrl_smem_raw[];
   ControlSmem& sm = *reinterpret_cast<ControlSmem*>(ctrl_smem_raw);
   NodeSmem& nd = sm.nd;
-  RowTable& t = sm.t;
   int (*s_emb)[2] = sm.emb;
-  int *s_sel_tok = sm.sel_tok, *s_sel_aux = sm.sel_aux;
-  float *s_sel_lse = sm.sel_lse, *s_sel_z2 = sm.sel_z2;
-  __shared__ int s_root[MAX_SEQS], s_nids[MAX_SEQS], s_ndec[MAX_SEQS], s_ntarget[MAX_SEQS], s_needv[MAX_SEQS];
-  __shared__ int s_nemb, s_err;
-  __shared__ unsigned long long s_steps;
-  __shared__ int s_trace_n;
+  __shared__ int s_root[MAX_SEQS], s_nids[MAX_SEQS], s_ndec[MAX_SEQS], s_ntarget[MAX_SEQS], s_needv[MAX_SEQS], s_keep[MAX_SEQS];
+  __shared__ int s_nemb, s_err, s_need, s_n_rows_new;
+  __shared__ unsigned long long s_part[CTRL_THREADS / 32];
   const int tid = threadIdx.x;
   const int n_nodes = p.S * p.NB;
   tune_mark(603, false);
   pdl_launch_dependents();
-  // Everything the serial bookkeeping reads is pulled into shared memory with one round of parallel loads.  The branch
-  // table, the row table and the sequence state were last written by the previous step, so they are read while this
-  // step's readout kernels are still running; only the selection results have to wait for them.
-  if (tid == CTRL_THREADS - 1) s_steps = p.ctr->steps;
-  if (tid == CTRL_THREADS - 2) s_trace_n = *p.trace_n;
+  // Everything the bookkeeping reads is pulled into shared memory with parallel loads.  The branch table, the row table and
+  // the sequence state were last written by the previous step, so they are read while this step's readout kernels are still
+  // running; only the selection results have to wait for them.
+  const int n_rows = p.tab->n_rows, n_readout = p.tab->n_readout;
+  const unsigned long long steps = p.ctr->steps;
+  const int trace_n = *p.trace_n;
   nodes_load(nd, p.nodes, n_nodes);
-  {
-    const int* src = reinterpret_cast<const int*>(p.tab);
-    int* dst = reinterpret_cast<int*>(&t);
-    for (int i = tid; i < (int)(sizeof(RowTable) / 4); i += CTRL_THREADS) dst[i] = src[i];
-  }
+  for (int i = tid; i < n_rows; i += CTRL_THREADS)
+    sm.seq[i] = p.tab->seq[i], sm.r[i] = p.tab->r[i], sm.node[i] = p.tab->node[i], sm.readout[i] = p.tab->readout[i];
   if (tid < p.S) {
     s_root[tid] = p.seqs.root[tid], s_nids[tid] = p.seqs.n_ids[tid], s_ndec[tid] = p.seqs.n_dec[tid];
     s_ntarget[tid] = p.seqs.n_target[tid], s_needv[tid] = p.seqs.need_verify[tid];
   }
+  if (tid == 0) s_nemb = 0, s_err = 0, s_need = 0, s_n_rows_new = n_rows;
   pdl_wait();
-  for (int i = tid; i < MAX_ROWS; i += CTRL_THREADS) {
-    s_sel_tok[i] = p.sel_tok[i], s_sel_aux[i] = p.sel_aux[i];
-    s_sel_lse[i] = p.sel_lse[i], s_sel_z2[i] = p.sel_z2[i];
-  }
-  if (tid == 0) s_nemb = 0, s_err = 0;
+  for (int i = tid; i < n_rows; i += CTRL_THREADS)
+    sm.sel_tok[i] = p.sel_tok[i], sm.sel_aux[i] = p.sel_aux[i], sm.sel_lse[i] = p.sel_lse[i], sm.sel_z2[i] = p.sel_z2[i];
   __syncthreads();
 
+  bool commit = false;  // this thread's sequence commits a token
   if (tid < p.S) {
     const int s = tid, o = s * p.NB;
     int* st = nd.state + o;
     // ---- advance, first proposal at d1, gated second proposal at d2 (Algorithm 1 main loop body) ----
+    int vrow = -1, from = 0;
     if (p.phases & PH_ADVANCE) {
-      for (int i = 0; i < t.n_rows; ++i)
-        if (t.seq[i] == s) nd.depth[t.node[i]] = t.r[i];
-      for (int i = 0; i < t.n_rows; ++i) {
-        if (t.seq[i] != s) continue;
-        const int gn = t.node[i], ro = t.readout[i];
-        if (ro == RO_D1 || (ro == RO_D2 && s_sel_aux[i])) {
-          int c = alloc_node(st, p.NB);
-          if (c < 0) { s_err = ERR_NODES; continue; }
-          st[c] = 1, nd.depth[o + c] = 0, nd.pos[o + c] = nd.pos[gn] + 1, nd.token[o + c] = s_sel_tok[i];
-          nd.parent[o + c] = gn - o, nd.child1[o + c] = nd.child2[o + c] = -1, nd.has2[o + c] = 0;
-          if (ro == RO_D1) {
-            nd.tok1[gn] = s_sel_tok[i], nd.child1[gn] = c, nd.lse1[gn] = s_sel_lse[i], nd.has2[gn] = 0, nd.child2[gn] = -1;
-            if (p.sel_flt) p.nodes.flt1[gn] = p.sel_flt[i];
-          } else {
-            nd.tok2[gn] = s_sel_tok[i], nd.child2[gn] = c, nd.lse2[gn] = s_sel_lse[i], nd.z2[gn] = s_sel_z2[i], nd.has2[gn] = 1;
-            if (p.sel_flt) p.nodes.flt2[gn] = p.sel_flt[i];
-            atomicAdd(&p.ctr->gate_opens, 1ull);
-          }
-          int e = atomicAdd(&s_nemb, 1);
-          s_emb[e][0] = o + c, s_emb[e][1] = s_sel_tok[i];
+      for (int i = 0; i < n_rows; ++i)
+        if (sm.seq[i] == s) nd.depth[sm.node[i]] = sm.r[i];
+    }
+    for (int i = 0; i < n_rows; ++i) {
+      const int ro = sm.readout[i];
+      if (ro == RO_NONE || sm.seq[i] != s) continue;
+      if (ro == RO_VERIFY) vrow = i;
+      if (!(p.phases & PH_ADVANCE)) continue;
+      const int gn = sm.node[i];
+      if (ro == RO_D1 || (ro == RO_D2 && sm.sel_aux[i])) {
+        const int c = alloc_node(st, p.NB, from);  // (nothing is freed here: nodes before the last one handed out are taken)
+        if (c < 0) { s_err = ERR_NODES; continue; }
+        from = c + 1;
+        st[c] = 1, nd.depth[o + c] = 0, nd.pos[o + c] = nd.pos[gn] + 1, nd.token[o + c] = sm.sel_tok[i];
+        nd.parent[o + c] = gn - o, nd.child1[o + c] = nd.child2[o + c] = -1, nd.has2[o + c] = 0;
+        if (ro == RO_D1) {
+          nd.tok1[gn] = sm.sel_tok[i], nd.child1[gn] = c, nd.lse1[gn] = sm.sel_lse[i], nd.has2[gn] = 0, nd.child2[gn] = -1;
+          if (p.sel_flt) p.nodes.flt1[gn] = p.sel_flt[i];
+        } else {
+          nd.tok2[gn] = sm.sel_tok[i], nd.child2[gn] = c, nd.lse2[gn] = sm.sel_lse[i], nd.z2[gn] = sm.sel_z2[i], nd.has2[gn] = 1;
+          if (p.sel_flt) p.nodes.flt2[gn] = p.sel_flt[i];
+          atomicAdd(&p.ctr->gate_opens, 1ull);
         }
-        if (ro == RO_D2) atomicAdd(&p.ctr->gate_evals, 1ull);
-        if (ro == RO_VERIFY) s_needv[s] = 1;
+        int e = atomicAdd(&s_nemb, 1);
+        s_emb[e][0] = o + c, s_emb[e][1] = sm.sel_tok[i];
       }
+      if (ro == RO_D2) atomicAdd(&p.ctr->gate_evals, 1ull);
+      if (ro == RO_VERIFY) s_needv[s] = 1;
     }
     // ---- the deepest branch reached R: commit and Reroot ---------------------------------------------
     p.kvcopy[s].n_planes = 0;
+    s_keep[s] = -2;  // nothing to prune
     if ((p.phases & PH_VERIFY) && s_needv[s]) {
-      int vrow = -1;
-      for (int i = 0; i < t.n_rows; ++i)
-        if (t.seq[i] == s && t.readout[i] == RO_VERIFY) vrow = i;
+      commit = true;
       const int rt = s_root[s];
-      const int tok = s_sel_tok[vrow], src = s_sel_aux[vrow];
+      const int tok = sm.sel_tok[vrow], src = sm.sel_aux[vrow];
       const int k = s_ndec[s];
       if (k < p.ids_cap) {
         p.out_ids[(size_t)s * p.ids_cap + k] = tok;
         int* cm = p.commits + ((size_t)s * p.ids_cap + k) * 8;
         cm[0] = s, cm[1] = 1, cm[2] = tok, cm[3] = src, cm[4] = (src == 1), cm[5] = (src == 2), cm[6] = nd.has2[o + rt];
-        cm[7] = (int)s_steps + ((p.phases & PH_ADVANCE) ? 1 : 0);
+        cm[7] = (int)steps + ((p.phases & PH_ADVANCE) ? 1 : 0);
       }
       s_ndec[s] = k + 1, s_nids[s] += 1;
       atomicAdd(&p.ctr->n_decode, 1ull);
       atomicAdd(src == 1 ? &p.ctr->n_accept1 : (src == 2 ? &p.ctr->n_accept2 : &p.ctr->n_restart), 1ull);
-      const int keep = src == 1 ? nd.child1[o + rt] : (src == 2 ? nd.child2[o + rt] : -1);
-      const int new_pos = nd.pos[o + rt] + 1;
-      for (int n = 0; n < p.NB; ++n) {
-        if (!st[n]) continue;
-        bool in = false;
-        for (int a = n; a >= 0; a = nd.parent[o + a])
-          if (a == keep) { in = true; break; }
-        if (!in) st[n] = 0;
-      }
-      if (keep < 0) {  // restart: fresh branch on the verified prefix
+      s_keep[s] = src == 1 ? nd.child1[o + rt] : (src == 2 ? nd.child2[o + rt] : -1);
+    }
+  }
+  __syncthreads();
+  for (int gn = tid; gn < n_nodes; gn += CTRL_THREADS) {  // branches outside the kept subtree are released
+    const int s = gn / p.NB, o = s * p.NB, keep = s_keep[s];
+    if (keep == -2 || !nd.state[gn]) continue;
+    bool in = false;
+    for (int a = gn - o; a >= 0; a = nd.parent[o + a])
+      if (a == keep) { in = true; break; }
+    if (!in) nd.state[gn] = 0;
+  }
+  __syncthreads();
+  if (tid < p.S) {
+    const int s = tid, o = s * p.NB;
+    if (commit) {
+      int* st = nd.state + o;
+      const int keep = s_keep[s];
+      if (keep < 0) {  // restart: fresh branch on the verified prefix (the committed token is the last of the ids written above)
+        int vrow = -1;
+        for (int i = 0; i < n_rows; ++i)
+          if (sm.readout[i] == RO_VERIFY && sm.seq[i] == s) vrow = i;
+        const int tok = sm.sel_tok[vrow], new_pos = nd.pos[o + s_root[s]] + 1;
         const int c = alloc_node(st, p.NB);
         st[c] = 1, nd.depth[o + c] = 0, nd.pos[o + c] = new_pos, nd.token[o + c] = tok, nd.parent[o + c] = -1;
         nd.child1[o + c] = nd.child2[o + c] = -1, nd.has2[o + c] = 0;
@@ -299,43 +334,30 @@ __global__ void __launch_bounds__(CTRL_THREADS) control_kernel(const __grid_cons
       }
       s_needv[s] = 0;
     }
+    if (s_needv[s]) atomicAdd(&s_need, s_needv[s]);
   }
   __syncthreads();
-  if (tid == 0) {
-    if (p.phases & PH_ADVANCE) {  // counters: no value is read back, so nothing here waits for memory
-      atomicAdd(&p.ctr->steps, 1ull), atomicAdd(&p.ctr->rows_total, (unsigned long long)t.n_rows);
-      atomicAdd(&p.ctr->readout_rows_total, (unsigned long long)t.n_readout);
-      atomicMax(&p.ctr->rows_max, (unsigned long long)t.n_rows);
-      const int k = s_trace_n;
-      if (k < p.trace_cap) p.row_trace[k] = t.n_rows;
-      *p.trace_n = k + 1;
-    }
-    int need = 0, min_dec = 0x7fffffff;
-    for (int s = 0; s < p.S; ++s) {
-      need += s_needv[s];
-      if (s_root[s] >= 0) min_dec = min(min_dec, s_ndec[s]);
-    }
-    int err = s_err;
-    // rows are rebuilt only when no verification is pending (the verify phase needs the current rows)
-    if ((p.phases & PH_BUILD) && need == 0) {
-      build_rows(t, nd, s_root, s_ndec, s_ntarget, p, &err);
-      if (p.tab_pre) derive_raven_tables(t, p.tab_pre, p.tab_coda, p.hid_coda_base, p.d2 > 0 ? 3 : 2);
-    }
-    p.host_flags[HF_MIN_DEC] = min_dec, p.host_flags[HF_N_ROWS] = t.n_rows, p.host_flags[HF_NEED_VERIFY] = need;
-    if (err) p.host_flags[HF_ERROR] = err;
-  }
-  __syncthreads();
+  // rows are rebuilt only when no verification is pending (the verify phase needs the current rows)
+  if ((p.phases & PH_BUILD) && s_need == 0) build_rows(p, nd, s_root, s_ndec, s_ntarget, s_part, &s_err, &s_n_rows_new);
   nodes_store(nd, p.nodes, n_nodes);
-  {
-    int* dst = reinterpret_cast<int*>(p.tab);
-    const int* src = reinterpret_cast<const int*>(&t);
-    for (int i = tid; i < (int)(sizeof(RowTable) / 4); i += CTRL_THREADS) dst[i] = src[i];
-  }
   if (tid < p.S) {
     p.seqs.root[tid] = s_root[tid], p.seqs.n_ids[tid] = s_nids[tid], p.seqs.n_dec[tid] = s_ndec[tid];
     p.seqs.need_verify[tid] = s_needv[tid];
   }
   embed_rows(s_emb, s_nemb, p.hid, p.H, p.embed, p.weight_dtype);
+  __syncthreads();
+  if (tid == 0) {
+    if (p.phases & PH_ADVANCE) {  // counters: no value is read back, so nothing here waits for memory
+      atomicAdd(&p.ctr->steps, 1ull), atomicAdd(&p.ctr->rows_total, (unsigned long long)n_rows);
+      atomicAdd(&p.ctr->readout_rows_total, (unsigned long long)n_readout);
+      atomicMax(&p.ctr->rows_max, (unsigned long long)n_rows);
+      if (trace_n < p.trace_cap) p.row_trace[trace_n] = n_rows;
+      *p.trace_n = trace_n + 1;
+    }
+    // the host reads these after a phase it launched by itself, not in a captured step
+    if ((p.phases & (PH_ADVANCE | PH_VERIFY)) != (PH_ADVANCE | PH_VERIFY)) p.host_flags[HF_N_ROWS] = s_n_rows_new, p.host_flags[HF_NEED_VERIFY] = s_need;
+    if (s_err) p.host_flags[HF_ERROR] = s_err;
+  }
   tune_mark(603, true);
 }
 
@@ -413,7 +435,7 @@ __global__ void __launch_bounds__(CTRL_THREADS) vanilla_control_kernel(const __g
       t.n_rows = n, t.n_readout = (r == p.R) ? n : 0, t.attn_items = items, t.att_mode = p.att_mode;
     }
     if (p.tab_coda) {  // the prelude pass of a vanilla token is the first table itself (every row enters recurrence 1)
-      derive_raven_tables(p.tabs[p.R - 1], nullptr, p.tab_coda, p.hid_coda_base, p.n_classes);
+      derive_coda_table(p.tabs[p.R - 1], p.tab_coda, p.hid_coda_base, p.n_classes);
     }
   }
   __syncthreads();
