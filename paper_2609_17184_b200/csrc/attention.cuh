@@ -3,10 +3,10 @@
 // committed slots [0, n_canon) of plane r plus the speculative slots of its uncommitted ancestors and itself.
 //
 // Three kernels, by regime:
-//   attn_kernel          work item = (row, kv head, chunk of ATT_CHUNK key positions): every chunk in parallel, for the few
-//                        rows and short contexts of a single sequence's decode pass (latency matters);
-//   attn_runs_kernel     work item = (row, kv head, run of chunks) streamed through a per-thread cp.async ring: long
-//                        contexts and contexts of several sequences (bandwidth matters);
+//   attn_kernel          work item = (row, kv head, chunk of ATT_CHUNK key positions): one CTA each, every chunk in parallel, for
+//                        the few rows and short contexts of a single sequence's decode pass (latency matters);
+//   attn_warp_kernel     work item = (row, kv head, run of chunks): one warp each, on the tensor cores; long contexts and
+//                        contexts of several sequences (bandwidth and the number of items matter);
 //   attn_prefill_mma_kernel  work item = (query head, block of rows, run of chunks) for the consecutive positions of a prefill
 //                        pass, which share their keys and values.
 // Chunks and runs are cut at fixed absolute positions (or as a function of the row's own context) and folded in
@@ -279,349 +279,383 @@ __global__ void __launch_bounds__(ATT_THREADS, 4) attn_kernel(const __grid_const
   timeline_mark(p.tl, p.tl_id, true);
 }
 
-// The same attention for contexts whose rows can have more chunks than single-chunk items are cut for (more than
-// ATT_MAX_RUNS chunks; more than ATT_BATCH_SINGLE in contexts of several sequences): a work item is a run of consecutive
-// chunks (a function of the row's own context only), so that the per-item costs (row lookup, partial write, counter) are paid
-// once per run and a (row, kv head) never has more than ATT_MAX_RUNS partials.  This is the kernel of the KV-bound
-// regime, built to stream: every thread owns a ring of (key piece, value piece) slots in shared memory that it fills
-// with cp.async and reads back itself, so the K/V of the next rounds are in flight while the current one is used and
-// the main loop has no block-wide barrier.  A key position is shared by the D/8 lanes of a group, 8 dims each (groups
-// of 4 lanes with D/4 dims each need fewer shuffles and softmax updates per byte but leave too few warps to hide
-// their longer dependent chains: 3.6 TB/s against 5.6 TB/s measured on 34 rows x 8192 positions).  Each lane group keeps
-// a running softmax (max, mass, weighted values) over the positions it is dealt - position j of a chunk always goes
-// to group j mod PPR - the groups of a warp are folded by a fixed butterfly, the warps in ascending order, once per
-// run.  Kept apart from attn_kernel, whose single-chunk items are the ones the batch-1 decode uses.
+// ======================= decode attention on the tensor cores, one warp per item =====================================
+// A work item is a run of consecutive chunks of one (row, kv head), cut as att_run_len says (a function of the row's own
+// context); ONE warp streams it in tiles of 16 keys and keeps the running softmax, so nothing is folded across warps and no block
+// barrier is met.  A CTA per item on the CUDA cores spends some 40 warp instructions on a key and 400 per item and warp; with many
+// rows of short contexts that, not the stream, bounds it.  Here a tile is one mma.sync per 16 dims for the scores and one per 16
+// dims for the values: K rows (V columns, by transposing ldmatrix) are the 16-row A operand, the query (the softmax weights) the
+// columns - for G = 1 its three exact bf16 planes as columns 0 .. 2, for G = 4 the heads as columns 0 .. 3 with the planes one
+// after the other into the same accumulator.  Every warp owns a ring of two tiles in shared memory, filled by its own cp.async
+// across items; rows are swizzled in 16-byte pieces (ldmatrix without bank conflicts).
+// A lone warp takes 1200 cycles per tile (310 issue the copies, 850 are the chain scores - softmax - values) and 4000 to 8000 per
+// item around them, so what counts is that all items are resident at once: 12 warps per SM with tiles of 16 keys beat 6 with
+// tiles of 32 [48 rows x 510 positions: 25.7 / 42.1 us] and 8 with three tiles each; deeper rings for few items change nothing.
+// Alone, one CTA per run (CUDA cores) -> this kernel: 40 rows x 536 positions 61 -> 43 us, 24 rows 39 -> 23, 48 rows x 446
+// 64 -> 26, 40 rows x 86 22 -> 12, 28 rows x 1036 69 -> 42, 14 rows x 8400 179 -> 154 us (6.25 TB/s).
 template <int D, int G>
-struct AtsCfg {
-  static constexpr int NP = 1;                     // 16-byte pieces of a key (and of a value) per lane
-  static constexpr int DPL = 8 * NP;               // dims per lane
-  static constexpr int LPP = D / DPL;              // lanes per key position
-  static constexpr int PPW = 32 / LPP;             // positions per warp per round
-  static constexpr int PPR = PPW * (ATT_THREADS / 32);  // positions per round of the whole CTA
-  static constexpr int UNIT_BYTES = 2 * NP * ATT_THREADS * 16;  // one round of the CTA: K and V pieces of every thread
-  static constexpr int MIN_CTAS = G == 1 ? 4 : 2;  // per SM (grouped-query attention keeps G accumulators per lane)
-  static constexpr int UNITS = (G == 1 ? 48 : 96) * 1024 / UNIT_BYTES;  // ring depth: 48 KB in flight per CTA
-  static constexpr int COMB_BYTES = (ATT_THREADS / 32) * G * (D + 2) * 4;
-  static constexpr int SMEM_BYTES = UNITS * UNIT_BYTES + COMB_BYTES;
+struct AtwCfg {
+    static constexpr int WARPS = 4, STAGES = 2, CTAS = 3, MT = 1;  // CTAS: per SM; MT: mma row tiles (of 16 keys) in a tile
+  static constexpr int ROWB = D * 2, KEYS = 16 * MT, TILE = KEYS * ROWB;  // bytes of a key row; keys of a tile and their bytes (values the same)
+  static constexpr int QBYTES = G * D * 4;                 // an item's queries
+  static constexpr int SMEM_BYTES = WARPS * STAGES * (2 * TILE + QBYTES);
 };
 
+__device__ __forceinline__ void att_ldsm4(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void att_ldsm4_t(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void att_mma(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
 template <int D, int G>
-__global__ void __launch_bounds__(ATT_THREADS, (AtsCfg<D, G>::MIN_CTAS)) attn_runs_kernel(const __grid_constant__ AttnParams p) {
-  using C = AtsCfg<D, G>;
-  constexpr int NP = C::NP, DPL = C::DPL, LPP = C::LPP, PPW = C::PPW, PPR = C::PPR, UNITS = C::UNITS;
-  constexpr int PSTRIDE = D + 2;
-  constexpr int EPT = (G * D + ATT_THREADS - 1) / ATT_THREADS;  // output elements (head, dim) a thread folds
-  constexpr unsigned PIECE = ATT_THREADS * 16, V_OFF = NP * PIECE, UNIT_BYTES = C::UNIT_BYTES, RING_BYTES = UNITS * UNIT_BYTES;
+__global__ void __launch_bounds__(AtwCfg<D, G>::WARPS * 32) attn_warp_kernel(const __grid_constant__ AttnParams p) {
+  using C = AtwCfg<D, G>;
+  static_assert(G == 1 || G == 4, "query heads per kv head");
+  constexpr int PSTRIDE = D + 2, KS = D / 16, PCS = D / 8, NP = G == 1 ? 1 : 3;  // NP: column sets of a k-step (G = 1: planes are columns)
+  constexpr int LI = C::KEYS * PCS / 32, MT = C::MT, RPI = 32 / PCS, SW = 8 / RPI;  // copies of keys per lane and tile, rows a copy of the warp covers, their swizzles
+  extern __shared__ __align__(128) unsigned char atw_smem[];
+  const RowTable* tab = p.tab;  // written before this pass started: safe to read ahead of the predecessor
+  const int n_rows = tab->n_rows, HQ = p.n_q_heads * D;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int total = tab->attn_items * p.n_kv_heads, n_warps = gridDim.x * C::WARPS, first = warp * gridDim.x + blockIdx.x;  // (few items: one per SM first)
+  const unsigned ring = (unsigned)__cvta_generic_to_shared(atw_smem) + warp * C::STAGES * 2 * C::TILE;
+  float* const qring = reinterpret_cast<float*>(atw_smem + C::WARPS * C::STAGES * 2 * C::TILE) + warp * C::STAGES * (G * D);
+  auto piece = [](int row, int c) { return (unsigned)(row * C::ROWB + ((c ^ (row & 7)) << 4)); };
+  // this lane's row address of the fragment loads (dims 0 .. 15; the piece of a later k-step is two on: an XOR, the tiles being aligned)
+  const unsigned k_lane = piece(lane & 15, lane >> 4), v_lane = piece((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1);
+  unsigned l_dst[SW];
+#pragma unroll
+  for (int i = 0; i < SW; ++i) l_dst[i] = (lane / PCS) * C::ROWB + (((lane % PCS) ^ ((lane / PCS + i * RPI) & 7)) << 4);
 
-  extern __shared__ __align__(16) unsigned char ats_smem[];
-  float* s_comb = reinterpret_cast<float*>(ats_smem + RING_BYTES);  // [warp][G][PSTRIDE]
-  __shared__ int s_last;
-
-  timeline_mark(p.tl, p.tl_id, false);
-  const RowTable* tab = p.tab;   // written before this pass started: safe to read ahead of the predecessor
-  const int n_rows = tab->n_rows;
-  const int HQ = p.n_q_heads * D;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int sub = lane / LPP, dl = lane % LPP;  // which position of the warp's group, which DPL-dim slice
-  const int jl = warp * PPW + sub;              // this lane group's position within a round
-  const int total = tab->attn_items * p.n_kv_heads;
-  const unsigned ring_s = (unsigned)__cvta_generic_to_shared(ats_smem) + tid * 16;
-  bool waited = false;
-
-  struct Cursor {  // a round of a chunk of the run, with the chunk's geometry
-    int chunk, rd, n_can, n_here, n_safe, rounds;
-  };
-  for (int item = blockIdx.x; item < total; item += gridDim.x) {
-    const int kvh = item % p.n_kv_heads;
+  // an item's keys: n_can committed ones from position p0 on, then (last run of the row) the speculative slots
+  auto locate = [&](int item, int& row, int& kvh, int& run, int& p0, int& n_can, int& n_keys) {
     const int rr = item / p.n_kv_heads;
-    int row = 0;
-    {  // the row whose items contain rr (binary search over the prefix sums)
-      int hi = n_rows - 1;
-      while (row < hi) {
-        const int mid = (row + hi + 1) >> 1;
-        if (tab->chunk_start[mid] <= rr) row = mid;
-        else hi = mid - 1;
+    kvh = item - rr * p.n_kv_heads;
+    row = -1;  // the row whose items contain rr: as many rows start at or before it (one round trip to the table, not a search's five)
+    for (int b = 0; b < n_rows; b += 32) row += __popc(__ballot_sync(0xffffffffu, b + lane < n_rows && tab->chunk_start[b + lane] <= rr));
+    run = rr - tab->chunk_start[row];
+    const int nc = tab->n_canon[row], len = att_run_len(nc, tab->att_mode) * ATT_CHUNK;
+    p0 = run * len;
+    n_can = min(len, nc - p0);
+    n_keys = n_can + (p0 + len >= nc ? tab->n_spec[row] : 0);
+  };
+  // ---- ring, issue side: tiles of this warp's items in order, running ahead across items ----------------------------------
+  int i_item = first, i_row = 0, i_p0 = 0, i_can = 0, i_keys = 0, i_j = 0;
+  const __nv_bfloat16* i_kb = p.kv;
+  auto i_setup = [&]() {
+    int kvh, run;
+    locate(i_item, i_row, kvh, run, i_p0, i_can, i_keys);
+    i_kb = p.kv + (size_t)(tab->r[i_row] - 1) * p.kv_plane_stride + (size_t)(tab->seq[i_row] * p.n_kv_heads + kvh) * p.slots * D;
+    i_j = 0;
+  };
+  if (i_item < total) i_setup();
+  unsigned i_st = 0, c_st = 0;
+  int i_q = 0, c_q = 0;        // query slot of the item being issued / consumed
+  bool queries = false;        // the queries exist (they are this pass's: not ahead of the dependency wait)
+  auto issue_q = [&](int row, int kvh, int qs) {
+    for (int i = lane; i < G * D / 4; i += 32)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(qring + qs * (G * D) + i * 4)),
+                   "l"(p.qbuf + (size_t)row * HQ + (size_t)kvh * G * D + i * 4)
+                   : "memory");
+  };
+  auto issue = [&]() {
+    if (i_item < total) {
+      if (i_j == 0 && queries) issue_q(i_row, i_item % p.n_kv_heads, i_q);
+      if (i_j + C::KEYS <= i_can) {  // a full tile of committed keys: constant strides from this lane's first piece
+        const __nv_bfloat16* k0 = i_kb + (size_t)(i_p0 + i_j) * D + lane * 8;
+        const __nv_bfloat16* v0 = k0 + p.kv_sel_stride;
+#pragma unroll
+        for (int i = 0; i < LI; ++i) {
+          const unsigned dst = ring + i_st + i * RPI * C::ROWB + l_dst[i % SW];
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(k0 + i * 256) : "memory");
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + C::TILE), "l"(v0 + i * 256) : "memory");
+        }
+      } else {
+#pragma unroll 1
+        for (int i = 0; i < LI; ++i) {
+          const int r = lane / PCS + i * RPI, c = lane % PCS, j = i_j + r;
+          const bool live = j < i_keys;  // keys beyond the item: zeros
+          const int slot = j < i_can ? i_p0 + j : (live ? tab->spec_slot[i_row][j - i_can] : 0);
+          const __nv_bfloat16* src = i_kb + (size_t)slot * D + c * 8;
+          const unsigned dst = ring + i_st + piece(r, c);
+          const int n = live ? 16 : 0;
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + C::TILE), "l"(src + p.kv_sel_stride), "r"(n) : "memory");
+        }
+      }
+      i_j += C::KEYS;
+      if (i_j >= i_keys) {
+        i_item += n_warps;
+        if (++i_q == C::STAGES) i_q = 0;
+        if (i_item < total) i_setup();
       }
     }
-    const int run = rr - tab->chunk_start[row];
-    const int n_runs = tab->chunk_start[row + 1] - tab->chunk_start[row];
-    const int n_canon = tab->n_canon[row];
-    const int n_chunks = (n_canon + ATT_CHUNK - 1) / ATT_CHUNK;
-    const int run_len = att_run_len(n_canon, tab->att_mode);
-    const int chunk_lo = run * run_len, chunk_hi = min(n_chunks, chunk_lo + run_len);
-    const int row_spec = tab->n_spec[row], row_safe = tab->n_safe[row];
-
-    const size_t plane = (size_t)(tab->r[row] - 1) * p.kv_plane_stride;
-    const size_t headbase = (size_t)(tab->seq[row] * p.n_kv_heads + kvh) * p.slots * D;
-    const __nv_bfloat16* Kb = p.kv + plane + headbase + dl * DPL;
-    const __nv_bfloat16* Vb = Kb + p.kv_sel_stride;
-
-    auto setup = [&](Cursor& c, int chunk) {
-      const int p0 = chunk * ATT_CHUNK;
-      const int n_spec = (chunk == n_chunks - 1) ? row_spec : 0;  // the last chunk of a row also carries its speculative slots
-      c.chunk = chunk, c.rd = 0;
-      c.n_can = min(ATT_CHUNK, n_canon - p0);
-      c.n_here = c.n_can + n_spec;
-      // positions below n_safe were cached by earlier passes; the others are written by this pass's QKV kernel
-      c.n_safe = (n_spec > 0) ? c.n_can + n_spec - 1 : min(c.n_can, max(0, row_safe - p0));
-      c.rounds = (c.n_here + PPR - 1) / PPR;
-    };
-    auto advance = [&](Cursor& c) {
-      if (++c.rd == c.rounds) {
-        if (c.chunk + 1 < chunk_hi) setup(c, c.chunk + 1);
-        else c.chunk = chunk_hi;
-      }
-    };
-    // ---- ring, issue side: one unit = this thread's pieces of a key and of a value of one round ------------------
-    Cursor ic;
-    setup(ic, chunk_lo);
-    unsigned i_slot = 0, c_slot = 0;
-    auto issue = [&]() {
-      if (ic.chunk < chunk_hi) {
-        const int jpos = ic.rd * PPR + jl;
-        if (jpos < ic.n_here) {
-          const int slot = jpos < ic.n_can ? ic.chunk * ATT_CHUNK + jpos : tab->spec_slot[row][jpos - ic.n_can];
-          const size_t off = (size_t)slot * D;
-#pragma unroll
-          for (int pc = 0; pc < NP; ++pc) {
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ring_s + i_slot + pc * PIECE), "l"(Kb + off + pc * 8) : "memory");
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ring_s + i_slot + V_OFF + pc * PIECE), "l"(Vb + off + pc * 8)
-                         : "memory");
-          }
-        }
-        advance(ic);
-      }
-      i_slot += UNIT_BYTES;
-      if (i_slot == RING_BYTES) i_slot = 0;
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
+    i_st += 2 * C::TILE;
+    if (i_st == C::STAGES * 2 * C::TILE) i_st = 0;
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  {
     int issued = 0;
-    if (!waited) {
-      // rounds whose positions were all cached by earlier passes are requested ahead of the predecessor's completion
-      while (issued < UNITS - 1 && ic.chunk < chunk_hi && min((ic.rd + 1) * PPR, ic.n_here) <= ic.n_safe) issue(), ++issued;
-      pdl_launch_dependents();
-      pdl_wait();
-      waited = true;
-      timeline_mark(p.tl, p.tl_id + 256, false);
+    // tiles whose keys were all cached by earlier passes are requested ahead of the predecessor's completion (committed
+    // positions below n_safe, and every speculative slot but the row's own; the others are written by this pass's QKV kernel)
+    while (issued < C::STAGES - 1 && i_item < total) {
+      const int n_safe = i_keys > i_can ? i_keys - 1 : min(i_can, max(0, tab->n_safe[i_row] - i_p0));
+      if (min(i_j + C::KEYS, i_keys) > n_safe) break;
+      issue(), ++issued;
     }
-    for (; issued < UNITS - 1; ++issued) issue();
-
-    float q[G][DPL];
-#pragma unroll
-    for (int gq = 0; gq < G; ++gq) {
-      const float4* qp =
-          reinterpret_cast<const float4*>(p.qbuf + (size_t)row * p.n_q_heads * D + (size_t)(kvh * G + gq) * D + dl * DPL);
-#pragma unroll
-      for (int i = 0; i < DPL / 4; ++i) {
-        const float4 a = qp[i];
-        q[gq][4 * i] = a.x, q[gq][4 * i + 1] = a.y, q[gq][4 * i + 2] = a.z, q[gq][4 * i + 3] = a.w;
-      }
-    }
-
-    // ---- main loop: running softmax of this lane group over its positions of the run ----------------------------
-    float gm[G], gl[G], o[G][DPL];
-#pragma unroll
-    for (int gq = 0; gq < G; ++gq) {
-      gm[gq] = -INFINITY, gl[gq] = 0.f;
-#pragma unroll
-      for (int i = 0; i < DPL; ++i) o[gq][i] = 0.f;
-    }
-    auto lds128 = [](unsigned addr) {
-      uint4 v;
-      asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-      return v;
-    };
-    Cursor cc;
-    setup(cc, chunk_lo);
-    while (cc.chunk < chunk_hi) {
-      issue();
-      asm volatile("cp.async.wait_group %0;" ::"n"(UNITS - 1) : "memory");
-      const bool valid = cc.rd * PPR + jl < cc.n_here;
-      float sc[G];
-#pragma unroll
-      for (int gq = 0; gq < G; ++gq) sc[gq] = 0.f;
-#pragma unroll
-      for (int pc = 0; pc < NP; ++pc) {  // one chain per piece, folded in piece order
-        const uint4 kk = valid ? lds128(ring_s + c_slot + pc * PIECE) : make_uint4(0, 0, 0, 0);
-        const unsigned kw[4] = {kk.x, kk.y, kk.z, kk.w};
-        float sp[G];
-#pragma unroll
-        for (int gq = 0; gq < G; ++gq) sp[gq] = 0.f;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float k0 = __uint_as_float(kw[i] << 16), k1 = __uint_as_float(kw[i] & 0xffff0000u);
-#pragma unroll
-          for (int gq = 0; gq < G; ++gq) sp[gq] = fmaf(q[gq][pc * 8 + 2 * i + 1], k1, fmaf(q[gq][pc * 8 + 2 * i], k0, sp[gq]));
-        }
-#pragma unroll
-        for (int gq = 0; gq < G; ++gq) sc[gq] += sp[gq];
-      }
-      float wb[G];
-#pragma unroll
-      for (int gq = 0; gq < G; ++gq) {
-#pragma unroll
-        for (int off = LPP / 2; off > 0; off >>= 1) sc[gq] += __shfl_xor_sync(0xffffffffu, sc[gq], off);  // (every lane takes part)
-        wb[gq] = 0.f;
-        if (valid) {
-          const float sv = sc[gq] * p.scale;
-          if (sv > gm[gq]) {  // a new maximum: rescale what has been gathered (the first position finds -inf: weight 0)
-            const float wa = expf(gm[gq] - sv);
-            gl[gq] *= wa;
-#pragma unroll
-            for (int i = 0; i < DPL; ++i) o[gq][i] *= wa;
-            gm[gq] = sv;
-          }
-          wb[gq] = expf(sv - gm[gq]);
-          gl[gq] += wb[gq];
-        }
-      }
-      if (valid) {
-#pragma unroll
-        for (int pc = 0; pc < NP; ++pc) {
-          const uint4 vv = lds128(ring_s + c_slot + V_OFF + pc * PIECE);
-          const unsigned vw[4] = {vv.x, vv.y, vv.z, vv.w};
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float v0 = __uint_as_float(vw[i] << 16), v1 = __uint_as_float(vw[i] & 0xffff0000u);
-#pragma unroll
-            for (int gq = 0; gq < G; ++gq) {
-              o[gq][pc * 8 + 2 * i] = fmaf(wb[gq], v0, o[gq][pc * 8 + 2 * i]);
-              o[gq][pc * 8 + 2 * i + 1] = fmaf(wb[gq], v1, o[gq][pc * 8 + 2 * i + 1]);
-            }
-          }
-        }
-      }
-      c_slot += UNIT_BYTES;
-      if (c_slot == RING_BYTES) c_slot = 0;
-      advance(cc);
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");  // (only empty groups are left)
-
-    // ---- fold the lane groups of a warp: a butterfly in which the lower lane's state always comes first ---------
-#pragma unroll
-    for (int off = LPP; off < 32; off <<= 1) {
-      const bool upper = (lane & off) != 0;
-#pragma unroll
-      for (int gq = 0; gq < G; ++gq) {
-        const float m2 = __shfl_xor_sync(0xffffffffu, gm[gq], off), l2 = __shfl_xor_sync(0xffffffffu, gl[gq], off);
-        const float ma = upper ? m2 : gm[gq], mb = upper ? gm[gq] : m2;  // a: the lower lane's state
-        const float la = upper ? l2 : gl[gq], lb = upper ? gl[gq] : l2;
-        const float mn = fmaxf(ma, mb);
-        const float wa = ma == -INFINITY ? 0.f : expf(ma - mn), wb2 = mb == -INFINITY ? 0.f : expf(mb - mn);
-        gl[gq] = fmaf(la, wa, lb * wb2), gm[gq] = mn;
-#pragma unroll
-        for (int i = 0; i < DPL; ++i) {
-          const float o2 = __shfl_xor_sync(0xffffffffu, o[gq][i], off);
-          const float oa = upper ? o2 : o[gq][i], ob = upper ? o[gq][i] : o2;
-          o[gq][i] = fmaf(oa, wa, ob * wb2);
-        }
-      }
-    }
-    // ---- ... and the warps in ascending order -----------------------------------------------------------------
-    __syncthreads();  // the previous item's readers are done with s_comb
-    if (sub == 0) {
-#pragma unroll
-      for (int gq = 0; gq < G; ++gq) {
-        float* dst = s_comb + ((size_t)warp * G + gq) * PSTRIDE;
-#pragma unroll
-        for (int i = 0; i < DPL; ++i) dst[dl * DPL + i] = o[gq][i];
-        if (dl == 0) dst[D] = gm[gq], dst[D + 1] = gl[gq];
-      }
-    }
-    __syncthreads();
-    float run_m[EPT], run_l[EPT], run_a[EPT];
-#pragma unroll
-    for (int e = 0; e < EPT; ++e) {
-      const int idx = tid + e * ATT_THREADS;
-      run_m[e] = -INFINITY, run_l[e] = 0.f, run_a[e] = 0.f;
-      if (idx < G * D) {
-        const int gq = idx / D, dd = idx % D;
-        const float* src = s_comb + (size_t)gq * PSTRIDE;
-        float m = -INFINITY;
-#pragma unroll
-        for (int w2 = 0; w2 < ATT_THREADS / 32; ++w2) m = fmaxf(m, src[(size_t)w2 * G * PSTRIDE + D]);
-        float l = 0.f, acc = 0.f;
-#pragma unroll
-        for (int w2 = 0; w2 < ATT_THREADS / 32; ++w2) {
-          const float* pc = src + (size_t)w2 * G * PSTRIDE;
-          const float wgt = pc[D] == -INFINITY ? 0.f : expf(pc[D] - m);  // a warp that was dealt no position
-          l = fmaf(pc[D + 1], wgt, l);
-          acc = fmaf(pc[dd], wgt, acc);
-        }
-        run_m[e] = m, run_l[e] = l, run_a[e] = acc;
-      }
-    }
-
-    const int pair = row * p.n_kv_heads + kvh;
-    float* mypart = p.part + ((size_t)pair * p.max_chunks + run) * G * PSTRIDE;
-    if (n_runs == 1) {
-#pragma unroll
-      for (int e = 0; e < EPT; ++e) {
-        const int idx = tid + e * ATT_THREADS;
-        if (idx < G * D) {
-          const int gq = idx / D, dd = idx % D;
-          store_split(p.aplanes + (size_t)row * 3 * HQ, HQ, (kvh * G + gq) * D + dd, run_a[e] / run_l[e]);
-        }
-      }
-      continue;
-    }
-#pragma unroll
-    for (int e = 0; e < EPT; ++e) {
-      const int idx = tid + e * ATT_THREADS;
-      if (idx < G * D) {
-        const int gq = idx / D, dd = idx % D;
-        __stcg(mypart + gq * PSTRIDE + dd, run_a[e]);
-        if (dd == 0) __stcg(mypart + gq * PSTRIDE + D, run_m[e]), __stcg(mypart + gq * PSTRIDE + D + 1, run_l[e]);
-      }
-    }
-    __syncthreads();
-    if (tid == 0) {
-      __threadfence();
-      int old = atomicAdd(p.counters + pair, 1);
-      s_last = (old == n_runs - 1);
-      __threadfence();
-    }
-    __syncthreads();
-    if (s_last) {  // combine the runs in ascending order
-      const float* base = p.part + (size_t)pair * p.max_chunks * G * PSTRIDE;
-      for (int idx = tid; idx < G * D; idx += ATT_THREADS) {
-        int gq = idx / D, dd = idx % D;
-        float m = -INFINITY;
-        for (int c0 = 0; c0 < n_runs; c0 += 8) {
-          float mm[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) mm[u] = (c0 + u < n_runs) ? __ldcg(base + ((size_t)(c0 + u) * G + gq) * PSTRIDE + D) : -INFINITY;
-#pragma unroll
-          for (int u = 0; u < 8; ++u) m = fmaxf(m, mm[u]);
-        }
-        float l = 0.f, acc = 0.f;
-        for (int c0 = 0; c0 < n_runs; c0 += 8) {
-          float mc[8], lc[8], oc[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const bool ok = c0 + u < n_runs;
-            const float* pc = base + ((size_t)(ok ? c0 + u : 0) * G + gq) * PSTRIDE;
-            mc[u] = ok ? __ldcg(pc + D) : -INFINITY;
-            lc[u] = ok ? __ldcg(pc + D + 1) : 0.f;
-            oc[u] = ok ? __ldcg(pc + dd) : 0.f;
-          }
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            float wgt = expf(mc[u] - m);
-            l = fmaf(lc[u], wgt, l);
-            acc = fmaf(oc[u], wgt, acc);
-          }
-        }
-        store_split(p.aplanes + (size_t)row * 3 * HQ, HQ, (kvh * G + gq) * D + dd, acc / l);
-      }
-      if (tid == 0) p.counters[pair] = 0;
-    }
-  }
-  if (!waited) {
     pdl_launch_dependents();
     pdl_wait();
+    queries = true;
+    if (issued > 0) {  // the queries of the items whose tiles went out above
+      int qs = 0;
+      for (int it = first; it < total && (it < i_item || (it == i_item && i_j > 0)); it += n_warps, ++qs) {
+        int row, kvh, run, p0, n_can, n_keys;
+        locate(it, row, kvh, run, p0, n_can, n_keys);
+        issue_q(row, kvh, qs);
+      }
+      asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    }
+    for (; issued < C::STAGES - 1; ++issued) issue();
   }
-  timeline_mark(p.tl, p.tl_id, true);
+  // A finished item's arrival is announced one item later, when its stores have long landed; the warp that announces the last
+  // run of a (row, kv head) folds the runs in ascending order, D / 32 dims per lane
+  int pend_row = -1, pend_kvh = 0;
+  auto arrive = [&]() {
+    const int row = pend_row, kvh = pend_kvh, pair = row * p.n_kv_heads + kvh, n_runs = tab->chunk_start[row + 1] - tab->chunk_start[row];
+    __threadfence();
+    __syncwarp();
+    int old = 0;
+    if (lane == 0) old = atomicAdd(p.counters + pair, 1);
+    old = __shfl_sync(0xffffffffu, old, 0);
+    if (old != n_runs - 1) return;
+    __threadfence();
+    constexpr int DPV = D / 32;
+    for (int gq = 0; gq < G; ++gq) {
+      const float* base = p.part + ((size_t)pair * p.max_chunks * G + gq) * PSTRIDE;
+      constexpr size_t RS = (size_t)G * PSTRIDE;
+      float mx = -INFINITY, ll = 0.f, acc[DPV];
+#pragma unroll
+      for (int d = 0; d < DPV; ++d) acc[d] = 0.f;
+      for (int c0 = 0; c0 < n_runs; c0 += 8) {
+        float mc[8], lc[8];
+        float2 oc[8][DPV / 2];  // (a partial's D + 2 floats keep 8-byte alignment only)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const bool live = c0 + u < n_runs;
+          const float* pc = base + (size_t)(live ? c0 + u : 0) * RS;
+          mc[u] = live ? __ldcg(pc + D) : -INFINITY, lc[u] = live ? __ldcg(pc + D + 1) : 0.f;
+#pragma unroll
+          for (int d = 0; d < DPV / 2; ++d) oc[u][d] = live ? __ldcg(reinterpret_cast<const float2*>(pc + lane * DPV) + d) : make_float2(0.f, 0.f);
+        }
+        float mn = mx;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) mn = fmaxf(mn, mc[u]);
+        const float wa = mx == -INFINITY ? 0.f : expf(mx - mn);
+        mx = mn, ll *= wa;
+#pragma unroll
+        for (int d = 0; d < DPV; ++d) acc[d] *= wa;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const float wgt = mc[u] == -INFINITY ? 0.f : expf(mc[u] - mx);
+          ll = fmaf(lc[u], wgt, ll);
+#pragma unroll
+          for (int d = 0; d < DPV / 2; ++d) acc[2 * d] = fmaf(oc[u][d].x, wgt, acc[2 * d]), acc[2 * d + 1] = fmaf(oc[u][d].y, wgt, acc[2 * d + 1]);
+        }
+      }
+#pragma unroll
+      for (int d = 0; d < DPV; d += 2) store_split2(p.aplanes + (size_t)row * 3 * HQ, HQ, (kvh * G + gq) * D + lane * DPV + d, acc[d] / ll, acc[d + 1] / ll);
+    }
+    if (lane == 0) p.counters[pair] = 0;
+  };
+
+  for (int item = first; item < total; item += n_warps) {
+    int row, kvh, run, p0, n_can, n_keys;
+    locate(item, row, kvh, run, p0, n_can, n_keys);
+    constexpr int NH = G == 1 ? 1 : 2;  // heads a lane keeps the softmax state of (G = 4: heads 2 t, 2 t + 1 in lanes t < 2)
+    float m[NH], l[NH], o[KS][4];
+#pragma unroll
+    for (int h = 0; h < NH; ++h) m[h] = -INFINITY, l[h] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) o[ks][i] = 0.f;
+
+    unsigned qf[KS][NP][2];
+    for (int j0 = 0; j0 < n_keys; j0 += C::KEYS) {
+      issue();
+      asm volatile("cp.async.wait_group %0;" ::"n"(C::STAGES - 1) : "memory");
+      __syncwarp();
+      if (j0 == 0) {  // the queries came with the first tile: dims 16 ks + 2 t, + 1 (first register) and + 8, + 9 (second) of column g
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+          const bool live = G == 1 ? g < 3 : g < 4;
+          float2 a = make_float2(0.f, 0.f), b = a;
+          if (live) {
+            const float* qp = qring + c_q * (G * D) + (G == 1 ? 0 : g) * D + 16 * ks + 2 * t;
+            a = *reinterpret_cast<const float2*>(qp), b = *reinterpret_cast<const float2*>(qp + 8);
+          }
+          unsigned pa[3], pb[3];
+          split3_pair(a.x, a.y, pa), split3_pair(b.x, b.y, pb);
+          if constexpr (G == 1) {
+            qf[ks][0][0] = g == 0 ? pa[0] : g == 1 ? pa[1] : pa[2];
+            qf[ks][0][1] = g == 0 ? pb[0] : g == 1 ? pb[1] : pb[2];
+          } else {
+#pragma unroll
+            for (int s = 0; s < 3; ++s) qf[ks][s][0] = pa[s], qf[ks][s][1] = pb[s];
+          }
+        }
+        if (++c_q == C::STAGES) c_q = 0;
+      }
+      const unsigned kt = ring + c_st, vt = kt + C::TILE;
+      // ---- scores of keys g and g + 8 of every row tile ----
+      unsigned fr[MT][KS][4];  // every fragment is requested before the first is used: a load waited for is 30 cycles of a lone warp's chain
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) att_ldsm4(fr[mt][ks], (kt + mt * 16 * C::ROWB + k_lane) ^ (ks << 5));
+      float sc[MT][4];
+      {
+        float c[MT][4][4];  // four chains over the k-steps
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) c[mt][x][i] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+          for (int s = 0; s < NP; ++s)
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) att_mma(c[mt][ks & 3], fr[mt][ks], qf[ks][s][0], qf[ks][s][1]);
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) sc[mt][i] = (c[mt][0][i] + c[mt][1][i]) + (c[mt][2][i] + c[mt][3][i]);
+      }
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)  // (the value columns arrive under the softmax)
+          att_ldsm4_t(fr[mt][ks], (vt + mt * 16 * C::ROWB + v_lane) ^ (ks << 5));
+      float e0[MT][NH], e1[MT][NH], wa[NH];  // (key g, key g + 8) of this lane's heads: score, then softmax weight
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) {
+        if constexpr (G == 1) {  // columns 0, 1 (planes hi, mid) sit in lane t = 0, column 2 (lo) in t = 1; every lane takes the sum
+          const int b = lane & ~3;
+          e0[mt][0] = __shfl_sync(0xffffffffu, sc[mt][0], b) + (__shfl_sync(0xffffffffu, sc[mt][1], b) + __shfl_sync(0xffffffffu, sc[mt][0], b + 1));
+          e1[mt][0] = __shfl_sync(0xffffffffu, sc[mt][2], b) + (__shfl_sync(0xffffffffu, sc[mt][3], b) + __shfl_sync(0xffffffffu, sc[mt][2], b + 1));
+        } else {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) e0[mt][h] = sc[mt][h], e1[mt][h] = sc[mt][2 + h];
+        }
+      }
+      bool moved = false;
+#pragma unroll
+      for (int h = 0; h < NH; ++h) {  // running softmax
+        float mx = -INFINITY;
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+          e0[mt][h] = j0 + 16 * mt + g < n_keys ? e0[mt][h] * p.scale : -INFINITY;
+          e1[mt][h] = j0 + 16 * mt + g + 8 < n_keys ? e1[mt][h] * p.scale : -INFINITY;
+          mx = fmaxf(mx, fmaxf(e0[mt][h], e1[mt][h]));
+        }
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+        mx = fmaxf(mx, m[h]);  // (finite: every tile holds a key)
+        wa[h] = m[h] == -INFINITY ? 0.f : expf(m[h] - mx);
+        moved |= mx != m[h];
+        m[h] = mx;
+        float sum = 0.f;
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+          e0[mt][h] = expf(e0[mt][h] - mx), e1[mt][h] = expf(e1[mt][h] - mx);
+          sum += e0[mt][h] + e1[mt][h];
+        }
+        l[h] = fmaf(l[h], wa[h], sum);  // (this lane's keys; summed over the lanes when the run is done)
+      }
+      if (G == 1 ? moved : __any_sync(0xffffffffu, moved)) {
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) o[ks][i] *= wa[G == 1 ? 0 : (i & 1)];
+      }
+      // ---- softmax weights as columns: keys 2 t, 2 t + 1 (first register), + 8, + 9 (second) of column g ----
+      unsigned pf[MT][NP][2];
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) {
+        float a[2], b[2];
+        const int l0 = 8 * t, l1 = 8 * t + 4;  // lanes (key 2 t, .) and (key 2 t + 1, .)
+        if constexpr (G == 1) {
+          a[0] = __shfl_sync(0xffffffffu, e0[mt][0], l0), a[1] = __shfl_sync(0xffffffffu, e0[mt][0], l1);
+          b[0] = __shfl_sync(0xffffffffu, e1[mt][0], l0), b[1] = __shfl_sync(0xffffffffu, e1[mt][0], l1);
+        } else {  // column g = head g: state in lane t = g / 2, register g & 1
+          const int src = (g >> 1) & 1;
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            const int from = (x ? l1 : l0) + src;
+            const float u0 = __shfl_sync(0xffffffffu, e0[mt][0], from), u1 = __shfl_sync(0xffffffffu, e0[mt][NH - 1], from);
+            const float w0 = __shfl_sync(0xffffffffu, e1[mt][0], from), w1 = __shfl_sync(0xffffffffu, e1[mt][NH - 1], from);
+            a[x] = g >= 4 ? 0.f : (g & 1) ? u1 : u0, b[x] = g >= 4 ? 0.f : (g & 1) ? w1 : w0;
+          }
+        }
+        unsigned pa[3], pb[3];
+        split3_pair(a[0], a[1], pa), split3_pair(b[0], b[1], pb);
+        if constexpr (G == 1) {
+          pf[mt][0][0] = g == 0 ? pa[0] : g == 1 ? pa[1] : g == 2 ? pa[2] : 0u;
+          pf[mt][0][1] = g == 0 ? pb[0] : g == 1 ? pb[1] : g == 2 ? pb[2] : 0u;
+        } else {
+#pragma unroll
+          for (int s = 0; s < 3; ++s) pf[mt][s][0] = pa[s], pf[mt][s][1] = pb[s];
+        }
+      }
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int s = 0; s < NP; ++s)
+#pragma unroll
+          for (int ks = 0; ks < KS; ++ks) att_mma(o[ks], fr[mt][ks], pf[mt][s][0], pf[mt][s][1]);  // dims 16 ks .. + 15
+      __syncwarp();  // the tile may be overwritten
+      c_st += 2 * C::TILE;
+      if (c_st == C::STAGES * 2 * C::TILE) c_st = 0;
+    }
+
+    // ---- the run is done: dims 16 ks + g and + 8 of this lane's heads ----
+#pragma unroll
+    for (int h = 0; h < NH; ++h)
+#pragma unroll
+      for (int off = 4; off < 32; off <<= 1) l[h] += __shfl_xor_sync(0xffffffffu, l[h], off);
+    const int pair = row * p.n_kv_heads + kvh, n_runs = tab->chunk_start[row + 1] - tab->chunk_start[row];
+    float* mypart = p.part + ((size_t)pair * p.max_chunks + run) * G * PSTRIDE;
+    auto out = [&](int gq, int dd, float v, float mass) {
+      if (n_runs == 1) store_split(p.aplanes + (size_t)row * 3 * HQ, HQ, (kvh * G + gq) * D + dd, v / mass);
+      else __stcg(mypart + gq * PSTRIDE + dd, v);
+    };
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks) {
+      if constexpr (G == 1) {
+        const float lo0 = __shfl_sync(0xffffffffu, o[ks][0], (lane & ~3) + 1), lo1 = __shfl_sync(0xffffffffu, o[ks][2], (lane & ~3) + 1);
+        if (t == 0) out(0, 16 * ks + g, o[ks][0] + (o[ks][1] + lo0), l[0]), out(0, 16 * ks + g + 8, o[ks][2] + (o[ks][3] + lo1), l[0]);
+      } else if (t < 2) {
+#pragma unroll
+        for (int h = 0; h < NH; ++h) out(2 * t + h, 16 * ks + g, o[ks][h], l[h]), out(2 * t + h, 16 * ks + g + 8, o[ks][2 + h], l[h]);
+      }
+    }
+    if (n_runs == 1) continue;
+    if (g == 0 && t < (G == 1 ? 1 : 2)) {
+#pragma unroll
+      for (int h = 0; h < NH; ++h) __stcg(mypart + (NH * t + h) * PSTRIDE + D, m[h]), __stcg(mypart + (NH * t + h) * PSTRIDE + D + 1, l[h]);
+    }
+    if (pend_row >= 0) arrive();
+    pend_row = row, pend_kvh = kvh;
+  }
+  if (pend_row >= 0) arrive();
+  asm volatile("cp.async.wait_group 0;" ::: "memory");  // (only empty groups are left)
 }
 
 // ======================= prefill attention: the rows of a pass share every key / value chunk ========================
@@ -661,12 +695,6 @@ struct AtmCfg {
   static constexpr int ST_OFF = S_OFF + IR * SS * 4;                // [IR][4] fp32
   static constexpr int SMEM_BYTES = ST_OFF + IR * 4 * 4;
 };
-
-__device__ __forceinline__ void att_mma(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 
 template <int D>
 __global__ void __launch_bounds__(ATT_THREADS, 2) attn_prefill_mma_kernel(const __grid_constant__ AttnParams p) {

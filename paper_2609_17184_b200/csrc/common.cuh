@@ -21,17 +21,22 @@ constexpr int GROUP_ROWS = 64;  // token columns one GEMM launch carries
 constexpr int MAX_SEQS = 64;  // sequences a context can hold
 constexpr int MAX_SPEC = 16;  // speculative ancestors (incl. the row itself) a row can attend to: R/d1 levels
 constexpr int ATT_CHUNK = 64; // key positions per attention chunk (cut at fixed absolute positions)
-constexpr int ATT_MAX_RUNS = 40;  // attention work items per (row, kv head) at most (contexts up to 2560: one chunk each)
-constexpr int ATT_LONG_RUNS = 8;  // ... and for longer contexts
-constexpr int ATT_BATCH_SINGLE = 8;  // contexts that hold several sequences: single-chunk items only up to 8 chunks
-// A work item covers a run of consecutive chunks.  mode 0 (a context of one sequence: few rows per pass, every chunk in
-// parallel matters): one chunk for contexts up to ATT_MAX_RUNS chunks, beyond that as many as leave ATT_LONG_RUNS items.
-// mode 1 (contexts of several sequences: many rows per pass, the stream matters): one chunk up to ATT_BATCH_SINGLE
-// chunks, beyond that as many as leave ATT_LONG_RUNS items.  Either way a function of the row's own context only, so a
-// row's arithmetic does not depend on what shares the pass.
+constexpr int ATT_MAX_RUNS = 40;   // contexts of one sequence: one chunk per attention work item up to 2560 positions ...
+constexpr int ATT_LONG_RUNS = 16;  // ... and this many items at most for longer ones
+constexpr int ATT_BATCH_RUNS = 12;   // contexts of several sequences: items per (row, kv head) at most ...
+constexpr int ATT_BATCH_CHUNKS = 4;  // ... and their shortest run: as many chunks as there are sequences, up to 4
+// A work item covers a run of consecutive chunks.  mode 1 (a context of one sequence: few rows per pass, every chunk in
+// parallel matters): one chunk for contexts up to ATT_MAX_RUNS chunks, beyond that as many as leave ATT_LONG_RUNS items
+// [7 rows x 8400 positions, 8 / 16 / 32 items each: 65 / 51 / 86 us; 1 row: 53 / 33 / 24].  mode 2 .. 4 (contexts of that many
+// sequences and more: many rows per pass; an item has a fixed cost of some 4 us of its warp, and all items should be resident
+// at once): runs of `mode` chunks at least [48 rows x 510 positions, runs of 2 / 3 / 4 chunks: 34.5 / 38.0 / 25.7 us; 8 rows x
+// 300: 11.7 / 13.9 / 16.0] and ATT_BATCH_RUNS items at most.  Either way a function of the row's own context only, so a row's
+// arithmetic does not depend on what shares the pass.
 __host__ __device__ inline int att_run_len(int n_canon, int mode) {
   const int nc = (n_canon + ATT_CHUNK - 1) / ATT_CHUNK;
-  return nc <= (mode ? ATT_BATCH_SINGLE : ATT_MAX_RUNS) ? 1 : (nc + ATT_LONG_RUNS - 1) / ATT_LONG_RUNS;
+  if (mode == 1) return nc <= ATT_MAX_RUNS ? 1 : (nc + ATT_LONG_RUNS - 1) / ATT_LONG_RUNS;
+  const int rl = (nc + ATT_BATCH_RUNS - 1) / ATT_BATCH_RUNS;
+  return rl > mode ? rl : mode;
 }
 __host__ __device__ inline int att_items(int n_canon, int mode) {
   const int nc = (n_canon + ATT_CHUNK - 1) / ATT_CHUNK, rl = att_run_len(n_canon, mode);
@@ -134,24 +139,31 @@ __device__ __forceinline__ void store_split(__nv_bfloat16* row_planes, int ld, i
   row_planes[2 * ld + k] = __ushort_as_bfloat16(l);
 }
 
-// the same for two / four neighbouring values (k even / a multiple of 4): 4- and 8-byte stores
+// the split of two neighbouring values, one register of each plane (the low half is `a`'s): packed conversions, half the instructions
+__device__ __forceinline__ void split3_pair(float a, float b, unsigned (&pl)[3]) {
+  auto pack = [](float x, float y) {  // (round-to-nearest, as split3)
+    const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
+    return *reinterpret_cast<const unsigned*>(&v);
+  };
+  pl[0] = pack(a, b);
+  a -= __uint_as_float(pl[0] << 16), b -= __uint_as_float(pl[0] & 0xffff0000u);
+  pl[1] = pack(a, b);
+  a -= __uint_as_float(pl[1] << 16), b -= __uint_as_float(pl[1] & 0xffff0000u);
+  pl[2] = pack(a, b);
+}
+// store_split for two / four neighbouring values (k even / a multiple of 4): 4- and 8-byte stores
 __device__ __forceinline__ void store_split2(__nv_bfloat16* row_planes, int ld, int k, float a, float b) {
-  unsigned short h0, m0, l0, h1, m1, l1;
-  split3(a, h0, m0, l0);
-  split3(b, h1, m1, l1);
-  *reinterpret_cast<unsigned*>(row_planes + k) = h0 | ((unsigned)h1 << 16);
-  *reinterpret_cast<unsigned*>(row_planes + ld + k) = m0 | ((unsigned)m1 << 16);
-  *reinterpret_cast<unsigned*>(row_planes + 2 * ld + k) = l0 | ((unsigned)l1 << 16);
+  unsigned pl[3];
+  split3_pair(a, b, pl);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) *reinterpret_cast<unsigned*>(row_planes + (size_t)i * ld + k) = pl[i];
 }
 __device__ __forceinline__ void store_split4(__nv_bfloat16* row_planes, int ld, int k, float4 v) {
-  unsigned short h[4], m[4], l[4];
-  split3(v.x, h[0], m[0], l[0]);
-  split3(v.y, h[1], m[1], l[1]);
-  split3(v.z, h[2], m[2], l[2]);
-  split3(v.w, h[3], m[3], l[3]);
-  *reinterpret_cast<uint2*>(row_planes + k) = make_uint2(h[0] | ((unsigned)h[1] << 16), h[2] | ((unsigned)h[3] << 16));
-  *reinterpret_cast<uint2*>(row_planes + ld + k) = make_uint2(m[0] | ((unsigned)m[1] << 16), m[2] | ((unsigned)m[3] << 16));
-  *reinterpret_cast<uint2*>(row_planes + 2 * ld + k) = make_uint2(l[0] | ((unsigned)l[1] << 16), l[2] | ((unsigned)l[3] << 16));
+  unsigned a[3], b[3];
+  split3_pair(v.x, v.y, a);
+  split3_pair(v.z, v.w, b);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) *reinterpret_cast<uint2*>(row_planes + (size_t)i * ld + k) = make_uint2(a[i], b[i]);
 }
 
 // tuning aid: earliest CTA start / latest CTA end of kernel `id` on the global nanosecond timer

@@ -247,8 +247,9 @@ struct Layout {  // byte offsets into the workspace
 };
 
 struct Derived {
-  int att_mode;   // attention work items: 0 one sequence per context, 1 several (see att_run_len)
-  int att_runs;   // the context's rows can have items of several chunks: the streaming attention kernel runs
+  int att_mode;   // how attention work items are cut (see att_run_len)
+  int att_long;   // what loopspec_decode_paths reports of the context capacity
+  int att_warps;  // decode attention by one warp per item (attn_warp_kernel)
   int S, NB, B, max_rows_dec, max_rows_pf, max_rows, slots, ids_cap, n_hid, n_logit_vecs, p_logit_base, n_sq, sq_stride, max_chunks,
       trace_cap, Hq, Hkv, d1, d2;
   // Raven-style layout (P and C hold transformer blocks): all layers in one list - prelude, recurrent, coda
@@ -351,8 +352,12 @@ bool resolve_sched(const loopspec_model* m, const loopspec_sched* s, Derived* d,
   d->n_sq = m->hidden / 128;  // row blocks of the residual GEMMs = partial sums of squares per row
   d->sq_stride = std::max(d->n_sq, 64);  // room for one partial per cluster of the persistent pass kernel
   d->max_chunks = (s->max_ctx + ATT_CHUNK - 1) / ATT_CHUNK;
-  d->att_mode = d->S >= 2 ? 1 : 0;
-  d->att_runs = d->max_chunks > (d->att_mode ? ATT_BATCH_SINGLE : ATT_MAX_RUNS) ? 1 : 0;
+  d->att_mode = std::min(d->S, ATT_BATCH_CHUNKS);
+  d->att_long = d->max_chunks > (d->S > 1 ? 8 : ATT_MAX_RUNS) ? 1 : 0;
+  // One CTA per item only for the few items of a lone sequence of short capacity, where the work of an item is its latency
+  // [us, attn_kernel / attn_warp_kernel, 536 positions: 1 row 6.5 / 9.5, 4 rows 8.2 / 10.5, 7 rows 14.2 / 11.5; 3000 positions, against
+  // the best of runs of chunks by one CTA: 4 rows 24 / 22, 7 rows 47 / 36; batches: attn_warp_kernel's comment]
+  d->att_warps = d->S > 1 || d->att_long ? 1 : 0;
   d->trace_cap = m->R * s->max_ctx + 64;  // a token can take R passes (restart)
   d->Hq = m->n_q_heads * m->head_dim;
   d->Hkv = m->n_kv_heads * m->head_dim;
@@ -623,23 +628,22 @@ cudaError_t launch_gemm(int wdt, int ng, int epi, const GemmParams& p, cudaStrea
 }
 
 using AttnFn = void (*)(const AttnParams);
-AttnFn attn_fn(int d, int G, bool runs) {  // runs: rows of this context can have work items of several chunks
-  if (runs) {
-    if (d == 128) return G == 1 ? attn_runs_kernel<128, 1> : attn_runs_kernel<128, 4>;
-    return G == 1 ? attn_runs_kernel<64, 1> : attn_runs_kernel<64, 4>;
-  }
-  if (d == 128) return G == 1 ? attn_kernel<128, 1> : attn_kernel<128, 4>;
-  return G == 1 ? attn_kernel<64, 1> : attn_kernel<64, 4>;
+// The decode attention of a context: kernel, grid, block and dynamic shared memory
+struct AttnLaunch {
+  AttnFn fn;
+  int grid, block;
+  size_t smem;
+};
+template <int D, int G>
+AttnLaunch attn_launch_of(int n_sm, bool warps) {
+  using C = AtwCfg<D, G>;
+  if (warps) return {attn_warp_kernel<D, G>, n_sm * C::CTAS, C::WARPS * 32, (size_t)C::SMEM_BYTES};
+  return {attn_kernel<D, G>, n_sm * 8, ATT_THREADS, 0};
 }
-
-// dynamic shared memory and grid of the attention launch (the streaming kernel of long contexts: its rings, and one
-// CTA per slot the SMs offer)
-size_t attn_smem(int d, int G, bool runs) {
-  if (!runs) return 0;
-  if (d == 128) return G == 1 ? AtsCfg<128, 1>::SMEM_BYTES : AtsCfg<128, 4>::SMEM_BYTES;
-  return G == 1 ? AtsCfg<64, 1>::SMEM_BYTES : AtsCfg<64, 4>::SMEM_BYTES;
+AttnLaunch attn_launch(int d, int G, int n_sm, bool warps) {
+  if (d == 128) return G == 1 ? attn_launch_of<128, 1>(n_sm, warps) : attn_launch_of<128, 4>(n_sm, warps);
+  return G == 1 ? attn_launch_of<64, 1>(n_sm, warps) : attn_launch_of<64, 4>(n_sm, warps);
 }
-int attn_grid(int n_sm, int G, bool runs) { return runs ? n_sm * (G == 1 ? AtsCfg<128, 1>::MIN_CTAS : AtsCfg<128, 4>::MIN_CTAS) : n_sm * 8; }
 
 // tuning builds (-DLOOPSPEC_TUNE) with LOOPSPEC_DBG set record a kernel timeline in a workspace region of their own
 unsigned long long* tune_timeline(loopspec_ctx* c) {
@@ -863,9 +867,8 @@ cudaError_t launch_attention(loopspec_ctx* c, const RowTable* tab, int l, unsign
       return e;
     return launch_k(attn_prefill_fold_kernel<64>, fold_grid, dim3(16), 0, c->stream, a, c->use_pdl);
   }
-  const bool runs = d.att_runs != 0;
-  return launch_k(attn_fn(m.head_dim, G, runs), dim3(attn_grid(c->n_sm, G, runs)), dim3(ATT_THREADS), attn_smem(m.head_dim, G, runs), c->stream, a,
-                  c->use_pdl);
+  const AttnLaunch k = attn_launch(m.head_dim, G, c->n_sm, d.att_warps != 0);
+  return launch_k(k.fn, dim3(k.grid), dim3(k.block), k.smem, c->stream, a, c->use_pdl);
 }
 
 // the blocks [l0, l0 + count) of the layer list on the rows of `tab`
@@ -1375,7 +1378,7 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
   // Every kernel of the chain asks for the same (largest) shared-memory carve-out: the GEMM CTAs need it, and an SM
   // whose partition was set by a small-shared-memory kernel would have to drain before it can host one.
   {
-    const void* small_fns[] = {(const void*)attn_fn(m->head_dim, m->n_q_heads / m->n_kv_heads, d.att_runs != 0), (const void*)prep_planes_kernel,
+    const void* small_fns[] = {(const void*)attn_launch(m->head_dim, m->n_q_heads / m->n_kv_heads, c->n_sm, d.att_warps != 0).fn, (const void*)prep_planes_kernel,
                                (const void*)select_kernel, (const void*)control_kernel, (const void*)vanilla_control_kernel,
                                (const void*)kv_commit_kernel};
     for (const void* f : small_fns)
@@ -1383,10 +1386,8 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
         (void)cudaGetLastError();
   }
   {
-    const int G = m->n_q_heads / m->n_kv_heads;
-    const bool runs = d.att_runs != 0;
-    if (runs && cudaFuncSetAttribute((const void*)attn_fn(m->head_dim, G, runs), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)attn_smem(m->head_dim, G, runs)) != cudaSuccess) {
+    const AttnLaunch k = attn_launch(m->head_dim, m->n_q_heads / m->n_kv_heads, c->n_sm, d.att_warps != 0);
+    if (k.smem && cudaFuncSetAttribute((const void*)k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem) != cudaSuccess) {
       delete c;
       return LOOPSPEC_ECUDA;
     }
@@ -1907,7 +1908,7 @@ int loopspec_launches_per_step(loopspec_ctx* c, int32_t* out) {
 int loopspec_decode_paths(loopspec_ctx* c, int32_t* gemm_path, int32_t* attention_path) {
   if (!c) return LOOPSPEC_EINVAL;
   if (gemm_path) *gemm_path = c->tc[1].on ? 1 : 0;
-  if (attention_path) *attention_path = c->d.att_runs != 0 ? 1 : 0;
+  if (attention_path) *attention_path = c->d.att_long;
   return LOOPSPEC_OK;
 }
 

@@ -474,12 +474,6 @@ struct PfAttnParams {
   int n_rows, p0, slots, n_kv_heads, n_q_heads;
   float scale;
 };
-__device__ __forceinline__ void pfa_ldsm4(unsigned (&r)[4], unsigned addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void pfa_ldsm4_t(unsigned (&r)[4], unsigned addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
 __device__ __forceinline__ unsigned pfa_pack(unsigned short a, unsigned short b) { return a | ((unsigned)b << 16); }
 
 template <int D>
@@ -559,11 +553,11 @@ __global__ void __launch_bounds__(PFA_THREADS, 2) pf_attn_kernel(const __grid_co
       for (int ks = 0; ks < D / 16; ++ks) {
         unsigned a[3][4];
 #pragma unroll
-        for (int pl = 0; pl < 3; ++pl) pfa_ldsm4(a[pl], sq + pl * PFA_ROWS * C::ROWB + piece(wr + (lane & 15), 2 * ks + (lane >> 4)));
+        for (int pl = 0; pl < 3; ++pl) att_ldsm4(a[pl], sq + pl * PFA_ROWS * C::ROWB + piece(wr + (lane & 15), 2 * ks + (lane >> 4)));
 #pragma unroll
         for (int jj = 0; jj < 4; ++jj) {  // two tiles of eight keys
           unsigned kb[4];
-          pfa_ldsm4(kb, sk + b * C::KV_BYTES + piece(16 * jj + (lane & 7) + 8 * (lane >> 4), 2 * ks + ((lane >> 3) & 1)));
+          att_ldsm4(kb, sk + b * C::KV_BYTES + piece(16 * jj + (lane & 7) + 8 * (lane >> 4), 2 * ks + ((lane >> 3) & 1)));
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             att_mma(s0[2 * jj + e], a[0], kb[2 * e], kb[2 * e + 1]);
@@ -624,7 +618,7 @@ __global__ void __launch_bounds__(PFA_THREADS, 2) pf_attn_kernel(const __grid_co
 #pragma unroll
         for (int kk = 0; kk < PFA_KEYS / 16; ++kk) {
           unsigned vb[4];
-          pfa_ldsm4_t(vb, sv + b * C::KV_BYTES + piece(16 * kk + (lane & 15), 2 * dt + (lane >> 4)));
+          att_ldsm4_t(vb, sv + b * C::KV_BYTES + piece(16 * kk + (lane & 15), 2 * dt + (lane >> 4)));
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             att_mma(a0[e], pa[kk][0], vb[2 * e], vb[2 * e + 1]);

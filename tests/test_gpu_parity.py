@@ -423,6 +423,23 @@ def test_batch_of_mid_length_contexts_streams_runs_of_chunks(name, T):
     ctx.close()
 
 
+@pytest.mark.parametrize("name,S,lens", [("tiny_bf16", 2, [15, 113]), ("tiny_bf16", 3, [62, 127, 176]), ("small_bf16", 2, [31, 111]),
+                                          ("tiny_gqa", 4, [1, 16, 240, 255])])
+def test_attention_of_several_sequences_at_the_edges_of_tiles_and_runs(name, S, lens):
+    """One warp per run of chunks: contexts of a single key, that grow over the edge of a 16-key tile, of a chunk and of a run
+    (2 to 4 chunks, as many as the context has sequences) while speculative keys follow the committed ones; head sizes 64 and 128,
+    one and four query heads per kv head."""
+    n = 20
+    refs = [U.oracle_run(name, lens[s], n, 1, 2, seed=4, seq=s) for s in range(S)]
+    ctx = U.make_ctx(name, 1, 2, seed=4, max_seqs=S, max_ctx=300)
+    for s in range(S):
+        assert ctx.prefill(refs[s]["prompt"], seq=s) == refs[s]["first"]
+    out = ctx.decode(n)
+    for s in range(S):
+        assert out[s].tolist() == refs[s]["tokens"], (s, U.min_margin(refs[s]["dec"]))
+    ctx.close()
+
+
 def test_prefill_chunking_does_not_change_results():
     name = "tiny_bf16"
     ref = U.oracle_run(name, 37, 16, 1, 2)
