@@ -96,6 +96,13 @@ __device__ __forceinline__ void tc_mma(unsigned d_tmem, unsigned long long adesc
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// One lane of a converged warp, always the same.  tcgen05.mma takes its operands from uniform registers: issued under a branch on
+// the lane number every MMA first moves them there, about 60 cycles each; under this one the compiler keeps them uniform.
+__device__ __forceinline__ bool tc_elect_one() {
+  unsigned e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+  return e != 0;
+}
 __device__ __forceinline__ void tc_commit(unsigned bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }

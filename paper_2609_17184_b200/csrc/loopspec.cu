@@ -487,7 +487,7 @@ struct loopspec_ctx {
   // prompt passes of the wide kernels: tensor maps of the weights (4 per block, then the adapter) and of the four plane buffers
   bool pf = false;
   std::vector<CUtensorMap> pf_wmaps;
-  CUtensorMap pf_x1[4], pf_x2[4];     // planes read by QKV and gate/up, by O, by down, by the adapter: boxes of 128 / 64 rows
+  PgMaps pf_x[4];                     // planes read by QKV and gate/up, by O, by down, by the adapter
   // readout GEMM of the decode passes on the tcgen05 kernel (bf16 weights): plan, tensor maps of the row-major lm_head
   // (one box per 128-row tile) and of the hidden-state planes (all three planes of dg_mp rows in one box)
   bool dg = false;
@@ -1072,13 +1072,29 @@ template <int EPI>
 cudaError_t launch_pf_gemm_epi(loopspec_ctx* c, const CUtensorMap& w, int xi, const PfGemmParams& p) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
-  const int items = p.n_rp * p.n_tt * p.n_split;
+  const int items = p.n_rp * p.n_split * (p.n_full + p.n_tail);
   cfg.gridDim = dim3(2 * std::min(c->n_sm / 2, items)), cfg.blockDim = dim3(PG_THREADS), cfg.dynamicSmemBytes = PG_SMEM, cfg.stream = c->stream;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at, cfg.numAttrs = c->use_pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, pf_gemm_kernel<EPI>, w, c->pf_x1[xi], c->pf_x2[xi], p);
+  return cudaLaunchKernelEx(&cfg, pf_gemm_kernel<EPI>, w, c->pf_x[xi], p);
+}
+// Token columns of a tile for a pass of n tokens over `blocks` weight-block pairs x k-splits on `pairs` pairs of CTAs: the width whose
+// rounds of full tiles, and of the leftover ones beyond those that fill the last round, are estimated shortest.  A tile's time
+// is its MMAs' or its operands' way through the L2 (16 KB of weights and 192 B per column and k-block), whichever is longer.
+int pg_tile_width(int n, int blocks, int pairs) {
+  auto cost = [](int cols) { return std::max(6.0 * cols, (PG_A_BYTES + 192.0 * pg_width(pg_width_of(cols))) / 56.0); };  // cycles per k-block
+  int best = PG_TOK;
+  double best_t = 1e30;
+  for (int w = 0; w < PG_WIDTHS; ++w) {
+    const int tok = pg_width(w), full = blocks * (n / tok), rest = n % tok;
+    const int rounds = (full + pairs - 1) / pairs, gap = rounds * pairs - full;  // pairs that idle in the last round of full tiles
+    const int tail = rest ? std::max(0, blocks - gap) : 0;
+    const double t = rounds * cost(tok) + (tail + pairs - 1) / pairs * cost((rest + 31) / 32 * 32);
+    if (t < best_t * 0.98) best_t = t, best = tok;
+  }
+  return best;
 }
 struct PfPass {  // rows of a pass: positions p0 .. p0 + n - 1 of sequence seq
   int seq, p0, n;
@@ -1090,9 +1106,10 @@ cudaError_t launch_pf_gemm(loopspec_ctx* c, int which, int layer, const PfPass& 
   PfGemmParams p;
   memset(&p, 0, sizeof p);
   const int Ns[6] = {d.Hq + 2 * d.Hkv, m.hidden, 2 * m.ffn, m.hidden, 0, m.hidden}, Ks[6] = {m.hidden, d.Hq, m.hidden, m.ffn, 0, 2 * m.hidden};
-  p.N = Ns[which], p.n_kb = (Ks[which] + TC_BK - 1) / TC_BK, p.n_tok = ps.n, p.n_tt = (ps.n + PG_TOK - 1) / PG_TOK;
+  p.N = Ns[which], p.n_kb = (Ks[which] + TC_BK - 1) / TC_BK, p.n_tok = ps.n;
   p.n_rp = which == G_GU ? (m.ffn + 127) / 128 : (p.N + 255) / 256;
   p.n_split = (which == G_QKV || which == G_GU) ? 1 : pf_splits(Ks[which]);
+  p.tok = pg_tile_width(ps.n, p.n_rp * p.n_split, c->n_sm / 2), p.n_full = ps.n / p.tok, p.n_tail = ps.n % p.tok ? 1 : 0;
   p.err = const_cast<int*>(c->host_flags_dev + HF_ERROR), p.err_code = ERR_WAIT_PF;
   p.sumsq = c->at<float>(c->L.pf_sumsq), p.H = m.hidden, p.eps = m.rms_eps;
   const CUtensorMap& w = which == G_ADAPT ? c->pf_wmaps[4 * d.NL] : c->pf_wmaps[4 * layer + which];
@@ -1482,8 +1499,9 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
     const size_t x_off[4] = {L.pf_x, L.pf_a, L.pf_s, L.pf_c};
     const int x_k[4] = {m->hidden, d.Hq, m->ffn, 2 * m->hidden};
     for (int i = 0; i < (d.raven ? 4 : 3) && ok; ++i)
-      ok = make_map_pf_planes(&c->pf_x1[i], c->ws + x_off[i], x_k[i], d.pf_rows, PG_TOK) &&
-           make_map_pf_planes(&c->pf_x2[i], c->ws + x_off[i], x_k[i], d.pf_rows, PG_TOK / 2);
+      for (int w = 0; w < PG_WIDTHS && ok; ++w)
+        ok = make_map_pf_planes(&c->pf_x[i].x1[w], c->ws + x_off[i], x_k[i], d.pf_rows, pg_width(w)) &&
+             make_map_pf_planes(&c->pf_x[i].x2[w], c->ws + x_off[i], x_k[i], d.pf_rows, pg_width(w) / 2);
     ok = ok && cudaFuncSetAttribute(pf_gemm_kernel<PG_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, PG_SMEM) == cudaSuccess &&
          cudaFuncSetAttribute(pf_gemm_kernel<PG_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, PG_SMEM) == cudaSuccess &&
          cudaFuncSetAttribute(pf_gemm_kernel<PG_PART>, cudaFuncAttributeMaxDynamicSharedMemorySize, PG_SMEM) == cudaSuccess &&

@@ -12,8 +12,8 @@
 // A row's arithmetic is a function of its own operands and of the model's shapes: k-splits depend on the matrix alone, every
 // accumulation chain runs over the whole k-range of its split, so results do not depend on how the prompt is cut into passes.
 //
-// Prompt of the 1.4B shape, wall clock of loopspec_prefill: 512 tokens 100 ms (passes of 32 rows; 61 ms with 64) -> 21.5 ms, 1024
-// tokens 132 -> 35 ms, 3001 tokens 716 -> 128 ms; three-plane products at the measured GEMM peak would take 9 / 19 / 56 ms.
+// Prompt of the 1.4B shape, wall clock of loopspec_prefill: 512 tokens 100 ms (passes of 32 rows; 61 ms with 64) -> 17.9 ms, 3001
+// tokens 716 -> 117 ms; three-plane products at the measured GEMM peak would take 9 / 56 ms.
 #pragma once
 #include <cuda.h>
 
@@ -111,13 +111,21 @@ __global__ void __launch_bounds__(256) pf_concat_kernel(const __grid_constant__ 
 // y[token][n] = sum_k x[token][k] W[n][k] for a whole pass.  Bound by the tensor cores: 3 x 2 x rows x N x K operations, so
 // everything here serves to keep tcgen05 fed.  A pair of CTAs (cluster of two, cta_group::2) owns 256 weight rows x 128 token
 // columns: each CTA holds its 128 weight rows and half of the columns' operand, so a k-block of 64 costs an SM 40 KB of L2
-// reads for 768 cycles of MMA (52 B per cycle; one CTA alone with 128 x 128 would need 83).  Per 16-wide k-step two MMAs:
+// reads for 740 cycles of MMA (55 B per cycle; one CTA alone with 128 x 128 would need 83).  Per 16-wide k-step two MMAs:
 // [hi | mid] as 256 columns (CTA 0 holds the hi rows, CTA 1 the mid rows of all 128 tokens) and lo as 128 columns that
 // accumulate onto mid's - two chains, hi and (mid + lo), folded when the accumulator is read.  256 TMEM columns per
 // accumulator, two accumulators: the epilogue of a tile runs under the main loop of the next (persistent CTAs, tiles dealt
 // round robin, the token tiles of one weight block next to each other so that its weights come from HBM once).
-constexpr int PG_THREADS = 256;
-constexpr int PG_TOK = 128;                        // token columns of a tile
+// A k-block takes 740 cycles at 128 columns, 560 at 96 and 540 at 64, where the operands' way through the L2 bounds it (more
+// stages change nothing); the MMAs are issued by a converged warp (see tc_elect_one: 840 cycles at any width before).  A pass of a
+// few hundred tokens has one to three tiles per pair, so their width is chosen for even rounds (pg_tile_width), and what stands
+// around the MMAs counts: 7000 cycles before the first (4000 of them after the predecessor's end) and 8000 to 10000 after the last.
+// us per launch on the 1.4B shape: 368 tokens QKV 61 -> 27, gate/up 60 -> 44, down 31 -> 25; 512 tokens QKV 61 -> 36, gate/up 65 -> 60.
+constexpr int PG_THREADS = 384;
+constexpr int PG_TOK = 128;                        // token columns of a tile at most
+constexpr int PG_WIDTHS = 3;                       // widths a tile can have: 128, 96 or 64 token columns (see pg_tile_width)
+__host__ __device__ constexpr int pg_width(int i) { return PG_TOK - 32 * i; }
+__host__ __device__ constexpr int pg_width_of(int cols) { return cols > 96 ? 0 : cols > 64 ? 1 : 2; }  // the narrowest that holds `cols`
 constexpr int PG_A_BYTES = 128 * TC_BK * 2;        // a CTA's weight rows of a stage
 constexpr int PG_B1_BYTES = PG_TOK * TC_BK * 2;    // hi (rank 0) or mid (rank 1) of all tokens
 constexpr int PG_B2_BYTES = PG_TOK / 2 * TC_BK * 2;  // lo of half the tokens
@@ -125,11 +133,16 @@ constexpr int PG_STAGE_BYTES = PG_A_BYTES + PG_B1_BYTES + PG_B2_BYTES;
 constexpr int PG_STAGES = 5;
 constexpr int PG_ST_LD = 132;                      // floats per token of the epilogue's exchange buffer
 constexpr int PG_ST_TOK = 16;                      // tokens exchanged at a time
-constexpr int PG_SMEM = 1024 + PG_STAGES * PG_STAGE_BYTES + 2 * PG_ST_TOK * PG_ST_LD * 4;
+constexpr int PG_SMEM = 1024 + PG_STAGES * PG_STAGE_BYTES + 2 * PG_ST_TOK * PG_ST_LD * 4;  // (an exchange buffer per epilogue team)
 enum { PG_QKV = 0, PG_SWIGLU = 1, PG_PART = 2 };
 
+// The planes read by a GEMM as (k, token, plane), one pair of maps per tile width: boxes of the width (hi, mid) and of half of it (lo)
+struct PgMaps {
+  CUtensorMap x1[PG_WIDTHS], x2[PG_WIDTHS];
+};
 struct PfGemmParams {
-  int n_rp, n_tt, n_split;  // pairs of 128-row weight blocks, token tiles, k-splits
+  int n_rp, n_split;        // pairs of 128-row weight blocks, k-splits
+  int tok, n_full, n_tail;  // token columns of a tile, tiles of that width, 1 when a narrower one is left over
   int n_kb;                 // 64-wide k-blocks of the matrix
   int n_tok, N;             // live rows of the pass, weight rows
   int* err;
@@ -169,7 +182,7 @@ __device__ __forceinline__ void pg_commit(unsigned bar) {
                : "memory");
 }
 __device__ __forceinline__ void pg_cluster_sync() { asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory"); }
-__device__ __forceinline__ void pg_team_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }  // the epilogue's four warps
+__device__ __forceinline__ void pg_team_sync(int team) { asm volatile("bar.sync %0, 128;" ::"r"(1 + team) : "memory"); }  // four warps of the epilogue
 __device__ __forceinline__ void pg_ld16(unsigned (&w)[16], unsigned taddr) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]), "=r"(w[8]), "=r"(w[9]),
@@ -181,29 +194,25 @@ __device__ __forceinline__ void pg_ld16(unsigned (&w)[16], unsigned taddr) {
 template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
     pf_gemm_kernel(const __grid_constant__ CUtensorMap map_w,   // weights: box 64 k x 128 rows; gate/up: (k, f, gate | up), box 64 x 64 x 2
-                   const __grid_constant__ CUtensorMap map_x1,  // planes as (k, token, plane): box 64 x 128 x 1
-                   const __grid_constant__ CUtensorMap map_x2,  // ... box 64 x 64 x 1
+                   const __grid_constant__ PgMaps maps,
                    const __grid_constant__ PfGemmParams p) {
   extern __shared__ unsigned char pg_smem_raw[];
   __shared__ __align__(8) unsigned long long s_full[PG_STAGES], s_empty[PG_STAGES], s_accf[2], s_acce[2];
   __shared__ unsigned s_tmem;
   __shared__ int s_fail;
-  __shared__ float s_rstd[PG_TOK];
+  __shared__ float s_rstd[2][PG_TOK];
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // (warp: uniform to the compiler)
   const unsigned rank = blockIdx.x & 1u;  // the pair's leader (rank 0) issues the MMAs and owns the full barriers
   const int cid = blockIdx.x >> 1, n_cl = gridDim.x >> 1;
   const unsigned base = (tc_smem_u32(pg_smem_raw) + 1023u) & ~1023u;
-  float* st = reinterpret_cast<float*>(pg_smem_raw + (base - tc_smem_u32(pg_smem_raw)) + PG_STAGES * PG_STAGE_BYTES);
-  const int n_items = p.n_rp * p.n_tt * p.n_split;
+  const int n_full_items = p.n_rp * p.n_split * p.n_full, n_items = n_full_items + p.n_rp * p.n_split * p.n_tail;
 
   pdl_launch_dependents();
   if (tid == 0) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<unsigned long long>(&map_w)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<unsigned long long>(&map_x1)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<unsigned long long>(&map_x2)) : "memory");
     for (int s = 0; s < PG_STAGES; ++s) tc_mbar_init(tc_smem_u32(&s_full[s]), 1), tc_mbar_init(tc_smem_u32(&s_empty[s]), 1);
-    for (int b = 0; b < 2; ++b) tc_mbar_init(tc_smem_u32(&s_accf[b]), 1), tc_mbar_init(tc_smem_u32(&s_acce[b]), 8);  // four warps of each CTA
+    for (int b = 0; b < 2; ++b) tc_mbar_init(tc_smem_u32(&s_accf[b]), 1), tc_mbar_init(tc_smem_u32(&s_acce[b]), 16);  // eight warps of each CTA
     s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -219,19 +228,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const unsigned tmem = s_tmem;
 
-  // item -> (weight block pair, token tile, split): token tiles vary fastest
+  // item -> (weight block pair, split, token tile): the full tiles first, token tiles fastest; the narrow ones of the leftover tokens
+  // come last and fill what the full ones leave of the last round
   struct Item {
-    int rp, tt, sp, kb_lo, n_kb, cols;  // cols: MMA columns of the tile (its live tokens rounded up to 32)
+    int rp, sp, t0, live, kb_lo, n_kb, cols;  // cols: MMA columns of the tile (its live tokens rounded up to 32)
   };
   auto item_of = [&](int it) {
     Item r;
-    r.tt = it % p.n_tt;
-    const int q = it / p.n_tt;
+    int q, tt;
+    if (it < n_full_items) q = it / p.n_full, tt = it - q * p.n_full;
+    else q = it - n_full_items, tt = p.n_full;
     r.rp = q % p.n_rp, r.sp = q / p.n_rp;
     r.kb_lo = (int)((long long)p.n_kb * r.sp / p.n_split);
     r.n_kb = (int)((long long)p.n_kb * (r.sp + 1) / p.n_split) - r.kb_lo;
-    const int live = min(PG_TOK, p.n_tok - r.tt * PG_TOK);
-    r.cols = (live + 31) & ~31;
+    r.t0 = tt * p.tok, r.live = min(p.tok, p.n_tok - r.t0);
+    r.cols = (r.live + 31) & ~31;
     return r;
   };
   bool ok = true;
@@ -244,15 +255,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
       // ---- producer: this CTA's weight rows and its share of the planes; both CTAs complete on the leader's barrier --------
       auto load_w = [&](const Item& r, int kb, int s) {
         const unsigned bar = tc_smem_u32(&s_full[s]) & 0xFEFFFFFFu, a = base + s * PG_STAGE_BYTES;
-        if (rank == 0) tc_mbar_expect_tx(tc_smem_u32(&s_full[s]), 2u * PG_STAGE_BYTES);
+        if (rank == 0) tc_mbar_expect_tx(tc_smem_u32(&s_full[s]), 2u * (PG_A_BYTES + pg_width(pg_width_of(r.cols)) * (3u * TC_BK)));
         if (EPI == PG_SWIGLU) pg_tma_3d(a, &map_w, bar, kb * TC_BK, (2 * r.rp + (int)rank) * 64, 0);
         else pg_tma_2d(a, &map_w, bar, kb * TC_BK, (2 * r.rp + (int)rank) * 128);
       };
       auto load_x = [&](const Item& r, int kb, int s) {
         const unsigned bar = tc_smem_u32(&s_full[s]) & 0xFEFFFFFFu, b = base + s * PG_STAGE_BYTES + PG_A_BYTES;
-        const int row = r.tt * PG_TOK;
-        pg_tma_3d(b, &map_x1, bar, kb * TC_BK, row, (int)rank);
-        pg_tma_3d(b + PG_B1_BYTES, &map_x2, bar, kb * TC_BK, row + (int)rank * (r.cols >> 1), 2);
+        const int w = pg_width_of(r.cols);
+        pg_tma_3d(b, &maps.x1[w], bar, kb * TC_BK, r.t0, (int)rank);
+        pg_tma_3d(b + PG_B1_BYTES, &maps.x2[w], bar, kb * TC_BK, r.t0 + (int)rank * (r.cols >> 1), 2);
       };
       // the first ring-full of weights is requested ahead of the predecessor's completion
       int pre = 0;
@@ -282,8 +293,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
       if (!ok) s_fail = 1, *p.err = p.err_code;
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
-      // ---- MMA issuer of the pair --------------------------------------------------------------------------------------
+    if (rank == 0) {
+      // ---- MMA issuer of the pair: the warp walks the k-blocks together, one elected lane issues (see tc_elect_one) ------------
       const unsigned long long desc0 = tc_smem_desc(0);
       int s = 0, n = 0;
       unsigned par = 0;
@@ -297,38 +308,56 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
         for (int kb = 0; kb < r.n_kb; ++kb) {
           wait(&s_full[s], par);
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const unsigned a = base + s * PG_STAGE_BYTES, b1 = a + PG_A_BYTES, b2 = b1 + PG_B1_BYTES;
-          const unsigned long long ad = desc0 | ((a >> 4) & 0x3FFF), bd1 = desc0 | ((b1 >> 4) & 0x3FFF), bd2 = desc0 | ((b2 >> 4) & 0x3FFF);
+          if (tc_elect_one()) {
+            const unsigned a = base + s * PG_STAGE_BYTES, b1 = a + PG_A_BYTES, b2 = b1 + PG_B1_BYTES;
+            const unsigned long long ad = desc0 | ((a >> 4) & 0x3FFF), bd1 = desc0 | ((b1 >> 4) & 0x3FFF), bd2 = desc0 | ((b2 >> 4) & 0x3FFF);
 #pragma unroll
-          for (int ks = 0; ks < TC_BK / 16; ++ks) {
-            pg_mma(d, ad + 2 * ks, bd1 + 2 * ks, idesc1, (kb | ks) != 0);
-            pg_mma(d + r.cols, ad + 2 * ks, bd2 + 2 * ks, idesc2, 1);
+            for (int ks = 0; ks < TC_BK / 16; ++ks) {
+              pg_mma(d, ad + 2 * ks, bd1 + 2 * ks, idesc1, (kb | ks) != 0);
+              pg_mma(d + r.cols, ad + 2 * ks, bd2 + 2 * ks, idesc2, 1);
+            }
+            pg_commit(tc_smem_u32(&s_empty[s]));
+            if (kb == r.n_kb - 1) pg_commit(tc_smem_u32(&s_accf[buf]));
           }
-          pg_commit(tc_smem_u32(&s_empty[s]));
+          __syncwarp();
           if (++s == PG_STAGES) s = 0, par ^= 1u;
         }
-        pg_commit(tc_smem_u32(&s_accf[buf]));
       }
-      if (!ok) s_fail = 1, *p.err = p.err_code;
+      if (!ok && lane == 0) s_fail = 1, *p.err = p.err_code;
     }
   } else if (warp >= 4) {
-    // ---- epilogue: thread = weight row of this CTA's block --------------------------------------------------------------
+    // ---- epilogue: thread = weight row of this CTA's block.  Two teams of four warps take 16 tokens each in turn: with one, the
+    // epilogue of a QKV tile (its rotary factors waited for one by one) took as long as two tiles of MMAs, and a pass of a few
+    // hundred tokens has one or two tiles per pair to hide it behind [QKV of 400 tokens: 61 us with both] ----------------
     pdl_wait();
-    const int j = tid - 128, ew = warp - 4;
+    const int team = (warp - 4) >> 2, ew = warp & 3, j = (tid - 128) & 127;
     const unsigned lane_off = (unsigned)(ew * 32) << 16;
-    int n = 0, sb = 0;
+    float* const sx = reinterpret_cast<float*>(pg_smem_raw + (base - tc_smem_u32(pg_smem_raw)) + PG_STAGES * PG_STAGE_BYTES) + team * (PG_ST_TOK * PG_ST_LD);
+    int n = 0;
     for (int it = cid; it < n_items; it += n_cl, ++n) {
       const Item r = item_of(it);
       const int buf = n & 1, uses = n >> 1;
-      const int t0 = r.tt * PG_TOK, live = min(PG_TOK, p.n_tok - t0);
+      const int t0 = r.t0, live = r.live;
       const int n0 = (2 * r.rp + (int)rank) * (EPI == PG_SWIGLU ? 64 : 128);
+      // QKV: a thread's rotary pair, its eight tokens of a step, and their rotary factors (requested a step ahead)
+      const int d = p.head_dim, hd2 = d >> 1, Hq = p.n_q_heads * d, Hk = p.n_kv_heads * d;
+      const int region = n0 < Hq ? 0 : (n0 < Hq + Hk ? 1 : 2);
+      const int rbase = region == 0 ? 0 : (region == 1 ? Hq : Hq + Hk);
+      const int pj = j & 63, hh = EPI == PG_QKV ? pj / hd2 : 0, i = pj - hh * hd2, head = EPI == PG_QKV ? (n0 - rbase) / d + hh : 0, tq = (j >> 6) * 8;
+      float2 cs[8];
+      auto load_cs = [&](int c0) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          cs[q] = region < 2 && c0 + tq + q < live ? p.rope[(size_t)(p.p0 + t0 + c0 + tq + q) * hd2 + i] : make_float2(1.f, 0.f);
+      };
+      if (EPI == PG_QKV) load_cs(team * PG_ST_TOK);
       if (EPI != PG_PART) {
-        pg_team_sync();  // the previous tile's readers of s_rstd are done
-        if (j < live) s_rstd[j] = 1.0f / sqrtf(p.sumsq[t0 + j] / (float)p.H + p.eps);
+        pg_team_sync(team);  // the previous tile's readers of s_rstd are done
+        if (j < live) s_rstd[team][j] = 1.0f / sqrtf(p.sumsq[t0 + j] / (float)p.H + p.eps);
       }
       wait(&s_accf[buf], uses & 1);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      for (int c0 = 0; c0 < live; c0 += PG_ST_TOK) {
+      for (int c0 = team * PG_ST_TOK; c0 < live; c0 += 2 * PG_ST_TOK) {
         unsigned hi[16], ml[16];
         pg_ld16(hi, tmem + lane_off + buf * 256 + c0);
         pg_ld16(ml, tmem + lane_off + buf * 256 + r.cols + c0);
@@ -342,50 +371,42 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
           }
           continue;
         }
-        float* sx = st + sb * (PG_ST_TOK * PG_ST_LD);
-        sb ^= 1;
+        pg_team_sync(team);  // the readers of the step before are done
 #pragma unroll
         for (int c = 0; c < 16; ++c) sx[c * PG_ST_LD + j] = __uint_as_float(hi[c]) + __uint_as_float(ml[c]);
-        pg_team_sync();  // (two buffers: the readers of the one before are past their own barrier by the time it is written again)
+        pg_team_sync(team);
         if (EPI == PG_SWIGLU) {  // two neighbouring features, four tokens per thread
           const int f2 = 2 * lane, f = n0 + f2;
           if (f < p.F) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               const int c = ew * 4 + q;
-              if (c0 + c >= live) break;
-              const float rs = s_rstd[c0 + c];
+              const float rs = s_rstd[team][c0 + c];
               const float2 gt = *reinterpret_cast<const float2*>(sx + c * PG_ST_LD + f2), up = *reinterpret_cast<const float2*>(sx + c * PG_ST_LD + 64 + f2);
               const float g0 = gt.x * rs, g1 = gt.y * rs;
-              store_split2(p.planes + (size_t)(t0 + c0 + c) * 3 * p.F, p.F, f, g0 / (1.0f + expf(-g0)) * (up.x * rs), g1 / (1.0f + expf(-g1)) * (up.y * rs));
+              const float y0 = g0 / (1.0f + expf(-g0)) * (up.x * rs), y1 = g1 / (1.0f + expf(-g1)) * (up.y * rs);
+              if (c0 + c < live) store_split2(p.planes + (size_t)(t0 + c0 + c) * 3 * p.F, p.F, f, y0, y1);
             }
           }
-        } else {  // QKV: rotary pairs, eight tokens per thread
-          const int d = p.head_dim, hd2 = d >> 1, Hq = p.n_q_heads * d, Hk = p.n_kv_heads * d;
-          const int region = n0 < Hq ? 0 : (n0 < Hq + Hk ? 1 : 2);
-          const int rbase = region == 0 ? 0 : (region == 1 ? Hq : Hq + Hk);
-          const int pj = j & 63, hh = pj / hd2, i = pj - hh * hd2, head = (n0 - rbase) / d + hh;
-          if (n0 < p.N) {
+        } else if (n0 < p.N) {  // QKV: a rotary pair, eight tokens per thread
+          float2 y[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              const int c = (j >> 6) * 8 + q;
-              if (c0 + c >= live) break;
-              const float rs = s_rstd[c0 + c];
-              const float x1 = sx[c * PG_ST_LD + hh * d + i] * rs, x2 = sx[c * PG_ST_LD + hh * d + i + hd2] * rs;
-              float y1 = x1, y2 = x2;
-              const int pos = p.p0 + t0 + c0 + c;
-              if (region < 2) {
-                const float2 cs = p.rope[(size_t)pos * hd2 + i];
-                y1 = x1 * cs.x - x2 * cs.y;
-                y2 = x2 * cs.x + x1 * cs.y;
-              }
-              if (region == 0) {
-                float* qd = p.qbuf + (size_t)(t0 + c0 + c) * Hq + head * d + i;
-                qd[0] = y1, qd[hd2] = y2;
-              } else {
-                __nv_bfloat16* dst = p.kv + (size_t)(region - 1) * p.kv_sel_stride + ((size_t)(p.seq * p.n_kv_heads + head) * p.slots + pos) * d + i;
-                dst[0] = __float2bfloat16_rn(y1), dst[hd2] = __float2bfloat16_rn(y2);
-              }
+          for (int q = 0; q < 8; ++q) {
+            const float rs = s_rstd[team][c0 + tq + q];
+            const float x1 = sx[(tq + q) * PG_ST_LD + hh * d + i] * rs, x2 = sx[(tq + q) * PG_ST_LD + hh * d + i + hd2] * rs;
+            y[q] = region < 2 ? make_float2(x1 * cs[q].x - x2 * cs[q].y, x2 * cs[q].x + x1 * cs[q].y) : make_float2(x1, x2);
+          }
+          load_cs(c0 + 2 * PG_ST_TOK);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const int c = c0 + tq + q;
+            if (c >= live) continue;
+            if (region == 0) {
+              float* qd = p.qbuf + (size_t)(t0 + c) * Hq + head * d + i;
+              qd[0] = y[q].x, qd[hd2] = y[q].y;
+            } else {
+              __nv_bfloat16* dst = p.kv + (size_t)(region - 1) * p.kv_sel_stride + ((size_t)(p.seq * p.n_kv_heads + head) * p.slots + p.p0 + t0 + c) * d + i;
+              dst[0] = __float2bfloat16_rn(y[q].x), dst[hd2] = __float2bfloat16_rn(y[q].y);
             }
           }
         }

@@ -673,3 +673,15 @@ def test_wide_prompt_passes_match_oracle(name, n_prompt, T):
     ctx.decode(12)
     U.assert_same_run(ctx, ref, 12)
     ctx.close()
+
+
+@pytest.mark.parametrize("n_prompt", [96, 97, 160, 192, 224, 257])
+def test_prompt_tiles_of_every_width_match_oracle(n_prompt):
+    """The token tiles of a wide pass are 128, 96 or 64 columns (whichever fills the pairs of CTAs evenly) with a narrower one for the
+    leftover tokens: prompts at the edges of the widths, against the oracle's logits."""
+    ref = U.oracle_run("small_bf16", n_prompt, 6, 1, 2, seed=3)
+    ctx = U.make_ctx("small_bf16", 1, 2, seed=3, max_ctx=320)
+    assert ctx.prefill(ref["prompt"]) == ref["first"]
+    assert ctx.decode(6)[0].tolist() == ref["tokens"], U.min_margin(ref["dec"])
+    U.assert_same_run(ctx, ref, 6)
+    ctx.close()
