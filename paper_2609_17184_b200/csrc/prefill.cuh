@@ -12,8 +12,8 @@
 // A row's arithmetic is a function of its own operands and of the model's shapes: k-splits depend on the matrix alone, every
 // accumulation chain runs over the whole k-range of its split, so results do not depend on how the prompt is cut into passes.
 //
-// Prompt of the 1.4B shape, wall clock of loopspec_prefill: 512 tokens 100 ms (passes of 32 rows; 61 ms with 64) -> 17.9 ms, 3001
-// tokens 716 -> 117 ms; three-plane products at the measured GEMM peak would take 9 / 56 ms.
+// Prompt of the 1.4B shape, wall clock of loopspec_prefill: 512 tokens 100 ms (passes of 32 rows; 61 ms with 64) -> 15.6 ms, 3001
+// tokens 716 -> 110 ms; three-plane products at the measured GEMM peak would take 9 / 56 ms.
 #pragma once
 #include <cuda.h>
 
@@ -475,17 +475,23 @@ __global__ void __launch_bounds__(256) pf_reduce_kernel(const __grid_constant__ 
 }
 
 // ---- attention ---------------------------------------------------------------------------------------------------------
-// A CTA owns 64 rows of the pass (16 per warp) and one query head and walks the keys 64 at a time; every row keeps a running
-// softmax.  Both contractions are mma.sync on exact three-plane splits, chains hi and (mid + lo) of one chunk folded in fp32
-// (a row's result depends on its own prefix only).  The softmax weights never leave registers: an accumulator fragment of the
-// scores is the A fragment of the second contraction.  Keys and values are double-buffered (cp.async); rows of shared memory
-// are swizzled in 16-byte pieces so that ldmatrix is free of bank conflicts.  Blocks with the longest prefixes start first.
-constexpr int PFA_ROWS = 64, PFA_KEYS = 64, PFA_THREADS = 128;
+// A CTA owns 64 rows of the pass and one query head.  Two groups of four warps (16 rows per warp) walk the keys 64 at a time, one the
+// even chunks and one the odd; every row keeps a running softmax per group, and the two are folded at the end.  Both
+// contractions are mma.sync on exact three-plane splits, chains hi and (mid + lo) of one chunk folded in fp32 (a row's result
+// depends on its own prefix only: chunks lie at absolute positions).  The softmax weights never leave registers: an accumulator
+// fragment of the scores is the A fragment of the second contraction.  Keys and values are double-buffered (cp.async) per
+// group; rows of shared memory are swizzled in 16-byte pieces so that ldmatrix is free of bank conflicts.  Blocks with the
+// longest prefixes start first.  A chunk is a chain of some 7800 cycles of one warp against 3100 of its MMAs, so a prompt of a few
+// hundred positions is bound by the longest block's chain, which the two groups halve.
+// Of the 1.4B shape, one group of four warps -> two: 512 positions 36 -> 28 us, the last pass of 3001 positions 237 -> 207 us.
+constexpr int PFA_ROWS = 64, PFA_KEYS = 64, PFA_GROUPS = 2, PFA_THREADS = PFA_GROUPS * 128;
 template <int D>
 struct PfaCfg {
   static constexpr int ROWB = D * 2;                                // bytes of a row of Q, K, V
   static constexpr int Q_BYTES = 3 * PFA_ROWS * ROWB, KV_BYTES = PFA_KEYS * ROWB;
-  static constexpr int SMEM_BYTES = Q_BYTES + 4 * KV_BYTES;         // Q planes, two buffers of K and V
+  static constexpr int SMEM_BYTES = Q_BYTES + PFA_GROUPS * 4 * KV_BYTES;  // Q planes, two buffers of K and V per group
+  static constexpr int FOLD_LD = D + 4;                             // floats per row of the fold's buffer (over a group's K and V)
+  static_assert(PFA_ROWS * FOLD_LD * 4 <= 4 * KV_BYTES, "the second group's rows fit its buffers");
 };
 struct PfAttnParams {
   const float* qbuf;         // [row][n_q_heads * D], rotary applied, unscaled
@@ -495,15 +501,15 @@ struct PfAttnParams {
   int n_rows, p0, slots, n_kv_heads, n_q_heads;
   float scale;
 };
-__device__ __forceinline__ unsigned pfa_pack(unsigned short a, unsigned short b) { return a | ((unsigned)b << 16); }
 
 template <int D>
-__global__ void __launch_bounds__(PFA_THREADS, 2) pf_attn_kernel(const __grid_constant__ PfAttnParams p) {
+__global__ void __launch_bounds__(PFA_THREADS, 1) pf_attn_kernel(const __grid_constant__ PfAttnParams p) {
   using C = PfaCfg<D>;
   constexpr int PCS = D / 8;  // 16-byte pieces per row
   extern __shared__ __align__(128) unsigned char pfa_smem[];
-  const unsigned sq = (unsigned)__cvta_generic_to_shared(pfa_smem), sk = sq + C::Q_BYTES, sv = sk + 2 * C::KV_BYTES;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int tid = threadIdx.x, grp = tid >> 7, gtid = tid & 127, warp = (tid >> 5) & 3, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const unsigned sq = (unsigned)__cvta_generic_to_shared(pfa_smem), sk = sq + C::Q_BYTES + grp * 4 * C::KV_BYTES, sv = sk + 2 * C::KV_BYTES;
+  auto group_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory"); };
   pdl_launch_dependents();
   const int h = blockIdx.x % p.n_q_heads, n_blocks = (p.n_rows + PFA_ROWS - 1) / PFA_ROWS;
   const int blk = n_blocks - 1 - blockIdx.x / p.n_q_heads;
@@ -517,8 +523,8 @@ __global__ void __launch_bounds__(PFA_THREADS, 2) pf_attn_kernel(const __grid_co
   auto load_chunk = [&](int chunk, int b) {
     const int k0 = chunk * PFA_KEYS;
 #pragma unroll
-    for (int i = 0; i < PFA_KEYS * PCS / PFA_THREADS; ++i) {
-      const int idx = tid + i * PFA_THREADS, key = idx / PCS, c = idx % PCS;
+    for (int i = 0; i < PFA_KEYS * PCS / 128; ++i) {
+      const int idx = gtid + i * 128, key = idx / PCS, c = idx % PCS;
       const bool live = k0 + key < n_keys;
       const size_t off = (size_t)(live ? k0 + key : 0) * D + c * 8;
       const int n = live ? 16 : 0;  // keys beyond the block's last position: zeros
@@ -528,7 +534,7 @@ __global__ void __launch_bounds__(PFA_THREADS, 2) pf_attn_kernel(const __grid_co
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   pdl_wait();
-  load_chunk(0, 0);
+  if (grp < n_chunks) load_chunk(grp, 0);
   // the block's queries, split into three planes (rows the pass does not have: zeros)
   for (int idx = tid; idx < PFA_ROWS * PCS; idx += PFA_THREADS) {
     const int lr = idx / PCS, c = idx % PCS;
@@ -538,14 +544,14 @@ __global__ void __launch_bounds__(PFA_THREADS, 2) pf_attn_kernel(const __grid_co
       const float4 a = src[0], b = src[1];
       x[0] = a.x, x[1] = a.y, x[2] = a.z, x[3] = a.w, x[4] = b.x, x[5] = b.y, x[6] = b.z, x[7] = b.w;
     }
-    unsigned short s[3][8];
+    unsigned s[4][3];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) split3(x[i], s[0][i], s[1][i], s[2][i]);
+    for (int i = 0; i < 4; ++i) split3_pair(x[2 * i], x[2 * i + 1], s[i]);
 #pragma unroll
     for (int pl = 0; pl < 3; ++pl)
-      *reinterpret_cast<uint4*>(pfa_smem + pl * PFA_ROWS * C::ROWB + piece(lr, c)) =
-          make_uint4(pfa_pack(s[pl][0], s[pl][1]), pfa_pack(s[pl][2], s[pl][3]), pfa_pack(s[pl][4], s[pl][5]), pfa_pack(s[pl][6], s[pl][7]));
+      *reinterpret_cast<uint4*>(pfa_smem + pl * PFA_ROWS * C::ROWB + piece(lr, c)) = make_uint4(s[0][pl], s[1][pl], s[2][pl], s[3][pl]);
   }
+  __syncthreads();
   float o[D / 8][4], m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
 #pragma unroll
   for (int j = 0; j < D / 8; ++j)
@@ -555,15 +561,15 @@ __global__ void __launch_bounds__(PFA_THREADS, 2) pf_attn_kernel(const __grid_co
   const int last_pos = p.p0 + row0 + wr + 15;  // ... and the last position any of them has
   // ldmatrix lane addresses: A tiles (16 x 16): rows lane & 15, piece half lane >> 4; B tiles of K (two 8-key tiles x 16 dims):
   // keys (lane & 7) + 8 (lane >> 4), piece half (lane >> 3) & 1; V, transposed: keys lane & 15, piece half lane >> 4
-  for (int chunk = 0; chunk < n_chunks; ++chunk) {
-    const int b = chunk & 1, k0 = chunk * PFA_KEYS;
-    if (chunk + 1 < n_chunks) {
-      load_chunk(chunk + 1, b ^ 1);
+  for (int chunk = grp; chunk < n_chunks; chunk += PFA_GROUPS) {
+    const int b = (chunk / PFA_GROUPS) & 1, k0 = chunk * PFA_KEYS;
+    if (chunk + PFA_GROUPS < n_chunks) {
+      load_chunk(chunk + PFA_GROUPS, b ^ 1);
       asm volatile("cp.async.wait_group 1;" ::: "memory");
     } else {
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-    __syncthreads();
+    group_sync();
     if (k0 <= last_pos) {  // (uniform over the warp) some row of the warp sees this chunk
       float s0[8][4], s1[8][4];
 #pragma unroll
@@ -600,13 +606,14 @@ __global__ void __launch_bounds__(PFA_THREADS, 2) pf_attn_kernel(const __grid_co
           s0[j][i] = sv_;
           mn[hf] = fmaxf(mn[hf], sv_);
         }
-      float wa[2], lc[2] = {0.f, 0.f};
+      float wa[2], m0[2], lc[2] = {0.f, 0.f};
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
         mn[hf] = fmaxf(mn[hf], __shfl_xor_sync(0xffffffffu, mn[hf], 1));
         mn[hf] = fmaxf(mn[hf], __shfl_xor_sync(0xffffffffu, mn[hf], 2));
         wa[hf] = m[hf] == -INFINITY ? 0.f : expf(m[hf] - mn[hf]);
         m[hf] = mn[hf];
+        m0[hf] = mn[hf] == -INFINITY ? 0.f : mn[hf];  // (a row that sees none of the group's chunks so far: every weight is zero)
       }
       // weights, split into three planes as A fragments: keys 16 kk + 2 t (+ 1) from tile 2 kk, + 8 from tile 2 kk + 1
       unsigned pa[PFA_KEYS / 16][3][4];
@@ -614,13 +621,12 @@ __global__ void __launch_bounds__(PFA_THREADS, 2) pf_attn_kernel(const __grid_co
       for (int j = 0; j < 8; ++j)
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
-          const float e0 = expf(s0[j][2 * hf] - m[hf]), e1 = expf(s0[j][2 * hf + 1] - m[hf]);  // (key 0 is visible to every row: m is finite)
+          const float e0 = expf(s0[j][2 * hf] - m0[hf]), e1 = expf(s0[j][2 * hf + 1] - m0[hf]);
           lc[hf] += e0 + e1;
-          unsigned short h0, m0, l0, h1, m1, l1;
-          split3(e0, h0, m0, l0);
-          split3(e1, h1, m1, l1);
-          const int r = hf + 2 * (j & 1);
-          pa[j >> 1][0][r] = pfa_pack(h0, h1), pa[j >> 1][1][r] = pfa_pack(m0, m1), pa[j >> 1][2][r] = pfa_pack(l0, l1);
+          unsigned w[3];
+          split3_pair(e0, e1, w);
+#pragma unroll
+          for (int pl = 0; pl < 3; ++pl) pa[j >> 1][pl][hf + 2 * (j & 1)] = w[pl];
         }
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
@@ -653,15 +659,34 @@ __global__ void __launch_bounds__(PFA_THREADS, 2) pf_attn_kernel(const __grid_co
           for (int i = 0; i < 4; ++i) o[2 * dt + e][i] = fmaf(o[2 * dt + e][i], wa[i >> 1], a0[e][i] + a1[e][i]);
       }
     }
-    __syncthreads();  // the buffer may be refilled
+    group_sync();  // the buffer may be refilled
   }
+  // ---- the odd chunks' sums join the even chunks' ----
+  float* const fold = reinterpret_cast<float*>(pfa_smem + C::Q_BYTES + 4 * C::KV_BYTES);
+  if (grp == 1) {  // (all of this group's reads of its buffers are behind its last barrier)
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      float* row = fold + (wr + g + 8 * hf) * C::FOLD_LD;
+      if (t == 0) row[D] = m[hf], row[D + 1] = l[hf];
+#pragma unroll
+      for (int j = 0; j < D / 8; ++j) *reinterpret_cast<float2*>(row + 8 * j + 2 * t) = make_float2(o[j][2 * hf], o[j][2 * hf + 1]);
+    }
+  }
+  __syncthreads();
+  if (grp == 1) return;
 #pragma unroll
   for (int hf = 0; hf < 2; ++hf) {
     const int lr = wr + g + 8 * hf;
     if (lr >= rows_here) continue;
+    const float* row = fold + lr * C::FOLD_LD;
+    const float m1 = row[D], mx = fmaxf(m[hf], m1);  // (key 0 is among the even chunks' and visible to every row: finite)
+    const float w0 = expf(m[hf] - mx), w1 = m1 == -INFINITY ? 0.f : expf(m1 - mx), mass = fmaf(l[hf], w0, row[D + 1] * w1);
     __nv_bfloat16* dst = p.aplanes + (size_t)(row0 + lr) * 3 * HQ;
 #pragma unroll
-    for (int j = 0; j < D / 8; ++j) store_split2(dst, HQ, h * D + 8 * j + 2 * t, o[j][2 * hf] / l[hf], o[j][2 * hf + 1] / l[hf]);
+    for (int j = 0; j < D / 8; ++j) {
+      const float2 o1 = *reinterpret_cast<const float2*>(row + 8 * j + 2 * t);
+      store_split2(dst, HQ, h * D + 8 * j + 2 * t, fmaf(o[j][2 * hf], w0, o1.x * w1) / mass, fmaf(o[j][2 * hf + 1], w0, o1.y * w1) / mass);
+    }
   }
 }
 
