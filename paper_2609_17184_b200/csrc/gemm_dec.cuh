@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(DG_THREADS) dgemm_kernel(const __grid_constant
 
   const GemmParams& p = q.g;
   cg::cluster_group cluster = cg::this_cluster();
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // (warp: uniform to the compiler)
   const int cs = p.cluster_size, rank = cs > 1 ? (int)cluster.block_rank() : 0, cid = blockIdx.x / cs;
   const int MP = q.MP, S = q.stages;
   const int own_max = (MP + cs - 1) / cs;
@@ -279,37 +279,42 @@ __global__ void __launch_bounds__(DG_THREADS) dgemm_kernel(const __grid_constant
       if (!ok) s_fail = 1, *p.err = q.err_code;
     }
   } else if (warp == 5 || warp == 7) {
-    if (lane == 0) {
-      // ---- MMA issuers: issuing an MMA of so few columns costs its thread ~150 cycles, so two threads share a k-block:
-      // thread ch issues the 16-wide k-steps ch, ch + 2 into its own accumulation chain (the chains are added in fixed
-      // order when the accumulator is read); a stage is free when both have committed ----
-      const int ch = warp == 5 ? 0 : 1;
-      const unsigned idesc = tc_idesc(TC_BM, (int)mma_n);
-      const unsigned long long desc0 = tc_smem_desc(0);  // the fixed bits of a shared-memory descriptor
-      bool ok = true;
-      int s = 0;
-      unsigned par = 0;
-      for (int task = 0; task < n_tasks; ++task) {
-        const int buf = q.acc_bufs > 1 ? (task & 1) : 0;
-        const int uses = q.acc_bufs > 1 ? (task >> 1) : task;  // earlier uses of this accumulator buffer
-        if (uses > 0 && !dg_wait(tc_smem_u32(&s_acce[buf]), (uses - 1) & 1, limit)) ok = false;  // its readers are done
+    // ---- MMA issuers: two warps share a k-block, an elected lane of each issuing (see tc_elect_one).  Warp ch issues the 16-wide
+    // k-steps ch, ch + 2 into its own accumulation chain (the chains are added in fixed order when the accumulator is read);
+    // a stage is free when both have committed ----
+    const int ch = warp == 5 ? 0 : 1;
+    const unsigned idesc = tc_idesc(TC_BM, (int)mma_n);
+    const unsigned long long desc0 = tc_smem_desc(0);  // the fixed bits of a shared-memory descriptor
+    bool ok = true;
+    int s = 0;
+    unsigned par = 0;
+    for (int task = 0; task < n_tasks; ++task) {
+      const int buf = q.acc_bufs > 1 ? (task & 1) : 0;
+      const int uses = q.acc_bufs > 1 ? (task >> 1) : task;  // earlier uses of this accumulator buffer
+      if (uses > 0 && !dg_wait(tc_smem_u32(&s_acce[buf]), (uses - 1) & 1, limit)) ok = false;  // its readers are done
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const unsigned d_tmem = tmem + (unsigned)buf * acc_stride + (unsigned)ch * mma_n;
+      for (int kbl = 0; kbl < n_kb; ++kbl) {
+        if (!dg_wait(tc_smem_u32(&s_full[s]), par, limit)) ok = false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const unsigned d_tmem = tmem + (unsigned)buf * acc_stride + (unsigned)ch * mma_n;
-        for (int kbl = 0; kbl < n_kb; ++kbl) {
-          if (!dg_wait(tc_smem_u32(&s_full[s]), par, limit)) ok = false;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (tc_elect_one()) {
           const unsigned b = base + s * stage_bytes;
           const unsigned long long bdesc = desc0 | (unsigned long long)((b >> 4) & 0x3FFF);
           const unsigned long long adesc = desc0 | (unsigned long long)(((b + x_bytes) >> 4) & 0x3FFF);
 #pragma unroll
-          for (int ks = ch; ks < TC_BK / 16; ks += DG_CHAINS) tc_mma(d_tmem, adesc + 2 * ks, bdesc + 2 * ks, idesc, (kbl | (ks / DG_CHAINS)) != 0);
+          for (int k2 = 0; k2 < TC_BK / 16 / DG_CHAINS; ++k2) {
+            const int ks = ch + k2 * DG_CHAINS;
+            tc_mma(d_tmem, adesc + 2 * ks, bdesc + 2 * ks, idesc, (kbl | k2) != 0);
+          }
           tc_commit(tc_smem_u32(&s_empty[s]));
-          if (++s == S) s = 0, par ^= 1u;
         }
-        tc_commit(tc_smem_u32(&s_accf[buf]));
+        __syncwarp();
+        if (++s == S) s = 0, par ^= 1u;
       }
-      if (!ok) s_fail = 1, *p.err = q.err_code;
+      if (tc_elect_one()) tc_commit(tc_smem_u32(&s_accf[buf]));
+      __syncwarp();
     }
+    if (!ok && lane == 0) s_fail = 1, *p.err = q.err_code;
   } else {
     // ---- accumulator readers / epilogue team: thread j = row j of the block ----
     pdl_wait();

@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
   __shared__ unsigned s_tmem;
   __shared__ int s_fail;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // (warp: uniform to the compiler)
   const unsigned base = (tc_smem_u32(tc_smem_raw) + 1023u) & ~1023u;  // swizzled tiles sit on 1024-byte boundaries
   const int stage_bytes = tc_stage_bytes(p.MP);
   const int n0 = blockIdx.x * TC_BM;
@@ -192,8 +192,9 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
     }
     if (!ok) s_fail = 1, *p.err = p.err_code;
   }
-  if (tid == 0 && n_kb > 0) {
-    // ---- MMA issuer: one thread, the accumulator lives in tensor memory ----
+  __syncwarp();  // (the other lanes do not poll for the end next to the producer)
+  if (warp == 0 && n_kb > 0) {
+    // ---- MMA issuer: one elected lane, the accumulator lives in tensor memory ----
     const unsigned idesc = tc_idesc(TC_BM, 3 * p.MP);
     bool ok = true;
     for (int kb = 0; kb < n_kb && ok; ++kb) {
@@ -201,15 +202,18 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
       ok = tc_mbar_wait(tc_smem_u32(&s_full[s]), (kb / p.stages) & 1);
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const unsigned a = base + s * stage_bytes, b = a + TC_BM * TC_BK * 2;
-      const unsigned long long adesc = tc_smem_desc(a);
-      const unsigned long long bdesc = tc_smem_desc(b);  // rows pl * MP + column: the hi, mid, lo planes stacked
+      if (tc_elect_one()) {
+        const unsigned a = base + s * stage_bytes, b = a + TC_BM * TC_BK * 2;
+        const unsigned long long adesc = tc_smem_desc(a);
+        const unsigned long long bdesc = tc_smem_desc(b);  // rows pl * MP + column: the hi, mid, lo planes stacked
 #pragma unroll
-      for (int ks = 0; ks < TC_BK / 16; ++ks) tc_mma(tmem, adesc + 2 * ks, bdesc + 2 * ks, idesc, (kb | ks) != 0);
-      tc_commit(tc_smem_u32(&s_empty[s]));  // arrives when the MMAs issued so far have read their operands
+        for (int ks = 0; ks < TC_BK / 16; ++ks) tc_mma(tmem, adesc + 2 * ks, bdesc + 2 * ks, idesc, (kb | ks) != 0);
+        tc_commit(tc_smem_u32(&s_empty[s]));  // arrives when the MMAs issued so far have read their operands
+        if (kb == n_kb - 1) tc_commit(tc_smem_u32(&s_done));
+      }
+      __syncwarp();
     }
-    if (ok) tc_commit(tc_smem_u32(&s_done));
-    else s_fail = 1, *p.err = p.err_code;
+    if (!ok && lane == 0) s_fail = 1, *p.err = p.err_code;
   }
   // everyone: the accumulator is complete when the last commit arrives
   bool have = n_kb > 0;
