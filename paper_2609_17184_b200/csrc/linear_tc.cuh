@@ -141,7 +141,11 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
   __syncthreads();
   pdl_launch_dependents();
   const int row0 = p.row0 + (int)blockIdx.z * p.group_cols;
-  if (p.n_live && *p.n_live <= row0) {  // (final before the pass starts; uniform over the CTA) this group of columns is empty
+  // columns that carry a token (final before the pass starts; uniform over the CTA): the others are neither loaded for nor written.  A pass
+  // whose group is empty - the second group of a small batch, the prelude and coda blocks of a Raven pass without rows at their
+  // depths - requests no weights at all
+  const int live = p.n_live ? min(p.M, *p.n_live - row0) : p.M;
+  if (live <= 0) {
     pdl_wait();  // a kernel that ended before its predecessor would release its own dependents too early
     return;
   }
@@ -222,10 +226,10 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
   const int n = n0 + warp * 32 + lane;  // this thread's weight row = its TMEM lane
   float* out = p.out + (size_t)blockIdx.z * p.group_stride + (size_t)blockIdx.y * p.M * p.N;
   if (n_kb <= 0) {
-    for (int m = 0; m < p.M; ++m)
+    for (int m = 0; m < live; ++m)
       if (n < p.N) out[(size_t)m * p.N + n] = 0.f;
   } else if (have) {
-    for (int c0 = 0; c0 < p.MP; c0 += 16) {
+    for (int c0 = 0; c0 < live; c0 += 16) {
       unsigned w[3][16];
 #pragma unroll
       for (int pl = 0; pl < 3; ++pl) {
@@ -245,7 +249,7 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
         v[j] = __float_as_uint(__uint_as_float(w[0][j]) + (__uint_as_float(w[1][j]) + __uint_as_float(w[2][j])));
 #pragma unroll
       for (int j = 0; j < 16; ++j)
-        if (c0 + j < p.M && n < p.N) out[(size_t)(c0 + j) * p.N + n] = __uint_as_float(v[j]);
+        if (c0 + j < live && n < p.N) out[(size_t)(c0 + j) * p.N + n] = __uint_as_float(v[j]);
     }
   } else if (tid == 0) {
     *p.err = p.err_code;

@@ -756,9 +756,9 @@ cudaError_t launch_prep(loopspec_ctx* c, const RowTable* tab, int first_layer = 
 int col_groups(loopspec_ctx* c, const RowTable* tab);
 // one layer GEMM of a prefill pass on the tcgen05 kernel: raw k-split sums, then the fused epilogue
 template <int EPI>
-cudaError_t launch_tc_epi(const TcEpiParams& q, int groups, cudaStream_t st, bool pdl) {
+cudaError_t launch_tc_epi(const TcEpiParams& q, int groups, int rows, cudaStream_t st, bool pdl) {  // rows: a pass carries at most
   if (groups > 1) return launch_k(tc_epilogue_kernel<EPI, true>, dim3(q.g.n_rb, TCE_GROUPS, groups), dim3(GEMM_THREADS), 0, st, q, pdl);
-  return launch_k(tc_epilogue_kernel<EPI, false>, dim3(q.g.n_rb, TCE_GROUPS), dim3(GEMM_THREADS), 0, st, q, pdl);
+  return launch_k(tc_epilogue_kernel<EPI, false>, dim3(q.g.n_rb, std::min(TCE_GROUPS, rows)), dim3(GEMM_THREADS), 0, st, q, pdl);
 }
 cudaError_t launch_tc_gemm(loopspec_ctx* c, int which, int layer, const RowTable* tab, int cfg_i) {
   const loopspec_ctx::TcCfg& tc = c->tc[cfg_i];
@@ -776,8 +776,7 @@ cudaError_t launch_tc_gemm(loopspec_ctx* c, int which, int layer, const RowTable
   p.M = tc.cols, p.MP = tc.cols, p.N = q.g.N, p.K = q.g.K, p.kb_per_split = t.kb_per_split, p.stages = tc.stages;
   p.err = const_cast<int*>(c->host_flags_dev + HF_ERROR), p.err_code = 5, p.x3d = 1;
   p.row0 = 0, p.group_cols = GROUP_ROWS, p.group_stride = (long long)t.n_split * tc.cols * q.g.N;
-  // (only a pass of several groups can have an empty one worth skipping)
-  p.n_live = groups > 1 ? reinterpret_cast<const int*>(reinterpret_cast<const char*>(tab) + offsetof(RowTable, n_rows)) : nullptr;
+  p.n_live = cfg_i == 1 ? reinterpret_cast<const int*>(reinterpret_cast<const char*>(tab) + offsetof(RowTable, n_rows)) : nullptr;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = dim3(t.n_tiles, t.n_split, groups), cfg.blockDim = dim3(TC_THREADS), cfg.dynamicSmemBytes = tc.smem, cfg.stream = c->stream;
@@ -790,9 +789,9 @@ cudaError_t launch_tc_gemm(loopspec_ctx* c, int which, int layer, const RowTable
   cudaError_t e = cudaLaunchKernelEx(&cfg, linear_tc_kernel, wm, tc.xmaps[xi], p);
   if (e != cudaSuccess) return e;
   switch (which) {
-    case G_QKV: return launch_tc_epi<EPI_QKV>(q, groups, c->stream, c->use_pdl);
-    case G_GU: return launch_tc_epi<EPI_SWIGLU>(q, groups, c->stream, c->use_pdl);
-    default: return launch_tc_epi<EPI_RESID>(q, groups, c->stream, c->use_pdl);
+    case G_QKV: return launch_tc_epi<EPI_QKV>(q, groups, table_rows(c, tab), c->stream, c->use_pdl);
+    case G_GU: return launch_tc_epi<EPI_SWIGLU>(q, groups, table_rows(c, tab), c->stream, c->use_pdl);
+    default: return launch_tc_epi<EPI_RESID>(q, groups, table_rows(c, tab), c->stream, c->use_pdl);
   }
 }
 
