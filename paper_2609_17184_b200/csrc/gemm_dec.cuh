@@ -12,8 +12,8 @@
 // the token rows are its N columns.  Activations arrive as three bf16 planes (an exact split of the fp32 value); the
 // planes sit side by side as accumulator columns (row r, plane pl -> column 3 r + pl), so one MMA per 16-wide k-step
 // feeds three separate accumulation chains, folded hi + (mid + lo) when the accumulator is read; the even and the odd
-// k-steps go to two accumulators of their own, issued by two threads (an MMA of so few columns costs its issuing thread
-// ~150 cycles) and added in fixed order.  A token's arithmetic therefore does not depend on which other tokens share
+// k-steps go to two accumulators of their own, issued by two warps and added in
+// fixed order.  A token's arithmetic therefore does not depend on which other tokens share
 // the pass, nor on the pass width.
 //
 // Work split.  A cluster of `cs` CTAs owns row blocks rb = cluster, cluster + n_clusters, ... (128 output rows each);
