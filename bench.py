@@ -32,11 +32,11 @@ import workloads as W  # noqa: E402
 # launch configuration (`bench.py --kernel-only gate_up`), reported with its source and only for that model shape.
 NCU_TRAFFIC = {"ouro_1p4b": (46226944, "ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch, captured on "
                                        "`bench.py --kernel-only gate_up --rows 4` (not measured in this run)")}
-# the streaming attention kernel: ncu DRAM bytes of one launch on a small case (4 rows x 4096 cached positions: 137.7 MB
-# against 134.2 MB algorithmic); its traffic grows in proportion to rows x context, so a full-size launch is scaled by
-# the units it processes
-ATTN_TRAFFIC = (137.7e6 / 134.2e6, "ncu dram__bytes.sum of one launch of `bench.py --kernel-only attention --rows 4 --prompt-len 4096` "
-                                   "(137.7 MB for 134.2 MB algorithmic), scaled to this launch's rows x context (not measured in this run)")
+# the decode attention kernel of long contexts and batches: ncu DRAM bytes of one launch on a small case (4 rows x 4096 cached
+# positions: 136.0 MB, mean of two launches, against 134.2 MB algorithmic); its traffic grows in proportion to rows x context,
+# so a full-size launch is scaled by the units it processes
+ATTN_TRAFFIC = (136.0e6 / 134.2e6, "ncu dram__bytes.sum of one launch of `bench.py --kernel-only attention --rows 4 --prompt-len 4096` "
+                                   "(136.0 MB for 134.2 MB algorithmic), scaled to this launch's rows x context (not measured in this run)")
 NOMINAL_HBM_GBS = 8000.0  # datasheet figure, for context beside the measured copy bandwidth
 
 

@@ -108,45 +108,44 @@ __device__ __forceinline__ void dg_arrive(unsigned bar) {
 }
 __device__ __forceinline__ void dg_team_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }  // warps 0-3
 
-// ---- the epilogue team (threads 0..127, thread j = row j of the block) finishes this rank's columns -------------
+// ---- the epilogue team (warps 0..3) finishes this rank's columns, a warp per column, four rows of the block per lane ----
 // recv holds, for every rank rk and owned slot, the 128 partial sums that rank pushed: [rk][slot][128].
+// With a thread per row and the team walking the columns together, the largest logit of every column cost a barrier and a fold
+// over the warps [lm_head of the 1.4B shape, 8 rows 35.9 -> 33.6 us, 40 rows 96 -> 79, 56 rows 123 -> 88 us].
 template <int EPI>
 __device__ __forceinline__ void dg_epilogue(const GemmParams& p, const int* ct, int rb, int n_cols, const float* recv, int own_max,
-                                            const float* s_rstd, float* s_red, int rank, int cs) {
+                                            const float* s_rstd, int rank, int cs) {
   static_assert(EPI == EPI_PLAIN || EPI == EPI_LOGITS, "the tcgen05 decode kernel finishes plain outputs and logits");
-  const int j = threadIdx.x, lane = j & 31, hw = j >> 5;
-  constexpr int NT = DG_MAX_COLS;  // column stride of the table
-  int it = 0;
-  for (int c = rank; c < n_cols; c += cs, ++it) {
-    const float* src = recv + (size_t)(c / cs) * RB_ROWS + j;
-    float v = src[0];
-    for (int rk = 1; rk < cs; ++rk) v += src[(size_t)rk * own_max * RB_ROWS];  // rank order, the same in every launch
-    v *= s_rstd[c];
-    const int n = rb * RB_ROWS + j;
-    if (n < p.N) {
-      if (EPI == EPI_PLAIN) p.out[(size_t)c * p.out_ld + n] = v;
-      else p.logits[(size_t)ct[CT_LOGIT * NT + c] * p.N + n] = v;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int NT = DG_MAX_COLS, RPL = RB_ROWS / 32;  // column stride of the table; rows per lane
+  for (int c = rank + cs * warp; c < n_cols; c += 4 * cs) {
+    const float* src = recv + (size_t)(c / cs) * RB_ROWS + lane;
+    float v[RPL];
+#pragma unroll
+    for (int i = 0; i < RPL; ++i) v[i] = src[32 * i];
+    for (int rk = 1; rk < cs; ++rk)  // rank order, the same in every launch
+#pragma unroll
+      for (int i = 0; i < RPL; ++i) v[i] += src[(size_t)rk * own_max * RB_ROWS + 32 * i];
+    float* out = EPI == EPI_PLAIN ? p.out + (size_t)c * p.out_ld : p.logits + (size_t)ct[CT_LOGIT * NT + c] * p.N;
+    float bv = -INFINITY;
+    int bi = rb * RB_ROWS + lane;
+#pragma unroll
+    for (int i = 0; i < RPL; ++i) {
+      const int n = rb * RB_ROWS + 32 * i + lane;
+      v[i] *= s_rstd[c];
+      if (n < p.N) {
+        out[n] = v[i];
+        if (v[i] > bv) bv = v[i], bi = n;  // (rows ascend: ties keep the lowest)
+      }
     }
     if (EPI == EPI_LOGITS) {  // the block's largest logit (ties: lowest index) for the greedy selection
-      float bv = n < p.N ? v : -INFINITY;
-      int bi = n;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ov > bv || (ov == bv && oi < bi)) bv = ov, bi = oi;
       }
-      float* av = s_red + (it & 1) * 8;
-      if (lane == 0) av[hw] = bv, av[4 + hw] = __int_as_float(bi);
-      dg_team_sync();
-      if (j == 0) {
-        for (int w = 1; w < 4; ++w) {
-          const float ov = av[w];
-          const int oi = __float_as_int(av[4 + w]);
-          if (ov > bv || (ov == bv && oi < bi)) bv = ov, bi = oi;
-        }
-        p.argpart[(size_t)c * p.n_rb + rb] = make_float2(bv, __int_as_float(bi));
-      }
+      if (lane == 0) p.argpart[(size_t)c * p.n_rb + rb] = make_float2(bv, __int_as_float(bi));
     }
   }
 }
@@ -163,7 +162,6 @@ __global__ void __launch_bounds__(DG_THREADS) dgemm_kernel(const __grid_constant
   __shared__ float s_rstd[DG_MAX_COLS];
   __shared__ int s_ct[CT_FIELDS * DG_MAX_COLS];
   __shared__ int s_colof[DG_MAX_COLS];   // pass row (= MMA column) -> output column, -1: not finished by this GEMM
-  __shared__ float s_red[16];
 
   const GemmParams& p = q.g;
   cg::cluster_group cluster = cg::this_cluster();
@@ -383,7 +381,7 @@ __global__ void __launch_bounds__(DG_THREADS) dgemm_kernel(const __grid_constant
       } else {
         dg_team_sync();
       }
-      dg_epilogue<EPI>(p, s_ct, rb, n_cols, recv, own_max, s_rstd, s_red, rank, cs);
+      dg_epilogue<EPI>(p, s_ct, rb, n_cols, recv, own_max, s_rstd, rank, cs);
       if (cs == 1 && q.recv_bufs == 1) dg_team_sync();  // the one receive buffer is free again
     }
     if (!ok && lane == 0) s_fail = 1, *p.err = q.err_code;
