@@ -1095,6 +1095,15 @@ int pg_tile_width(int n, int blocks, int pairs) {
   }
   return best;
 }
+// k-blocks of an accumulation chain: never more than the passes of up to 64 rows have for this matrix, so that a prompt's sums are no
+// further from the exact ones there than here - their k-split on the tcgen05 kernel, or three where they run the cluster kernels of
+// mma.sync (clusters of up to 8 ranks).  Matrices of fewer than 32 k-blocks get at least four chains: their launches are bound by latency.
+// [error against float64, passes of up to 64 rows / this rule / chains of up to 4 for every matrix: the 768-wide model at 130 tokens
+// 1.46e-4 / 1.19e-4 / 1.59e-4]
+int pg_chain_kb(const loopspec_model& m, int N, int n_kb) {
+  const int narrow = tc_prefill_shapes_ok(&m) ? tc_pf_plan(N, n_kb * TC_BK).kb_per_split : 3;
+  return std::min(std::min(PG_SEG_MAX, narrow), std::max(2, n_kb / 4));
+}
 struct PfPass {  // rows of a pass: positions p0 .. p0 + n - 1 of sequence seq
   int seq, p0, n;
 };
@@ -1108,6 +1117,7 @@ cudaError_t launch_pf_gemm(loopspec_ctx* c, int which, int layer, const PfPass& 
   p.N = Ns[which], p.n_kb = (Ks[which] + TC_BK - 1) / TC_BK, p.n_tok = ps.n;
   p.n_rp = which == G_GU ? (m.ffn + 127) / 128 : (p.N + 255) / 256;
   p.n_split = (which == G_QKV || which == G_GU) ? 1 : pf_splits(Ks[which]);
+  p.seg_kb = pg_chain_kb(m, p.N, p.n_kb);
   p.tok = pg_tile_width(ps.n, p.n_rp * p.n_split, c->n_sm / 2), p.n_full = ps.n / p.tok, p.n_tail = ps.n % p.tok ? 1 : 0;
   p.err = const_cast<int*>(c->host_flags_dev + HF_ERROR), p.err_code = ERR_WAIT_PF;
   p.sumsq = c->at<float>(c->L.pf_sumsq), p.H = m.hidden, p.eps = m.rms_eps;

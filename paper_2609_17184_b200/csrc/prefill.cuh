@@ -9,8 +9,8 @@
 //   pf_reduce_kernel   k-split sums in split order + residual + planes of x * next gain + sum of squares
 //   pf_attn_kernel     causal attention of the pass's rows over the cached keys and values
 //
-// A row's arithmetic is a function of its own operands and of the model's shapes: k-splits depend on the matrix alone, every
-// accumulation chain runs over the whole k-range of its split, so results do not depend on how the prompt is cut into passes.
+// A row's arithmetic is a function of its own operands and of the model's shapes: k-splits and the accumulation chains within them
+// depend on the matrix alone, so results do not depend on how the prompt is cut into passes.
 //
 // Prompt of the 1.4B shape, wall clock of loopspec_prefill: 512 tokens 100 ms (passes of 32 rows; 61 ms with 64) -> 15.6 ms, 3001
 // tokens 716 -> 110 ms; three-plane products at the measured GEMM peak would take 9 / 56 ms.
@@ -114,8 +114,9 @@ __global__ void __launch_bounds__(256) pf_concat_kernel(const __grid_constant__ 
 // reads for 740 cycles of MMA (55 B per cycle; one CTA alone with 128 x 128 would need 83).  Per 16-wide k-step two MMAs:
 // [hi | mid] as 256 columns (CTA 0 holds the hi rows, CTA 1 the mid rows of all 128 tokens) and lo as 128 columns that
 // accumulate onto mid's - two chains, hi and (mid + lo), folded when the accumulator is read.  256 TMEM columns per
-// accumulator, two accumulators: the epilogue of a tile runs under the main loop of the next (persistent CTAs, tiles dealt
-// round robin, the token tiles of one weight block next to each other so that its weights come from HBM once).
+// accumulator, two accumulators in turn: the epilogue warps read one (chains of at most PG_SEG_MAX k-blocks, their sums kept in
+// registers) while the MMAs of the next chain fill the other, and finish a tile under the first chains of the next (persistent
+// CTAs, tiles dealt round robin, the token tiles of one weight block next to each other so that its weights come from HBM once).
 // A k-block takes 740 cycles at 128 columns, 560 at 96 and 540 at 64, where the operands' way through the L2 bounds it (more
 // stages change nothing); the MMAs are issued by a converged warp (see tc_elect_one: 840 cycles at any width before).  A pass of a
 // few hundred tokens has one to three tiles per pair, so their width is chosen for even rounds (pg_tile_width), and what stands
@@ -134,6 +135,13 @@ constexpr int PG_STAGES = 5;
 constexpr int PG_ST_LD = 132;                      // floats per token of the epilogue's exchange buffer
 constexpr int PG_ST_TOK = 16;                      // tokens exchanged at a time
 constexpr int PG_SMEM = 1024 + PG_STAGES * PG_STAGE_BYTES + 2 * PG_ST_TOK * PG_ST_LD * 4;  // (an exchange buffer per epilogue team)
+// k-blocks of one accumulation chain at most.  tcgen05 truncates its fp32 accumulator after every 16-wide step, so a sum's relative
+// error grows with the length of its chain and not with K; the k-range of an item is cut into chains of its own, which the epilogue adds
+// in order with rounded additions.  Relative error of the logits against float64 of one block of the 1.4B shape without its attention, 300
+// tokens: whole k-ranges 2.6e-6, chains of 8 (QKV 6, O 4, down 5) 7.9e-7, of 4 6.1e-7; the passes of up to 64 rows, whose k-splits
+// are such chains too, 9.1e-7.  Each chain costs the read of an accumulator: 70 tokens 6.97 -> 7.40 ms, 512
+// 16.8 -> 16.8, 3001 111 -> 112.
+constexpr int PG_SEG_MAX = 8;
 enum { PG_QKV = 0, PG_SWIGLU = 1, PG_PART = 2 };
 
 // The planes read by a GEMM as (k, token, plane), one pair of maps per tile width: boxes of the width (hi, mid) and of half of it (lo)
@@ -143,7 +151,7 @@ struct PgMaps {
 struct PfGemmParams {
   int n_rp, n_split;        // pairs of 128-row weight blocks, k-splits
   int tok, n_full, n_tail;  // token columns of a tile, tiles of that width, 1 when a narrower one is left over
-  int n_kb;                 // 64-wide k-blocks of the matrix
+  int n_kb, seg_kb;         // 64-wide k-blocks of the matrix, at most in one accumulation chain
   int n_tok, N;             // live rows of the pass, weight rows
   int* err;
   int err_code;
@@ -180,6 +188,11 @@ __device__ __forceinline__ void pg_mma(unsigned d_tmem, unsigned long long adesc
 __device__ __forceinline__ void pg_commit(unsigned bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"((unsigned short)3)
                : "memory");
+}
+// Arrival that hands over nothing but an accumulator that has been read: no store of this thread needs to be visible with it (as a
+// release at cluster scope it waited some 3500 cycles for the epilogue's stores)
+__device__ __forceinline__ void pg_arrive_relaxed(unsigned addr) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 __device__ __forceinline__ void pg_cluster_sync() { asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory"); }
 __device__ __forceinline__ void pg_team_sync(int team) { asm volatile("bar.sync %0, 128;" ::"r"(1 + team) : "memory"); }  // four warps of the epilogue
@@ -231,7 +244,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
   // item -> (weight block pair, split, token tile): the full tiles first, token tiles fastest; the narrow ones of the leftover tokens
   // come last and fill what the full ones leave of the last round
   struct Item {
-    int rp, sp, t0, live, kb_lo, n_kb, cols;  // cols: MMA columns of the tile (its live tokens rounded up to 32)
+    int rp, sp, t0, live, kb_lo, n_kb, n_seg, cols;  // n_seg: accumulation chains of (nearly) equal length; cols: MMA columns of the tile
+                                                     // (its live tokens rounded up to 32)
   };
   auto item_of = [&](int it) {
     Item r;
@@ -239,8 +253,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
     if (it < n_full_items) q = it / p.n_full, tt = it - q * p.n_full;
     else q = it - n_full_items, tt = p.n_full;
     r.rp = q % p.n_rp, r.sp = q / p.n_rp;
-    r.kb_lo = (int)((long long)p.n_kb * r.sp / p.n_split);
-    r.n_kb = (int)((long long)p.n_kb * (r.sp + 1) / p.n_split) - r.kb_lo;
+    r.kb_lo = p.n_kb * r.sp / p.n_split;
+    r.n_kb = p.n_kb * (r.sp + 1) / p.n_split - r.kb_lo;
+    r.n_seg = (r.n_kb + p.seg_kb - 1) / p.seg_kb;
     r.t0 = tt * p.tok, r.live = min(p.tok, p.n_tok - r.t0);
     r.cols = (r.live + 31) & ~31;
     return r;
@@ -296,31 +311,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
     if (rank == 0) {
       // ---- MMA issuer of the pair: the warp walks the k-blocks together, one elected lane issues (see tc_elect_one) ------------
       const unsigned long long desc0 = tc_smem_desc(0);
-      int s = 0, n = 0;
+      int s = 0, n = 0;  // n: segments so far
       unsigned par = 0;
-      for (int it = cid; it < n_items; it += n_cl, ++n) {
+      for (int it = cid; it < n_items; it += n_cl) {
         const Item r = item_of(it);
-        const int buf = n & 1, uses = n >> 1;
-        if (uses > 0) wait(&s_acce[buf], (uses - 1) & 1);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const unsigned d = tmem + buf * 256;
         const unsigned idesc1 = tc_idesc(256, 2 * r.cols), idesc2 = tc_idesc(256, r.cols);
-        for (int kb = 0; kb < r.n_kb; ++kb) {
-          wait(&s_full[s], par);
+        for (int sg = 0, kb = 0; sg < r.n_seg; ++sg, ++n) {
+          const int buf = n & 1, uses = n >> 1, first = kb, end = r.n_kb * (sg + 1) / r.n_seg;
+          if (uses > 0) wait(&s_acce[buf], (uses - 1) & 1);
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          if (tc_elect_one()) {
-            const unsigned a = base + s * PG_STAGE_BYTES, b1 = a + PG_A_BYTES, b2 = b1 + PG_B1_BYTES;
-            const unsigned long long ad = desc0 | ((a >> 4) & 0x3FFF), bd1 = desc0 | ((b1 >> 4) & 0x3FFF), bd2 = desc0 | ((b2 >> 4) & 0x3FFF);
+          const unsigned d = tmem + buf * 256;
+          for (; kb < end; ++kb) {
+            wait(&s_full[s], par);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (tc_elect_one()) {
+              const unsigned a = base + s * PG_STAGE_BYTES, b1 = a + PG_A_BYTES, b2 = b1 + PG_B1_BYTES;
+              const unsigned long long ad = desc0 | ((a >> 4) & 0x3FFF), bd1 = desc0 | ((b1 >> 4) & 0x3FFF), bd2 = desc0 | ((b2 >> 4) & 0x3FFF);
 #pragma unroll
-            for (int ks = 0; ks < TC_BK / 16; ++ks) {
-              pg_mma(d, ad + 2 * ks, bd1 + 2 * ks, idesc1, (kb | ks) != 0);
-              pg_mma(d + r.cols, ad + 2 * ks, bd2 + 2 * ks, idesc2, 1);
+              for (int ks = 0; ks < TC_BK / 16; ++ks) {
+                pg_mma(d, ad + 2 * ks, bd1 + 2 * ks, idesc1, kb > first || ks > 0);
+                pg_mma(d + r.cols, ad + 2 * ks, bd2 + 2 * ks, idesc2, 1);
+              }
+              pg_commit(tc_smem_u32(&s_empty[s]));
+              if (kb == end - 1) pg_commit(tc_smem_u32(&s_accf[buf]));
             }
-            pg_commit(tc_smem_u32(&s_empty[s]));
-            if (kb == r.n_kb - 1) pg_commit(tc_smem_u32(&s_accf[buf]));
+            __syncwarp();
+            if (++s == PG_STAGES) s = 0, par ^= 1u;
           }
-          __syncwarp();
-          if (++s == PG_STAGES) s = 0, par ^= 1u;
         }
       }
       if (!ok && lane == 0) s_fail = 1, *p.err = p.err_code;
@@ -333,10 +350,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
     const int team = (warp - 4) >> 2, ew = warp & 3, j = (tid - 128) & 127;
     const unsigned lane_off = (unsigned)(ew * 32) << 16;
     float* const sx = reinterpret_cast<float*>(pg_smem_raw + (base - tc_smem_u32(pg_smem_raw)) + PG_STAGES * PG_STAGE_BYTES) + team * (PG_ST_TOK * PG_ST_LD);
-    int n = 0;
-    for (int it = cid; it < n_items; it += n_cl, ++n) {
+    int n = 0;  // segments so far
+    for (int it = cid; it < n_items; it += n_cl) {
       const Item r = item_of(it);
-      const int buf = n & 1, uses = n >> 1;
       const int t0 = r.t0, live = r.live;
       const int n0 = (2 * r.rp + (int)rank) * (EPI == PG_SWIGLU ? 64 : 128);
       // QKV: a thread's rotary pair, its eight tokens of a step, and their rotary factors (requested a step ahead)
@@ -355,65 +371,90 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
         pg_team_sync(team);  // the previous tile's readers of s_rstd are done
         if (j < live) s_rstd[team][j] = 1.0f / sqrtf(p.sumsq[t0 + j] / (float)p.H + p.eps);
       }
-      wait(&s_accf[buf], uses & 1);
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      for (int c0 = team * PG_ST_TOK; c0 < live; c0 += 2 * PG_ST_TOK) {
-        unsigned hi[16], ml[16];
-        pg_ld16(hi, tmem + lane_off + buf * 256 + c0);
-        pg_ld16(ml, tmem + lane_off + buf * 256 + r.cols + c0);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (EPI == PG_PART) {
-          if (n0 + j < p.N) {
-            float* out = p.part + (size_t)r.sp * p.split_stride + (size_t)(t0 + c0) * p.N + n0 + j;
+      // the segments' sums, added in order: this thread's weight row, its team's token columns
+      constexpr int STEPS = PG_TOK / 2 / PG_ST_TOK;
+      float acc[STEPS][PG_ST_TOK];
+      for (int sg = 0; sg < r.n_seg; ++sg, ++n) {
+        const int buf = n & 1, uses = n >> 1;
+        wait(&s_accf[buf], uses & 1);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-            for (int c = 0; c < 16; ++c)
-              if (c0 + c < live) out[(size_t)c * p.N] = __uint_as_float(hi[c]) + __uint_as_float(ml[c]);
-          }
-          continue;
-        }
-        pg_team_sync(team);  // the readers of the step before are done
+        for (int q = 0; q < STEPS; ++q) {
+          const int c0 = (2 * q + team) * PG_ST_TOK;
+          if (c0 < live) {
+            unsigned hi[16], ml[16];
+            pg_ld16(hi, tmem + lane_off + buf * 256 + c0);
+            pg_ld16(ml, tmem + lane_off + buf * 256 + r.cols + c0);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-        for (int c = 0; c < 16; ++c) sx[c * PG_ST_LD + j] = __uint_as_float(hi[c]) + __uint_as_float(ml[c]);
-        pg_team_sync(team);
-        if (EPI == PG_SWIGLU) {  // two neighbouring features, four tokens per thread
-          const int f2 = 2 * lane, f = n0 + f2;
-          if (f < p.F) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const int c = ew * 4 + q;
-              const float rs = s_rstd[team][c0 + c];
-              const float2 gt = *reinterpret_cast<const float2*>(sx + c * PG_ST_LD + f2), up = *reinterpret_cast<const float2*>(sx + c * PG_ST_LD + 64 + f2);
-              const float g0 = gt.x * rs, g1 = gt.y * rs;
-              const float y0 = g0 / (1.0f + expf(-g0)) * (up.x * rs), y1 = g1 / (1.0f + expf(-g1)) * (up.y * rs);
-              if (c0 + c < live) store_split2(p.planes + (size_t)(t0 + c0 + c) * 3 * p.F, p.F, f, y0, y1);
+            for (int c = 0; c < PG_ST_TOK; ++c) {
+              const float v = __uint_as_float(hi[c]) + __uint_as_float(ml[c]);
+              acc[q][c] = sg == 0 ? v : acc[q][c] + v;
             }
           }
-        } else if (n0 < p.N) {  // QKV: a rotary pair, eight tokens per thread
-          float2 y[8];
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) pg_arrive_relaxed(dg_mapa(tc_smem_u32(&s_acce[buf]), 0));  // the accumulator may be overwritten
+      }
+      if constexpr (EPI == PG_PART) {
+        if (n0 + j < p.N) {
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const float rs = s_rstd[team][c0 + tq + q];
-            const float x1 = sx[(tq + q) * PG_ST_LD + hh * d + i] * rs, x2 = sx[(tq + q) * PG_ST_LD + hh * d + i + hd2] * rs;
-            y[q] = region < 2 ? make_float2(x1 * cs[q].x - x2 * cs[q].y, x2 * cs[q].x + x1 * cs[q].y) : make_float2(x1, x2);
+          for (int q = 0; q < STEPS; ++q) {
+            const int c0 = (2 * q + team) * PG_ST_TOK;
+            float* out = p.part + (size_t)r.sp * p.split_stride + (size_t)(t0 + c0) * p.N + n0 + j;
+#pragma unroll
+            for (int c = 0; c < PG_ST_TOK; ++c)
+              if (c0 + c < live) out[(size_t)c * p.N] = acc[q][c];
           }
-          load_cs(c0 + 2 * PG_ST_TOK);
+        }
+      } else {
+        for (int c0 = team * PG_ST_TOK; c0 < live; c0 += 2 * PG_ST_TOK) {
+          pg_team_sync(team);  // the readers of the step before are done
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int c = c0 + tq + q;
-            if (c >= live) continue;
-            if (region == 0) {
-              float* qd = p.qbuf + (size_t)(t0 + c) * Hq + head * d + i;
-              qd[0] = y[q].x, qd[hd2] = y[q].y;
-            } else {
-              __nv_bfloat16* dst = p.kv + (size_t)(region - 1) * p.kv_sel_stride + ((size_t)(p.seq * p.n_kv_heads + head) * p.slots + p.p0 + t0 + c) * d + i;
-              dst[0] = __float2bfloat16_rn(y[q].x), dst[hd2] = __float2bfloat16_rn(y[q].y);
+          for (int q = 0; q < STEPS; ++q)  // (registers are addressed by constants)
+            if (c0 == (2 * q + team) * PG_ST_TOK) {
+#pragma unroll
+              for (int c = 0; c < PG_ST_TOK; ++c) sx[c * PG_ST_LD + j] = acc[q][c];
+            }
+          pg_team_sync(team);
+          if (EPI == PG_SWIGLU) {  // two neighbouring features, four tokens per thread
+            const int f2 = 2 * lane, f = n0 + f2;
+            if (f < p.F) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const int c = ew * 4 + q;
+                const float rs = s_rstd[team][c0 + c];
+                const float2 gt = *reinterpret_cast<const float2*>(sx + c * PG_ST_LD + f2), up = *reinterpret_cast<const float2*>(sx + c * PG_ST_LD + 64 + f2);
+                const float g0 = gt.x * rs, g1 = gt.y * rs;
+                const float y0 = g0 / (1.0f + expf(-g0)) * (up.x * rs), y1 = g1 / (1.0f + expf(-g1)) * (up.y * rs);
+                if (c0 + c < live) store_split2(p.planes + (size_t)(t0 + c0 + c) * 3 * p.F, p.F, f, y0, y1);
+              }
+            }
+          } else if (n0 < p.N) {  // QKV: a rotary pair, eight tokens per thread
+            float2 y[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const float rs = s_rstd[team][c0 + tq + q];
+              const float x1 = sx[(tq + q) * PG_ST_LD + hh * d + i] * rs, x2 = sx[(tq + q) * PG_ST_LD + hh * d + i + hd2] * rs;
+              y[q] = region < 2 ? make_float2(x1 * cs[q].x - x2 * cs[q].y, x2 * cs[q].x + x1 * cs[q].y) : make_float2(x1, x2);
+            }
+            load_cs(c0 + 2 * PG_ST_TOK);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const int c = c0 + tq + q;
+              if (c >= live) continue;
+              if (region == 0) {
+                float* qd = p.qbuf + (size_t)(t0 + c) * Hq + head * d + i;
+                qd[0] = y[q].x, qd[hd2] = y[q].y;
+              } else {
+                __nv_bfloat16* dst = p.kv + (size_t)(region - 1) * p.kv_sel_stride + ((size_t)(p.seq * p.n_kv_heads + head) * p.slots + p.p0 + t0 + c) * d + i;
+                dst[0] = __float2bfloat16_rn(y[q].x), dst[hd2] = __float2bfloat16_rn(y[q].y);
+              }
             }
           }
         }
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) dg_arrive_cluster(dg_mapa(tc_smem_u32(&s_acce[buf]), 0));  // the accumulator may be overwritten
     }
     if (!ok && lane == 0) s_fail = 1, *p.err = p.err_code;
   }

@@ -685,3 +685,37 @@ def test_prompt_tiles_of_every_width_match_oracle(n_prompt):
     assert ctx.decode(6)[0].tolist() == ref["tokens"], U.min_margin(ref["dec"])
     U.assert_same_run(ctx, ref, 6)
     ctx.close()
+
+
+def _prompt_error(shape, n_prompt, **kw):
+    """Relative error (2-norm) of a prompt's logits against the float64 oracle, of a model without attention (its keys and values are
+    zero, so no rounding to bf16 hides the GEMMs' own error)."""
+    import paper_2609_17184_b200 as ls
+    from oracle.loopspec import Decoder
+    from oracle.model import LoopedLM
+    w = W.make_weights(shape, seed=3, out_scale=1.0)
+    for k in w:
+        if k.endswith("wqkv"):
+            w[k][:] = 0
+    prompt = W.make_prompt(shape.vocab, n_prompt, seed=1)
+    ref = Decoder(LoopedLM(shape, w), temperature=0.0, seed=0)
+    ref.prefill(prompt, 4)
+    gw = ls.upload_weights(shape, w)
+    out = []
+    for rows in (0, 64):  # the wide passes, passes of up to 64 rows
+        ctx = ls.LoopSpec(shape, gw, d1=1, d2=0, max_ctx=n_prompt + 16, max_prefill_rows=rows)
+        ctx.prefill(prompt)
+        z = ctx.debug_logits(0, 0).astype(np.float64)
+        out.append(np.linalg.norm(z - ref.first_logits) / np.linalg.norm(ref.first_logits))
+        ctx.close()
+    return out
+
+
+@pytest.mark.parametrize("hidden,ffn,n_prompt", [(2048, 5632, 70), (2048, 5632, 130), (768, 2000, 97)])
+def test_wide_prompt_passes_are_as_exact_as_narrow_ones(hidden, ffn, n_prompt):
+    """The tensor cores truncate their fp32 accumulators after every 16 values of k, so a GEMM's error grows with the length of its
+    accumulation chains: the wide passes may not have longer ones than the passes of up to 64 rows.  A chain of c steps of a random
+    walk loses about 2/3 c 2^-24: 1.3e-6 at the 32 steps allowed at most (whole k-ranges: 2.7e-6 at these widths)."""
+    shape = W.CONFIGS["ouro_1p4b"].with_(vocab=512, hidden=hidden, n_q_heads=hidden // 128, n_kv_heads=hidden // 128, ffn=ffn, n_recurrent=1, R=2)
+    wide, narrow = _prompt_error(shape, n_prompt)
+    assert wide < 1.3e-6 and wide < 1.25 * narrow, (wide, narrow)
