@@ -40,6 +40,8 @@ struct LinearTcParams {
   int group_cols;      //      group_stride floats to `out` (passes wider than one MMA's columns: one grid plane per
   long long group_stride;  //  group of columns)
   const int* n_live;   // x3d: number of live columns of the pass (may be null); a group beyond it has nothing to do
+  long long wait_cycles;
+  int drop_kb;         // test hook: the producer of CTA 0 skips this k-block (-1: none), so that the waits for it run out
 };
 
 __device__ __forceinline__ unsigned tc_smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -51,7 +53,7 @@ __device__ __forceinline__ void tc_mbar_expect_tx(unsigned bar, unsigned bytes) 
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 // bounded wait on a phase parity: false when it gave up
-__device__ __forceinline__ bool tc_mbar_wait(unsigned bar, unsigned parity) {
+__device__ __forceinline__ bool tc_mbar_wait(unsigned bar, unsigned parity, long long limit) {
   const long long t0 = clock64();
   for (;;) {
     unsigned ok;
@@ -61,7 +63,7 @@ __device__ __forceinline__ bool tc_mbar_wait(unsigned bar, unsigned parity) {
         : "r"(bar), "r"(parity)
         : "memory");
     if (ok) return true;
-    if (clock64() - t0 > TC_WAIT_CYCLES) return false;
+    if (clock64() - t0 > limit) return false;
   }
 }
 __device__ __forceinline__ void tc_tma_load_2d(unsigned dst, const CUtensorMap* map, unsigned bar, int x, int y) {
@@ -153,8 +155,10 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
   // completion - and while warp 0 still allocates the tensor memory; the activation tiles (which the predecessor may
   // still be writing) follow after the dependency wait, on the same barriers.
   const int pre = min(p.stages, n_kb);
+  const int drop_kb = (blockIdx.x | blockIdx.y | blockIdx.z) == 0 ? p.drop_kb : -1;
   if (tid == 32) {
     for (int kb = 0; kb < pre; ++kb) {
+      if (kb == drop_kb) continue;
       const unsigned bar = tc_smem_u32(&s_full[kb]);
       tc_mbar_expect_tx(bar, (unsigned)stage_bytes);
       tc_tma_load_2d(base + kb * stage_bytes, &map_w, bar, (kb0 + kb) * TC_BK, n0);
@@ -182,12 +186,13 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
   if (tid == 32 && n_kb > 0) {
     // ---- producer: one thread keeps the ring of stages filled by TMA ----
     for (int kb = 0; kb < pre; ++kb)
-      load_x(base + kb * stage_bytes + TC_BM * TC_BK * 2, tc_smem_u32(&s_full[kb]), (kb0 + kb) * TC_BK);
+      if (kb != drop_kb) load_x(base + kb * stage_bytes + TC_BM * TC_BK * 2, tc_smem_u32(&s_full[kb]), (kb0 + kb) * TC_BK);
     bool ok = true;
     for (int kb = pre; kb < n_kb && ok; ++kb) {
       const int s = kb % p.stages;
-      ok = tc_mbar_wait(tc_smem_u32(&s_empty[s]), ((kb / p.stages) - 1) & 1);  // the stage's MMAs are done
+      ok = tc_mbar_wait(tc_smem_u32(&s_empty[s]), ((kb / p.stages) - 1) & 1, p.wait_cycles);  // the stage's MMAs are done
       if (!ok) break;
+      if (kb == drop_kb) continue;
       const unsigned bar = tc_smem_u32(&s_full[s]);
       const unsigned a = base + s * stage_bytes, b = a + TC_BM * TC_BK * 2;
       tc_mbar_expect_tx(bar, (unsigned)stage_bytes);
@@ -203,7 +208,8 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
     bool ok = true;
     for (int kb = 0; kb < n_kb && ok; ++kb) {
       const int s = kb % p.stages;
-      ok = tc_mbar_wait(tc_smem_u32(&s_full[s]), (kb / p.stages) & 1);
+      // (one verdict for the warp: lanes that gave up alone would leave the others waiting for them)
+      ok = __all_sync(0xffffffffu, tc_mbar_wait(tc_smem_u32(&s_full[s]), (kb / p.stages) & 1, p.wait_cycles));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (tc_elect_one()) {
@@ -221,7 +227,7 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
   }
   // everyone: the accumulator is complete when the last commit arrives
   bool have = n_kb > 0;
-  if (have) have = tc_mbar_wait(tc_smem_u32(&s_done), 0);
+  if (have) have = __all_sync(0xffffffffu, tc_mbar_wait(tc_smem_u32(&s_done), 0, p.wait_cycles));
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const int n = n0 + warp * 32 + lane;  // this thread's weight row = its TMEM lane
   float* out = p.out + (size_t)blockIdx.z * p.group_stride + (size_t)blockIdx.y * p.M * p.N;
@@ -251,7 +257,7 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
       for (int j = 0; j < 16; ++j)
         if (c0 + j < live && n < p.N) out[(size_t)(c0 + j) * p.N + n] = __uint_as_float(v[j]);
     }
-  } else if (tid == 0) {
+  } else if (lane == 0) {
     *p.err = p.err_code;
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

@@ -580,6 +580,32 @@ def test_a_bounded_device_wait_that_runs_out_is_reported_and_survived():
     ctx.close()
 
 
+def test_a_bounded_wait_of_the_wide_decode_gemms_that_runs_out_is_reported_and_survived():
+    """The same for the layers' GEMMs of a context of several sequences (tcgen05 path): the issuing warp of CTA 0 gives up as one - lanes
+    that left alone would keep the others waiting - and so does every warp that waits for the accumulator."""
+    import time
+    import paper_2609_17184_b200 as ls
+    refs = [U.oracle_run("tiny_bf16", 16 + s, 12, 1, 2, seq=s) for s in range(4)]
+    ctx = U.make_ctx("tiny_bf16", 1, 2, max_seqs=4, max_ctx=64)
+    assert ctx.decode_paths()[0] == 1
+    prefill = lambda: [ctx.prefill(refs[s]["prompt"], seq=s) for s in range(4)]
+    prefill()
+    ctx.decode(12)                   # (every partial sum has been written once: what a dropped tile leaves behind is finite)
+    prefill()
+    ctx.debug_drop_tile(1, wait_us=100)
+    t0 = time.time()
+    with pytest.raises(ls.LoopSpecError) as e:
+        ctx.step()
+    assert e.value.status == "ETIMEOUT", e.value
+    assert time.time() - t0 < 5.0
+    ctx.debug_drop_tile(-1)
+    assert prefill() == [r["first"] for r in refs]
+    out = ctx.decode(12)
+    for s in range(4):
+        assert out[s].tolist() == refs[s]["tokens"], U.min_margin(refs[s]["dec"])
+    ctx.close()
+
+
 def test_depths_from_the_closed_form_are_used_when_none_are_given():
     """d1 = d2 = 0 at init: the library picks the admissible pair minimising Theorem 2's bound, like the oracle."""
     from oracle import depths as dp
