@@ -760,8 +760,10 @@ cudaError_t launch_tc_epi(const TcEpiParams& q, int groups, int rows, cudaStream
   if (groups > 1) return launch_k(tc_epilogue_kernel<EPI, true>, dim3(q.g.n_rb, TCE_GROUPS, groups), dim3(GEMM_THREADS), 0, st, q, pdl);
   return launch_k(tc_epilogue_kernel<EPI, false>, dim3(q.g.n_rb, std::min(TCE_GROUPS, rows)), dim3(GEMM_THREADS), 0, st, q, pdl);
 }
-cudaError_t launch_tc_gemm(loopspec_ctx* c, int which, int layer, const RowTable* tab, int cfg_i) {
+// (n_rows: rows of a table that may carry more than the passes of this configuration do)
+cudaError_t launch_tc_gemm(loopspec_ctx* c, int which, int layer, const RowTable* tab, int cfg_i, int n_rows = 0) {
   const loopspec_ctx::TcCfg& tc = c->tc[cfg_i];
+  const int epi_rows = std::max(n_rows, cfg_i == 1 ? c->d.max_rows_dec : c->d.max_rows_pf);
   const int pi = which == G_ADAPT ? 4 : which;
   const TcPfPlan& t = c->tc_plan[pi];
   TcEpiParams q;
@@ -790,9 +792,9 @@ cudaError_t launch_tc_gemm(loopspec_ctx* c, int which, int layer, const RowTable
   cudaError_t e = cudaLaunchKernelEx(&cfg, linear_tc_kernel, wm, tc.xmaps[xi], p);
   if (e != cudaSuccess) return e;
   switch (which) {
-    case G_QKV: return launch_tc_epi<EPI_QKV>(q, groups, table_rows(c, tab), c->stream, c->use_pdl);
-    case G_GU: return launch_tc_epi<EPI_SWIGLU>(q, groups, table_rows(c, tab), c->stream, c->use_pdl);
-    default: return launch_tc_epi<EPI_RESID>(q, groups, table_rows(c, tab), c->stream, c->use_pdl);
+    case G_QKV: return launch_tc_epi<EPI_QKV>(q, groups, epi_rows, c->stream, c->use_pdl);
+    case G_GU: return launch_tc_epi<EPI_SWIGLU>(q, groups, epi_rows, c->stream, c->use_pdl);
+    default: return launch_tc_epi<EPI_RESID>(q, groups, epi_rows, c->stream, c->use_pdl);
   }
 }
 
@@ -1995,7 +1997,7 @@ int loopspec_time_kernel(loopspec_ctx* c, int32_t which, int32_t rows, int32_t i
       GemmParams p = gemm_params(c, which, i % L, tab);
       if (kTune && tune_timeline(c)) p.dbg = reinterpret_cast<long long*>(tune_timeline(c));  // phase stamps of CTA 0 (tuning builds)
       cudaError_t e = (c->dg && which == G_LM)         ? launch_dg_lm(c, tab)
-                      : (c->tc[1].on && which != G_LM) ? launch_tc_gemm(c, which, i % L, tab, 1)
+                      : (c->tc[1].on && which != G_LM) ? launch_tc_gemm(c, which, i % L, tab, 1, rows)
                                                        : launch_gemm(c->m.weight_dtype, c->ng_dec, kEpiOf[which], p, c->stream, c->use_pdl);
       if (e) return e;
     }

@@ -68,3 +68,28 @@ def test_kernels_can_be_timed_alone_and_the_context_stays_usable(max_ctx):
     ctx.decode(12)
     U.assert_same_run(ctx, ref, 12)
     ctx.close()
+
+
+@pytest.mark.parametrize("which", [0, 2, 3])
+def test_a_timed_wide_gemm_finishes_every_row_whatever_bounds_a_prefill_pass(which):
+    """The timed launches run in the decode launch configuration: with prefill passes of at most 16 rows, 24 rows of a GEMM on the
+    tcgen05 path write as much of the workspace as with passes of 64 (the two contexts are otherwise in the same state)."""
+    import torch
+    name, S = "tiny_bf16", 8
+    refs = [U.oracle_run(name, 16, 12, 1, 2, seq=s) for s in range(S)]
+    changed = []
+    for rows_pf in (16, 64):
+        ctx = U.make_ctx(name, 1, 2, max_seqs=S, max_ctx=64, max_prefill_rows=rows_pf)
+        for s in range(S):
+            assert ctx.prefill(refs[s]["prompt"], seq=s) == refs[s]["first"]
+        ctx.decode(12)
+        assert ctx.decode_paths()[0] == 1 and ctx.stats()["rows_max"] >= 24
+        ctx.time_kernel(1, 24, 1)                       # the scratch table and states of the timed launches are in place
+        torch.cuda.synchronize()
+        before = ctx.workspace.clone()
+        ctx.time_kernel(which, 24, 1)
+        torch.cuda.synchronize()
+        n = before.numel() // 4 * 4
+        changed.append(int((before[:n].view(torch.int32) != ctx.workspace[:n].view(torch.int32)).sum()))
+        ctx.close()
+    assert changed[0] == changed[1], changed
