@@ -228,7 +228,7 @@ int loopspec_time_kernel(loopspec_ctx*, int32_t which, int32_t rows, int32_t ite
  * All pointers device; x, y fp32; scratch: device, 16-byte aligned, loopspec_linear_scratch_bytes(M, N, K)
  * bytes (it receives the bf16 planes of x where x is split by a launch of its own - more than 16 rows, fp32 weights; W is read
  * in place; contents on entry are
- * irrelevant).  M <= 64, N % 16 == 0, K % 8 == 0. */
+ * irrelevant).  M <= 64, N % 16 == 0, K % 8 == 0, W 16-byte aligned, else LOOPSPEC_EINVAL. */
 size_t loopspec_linear_scratch_bytes(int32_t M, int32_t N, int32_t K);
 int loopspec_op_linear(const void* W, int32_t weight_dtype, const float* x, float* y, int32_t M, int32_t N,
                        int32_t K, void* scratch, size_t scratch_bytes, void* cuda_stream);

@@ -2033,14 +2033,14 @@ int loopspec_op_linear(const void* W, int32_t weight_dtype, const float* x, floa
                        void* scratch, size_t scratch_bytes, void* cuda_stream) {
   if (!W || !x || !y || (weight_dtype != 0 && weight_dtype != 1)) return LOOPSPEC_EINVAL;
   size_t need = loopspec_linear_scratch_bytes(M, N, K);
-  if (!need) return LOOPSPEC_EINVAL;
+  if (!need || (reinterpret_cast<uintptr_t>(W) & 15)) return LOOPSPEC_EINVAL;  // (every kernel reads W with 16-byte accesses)
   if (!scratch || scratch_bytes < need || (reinterpret_cast<uintptr_t>(scratch) & 15)) return LOOPSPEC_ECAPACITY;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const int ng = ng_for_rows(M);
   GemmPlan g = weight_dtype ? plan_gemm((N + 127) / 128, K, 148 * kCtasPerSm, true) : plan_gemm_f32((N + 127) / 128, K, 148 * kCtasPerSm);
   // Up to 16 rows: one launch that splits x itself.  Beyond, every warp would read and split more of x than it reads of W, and
   // the cluster GEMM on planes made once is the faster one.
-  if (weight_dtype == 1 && ng <= 2 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(W)) & 15) == 0) {
+  if (weight_dtype == 1 && ng <= 2 && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
     LinearDirectParams q = {static_cast<const __nv_bfloat16*>(W), x, y, M, N, K, g.cs};
     const int tpc = 8 / g.cs, tiles = N / 16;
     // two tiles per warp share the split of x; below two CTAs per SM the parallelism is worth more [2048 x 2048, 4 rows: 5.0 us

@@ -76,3 +76,12 @@ def test_workspace_query_rejects_bad_shapes():
     s2 = Sched(3, 0, 0, 0, 1, 1, 0.0, 0, 1, 128, 0)      # d1 does not divide R
     assert ls.lib.loopspec_workspace_bytes(C.byref(m), C.byref(s2)) == 0
     assert ls.linear_scratch_bytes(4, 256, 256) > 0 and ls.linear_scratch_bytes(4, 250, 256) == 0
+
+
+def test_linear_refuses_weights_that_are_not_16_byte_aligned():
+    """The kernels read W with 16-byte accesses: the call ends with EINVAL before anything is launched (the addresses here are never
+    read)."""
+    for dtype in (0, 1):
+        for M in (1, 16, 17, 64):
+            for off in (2, 4, 8):
+                assert ls.lib.loopspec_op_linear((1 << 20) + off, dtype, 1 << 21, 1 << 22, M, 256, 256, 1 << 23, 1 << 20, None) == -1
