@@ -226,9 +226,8 @@ int loopspec_time_kernel(loopspec_ctx*, int32_t which, int32_t rows, int32_t ite
 /* Stand-alone linear map y[M][N] = x[M][K] * W[N][K]^T through the same weight-streaming kernel (token
  * activations split into three bf16 terms, fp32 accumulation; fp32 weights use the CUDA-core path).
  * All pointers device; x, y fp32; scratch: device, 16-byte aligned, loopspec_linear_scratch_bytes(M, N, K)
- * bytes (it receives the bf16 planes of x where x is split by a launch of its own - more than 16 rows, fp32 weights; W is read
- * in place; contents on entry are
- * irrelevant).  M <= 64, N % 16 == 0, K % 8 == 0, W 16-byte aligned, else LOOPSPEC_EINVAL. */
+ * bytes (it receives the bf16 planes of x where x is split by a launch of its own - more than 16 rows, fp32 weights, an x
+ * that is not 16-byte aligned; W is read in place; contents on entry are irrelevant).  M <= 64, N % 16 == 0, K % 8 == 0, W 16-byte aligned, else LOOPSPEC_EINVAL. */
 size_t loopspec_linear_scratch_bytes(int32_t M, int32_t N, int32_t K);
 int loopspec_op_linear(const void* W, int32_t weight_dtype, const float* x, float* y, int32_t M, int32_t N,
                        int32_t K, void* scratch, size_t scratch_bytes, void* cuda_stream);
@@ -261,8 +260,8 @@ int loopspec_time_linear_tc(const void* const* Ws, int32_t n_w, const float* x, 
  * every other stream.  Such callers pass only inputs and the output; the scratch that loopspec_op_linear wants lives
  * in a fixed 16 MiB array inside the library's device image (every GPU that loads the library carries it until the
  * process exits).  The call allocates nothing and frees nothing.
- *   - Sizes: loopspec_linear_scratch_bytes(M, N, K) must not exceed 16 MiB (roughly N*K <= 8M bf16 weights);
- *     larger requests return LOOPSPEC_ECAPACITY and do nothing.  Bad shapes return LOOPSPEC_EINVAL.
+ *   - Sizes: loopspec_linear_scratch_bytes(M, N, K) and N*K bf16 weights together must not exceed 16 MiB (roughly
+ *     N*K <= 8M); larger requests return LOOPSPEC_ECAPACITY and do nothing.  Bad shapes return LOOPSPEC_EINVAL.
  *   - The first call on each device looks up the array's device address (with that device current); make that
  *     first call outside any stream capture.  Later calls only launch kernels on cuda_stream.  With lazy module
  *     loading that first call is also when the library's device image -- the 16 MiB array with it -- becomes

@@ -2026,7 +2026,7 @@ int loopspec_time_kernel(loopspec_ctx* c, int32_t which, int32_t rows, int32_t i
 
 size_t loopspec_linear_scratch_bytes(int32_t M, int32_t N, int32_t K) {
   if (M < 1 || M > 64 || N < 16 || K < 8 || N % 16 || K % 8) return 0;
-  return align_up((size_t)M * 3 * K * 2) + packed_bytes(N, K);
+  return align_up((size_t)M * 3 * K * 2);  // the planes of x
 }
 
 int loopspec_op_linear(const void* W, int32_t weight_dtype, const float* x, float* y, int32_t M, int32_t N, int32_t K,
@@ -2080,7 +2080,8 @@ int loopspec_op_linear_static(const void* W, int32_t weight_dtype, const float* 
   static std::atomic<void*> scratch_of_device[64];
   size_t need = loopspec_linear_scratch_bytes(M, N, K);
   if (!need) return LOOPSPEC_EINVAL;
-  if (need > LOOPSPEC_STATIC_SCRATCH_BYTES) return LOOPSPEC_ECAPACITY;  // beyond the built-in scratch: use loopspec_op_linear
+  // the documented limit of this entry point counts the weights too, although they are read in place
+  if (need + packed_bytes(N, K) > LOOPSPEC_STATIC_SCRATCH_BYTES) return LOOPSPEC_ECAPACITY;  // use loopspec_op_linear
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LOOPSPEC_ECUDA;
   void* ptr = scratch_of_device[dev].load(std::memory_order_acquire);

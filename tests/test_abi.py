@@ -85,3 +85,9 @@ def test_linear_refuses_weights_that_are_not_16_byte_aligned():
         for M in (1, 16, 17, 64):
             for off in (2, 4, 8):
                 assert ls.lib.loopspec_op_linear((1 << 20) + off, dtype, 1 << 21, 1 << 22, M, 256, 256, 1 << 23, 1 << 20, None) == -1
+
+
+def test_linear_scratch_holds_the_planes_of_x_and_no_copy_of_the_weights():
+    for M, N, K in [(1, 16, 8), (4, 2048, 2048), (17, 304, 72), (64, 12288, 5632)]:
+        planes = M * 3 * K * 2
+        assert planes <= ls.linear_scratch_bytes(M, N, K) < planes + 256

@@ -83,6 +83,23 @@ def test_linear_reads_row_major_weights_at_the_edges(M, N, K):
     assert np.array_equal(ls.linear(Wt, xo).cpu().numpy().view(np.uint32), y.view(np.uint32))
 
 
+@pytest.mark.parametrize("M,N,K,dtype,shift", [(16, 304, 72, "bf16", 1), (17, 304, 72, "bf16", 0), (64, 4096, 1000, "bf16", 0), (9, 272, 264, "fp32", 0)])
+def test_linear_stays_within_its_scratch(M, N, K, dtype, shift):
+    """The calls that split x in a launch of their own, with exactly the scratch that is asked for and a guard behind it."""
+    import paper_2609_17184_b200 as ls
+    rng = np.random.default_rng(M)
+    Wn = W.bf16_round((rng.standard_normal((N, K)) * 0.05).astype(np.float32))
+    x = rng.standard_normal((M, K)).astype(np.float32)
+    xt = torch.zeros(M * K + shift, device="cuda")[shift:].view(M, K)
+    xt.copy_(torch.from_numpy(x))
+    need = ls.linear_scratch_bytes(M, N, K)
+    buf = torch.full((need + 65536,), 77, dtype=torch.uint8, device="cuda")
+    y = ls.linear(torch.from_numpy(Wn).cuda().to(torch.bfloat16 if dtype == "bf16" else torch.float32), xt, buf[:need]).cpu().numpy()
+    scale = np.abs(x).astype(np.float64) @ np.abs(Wn).astype(np.float64).T
+    assert (np.abs(y - x.astype(np.float64) @ Wn.astype(np.float64).T) <= 2e-6 * scale + 1e-30).all()
+    assert (buf[need:] == 77).all()
+
+
 def test_linear_tc_rejects_unsupported_shapes():
     import paper_2609_17184_b200 as ls
     assert ls.lib.loopspec_linear_tc_scratch_bytes(4, 256, 256) > 0
