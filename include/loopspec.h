@@ -194,9 +194,9 @@ int loopspec_debug_logits(loopspec_ctx*, int32_t seq, int32_t which, float* out_
  * core releases, a cluster partner's partial sums) is bounded by the clock; when one runs out the kernel raises a flag,
  * carries on with whatever data it has so that every barrier still receives its arrivals, and ends; the call that
  * launched it returns LOOPSPEC_ETIMEOUT, the results of that pass are void, the context stays usable (prefill the
- * sequence again).  This call makes such a wait run out: from now on CTA 0 of the readout GEMM - and, where a decode pass
- * runs its layers on the tcgen05 path (loopspec_decode_paths), CTA 0 of those GEMMs - never requests ring unit `unit`
- * (unit >= 0), so the wait for it gives up after about wait_us microseconds.  unit = -1 restores normal operation
+ * sequence again).  This call makes such a wait run out: from now on CTA 0 of the readout GEMM never requests ring unit
+ * `unit` (unit >= 0) - and, where a decode pass runs its layers on the tcgen05 path (loopspec_decode_paths), those GEMMs
+ * request no unit from this one on - so the wait for it gives up after about wait_us microseconds.  unit = -1 restores normal operation
  * (and the normal bound of ~0.2 s).  Nothing faults or hangs: the skipped copy is simply never issued. */
 int loopspec_debug_drop_tile(loopspec_ctx*, int32_t unit, int32_t wait_us);
 

@@ -41,7 +41,7 @@ struct LinearTcParams {
   long long group_stride;  //  group of columns)
   const int* n_live;   // x3d: number of live columns of the pass (may be null); a group beyond it has nothing to do
   long long wait_cycles;
-  int drop_kb;         // test hook: the producer of CTA 0 skips this k-block (-1: none), so that the waits for it run out
+  int stop_kb;         // test hook: no CTA requests its k-blocks from this one on (INT_MAX: all are), so that the waits for them run out
 };
 
 __device__ __forceinline__ unsigned tc_smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -154,11 +154,9 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
   // The weights are constants, so the first ring-full of weight tiles is requested ahead of the predecessor's
   // completion - and while warp 0 still allocates the tensor memory; the activation tiles (which the predecessor may
   // still be writing) follow after the dependency wait, on the same barriers.
-  const int pre = min(p.stages, n_kb);
-  const int drop_kb = (blockIdx.x | blockIdx.y | blockIdx.z) == 0 ? p.drop_kb : -1;
+  const int n_load = min(n_kb, p.stop_kb), pre = min(p.stages, n_load);
   if (tid == 32) {
     for (int kb = 0; kb < pre; ++kb) {
-      if (kb == drop_kb) continue;
       const unsigned bar = tc_smem_u32(&s_full[kb]);
       tc_mbar_expect_tx(bar, (unsigned)stage_bytes);
       tc_tma_load_2d(base + kb * stage_bytes, &map_w, bar, (kb0 + kb) * TC_BK, n0);
@@ -186,13 +184,12 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
   if (tid == 32 && n_kb > 0) {
     // ---- producer: one thread keeps the ring of stages filled by TMA ----
     for (int kb = 0; kb < pre; ++kb)
-      if (kb != drop_kb) load_x(base + kb * stage_bytes + TC_BM * TC_BK * 2, tc_smem_u32(&s_full[kb]), (kb0 + kb) * TC_BK);
+      load_x(base + kb * stage_bytes + TC_BM * TC_BK * 2, tc_smem_u32(&s_full[kb]), (kb0 + kb) * TC_BK);
     bool ok = true;
-    for (int kb = pre; kb < n_kb && ok; ++kb) {
+    for (int kb = pre; kb < n_load && ok; ++kb) {
       const int s = kb % p.stages;
       ok = tc_mbar_wait(tc_smem_u32(&s_empty[s]), ((kb / p.stages) - 1) & 1, p.wait_cycles);  // the stage's MMAs are done
       if (!ok) break;
-      if (kb == drop_kb) continue;
       const unsigned bar = tc_smem_u32(&s_full[s]);
       const unsigned a = base + s * stage_bytes, b = a + TC_BM * TC_BK * 2;
       tc_mbar_expect_tx(bar, (unsigned)stage_bytes);
@@ -205,36 +202,40 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
   if (warp == 0 && n_kb > 0) {
     // ---- MMA issuer: one elected lane, the accumulator lives in tensor memory ----
     const unsigned idesc = tc_idesc(TC_BM, 3 * p.MP);
+    // No lane leaves the loop when a wait runs out - the others would wait for it, without a bound, at the next instruction of the
+    // whole warp: the rest of the k-blocks is walked without MMAs, and every barrier still receives its arrival.
     bool ok = true;
-    for (int kb = 0; kb < n_kb && ok; ++kb) {
+    for (int kb = 0; kb < n_kb; ++kb) {
       const int s = kb % p.stages;
-      // (one verdict for the warp: lanes that gave up alone would leave the others waiting for them)
-      ok = __all_sync(0xffffffffu, tc_mbar_wait(tc_smem_u32(&s_full[s]), (kb / p.stages) & 1, p.wait_cycles));
-      if (!ok) break;
+      if (!tc_mbar_wait(tc_smem_u32(&s_full[s]), (kb / p.stages) & 1, ok ? p.wait_cycles : 0)) ok = false;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (tc_elect_one()) {
         const unsigned a = base + s * stage_bytes, b = a + TC_BM * TC_BK * 2;
         const unsigned long long adesc = tc_smem_desc(a);
         const unsigned long long bdesc = tc_smem_desc(b);  // rows pl * MP + column: the hi, mid, lo planes stacked
+        if (ok) {
 #pragma unroll
-        for (int ks = 0; ks < TC_BK / 16; ++ks) tc_mma(tmem, adesc + 2 * ks, bdesc + 2 * ks, idesc, (kb | ks) != 0);
+          for (int ks = 0; ks < TC_BK / 16; ++ks) tc_mma(tmem, adesc + 2 * ks, bdesc + 2 * ks, idesc, (kb | ks) != 0);
+        }
         tc_commit(tc_smem_u32(&s_empty[s]));  // arrives when the MMAs issued so far have read their operands
-        if (kb == n_kb - 1) tc_commit(tc_smem_u32(&s_done));
+        if (kb == n_kb - 1) {
+          if (!ok) s_fail = 1, *p.err = p.err_code, __threadfence_block();
+          tc_commit(tc_smem_u32(&s_done));
+        }
       }
       __syncwarp();
     }
-    if (!ok && lane == 0) s_fail = 1, *p.err = p.err_code;
   }
-  // everyone: the accumulator is complete when the last commit arrives
-  bool have = n_kb > 0;
-  if (have) have = __all_sync(0xffffffffu, tc_mbar_wait(tc_smem_u32(&s_done), 0, p.wait_cycles));
+  // everyone: the accumulator is complete when the last commit arrives.  It is read either way (the loads are the whole warp's); a
+  // lane that does not have it complete stores nothing.
+  const bool have = n_kb > 0 && tc_mbar_wait(tc_smem_u32(&s_done), 0, p.wait_cycles) && *const_cast<volatile int*>(&s_fail) == 0;
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const int n = n0 + warp * 32 + lane;  // this thread's weight row = its TMEM lane
   float* out = p.out + (size_t)blockIdx.z * p.group_stride + (size_t)blockIdx.y * p.M * p.N;
   if (n_kb <= 0) {
     for (int m = 0; m < live; ++m)
       if (n < p.N) out[(size_t)m * p.N + n] = 0.f;
-  } else if (have) {
+  } else {
     for (int c0 = 0; c0 < live; c0 += 16) {
       unsigned w[3][16];
 #pragma unroll
@@ -255,10 +256,9 @@ __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_cons
         v[j] = __float_as_uint(__uint_as_float(w[0][j]) + (__uint_as_float(w[1][j]) + __uint_as_float(w[2][j])));
 #pragma unroll
       for (int j = 0; j < 16; ++j)
-        if (c0 + j < live && n < p.N) out[(size_t)(c0 + j) * p.N + n] = __uint_as_float(v[j]);
+        if (c0 + j < live && n < p.N && have) out[(size_t)(c0 + j) * p.N + n] = __uint_as_float(v[j]);
     }
-  } else if (lane == 0) {
-    *p.err = p.err_code;
+    if (!have) s_fail = 1, *p.err = p.err_code;
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();

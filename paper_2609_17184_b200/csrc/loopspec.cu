@@ -3,6 +3,7 @@
 #include "../../include/loopspec.h"
 
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstddef>
@@ -778,7 +779,7 @@ cudaError_t launch_tc_gemm(loopspec_ctx* c, int which, int layer, const RowTable
   p.M = tc.cols, p.MP = tc.cols, p.N = q.g.N, p.K = q.g.K, p.kb_per_split = t.kb_per_split, p.stages = tc.stages;
   p.err = const_cast<int*>(c->host_flags_dev + HF_ERROR), p.err_code = 5, p.x3d = 1;
   p.row0 = 0, p.group_cols = GROUP_ROWS, p.group_stride = (long long)t.n_split * tc.cols * q.g.N;
-  p.wait_cycles = cfg_i == 1 ? c->dg_wait_cycles : TC_WAIT_CYCLES, p.drop_kb = cfg_i == 1 ? c->dg_drop_unit : -1;
+  p.wait_cycles = cfg_i == 1 ? c->dg_wait_cycles : TC_WAIT_CYCLES, p.stop_kb = cfg_i == 1 && c->dg_drop_unit >= 0 ? c->dg_drop_unit : INT_MAX;
   p.n_live = cfg_i == 1 ? reinterpret_cast<const int*>(reinterpret_cast<const char*>(tab) + offsetof(RowTable, n_rows)) : nullptr;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
@@ -2149,7 +2150,7 @@ int loopspec_op_linear_tc(const void* W, const float* x, float* y, int32_t M, in
   p.out = t.n_split > 1 ? reinterpret_cast<float*>(sc + t.part_off) : y;
   p.M = M, p.MP = t.MP, p.N = N, p.K = K, p.kb_per_split = t.kb_per_split, p.stages = t.stages;
   p.err = reinterpret_cast<int*>(sc), p.err_code = 1;
-  p.wait_cycles = TC_WAIT_CYCLES, p.drop_kb = -1;
+  p.wait_cycles = TC_WAIT_CYCLES, p.stop_kb = INT_MAX;
   if (!tc_allow_smem()) return LOOPSPEC_ECUDA;
   // programmatic dependent launches: the weights are requested while x is split, the sums start as the last tile ends
   cudaLaunchConfig_t cfg;
@@ -2187,7 +2188,7 @@ int loopspec_time_linear_tc(const void* const* Ws, int32_t n_w, const float* x, 
   p.out = reinterpret_cast<float*>(sc + t.part_off);
   p.M = M, p.MP = t.MP, p.N = N, p.K = K, p.kb_per_split = t.kb_per_split, p.stages = t.stages;
   p.err = reinterpret_cast<int*>(sc), p.err_code = 1;
-  p.wait_cycles = TC_WAIT_CYCLES, p.drop_kb = -1;
+  p.wait_cycles = TC_WAIT_CYCLES, p.stop_kb = INT_MAX;
   if (!tc_allow_smem()) return LOOPSPEC_ECUDA;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);

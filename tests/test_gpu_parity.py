@@ -597,9 +597,10 @@ def test_a_bounded_device_wait_that_runs_out_is_reported_and_survived():
     ctx.close()
 
 
-def test_a_bounded_wait_of_the_wide_decode_gemms_that_runs_out_is_reported_and_survived():
-    """The same for the layers' GEMMs of a context of several sequences (tcgen05 path): the issuing warp of CTA 0 gives up as one - lanes
-    that left alone would keep the others waiting - and so does every warp that waits for the accumulator."""
+@pytest.mark.parametrize("unit", [0, 1, 3])
+def test_a_bounded_wait_of_the_wide_decode_gemms_that_runs_out_is_reported_and_survived(unit):
+    """The same for the layers' GEMMs of a context of several sequences (tcgen05 path): no lane of an issuing warp leaves its loop
+    alone - the others would wait for it - and an accumulator that is not complete is not stored."""
     import time
     import paper_2609_17184_b200 as ls
     refs = [U.oracle_run("tiny_bf16", 16 + s, 12, 1, 2, seq=s) for s in range(4)]
@@ -609,7 +610,7 @@ def test_a_bounded_wait_of_the_wide_decode_gemms_that_runs_out_is_reported_and_s
     prefill()
     ctx.decode(12)                   # (every partial sum has been written once: what a dropped tile leaves behind is finite)
     prefill()
-    ctx.debug_drop_tile(1, wait_us=100)
+    ctx.debug_drop_tile(unit, wait_us=100)
     t0 = time.time()
     with pytest.raises(ls.LoopSpecError) as e:
         ctx.step()
