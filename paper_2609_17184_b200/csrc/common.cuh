@@ -24,23 +24,28 @@ constexpr int ATT_CHUNK = 64; // key positions per attention chunk (cut at fixed
 constexpr int ATT_MAX_RUNS = 40;   // contexts of one sequence: one chunk per attention work item up to 2560 positions ...
 constexpr int ATT_LONG_RUNS = 16;  // ... and this many items at most for longer ones
 constexpr int ATT_BATCH_RUNS = 12;  // contexts of several sequences: items per (row, kv head) at most
-enum { ATT_ONE = 1, ATT_FEW = 2, ATT_MANY = 3 };  // sequences a context holds: one, 2 to 4, 5 and more
-// A work item covers a run of consecutive chunks.  A context of one sequence (few rows per pass, every chunk in parallel
-// matters): one chunk for contexts up to ATT_MAX_RUNS chunks, beyond that as many as leave ATT_LONG_RUNS items [7 rows x 8400
-// positions, 8 / 16 / 32 items each: 65 / 51 / 86 us; 1 row: 53 / 33 / 24].  Contexts of several sequences: an item has a fixed cost
-// of some 4 us of its warp and all items of a full pass should be resident at once, but with few of the sequences live an item's
-// length is the kernel's time.  So runs of one chunk (two from six chunks on) for up to four sequences, of two chunks (four from nine
-// chunks on) for more, and ATT_BATCH_RUNS items at most [ms per pass of the 1.4B shape, shortest runs of 1 / 2 / 3 / 4 chunks: 4
-// sequences, contexts of 260 positions, one live 1.23 / 1.30 / 1.35 / 1.41, all 1.40 / 1.40 / 1.44 / 1.50; of 450, all 1.51 / 1.47 / 1.49 /
-// 1.54; 8 sequences of 260, one live 1.39 / 1.46 / 1.51 / 1.57, all 1.84 / 1.75 / 1.78 / 1.81; of 580, all 2.22 / 2.13 / 2.13 / 2.03].
+constexpr int ATT_BATCH_SEQS = 5;   // ... and the number of sequences from which on the rule is the same
+// A work item covers a run of consecutive chunks.  mode = sequences the context holds, up to ATT_BATCH_SEQS.  One (few rows per pass,
+// every chunk in parallel matters): one chunk for contexts up to ATT_MAX_RUNS chunks, beyond that as many as leave ATT_LONG_RUNS items
+// [7 rows x 8400 positions, 8 / 16 / 32 items each: 65 / 51 / 86 us; 1 row: 53 / 33 / 24].  Several: an item has a fixed cost of some
+// 4 us of its warp, a row of one item needs no fold, and all items of a full pass should be resident at once; but with few of the
+// sequences live the longest item is the kernel's time.  Two sequences: runs of two chunks.  Three or four: a single run up to three
+// chunks, runs of one chunk for four and five, of two up to eight, beyond that of as many as there are sequences.  More: of four chunks,
+// five and six chunks in two equal halves.  ATT_BATCH_RUNS items at most.
+// [ms per pass of the 1.4B shape, runs of 1 / 2 / 3 / 4 chunks: 4 sequences, contexts of 260 positions, one live 1.23 / 1.30 / 1.35 / 1.41, all
+// 1.40 / 1.40 / 1.44 / 1.50; of 450, one live 1.25 / 1.31 / 1.36 / 1.42, all 1.51 / 1.47 / 1.49 / 1.54.  Sampled (more rows): 4 sequences of 100,
+// all, 1 / 4 chunks 1.47 / 1.39; 8 sequences of 260 to 340, all, 2 / 4 chunks 2.11 / 1.97.  The rule is evaluated in front of every item
+// of attn_warp_kernel, so it divides by constants only (a balanced cut with two divisions: 1 to 5 % of a pass).]
 // Either way a function of the row's own context and of what the context can hold, so a row's arithmetic does not depend on
 // what shares the pass.
-__host__ __device__ inline int att_mode_of(int n_seqs) { return n_seqs == 1 ? ATT_ONE : n_seqs <= 4 ? ATT_FEW : ATT_MANY; }
 __host__ __device__ inline int att_run_len(int n_canon, int mode) {
   const int nc = (n_canon + ATT_CHUNK - 1) / ATT_CHUNK;
-  if (mode == ATT_ONE) return nc <= ATT_MAX_RUNS ? 1 : (nc + ATT_LONG_RUNS - 1) / ATT_LONG_RUNS;
-  const int rl = (nc + ATT_BATCH_RUNS - 1) / ATT_BATCH_RUNS, shortest = mode == ATT_FEW ? (nc <= 5 ? 1 : 2) : (nc <= 8 ? 2 : 4);
-  return rl > shortest ? rl : shortest;
+  if (mode == 1) return nc <= ATT_MAX_RUNS ? 1 : (nc + ATT_LONG_RUNS - 1) / ATT_LONG_RUNS;
+  int run = mode;
+  if (mode == ATT_BATCH_SEQS) run = nc == 5 || nc == 6 ? 3 : 4;
+  else if (mode > 2 && nc <= 8) run = nc <= 3 ? 3 : nc <= 5 ? 1 : 2;
+  const int rl = (nc + ATT_BATCH_RUNS - 1) / ATT_BATCH_RUNS;
+  return rl > run ? rl : run;
 }
 __host__ __device__ inline int att_items(int n_canon, int mode) {
   const int nc = (n_canon + ATT_CHUNK - 1) / ATT_CHUNK, rl = att_run_len(n_canon, mode);

@@ -353,7 +353,7 @@ bool resolve_sched(const loopspec_model* m, const loopspec_sched* s, Derived* d,
   d->n_sq = m->hidden / 128;  // row blocks of the residual GEMMs = partial sums of squares per row
   d->sq_stride = std::max(d->n_sq, 64);  // room for one partial per cluster of the persistent pass kernel
   d->max_chunks = (s->max_ctx + ATT_CHUNK - 1) / ATT_CHUNK;
-  d->att_mode = att_mode_of(d->S);
+  d->att_mode = std::min(d->S, ATT_BATCH_SEQS);
   d->att_long = d->max_chunks > (d->S > 1 ? 8 : ATT_MAX_RUNS) ? 1 : 0;
   // One CTA per item only for the few items of a lone sequence of short capacity, where the work of an item is its latency
   // [us, attn_kernel / attn_warp_kernel, 536 positions: 1 row 6.5 / 9.5, 4 rows 8.2 / 10.5, 7 rows 14.2 / 11.5; 3000 positions, against

@@ -457,6 +457,21 @@ def test_attention_of_several_sequences_at_the_edges_of_tiles_and_runs(name, S, 
     ctx.close()
 
 
+@pytest.mark.parametrize("S,lens", [(3, [185, 1, 505]), (4, [311, 180, 500, 319]), (5, [250, 100, 375, 20, 383])])
+def test_attention_runs_change_length_while_a_batch_decodes(S, lens):
+    """Contexts that grow over the edges of the rule that cuts attention runs while they decode: of a batch of three or four, past 3, 5 and
+    8 chunks; of a larger one, past 4 and 6 (five sequences are passes of up to 35 rows)."""
+    n = 20
+    refs = [U.oracle_run("tiny_bf16", lens[s], n, 1, 2, seed=4, seq=s) for s in range(S)]
+    ctx = U.make_ctx("tiny_bf16", 1, 2, seed=4, max_seqs=S, max_ctx=560)
+    for s in range(S):
+        assert ctx.prefill(refs[s]["prompt"], seq=s) == refs[s]["first"]
+    out = ctx.decode(n)
+    for s in range(S):
+        assert out[s].tolist() == refs[s]["tokens"], (s, U.min_margin(refs[s]["dec"]))
+    ctx.close()
+
+
 def test_prefill_chunking_does_not_change_results():
     name = "tiny_bf16"
     ref = U.oracle_run(name, 37, 16, 1, 2)
