@@ -110,6 +110,14 @@ __device__ __forceinline__ void tc_commit(unsigned bar) {
 }
 
 __host__ __device__ constexpr int tc_stage_bytes(int MP) { return TC_BM * TC_BK * 2 + 3 * MP * TC_BK * 2; }
+// Dynamic shared memory of a launch: the ring, and for more than 128 accumulator columns (256 of tensor memory) enough that no third CTA
+// fits an SM: it would hold its slot in the tensor-memory allocation until another CTA ends, ahead of the kernels that could run there
+// [decode passes of 35 to 48 rows, 2 stages of 34 KB each: 5 sequences of 260 positions 1.89 -> 1.56 ms per pass, one live 1.61 -> 1.41].
+// (Fewer columns: four and more CTAs share the 512 columns, and the rings keep them below that.)
+inline size_t tc_smem_bytes(int MP, int stages) {
+  const size_t ring = (size_t)stages * tc_stage_bytes(MP) + 1024;
+  return 3 * MP > 128 && ring < 78 * 1024 ? 78 * 1024 : ring;
+}
 
 __global__ void __launch_bounds__(TC_THREADS) linear_tc_kernel(const __grid_constant__ CUtensorMap map_w,
                                                                const __grid_constant__ CUtensorMap map_x,

@@ -1492,7 +1492,7 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
       tc.cols = tc_pf_cols(rows[k]);
       const int sb = tc_stage_bytes(tc.cols);
       tc.stages = std::max(2, std::min(TC_MAX_STAGES, (100 * 1024) / sb));
-      tc.smem = (size_t)tc.stages * sb + 1024;
+      tc.smem = tc_smem_bytes(tc.cols, tc.stages);
       for (int i = 0; i < (dd.raven ? 4 : 3) && ok; ++i)
         ok = make_map_planes3d(&tc.xmaps[i], c->ws + x_off[i], x_k[i], x_k[i], dd.max_rows, tc.cols);
     }
@@ -2114,7 +2114,7 @@ bool plan_tc(int M, int N, int K, TcPlan* t) {
   const int kb_budget = t->MP <= 16 ? 56 : 100;
   const int slots = t->MP <= 16 ? 592 : 296;
   t->stages = std::max(2, std::min(TC_MAX_STAGES, (kb_budget * 1024) / sb));
-  t->smem = (size_t)t->stages * sb + 1024;
+  t->smem = tc_smem_bytes(t->MP, t->stages);
   t->n_rb = (N + TC_BM - 1) / TC_BM;
   const int total_kb = K / TC_BK;
   int want = std::max(1, std::min(slots / t->n_rb, total_kb / 4));
