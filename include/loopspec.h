@@ -37,7 +37,7 @@ typedef enum {
   LOOPSPEC_ESTATE = -2,       /* call out of order (step before prefill, verify with nothing at depth R, ...) */
   LOOPSPEC_ECAPACITY = -3,    /* max_ctx, max_seqs, node table or workspace too small */
   LOOPSPEC_ECUDA = -4,        /* a CUDA call failed; see loopspec_last_error */
-  LOOPSPEC_ETIMEOUT = -5,     /* a bounded device-side wait (mbarrier, grid barrier) ran out; the pass's results are void */
+  LOOPSPEC_ETIMEOUT = -5,     /* a bounded device-side wait (mbarrier) ran out; the pass's results are void */
   LOOPSPEC_EUNSUPPORTED = -6  /* shape outside what the kernels support */
 } loopspec_status;
 

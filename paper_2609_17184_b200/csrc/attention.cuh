@@ -295,8 +295,8 @@ __global__ void __launch_bounds__(ATT_THREADS, 4) attn_kernel(const __grid_const
 // 64 -> 26, 40 rows x 86 22 -> 12, 28 rows x 1036 69 -> 42, 14 rows x 8400 179 -> 154 us (6.25 TB/s).
 template <int D, int G>
 struct AtwCfg {
-    static constexpr int WARPS = 4, STAGES = 2, CTAS = 3, MT = 1;  // CTAS: per SM; MT: mma row tiles (of 16 keys) in a tile
-  static constexpr int ROWB = D * 2, KEYS = 16 * MT, TILE = KEYS * ROWB;  // bytes of a key row; keys of a tile and their bytes (values the same)
+  static constexpr int WARPS = 4, STAGES = 2, CTAS = 3;  // CTAS: per SM
+  static constexpr int ROWB = D * 2, KEYS = 16, TILE = KEYS * ROWB;  // bytes of a key row; keys of a tile and their bytes (values the same)
   static constexpr int QBYTES = G * D * 4;                 // an item's queries
   static constexpr int SMEM_BYTES = WARPS * STAGES * (2 * TILE + QBYTES);
 };
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(AtwCfg<D, G>::WARPS * 32) attn_warp_kernel(con
   using C = AtwCfg<D, G>;
   static_assert(G == 1 || G == 4, "query heads per kv head");
   constexpr int PSTRIDE = D + 2, KS = D / 16, PCS = D / 8, NP = G == 1 ? 1 : 3;  // NP: column sets of a k-step (G = 1: planes are columns)
-  constexpr int LI = C::KEYS * PCS / 32, MT = C::MT, RPI = 32 / PCS, SW = 8 / RPI;  // copies of keys per lane and tile, rows a copy of the warp covers, their swizzles
+  constexpr int LI = C::KEYS * PCS / 32, RPI = 32 / PCS, SW = 8 / RPI;  // copies of keys per lane and tile, rows a copy of the warp covers, their swizzles
   extern __shared__ __align__(128) unsigned char atw_smem[];
   const RowTable* tab = p.tab;  // written before this pass started: safe to read ahead of the predecessor
   const int n_rows = tab->n_rows, HQ = p.n_q_heads * D;
@@ -513,58 +513,42 @@ __global__ void __launch_bounds__(AtwCfg<D, G>::WARPS * 32) attn_warp_kernel(con
       }
       const unsigned kt = ring + c_st, vt = kt + C::TILE;
       // ---- scores of keys g and g + 8 of every row tile ----
-      unsigned fr[MT][KS][4];  // every fragment is requested before the first is used: a load waited for is 30 cycles of a lone warp's chain
+      unsigned fr[KS][4];  // every fragment is requested before the first is used: a load waited for is 30 cycles of a lone warp's chain
 #pragma unroll
-      for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-        for (int ks = 0; ks < KS; ++ks) att_ldsm4(fr[mt][ks], (kt + mt * 16 * C::ROWB + k_lane) ^ (ks << 5));
-      float sc[MT][4];
+      for (int ks = 0; ks < KS; ++ks) att_ldsm4(fr[ks], (kt + k_lane) ^ (ks << 5));
+      float sc[4];
       {
-        float c[MT][4][4];  // four chains over the k-steps
+        float c[4][4];  // four chains over the k-steps
 #pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
+        for (int x = 0; x < 4; ++x)
 #pragma unroll
-          for (int x = 0; x < 4; ++x)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) c[mt][x][i] = 0.f;
+          for (int i = 0; i < 4; ++i) c[x][i] = 0.f;
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
-          for (int s = 0; s < NP; ++s)
+          for (int s = 0; s < NP; ++s) att_mma(c[ks & 3], fr[ks], qf[ks][s][0], qf[ks][s][1]);
 #pragma unroll
-            for (int mt = 0; mt < MT; ++mt) att_mma(c[mt][ks & 3], fr[mt][ks], qf[ks][s][0], qf[ks][s][1]);
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) sc[mt][i] = (c[mt][0][i] + c[mt][1][i]) + (c[mt][2][i] + c[mt][3][i]);
+        for (int i = 0; i < 4; ++i) sc[i] = (c[0][i] + c[1][i]) + (c[2][i] + c[3][i]);
       }
 #pragma unroll
-      for (int mt = 0; mt < MT; ++mt)
+      for (int ks = 0; ks < KS; ++ks)  // (the value columns arrive under the softmax)
+        att_ldsm4_t(fr[ks], (vt + v_lane) ^ (ks << 5));
+      float e0[NH], e1[NH], wa[NH];  // (key g, key g + 8) of this lane's heads: score, then softmax weight
+      if constexpr (G == 1) {  // columns 0, 1 (planes hi, mid) sit in lane t = 0, column 2 (lo) in t = 1; every lane takes the sum
+        const int b = lane & ~3;
+        e0[0] = __shfl_sync(0xffffffffu, sc[0], b) + (__shfl_sync(0xffffffffu, sc[1], b) + __shfl_sync(0xffffffffu, sc[0], b + 1));
+        e1[0] = __shfl_sync(0xffffffffu, sc[2], b) + (__shfl_sync(0xffffffffu, sc[3], b) + __shfl_sync(0xffffffffu, sc[2], b + 1));
+      } else {
 #pragma unroll
-        for (int ks = 0; ks < KS; ++ks)  // (the value columns arrive under the softmax)
-          att_ldsm4_t(fr[mt][ks], (vt + mt * 16 * C::ROWB + v_lane) ^ (ks << 5));
-      float e0[MT][NH], e1[MT][NH], wa[NH];  // (key g, key g + 8) of this lane's heads: score, then softmax weight
-#pragma unroll
-      for (int mt = 0; mt < MT; ++mt) {
-        if constexpr (G == 1) {  // columns 0, 1 (planes hi, mid) sit in lane t = 0, column 2 (lo) in t = 1; every lane takes the sum
-          const int b = lane & ~3;
-          e0[mt][0] = __shfl_sync(0xffffffffu, sc[mt][0], b) + (__shfl_sync(0xffffffffu, sc[mt][1], b) + __shfl_sync(0xffffffffu, sc[mt][0], b + 1));
-          e1[mt][0] = __shfl_sync(0xffffffffu, sc[mt][2], b) + (__shfl_sync(0xffffffffu, sc[mt][3], b) + __shfl_sync(0xffffffffu, sc[mt][2], b + 1));
-        } else {
-#pragma unroll
-          for (int h = 0; h < 2; ++h) e0[mt][h] = sc[mt][h], e1[mt][h] = sc[mt][2 + h];
-        }
+        for (int h = 0; h < 2; ++h) e0[h] = sc[h], e1[h] = sc[2 + h];
       }
       bool moved = false;
 #pragma unroll
       for (int h = 0; h < NH; ++h) {  // running softmax
         float mx = -INFINITY;
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-          e0[mt][h] = j0 + 16 * mt + g < n_keys ? e0[mt][h] * p.scale : -INFINITY;
-          e1[mt][h] = j0 + 16 * mt + g + 8 < n_keys ? e1[mt][h] * p.scale : -INFINITY;
-          mx = fmaxf(mx, fmaxf(e0[mt][h], e1[mt][h]));
-        }
+        e0[h] = j0 + g < n_keys ? e0[h] * p.scale : -INFINITY;
+        e1[h] = j0 + g + 8 < n_keys ? e1[h] * p.scale : -INFINITY;
+        mx = fmaxf(mx, fmaxf(e0[h], e1[h]));
 #pragma unroll
         for (int off = 4; off < 32; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
         mx = fmaxf(mx, m[h]);  // (finite: every tile holds a key)
@@ -572,11 +556,8 @@ __global__ void __launch_bounds__(AtwCfg<D, G>::WARPS * 32) attn_warp_kernel(con
         moved |= mx != m[h];
         m[h] = mx;
         float sum = 0.f;
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-          e0[mt][h] = expf(e0[mt][h] - mx), e1[mt][h] = expf(e1[mt][h] - mx);
-          sum += e0[mt][h] + e1[mt][h];
-        }
+        e0[h] = expf(e0[h] - mx), e1[h] = expf(e1[h] - mx);
+        sum += e0[h] + e1[h];
         l[h] = fmaf(l[h], wa[h], sum);  // (this lane's keys; summed over the lanes when the run is done)
       }
       if (G == 1 ? moved : __any_sync(0xffffffffu, moved)) {
@@ -586,40 +567,35 @@ __global__ void __launch_bounds__(AtwCfg<D, G>::WARPS * 32) attn_warp_kernel(con
           for (int i = 0; i < 4; ++i) o[ks][i] *= wa[G == 1 ? 0 : (i & 1)];
       }
       // ---- softmax weights as columns: keys 2 t, 2 t + 1 (first register), + 8, + 9 (second) of column g ----
-      unsigned pf[MT][NP][2];
+      unsigned pf[NP][2];
+      float a[2], b[2];
+      const int l0 = 8 * t, l1 = 8 * t + 4;  // lanes (key 2 t, .) and (key 2 t + 1, .)
+      if constexpr (G == 1) {
+        a[0] = __shfl_sync(0xffffffffu, e0[0], l0), a[1] = __shfl_sync(0xffffffffu, e0[0], l1);
+        b[0] = __shfl_sync(0xffffffffu, e1[0], l0), b[1] = __shfl_sync(0xffffffffu, e1[0], l1);
+      } else {  // column g = head g: state in lane t = g / 2, register g & 1
+        const int src = (g >> 1) & 1;
 #pragma unroll
-      for (int mt = 0; mt < MT; ++mt) {
-        float a[2], b[2];
-        const int l0 = 8 * t, l1 = 8 * t + 4;  // lanes (key 2 t, .) and (key 2 t + 1, .)
-        if constexpr (G == 1) {
-          a[0] = __shfl_sync(0xffffffffu, e0[mt][0], l0), a[1] = __shfl_sync(0xffffffffu, e0[mt][0], l1);
-          b[0] = __shfl_sync(0xffffffffu, e1[mt][0], l0), b[1] = __shfl_sync(0xffffffffu, e1[mt][0], l1);
-        } else {  // column g = head g: state in lane t = g / 2, register g & 1
-          const int src = (g >> 1) & 1;
-#pragma unroll
-          for (int x = 0; x < 2; ++x) {
-            const int from = (x ? l1 : l0) + src;
-            const float u0 = __shfl_sync(0xffffffffu, e0[mt][0], from), u1 = __shfl_sync(0xffffffffu, e0[mt][NH - 1], from);
-            const float w0 = __shfl_sync(0xffffffffu, e1[mt][0], from), w1 = __shfl_sync(0xffffffffu, e1[mt][NH - 1], from);
-            a[x] = g >= 4 ? 0.f : (g & 1) ? u1 : u0, b[x] = g >= 4 ? 0.f : (g & 1) ? w1 : w0;
-          }
-        }
-        unsigned pa[3], pb[3];
-        split3_pair(a[0], a[1], pa), split3_pair(b[0], b[1], pb);
-        if constexpr (G == 1) {
-          pf[mt][0][0] = g == 0 ? pa[0] : g == 1 ? pa[1] : g == 2 ? pa[2] : 0u;
-          pf[mt][0][1] = g == 0 ? pb[0] : g == 1 ? pb[1] : g == 2 ? pb[2] : 0u;
-        } else {
-#pragma unroll
-          for (int s = 0; s < 3; ++s) pf[mt][s][0] = pa[s], pf[mt][s][1] = pb[s];
+        for (int x = 0; x < 2; ++x) {
+          const int from = (x ? l1 : l0) + src;
+          const float u0 = __shfl_sync(0xffffffffu, e0[0], from), u1 = __shfl_sync(0xffffffffu, e0[NH - 1], from);
+          const float w0 = __shfl_sync(0xffffffffu, e1[0], from), w1 = __shfl_sync(0xffffffffu, e1[NH - 1], from);
+          a[x] = g >= 4 ? 0.f : (g & 1) ? u1 : u0, b[x] = g >= 4 ? 0.f : (g & 1) ? w1 : w0;
         }
       }
+      unsigned pa[3], pb[3];
+      split3_pair(a[0], a[1], pa), split3_pair(b[0], b[1], pb);
+      if constexpr (G == 1) {
+        pf[0][0] = g == 0 ? pa[0] : g == 1 ? pa[1] : g == 2 ? pa[2] : 0u;
+        pf[0][1] = g == 0 ? pb[0] : g == 1 ? pb[1] : g == 2 ? pb[2] : 0u;
+      } else {
 #pragma unroll
-      for (int mt = 0; mt < MT; ++mt)
+        for (int s = 0; s < 3; ++s) pf[s][0] = pa[s], pf[s][1] = pb[s];
+      }
 #pragma unroll
-        for (int s = 0; s < NP; ++s)
+      for (int s = 0; s < NP; ++s)
 #pragma unroll
-          for (int ks = 0; ks < KS; ++ks) att_mma(o[ks], fr[mt][ks], pf[mt][s][0], pf[mt][s][1]);  // dims 16 ks .. + 15
+        for (int ks = 0; ks < KS; ++ks) att_mma(o[ks], fr[ks], pf[s][0], pf[s][1]);  // dims 16 ks .. + 15
       __syncwarp();  // the tile may be overwritten
       c_st += 2 * C::TILE;
       if (c_st == C::STAGES * 2 * C::TILE) c_st = 0;

@@ -11,7 +11,7 @@ constexpr int CTRL_THREADS = 256;
 constexpr int MAX_NODES = 512;   // max_seqs * nodes-per-sequence
 enum { PH_ADVANCE = 1, PH_VERIFY = 2, PH_BUILD = 4 };
 enum { HF_ERROR = 0, HF_N_ROWS = 2, HF_NEED_VERIFY = 3, HF_FIRST_TOKEN = 4, HF_COUNT = 8 };
-enum { ERR_NODES = 1, ERR_CTX = 2, ERR_SPEC = 3, ERR_WAIT = 4 /* bounded wait, decode GEMM */, ERR_WAIT_PF = 5 /* prefill GEMM, grid barrier */ };
+enum { ERR_NODES = 1, ERR_CTX = 2, ERR_SPEC = 3, ERR_WAIT = 4 /* bounded wait, readout GEMM */, ERR_WAIT_PF = 5 /* GEMM of a prompt or of a wide decode pass */ };
 
 struct ControlParams {
   int att_mode;     // how attention work items are cut (att_run_len)
@@ -190,7 +190,7 @@ __device__ void build_rows(const ControlParams& p, const NodeSmem& nd, const int
     rows0 += (int)(s_tot[0] & 0xffff), ros0 += (int)((s_tot[0] >> 16) & 0xffff), items0 += (int)(s_tot[0] >> 32);
     if (pre) pres0 += (int)(s_tot[1] & 0xffff), pitems0 += (int)((s_tot[1] >> 16) & 0xffffff), citems0 += (int)(s_tot[1] >> 40);
   }
-  rows0 = min(rows0, MAX_ROWS), ros0 = min(ros0, MAX_ROWS);  // (more: the error flag is up)
+  rows0 = min(rows0, MAX_ROWS), ros0 = min(ros0, MAX_ROWS), pres0 = min(pres0, MAX_ROWS);  // (more: the error flag is up)
   if (threadIdx.x == 0) {
     t->n_rows = rows0, t->n_readout = ros0, t->attn_items = items0, t->chunk_start[rows0] = items0, t->att_mode = p.att_mode;
     if (pre) {

@@ -351,7 +351,7 @@ bool resolve_sched(const loopspec_model* m, const loopspec_sched* s, Derived* d,
   d->p_logit_base = d->S * d->NB * 2;
   d->n_logit_vecs = d->p_logit_base + d->S;
   d->n_sq = m->hidden / 128;  // row blocks of the residual GEMMs = partial sums of squares per row
-  d->sq_stride = std::max(d->n_sq, 64);  // room for one partial per cluster of the persistent pass kernel
+  d->sq_stride = std::max(d->n_sq, 64);  // row stride of the partial sums
   d->max_chunks = (s->max_ctx + ATT_CHUNK - 1) / ATT_CHUNK;
   d->att_mode = std::min(d->S, ATT_BATCH_SEQS);
   d->att_long = d->max_chunks > (d->S > 1 ? 8 : ATT_MAX_RUNS) ? 1 : 0;
@@ -777,7 +777,7 @@ cudaError_t launch_tc_gemm(loopspec_ctx* c, int which, int layer, const RowTable
   memset(&p, 0, sizeof p);
   p.out = c->at<float>(c->L.tcpart);
   p.M = tc.cols, p.MP = tc.cols, p.N = q.g.N, p.K = q.g.K, p.kb_per_split = t.kb_per_split, p.stages = tc.stages;
-  p.err = const_cast<int*>(c->host_flags_dev + HF_ERROR), p.err_code = 5, p.x3d = 1;
+  p.err = const_cast<int*>(c->host_flags_dev + HF_ERROR), p.err_code = ERR_WAIT_PF, p.x3d = 1;
   p.row0 = 0, p.group_cols = GROUP_ROWS, p.group_stride = (long long)t.n_split * tc.cols * q.g.N;
   p.wait_cycles = cfg_i == 1 ? c->dg_wait_cycles : TC_WAIT_CYCLES, p.stop_kb = cfg_i == 1 && c->dg_drop_unit >= 0 ? c->dg_drop_unit : INT_MAX;
   p.n_live = cfg_i == 1 ? reinterpret_cast<const int*>(reinterpret_cast<const char*>(tab) + offsetof(RowTable, n_rows)) : nullptr;
@@ -1065,7 +1065,7 @@ int check_device_error(loopspec_ctx* c) {
   if (!e) return LOOPSPEC_OK;
   c->host_flags[HF_ERROR] = 0;
   if (e == ERR_WAIT || e == ERR_WAIT_PF)  // a bounded wait inside a kernel ran out: the pass's results are void, the context is not
-    return fail(c, LOOPSPEC_ETIMEOUT, "a bounded device-side wait ran out (%s)", e == ERR_WAIT ? "decode-pass GEMM" : "prefill GEMM or grid barrier");
+    return fail(c, LOOPSPEC_ETIMEOUT, "a bounded device-side wait ran out (%s)", e == ERR_WAIT ? "readout GEMM" : "GEMM of a prompt or of a wide decode pass");
   return fail(c, LOOPSPEC_ECAPACITY, "device scheduler reported %s",
               e == ERR_NODES ? "node/row table overflow" : e == ERR_CTX ? "max_ctx exceeded" : "speculative chain too deep");
 }
