@@ -399,7 +399,7 @@ def run_ours(args):
         "kernels_alone": per_kernel,
         "prefill": {"ms_per_sequence": round(prefill_ms_seq, 2), "prompt_len": n_prompt,
                     "tok_per_s": round(n_prompt / (prefill_ms_seq / 1e3), 1), "what": "wall clock of loopspec_prefill (host ids in, first token out)"},
-        "prefill_tcgen05_kernels_alone": tc_alone,
+        "narrow_prefill_tcgen05_kernels_alone": tc_alone,  # linear_tc_kernel: prompts of up to 64 tokens, wide decode passes
         "step_roofline": {"achieved": round(step_gbs, 1), "peak": peak, "unit": "GB/s", "frac": round(step_gbs / peak, 4),
                           "ms_per_pass": round(statistics.mean(dec_ms) / max(stats["steps"], 1), 4),
                           "bytes_per_pass": int(total_b / max(stats["steps"], 1))},

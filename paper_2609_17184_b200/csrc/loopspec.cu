@@ -357,7 +357,8 @@ bool resolve_sched(const loopspec_model* m, const loopspec_sched* s, Derived* d,
   d->att_long = d->max_chunks > (d->S > 1 ? 8 : ATT_MAX_RUNS) ? 1 : 0;
   // One CTA per item only for the few items of a lone sequence of short capacity, where the work of an item is its latency
   // [us, attn_kernel / attn_warp_kernel, 536 positions: 1 row 6.5 / 9.5, 4 rows 8.2 / 10.5, 7 rows 14.2 / 11.5; 3000 positions, against
-  // the best of runs of chunks by one CTA: 4 rows 24 / 22, 7 rows 47 / 36; batches: attn_warp_kernel's comment]
+  // the best of runs of chunks by one CTA: 4 rows 24 / 22, 7 rows 47 / 36; ms per pass at 3.6 rows: capacity 320 0.952 / 1.025, 640
+  // 1.064 / 1.047, 1040 1.140 / 1.081, 2560 1.730 / 1.482 - the line could lie near 600 positions; batches: attn_warp_kernel's comment]
   d->att_warps = d->S > 1 || d->att_long ? 1 : 0;
   d->trace_cap = m->R * s->max_ctx + 64;  // a token can take R passes (restart)
   d->Hq = m->n_q_heads * m->head_dim;

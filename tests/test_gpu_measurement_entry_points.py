@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 def test_decode_paths_follow_the_row_and_context_capacity():
     """Passes of up to 8 rows: mma.sync cluster kernels; 9 to 64 rows of a bf16 model: the tcgen05 kernel + epilogue;
-    a context capacity beyond 2560 positions (512 when the context holds several sequences): the streaming attention kernel;
+    attention_path tells a long context capacity: beyond 2560 positions, 512 when the context holds several sequences;
     fp32 weights never leave the CUDA cores."""
     cases = [(dict(name="tiny_bf16", max_seqs=1, max_ctx=256), (0, 0)),
              (dict(name="tiny_bf16", max_seqs=4, max_ctx=256), (1, 0)),
