@@ -57,6 +57,7 @@ struct GemmParams {
   int N, K;
   int n_rb, kb_per_rb;    // row blocks; 32-wide k-blocks per row
   int cluster_size, n_clusters;
+  unsigned inv_cs;        // ceil(2^32 / cluster_size)
   // activations: bf16 planes [col][3][x_ld]
   const __nv_bfloat16* xplanes;
   int x_ld;
@@ -147,6 +148,8 @@ __device__ __forceinline__ int gemm_row0(const GemmParams& p, int rb, int warp) 
   return r < p.N ? r : -1;
 }
 
+// x / cs by the host's ceil(2^32 / cs), for x < 2^28 (an integer division is some forty instructions of cold code)
+__device__ __forceinline__ int gemm_div(int x, int cs, unsigned inv) { return cs == 1 ? x : (int)__umulhi((unsigned)x, inv); }
 // k-blocks [lo, hi) of cluster rank `rank`
 __device__ __forceinline__ void gemm_krange(int kpr, int cs, int rank, int& lo, int& hi) {
   int q = kpr / cs, r = kpr % cs;
@@ -165,6 +168,7 @@ __device__ __forceinline__ void gemm_reduce_epilogue(const GemmParams& p, const 
   const int tid = threadIdx.x, half = tid >> 7, j = tid & 127, lane = tid & 31, hw = (tid >> 5) & 3;
   const int cs = p.cluster_size, vcs = p.recv_ranks ? p.recv_ranks : cs * KH;
   __shared__ float s_ss[2][4];
+#pragma unroll 1
   for (int base = rank; base < n_cols; base += 2 * cs) {
     const int c = base + cs * half;
     const bool live = c < n_cols && j < RBW;
@@ -183,7 +187,7 @@ __device__ __forceinline__ void gemm_reduce_epilogue(const GemmParams& p, const 
     }
     float v = 0.f;
     if (live) {
-      const float* src = recv + (size_t)(c / cs) * RBW + j;
+      const float* src = recv + (size_t)gemm_div(c, cs, p.inv_cs) * RBW + j;
       v = src[0];
       for (int rk = 1; rk < vcs; ++rk) v += src[(size_t)rk * own_max * RBW];  // rank order, the same for every launch
       v *= s_rstd[c];
@@ -245,7 +249,7 @@ __device__ __forceinline__ void gemm_reduce_epilogue(const GemmParams& p, const 
           const int n0 = rb * RB_ROWS;
           const int region = n0 < Hq ? 0 : (n0 < Hq + Hk ? 1 : 2);
           const int rbase = region == 0 ? 0 : (region == 1 ? Hq : Hq + Hk);
-          const int hh = j / hd2, i = j - hh * hd2;
+          const int ld = d == 128 ? 7 : 6, hh = j >> (ld - 1), i = j & (hd2 - 1);  // (head sizes 64 and 128: shifts)
           const float x1 = col[hh * d + i], x2 = col[hh * d + i + hd2];
           float y1 = x1, y2 = x2;
           if (region < 2) {
@@ -253,7 +257,7 @@ __device__ __forceinline__ void gemm_reduce_epilogue(const GemmParams& p, const 
             y1 = x1 * csn.x - x2 * csn.y;
             y2 = x2 * csn.x + x1 * csn.y;
           }
-          const int head = (n0 - rbase) / d + hh;
+          const int head = ((n0 - rbase) >> ld) + hh;
           if (region == 0) {
             float* q = p.qbuf + (size_t)c * Hq + head * d + i;
             q[0] = y1;
@@ -275,11 +279,14 @@ __device__ __forceinline__ void gemm_reduce_epilogue(const GemmParams& p, const 
 // butterfly sum: the same order in every launch)
 __device__ __forceinline__ void gemm_rstd(const GemmParams& p, int n_cols, float* s_rstd, const int* ct, int ntok) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll 1
   for (int c = warp; c < n_cols; c += GEMM_THREADS / 32) {
     const int xr = p.cols_from_readout ? ct[CT_XROW * ntok + c] : c;  // the lm_head's columns are the reading-out rows
     float ss = 0.f;
-    if (p.sumsq)
+    if (p.sumsq) {
+#pragma unroll 1
       for (int j = lane; j < p.n_sq; j += 32) ss += p.sumsq[xr * p.sq_stride + j];
+    }
     ss = warp_sum(ss);
     if (lane == 0) s_rstd[c] = p.sumsq ? 1.0f / sqrtf(ss / (float)p.H + p.eps) : 1.0f;
   }
@@ -297,10 +304,44 @@ __device__ __forceinline__ void gemm_load_cols(const GemmParams& p, int n_cols, 
   }
 }
 
+// ---- hand-over of the partial columns inside a cluster without a cluster barrier (fp32 kernel): every rank that finishes columns has an
+// mbarrier in its shared memory, and the contributors' stores count their bytes on it (st.async).  [A job of the 256-wide model, passes
+// of 2 to 4 rows: 4 % shorter.  The bf16 kernels keep plain stores and the barrier: there the jobs with several rows per pass got 4 %
+// longer, those with one row no shorter.]
+__device__ __forceinline__ unsigned gemm_mapa(unsigned addr, unsigned rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void gemm_st_async(unsigned addr, float v, unsigned bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(__float_as_uint(v)), "r"(bar) : "memory");
+}
+// columns rank `rank` finishes
+__device__ __forceinline__ int gemm_owned(int n_cols, int cs, int rank, unsigned inv) { return rank < n_cols ? gemm_div(n_cols - rank + cs - 1, cs, inv) : 0; }
+__device__ __forceinline__ void gemm_arm(unsigned bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+constexpr int GEMM_ERR_WAIT = 6;  // what the host's flag shows of a wait that ran out (ERR_WAIT_DEC)
+constexpr long long GEMM_WAIT_CYCLES = 400000000LL;  // ~0.2 s
+__device__ __forceinline__ bool gemm_recv_wait(unsigned bar, unsigned parity) {
+  const long long t0 = clock64();
+  for (;;) {
+    unsigned ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if (clock64() - t0 > GEMM_WAIT_CYCLES) return false;
+  }
+}
+
 // push this thread's accumulator fragments (rows warp*16+g / +8, columns n*8+2t / +1) into the receive buffers of
-// the ranks that own the columns (distributed shared memory stores; made visible by the cluster barrier)
-template <int NG, int KH = 1>
-__device__ __forceinline__ void gemm_push_tile(const float (&acc)[NG][4], float* recv, int own_max, int n_cols, int cs, int rank,
+// the ranks that own the columns: stores to distributed shared memory, made visible by the cluster barrier or (ASYNC) counted on the
+// owner's mbarrier (`bar`: the address of this CTA's, the same in every CTA of the cluster)
+template <int NG, bool ASYNC, int KH = 1>
+__device__ __forceinline__ void gemm_push_tile(const float (&acc)[NG][4], float* recv, int own_max, int n_cols, int cs, unsigned inv, int rank, unsigned bar,
                                                cg::cluster_group& cluster) {
   constexpr int RBW = RB_ROWS / KH;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -312,15 +353,23 @@ __device__ __forceinline__ void gemm_push_tile(const float (&acc)[NG][4], float*
     for (int e = 0; e < 2; ++e) {
       const int c = n * 8 + 2 * t + e;
       if (c < n_cols) {
-        const int owner = c % cs, slot = c / cs;
-        float* dst = (cs > 1 ? cluster.map_shared_rank(recv, owner) : recv) + ((size_t)rank * own_max + slot) * RBW + rl;
-        dst[0] = acc[n][e];
-        dst[8] = acc[n][2 + e];
+        const int slot = gemm_div(c, cs, inv), owner = c - slot * cs;
+        if (!ASYNC || cs == 1) {  // (launches of single CTAs have no cluster)
+          float* const dst = (cs > 1 ? cluster.map_shared_rank(recv, owner) : recv) + ((size_t)rank * own_max + slot) * RBW + rl;
+          dst[0] = acc[n][e], dst[8] = acc[n][2 + e];
+          continue;
+        }
+        const unsigned dst = gemm_mapa((unsigned)__cvta_generic_to_shared(recv) + ((rank * own_max + slot) * RBW + rl) * 4, owner), b = gemm_mapa(bar, owner);
+        gemm_st_async(dst, acc[n][e], b);
+        gemm_st_async(dst + 32, acc[n][2 + e], b);
       }
     }
 }
 
 // ======================================= bf16 weights: tensor cores ========================================
+// A launch of the chain runs its code about once and cold in the instruction caches, so what does not stream is kept small: loops rolled,
+// divisions as multiplications [36 -> 20 KB of code for NG = 1; four passes of one row of the 1.4B shape 3.59 -> 3.47 ms, a pass of a
+// 3-layer model 4 to 5 % shorter; unrolling the main loop by 1, 2 or 4 by hand changes nothing].
 template <int NG, int EPI>
 __global__ void __launch_bounds__(GEMM_THREADS) __maxnreg__(NG == 1 ? LS_MAXREG : 255) gemm_bf16_kernel(const __grid_constant__ GemmParams p) {
   // KH = 2 (64-row blocks, the warps of a CTA in two groups that alternate k-blocks) is supported by the helpers below
@@ -340,8 +389,8 @@ __global__ void __launch_bounds__(GEMM_THREADS) __maxnreg__(NG == 1 ? LS_MAXREG 
 
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int cs = p.cluster_size, rank = (int)cluster.block_rank(), cid = blockIdx.x / cs;
-  const int own_max = (NTOK + cs - 1) / cs;
+  const int cs = p.cluster_size, rank = (int)cluster.block_rank(), cid = gemm_div(blockIdx.x, cs, p.inv_cs);
+  const int own_max = gemm_div(NTOK + cs - 1, cs, p.inv_cs);
   int dbg_n = 0;
   auto stamp = [&]() {
     if (kTune && p.dbg && blockIdx.x == 0 && tid == 0) p.dbg[dbg_n++] = clock64();
@@ -360,7 +409,10 @@ __global__ void __launch_bounds__(GEMM_THREADS) __maxnreg__(NG == 1 ? LS_MAXREG 
   }
   const int kpr = p.kb_per_rb;
   int kb_lo, kb_hi;
-  gemm_krange(kpr, cs, rank, kb_lo, kb_hi);
+  {  // gemm_krange
+    const int q = gemm_div(kpr, cs, p.inv_cs), r = kpr - q * cs;
+    kb_lo = rank * q + min(rank, r), kb_hi = kb_lo + q + (rank < r ? 1 : 0);
+  }
   const int upt = kb_hi - kb_lo;                                 // k-blocks per task (whole CTA)
   const int khalf = warp / (8 / KH);                             // which k-blocks of the range this warp takes
   const int my_upt = (upt - khalf + KH - 1) / KH;                // units per task of this warp
@@ -409,7 +461,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) __maxnreg__(NG == 1 ? LS_MAXREG 
     cp_async_commit();
   };
   auto drain = [&]() { cp_async_wait<0>(); };
-#pragma unroll
+#pragma unroll 1
   for (int s = 0; s < RING - 1; ++s) issue_unit();
 
   // the row table was written before this pass started, so the live row count can be read ahead of the predecessor
@@ -465,6 +517,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) __maxnreg__(NG == 1 ? LS_MAXREG 
   };
   float pre_h = 0.f, pre_g = 1.f;
   float2 pre_rope = make_float2(1.f, 0.f);
+#pragma unroll 1
   for (int task = 0; task < n_tasks; ++task) {
     const int rb = cid + task * p.n_clusters;
     const bool warp_valid = gemm_row0<EPI, KH>(p, rb, warp) >= 0;
@@ -474,6 +527,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) __maxnreg__(NG == 1 ? LS_MAXREG 
       for (int n = 0; n < NG; ++n)
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[h][n][i] = 0.f;
+#pragma unroll 1
     for (int ck = 0; ck < upt; ck += XCH) {
       const int nkb = min(XCH, upt - ck);
       const bool first = task == 0 && ck == 0;
@@ -493,7 +547,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) __maxnreg__(NG == 1 ? LS_MAXREG 
         }
         if (EPI == EPI_QKV && c < n_cols && jr < 64) {
           const int hd2 = p.head_dim >> 1;
-          pre_rope = p.rope[(size_t)s_ct[CT_POS * NTOK + c] * hd2 + jr % hd2];
+          pre_rope = p.rope[(size_t)s_ct[CT_POS * NTOK + c] * hd2 + (jr & (hd2 - 1))];
         }
       }
       const int kbl0 = (khalf + KH - (ck % KH)) % KH;  // this warp's first k-block of the chunk
@@ -543,7 +597,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) __maxnreg__(NG == 1 ? LS_MAXREG 
 #pragma unroll
       for (int i = 0; i < 4; ++i) tot[n][i] = acc[0][n][i] + (acc[1][n][i] + acc[2][n][i]);
     stamp();
-    gemm_push_tile<NG, KH>(tot, recv, own_max, n_cols, cs, rank, cluster);
+    gemm_push_tile<NG, false, KH>(tot, recv, own_max, n_cols, cs, p.inv_cs, rank, 0, cluster);
     cluster.sync();
     stamp();
     gemm_reduce_epilogue<EPI, KH>(p, s_ct, NTOK, rb, n_cols, recv, own_max, colbuf, s_rstd, rank, pre_h, pre_g, pre_rope,
@@ -588,6 +642,14 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_f32_kernel(const __grid_con
   const int upt = kb_hi - kb_lo;
   const int n_tasks = (p.n_rb - cid + p.n_clusters - 1) / p.n_clusters;
   const int own_max = (NTOK + cs - 1) / cs;
+  __shared__ __align__(8) unsigned long long s_recv_bar;
+  const unsigned recv_bar = (unsigned)__cvta_generic_to_shared(&s_recv_bar);
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(recv_bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncwarp();
+  if (cs > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   pdl_launch_dependents();
   float4 w[DEPTH][4];  // rows g and g + 8, eight k each
   int row0 = gemm_row0<EPI>(p, cid, warp);
@@ -609,7 +671,11 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_f32_kernel(const __grid_con
   if (n_cols > NTOK) n_cols = NTOK;
   gemm_load_cols(p, n_cols, NTOK, s_ct);
   pdl_wait();
+  if (cs > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (n_cols <= 0) return;
+  const int owned = gemm_owned(n_cols, cs, rank, p.inv_cs);
+  const unsigned recv_bytes = (unsigned)(cs * owned * RB_ROWS * 4);
+  if (tid == 0 && owned > 0) gemm_arm(recv_bar, recv_bytes);
   __syncthreads();
 
   for (int task = 0; task < n_tasks; ++task) {
@@ -694,8 +760,16 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_f32_kernel(const __grid_con
           if (c == 2 * t) tot[n][2 * h] = v;
           if (c == 2 * t + 1) tot[n][2 * h + 1] = v;
         }
-    gemm_push_tile<NG>(tot, recv, own_max, n_cols, cs, rank, cluster);
-    cluster.sync();
+    gemm_push_tile<NG, true>(tot, recv, own_max, n_cols, cs, p.inv_cs, rank, recv_bar, cluster);
+    if (cs == 1) {
+      __syncthreads();
+    } else if (owned > 0) {
+      if (!gemm_recv_wait(recv_bar, task & 1) && p.err) *p.err = GEMM_ERR_WAIT;
+      if (task + 1 < n_tasks) {
+        __syncthreads();
+        if (tid == 0) gemm_arm(recv_bar, recv_bytes);
+      }
+    }
     gemm_reduce_epilogue<EPI>(p, s_ct, NTOK, rb, n_cols, recv, own_max, colbuf, s_rstd, rank);
     if (task + 1 < n_tasks) cluster.sync();
   }

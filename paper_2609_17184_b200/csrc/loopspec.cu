@@ -94,6 +94,8 @@ GemmPlan plan_gemm_f32(int n_rb, int K, int slots) {
   return g;
 }
 
+unsigned inv_of(int cs) { return (unsigned)(((1ull << 32) + cs - 1) / cs); }  // GemmParams.inv_cs
+
 size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 
 // ---- plan of a decode-pass GEMM on the tcgen05 kernel (dgemm_kernel) ----
@@ -131,6 +133,7 @@ DgPlan plan_dg(int n_rb, int K, int MP, const int* max_clusters /* [9], by clust
 }
 int ng_for_rows(int rows) { return rows <= 8 ? 1 : rows <= 16 ? 2 : rows <= 32 ? 4 : 8; }
 
+static_assert(GEMM_ERR_WAIT == ERR_WAIT_DEC, "the flag a cluster GEMM raises");
 static_assert(SEL_ARG_BLOCK == RB_ROWS, "the selection reads one argmax partial per lm_head row block");
 
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -667,7 +670,7 @@ GemmParams gemm_params(loopspec_ctx* c, int which, int layer, const RowTable* ta
   GemmParams p;
   memset(&p, 0, sizeof p);
   const GemmPlan& g = c->cur_plan[which];
-  p.n_rb = g.n_rb, p.kb_per_rb = g.kpr, p.cluster_size = g.cs, p.n_clusters = g.n_clusters;
+  p.n_rb = g.n_rb, p.kb_per_rb = g.kpr, p.cluster_size = g.cs, p.n_clusters = g.n_clusters, p.inv_cs = inv_of(g.cs);
   p.hid = c->at<float>(c->L.hid), p.H = m.hidden, p.eps = m.rms_eps, p.tab = tab;
   p.err = c->host_flags_dev + HF_ERROR;
   const void* const* lp = (which == G_LM || which == G_ADAPT) ? nullptr : &c->layers[6 * layer];
@@ -772,7 +775,7 @@ cudaError_t launch_tc_gemm(loopspec_ctx* c, int which, int layer, const RowTable
   // one grid plane per group of 64 token columns (a plane whose group holds no row returns at once)
   const int groups = cfg_i == 1 ? col_groups(c, tab) : 1;
   q.g = gemm_params(c, which, layer, tab);
-  q.g.cluster_size = TCE_GROUPS, q.g.recv_ranks = 1, q.Hq = c->d.Hq;
+  q.g.cluster_size = TCE_GROUPS, q.g.inv_cs = inv_of(TCE_GROUPS), q.g.recv_ranks = 1, q.Hq = c->d.Hq;
   q.part = c->at<float>(c->L.tcpart), q.n_split = t.n_split, q.cols_ld = tc.cols;
   LinearTcParams p;
   memset(&p, 0, sizeof p);
@@ -828,7 +831,7 @@ cudaError_t launch_dg_lm(loopspec_ctx* c, const RowTable* tab, bool one_sum = fa
   DgParams q;
   memset(&q, 0, sizeof q);
   q.g = gemm_params(c, G_LM, 0, tab);
-  q.g.cluster_size = g.cs, q.g.n_clusters = g.n_clusters, q.g.n_rb = g.n_rb;
+  q.g.cluster_size = g.cs, q.g.inv_cs = inv_of(g.cs), q.g.n_clusters = g.n_clusters, q.g.n_rb = g.n_rb;
   if (one_sum) q.g.n_sq = 1;
   q.g.err = c->host_flags_dev + HF_ERROR, q.g.tl_id = 120;
   q.MP = c->dg_mp, q.stages = g.stages, q.acc_bufs = g.acc_bufs, q.recv_bufs = g.recv_bufs, q.err_code = ERR_WAIT;
@@ -1065,6 +1068,7 @@ int check_device_error(loopspec_ctx* c) {
   int e = c->host_flags[HF_ERROR];
   if (!e) return LOOPSPEC_OK;
   c->host_flags[HF_ERROR] = 0;
+  if (e == ERR_WAIT_DEC) return fail(c, LOOPSPEC_ETIMEOUT, "a bounded device-side wait ran out (GEMM of a decode pass's block)");
   if (e == ERR_WAIT || e == ERR_WAIT_PF)  // a bounded wait inside a kernel ran out: the pass's results are void, the context is not
     return fail(c, LOOPSPEC_ETIMEOUT, "a bounded device-side wait ran out (%s)", e == ERR_WAIT ? "readout GEMM" : "GEMM of a prompt or of a wide decode pass");
   return fail(c, LOOPSPEC_ECAPACITY, "device scheduler reported %s",
@@ -2058,7 +2062,7 @@ int loopspec_op_linear(const void* W, int32_t weight_dtype, const float* x, floa
   if (launch_k(prep_planes_kernel, dim3(M), dim3(256), 0, st, q, false) != cudaSuccess) return LOOPSPEC_ECUDA;
   GemmParams p;
   memset(&p, 0, sizeof p);
-  p.W = W, p.N = N, p.K = K, p.n_rb = g.n_rb, p.kb_per_rb = g.kpr, p.cluster_size = g.cs, p.n_clusters = g.n_clusters;
+  p.W = W, p.N = N, p.K = K, p.n_rb = g.n_rb, p.kb_per_rb = g.kpr, p.cluster_size = g.cs, p.n_clusters = g.n_clusters, p.inv_cs = inv_of(g.cs);
   p.xplanes = q.planes, p.x_ld = K, p.m_fixed = M;
   p.out = y, p.out_ld = N;
   GemmFn fn = gemm_fn(weight_dtype, ng, EPI_PLAIN);

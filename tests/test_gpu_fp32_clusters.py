@@ -1,0 +1,24 @@
+"""The fp32 GEMM's hand-over inside a cluster: every rank waits for the bytes of the columns it finishes, counted by the stores of the
+others.  Sizes at which that can go wrong: launches without a cluster (a single k-block; more row blocks than the device holds clusters),
+ranks that finish no column, one, and several, k-ranges that end inside a block, two rounds of row blocks per CTA."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 16, 8), (3, 19072, 24), (2, 48000, 40), (1, 128, 2048), (7, 128, 2048), (8, 304, 72), (9, 304, 1032), (64, 256, 688)])
+def test_fp32_linear_inside_clusters(M, N, K):
+    import paper_2609_17184_b200 as ls
+    rng = np.random.default_rng(N + K + M)
+    w = (rng.standard_normal((N, K)) * 0.05).astype(np.float32)
+    x = rng.standard_normal((M, K)).astype(np.float32)
+    wt, xt = torch.from_numpy(w).cuda(), torch.from_numpy(x).cuda()
+    y = ls.linear(wt, xt).cpu().numpy()
+    # products and sums in fp32 over chains of K / 8 terms at most: well below 2e-6 of the sum of magnitudes
+    scale = np.abs(x).astype(np.float64) @ np.abs(w).astype(np.float64).T
+    assert (np.abs(y - x.astype(np.float64) @ w.astype(np.float64).T) <= 2e-6 * scale + 1e-30).all()
+    for _ in range(3):  # bit for bit, and whatever shares the call
+        assert np.array_equal(ls.linear(wt, xt).cpu().numpy().view(np.uint32), y.view(np.uint32))
+    assert np.array_equal(ls.linear(wt, xt[:1].contiguous()).cpu().numpy()[0].view(np.uint32), y[0].view(np.uint32))
