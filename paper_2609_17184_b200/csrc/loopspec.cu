@@ -34,6 +34,7 @@ namespace {
 #ifndef LS_CTAS
 #define LS_CTAS 2
 #endif
+constexpr int ATT_LONE_CTX = 1000;  // context capacity up to which a lone sequence's passes of several rows run attn_kernel
 constexpr int kCtasPerSm = LS_CTAS;  // GEMM CTAs that fit one SM (shared memory and registers)
 
 struct GemmPlan {
@@ -254,6 +255,7 @@ struct Derived {
   int att_mode;   // how attention work items are cut (see att_run_len)
   int att_long;   // what loopspec_decode_paths reports of the context capacity
   int att_warps;  // decode attention by one warp per item (attn_warp_kernel)
+  int att_warps_one;  // ... of passes with one row per sequence
   int S, NB, B, max_rows_dec, max_rows_pf, max_rows, slots, ids_cap, n_hid, n_logit_vecs, p_logit_base, n_sq, sq_stride, max_chunks,
       trace_cap, Hq, Hkv, d1, d2;
   // Raven-style layout (P and C hold transformer blocks): all layers in one list - prelude, recurrent, coda
@@ -358,11 +360,13 @@ bool resolve_sched(const loopspec_model* m, const loopspec_sched* s, Derived* d,
   d->max_chunks = (s->max_ctx + ATT_CHUNK - 1) / ATT_CHUNK;
   d->att_mode = std::min(d->S, ATT_BATCH_SEQS);
   d->att_long = d->max_chunks > (d->S > 1 ? 8 : ATT_MAX_RUNS) ? 1 : 0;
-  // One CTA per item only for the few items of a lone sequence of short capacity, where the work of an item is its latency
-  // [us, attn_kernel / attn_warp_kernel, 536 positions: 1 row 6.5 / 9.5, 4 rows 8.2 / 10.5, 7 rows 14.2 / 11.5; 3000 positions, against
-  // the best of runs of chunks by one CTA: 4 rows 24 / 22, 7 rows 47 / 36; ms per pass at 3.6 rows: capacity 320 0.952 / 1.025, 640
-  // 1.064 / 1.047, 1040 1.140 / 1.081, 2560 1.730 / 1.482 - the line could lie near 600 positions; batches: attn_warp_kernel's comment]
-  d->att_warps = d->S > 1 || d->att_long ? 1 : 0;
+  // One CTA per item only where the work of an item is its latency: the few items of a lone sequence of short capacity, and - up to
+  // one chunk per item - every pass of one row (vanilla decoding) [us, attn_kernel / attn_warp_kernel, 536 positions: 1 row 6.5 / 9.5,
+  // 4 rows 8.2 / 10.5, 7 rows 14.2 / 11.5; 3000 positions, against the best of runs of chunks by one CTA: 4 rows 24 / 22, 7 rows 47 / 36;
+  // jobs of 64 greedy tokens of the 1.4B shape, prefill included, ms: 560 positions 100 / 107, 1000 130 / 127, 1600 166 / 157, 2200
+  // 215 / 200; 24 vanilla tokens: 1000 positions 115 / 126, 2200 178 / 184; batches: attn_warp_kernel's comment]
+  d->att_warps_one = d->S > 1 || d->att_long ? 1 : 0;
+  d->att_warps = d->att_warps_one || s->max_ctx > ATT_LONE_CTX ? 1 : 0;
   d->trace_cap = m->R * s->max_ctx + 64;  // a token can take R passes (restart)
   d->Hq = m->n_q_heads * m->head_dim;
   d->Hkv = m->n_kv_heads * m->head_dim;
@@ -848,6 +852,12 @@ int col_groups(loopspec_ctx* c, const RowTable* tab) {
   return (c->d.max_rows_dec + GROUP_ROWS - 1) / GROUP_ROWS;
 }
 
+// a pass of vanilla decoding: one row per sequence
+bool is_vanilla_table(loopspec_ctx* c, const RowTable* tab) {
+  const RowTable* const first = c->at<RowTable>(c->L.tab_van);
+  return (tab >= first && tab < first + c->m.R) || tab == c->at<RowTable>(c->L.tab_vanc);
+}
+
 // decode attention of block `l` on the rows of `tab`
 cudaError_t launch_attention(loopspec_ctx* c, const RowTable* tab, int l, unsigned long long* tl, int tl_id, bool prefill_rows = false) {
   const loopspec_model& m = c->m;
@@ -874,7 +884,7 @@ cudaError_t launch_attention(loopspec_ctx* c, const RowTable* tab, int l, unsign
       return e;
     return launch_k(attn_prefill_fold_kernel<64>, fold_grid, dim3(16), 0, c->stream, a, c->use_pdl);
   }
-  const AttnLaunch k = attn_launch(m.head_dim, G, c->n_sm, d.att_warps != 0);
+  const AttnLaunch k = attn_launch(m.head_dim, G, c->n_sm, (is_vanilla_table(c, tab) ? d.att_warps_one : d.att_warps) != 0);
   return launch_k(k.fn, dim3(k.grid), dim3(k.block), k.smem, c->stream, a, c->use_pdl);
 }
 
@@ -1413,7 +1423,8 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
   // Every kernel of the chain asks for the same (largest) shared-memory carve-out: the GEMM CTAs need it, and an SM
   // whose partition was set by a small-shared-memory kernel would have to drain before it can host one.
   {
-    const void* small_fns[] = {(const void*)attn_launch(m->head_dim, m->n_q_heads / m->n_kv_heads, c->n_sm, d.att_warps != 0).fn, (const void*)prep_planes_kernel,
+    const void* small_fns[] = {(const void*)attn_launch(m->head_dim, m->n_q_heads / m->n_kv_heads, c->n_sm, d.att_warps != 0).fn,
+                               (const void*)attn_launch(m->head_dim, m->n_q_heads / m->n_kv_heads, c->n_sm, d.att_warps_one != 0).fn, (const void*)prep_planes_kernel,
                                (const void*)select_kernel, (const void*)control_kernel, (const void*)vanilla_control_kernel,
                                (const void*)kv_commit_kernel};
     for (const void* f : small_fns)
