@@ -160,7 +160,9 @@ __device__ __forceinline__ void gemm_krange(int kpr, int cs, int rank, int& lo, 
 // ---- every rank has pushed its partial columns into the owners' receive buffers: sum them in rank order and
 // finish this CTA's columns.  Column c of row block rb is finished by rank (c mod cluster size); threads 0..127
 // take one column, threads 128..255 the next one of this rank, one output row each.
-template <int EPI, int KH = 1>
+// SMALL: the cluster kernels' divisions as multiplications and shifts (their code runs cold); the epilogue kernel of the wide passes keeps
+// the divisions [eight sequences: 268 ms with, 271 without; one row per pass on the cluster kernels: 139.4 / 138.3 ms].
+template <int EPI, int KH = 1, bool SMALL = true>
 __device__ __forceinline__ void gemm_reduce_epilogue(const GemmParams& p, const int* ct, int ntok, int rb, int n_cols, const float* recv,
                                                      int own_max, float* colbuf, const float* s_rstd, int rank, float pre_h = 0.f,
                                                      float pre_g = 1.f, float2 pre_rope = make_float2(1.f, 0.f), bool pre_valid = false) {
@@ -186,7 +188,7 @@ __device__ __forceinline__ void gemm_reduce_epilogue(const GemmParams& p, const 
     }
     float v = 0.f;
     if (live) {
-      const float* src = recv + (size_t)gemm_div(c, cs, p.inv_cs) * RBW + j;
+      const float* src = recv + (size_t)(SMALL ? gemm_div(c, cs, p.inv_cs) : c / cs) * RBW + j;
       v = src[0];
       for (int rk = 1; rk < vcs; ++rk) v += src[(size_t)rk * own_max * RBW];  // rank order, the same for every launch
       v *= s_rstd[c];
@@ -248,7 +250,8 @@ __device__ __forceinline__ void gemm_reduce_epilogue(const GemmParams& p, const 
           const int n0 = rb * RB_ROWS;
           const int region = n0 < Hq ? 0 : (n0 < Hq + Hk ? 1 : 2);
           const int rbase = region == 0 ? 0 : (region == 1 ? Hq : Hq + Hk);
-          const int ld = d == 128 ? 7 : 6, hh = j >> (ld - 1), i = j & (hd2 - 1);  // (head sizes 64 and 128: shifts)
+          const int ld = d == 128 ? 7 : 6;  // (head sizes 64 and 128)
+          const int hh = SMALL ? j >> (ld - 1) : j / hd2, i = SMALL ? j & (hd2 - 1) : j - hh * hd2;
           const float x1 = col[hh * d + i], x2 = col[hh * d + i + hd2];
           float y1 = x1, y2 = x2;
           if (region < 2) {
@@ -256,7 +259,7 @@ __device__ __forceinline__ void gemm_reduce_epilogue(const GemmParams& p, const 
             y1 = x1 * csn.x - x2 * csn.y;
             y2 = x2 * csn.x + x1 * csn.y;
           }
-          const int head = ((n0 - rbase) >> ld) + hh;
+          const int head = (SMALL ? (n0 - rbase) >> ld : (n0 - rbase) / d) + hh;
           if (region == 0) {
             float* q = p.qbuf + (size_t)c * Hq + head * d + i;
             q[0] = y1;
@@ -979,7 +982,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, GROUPED ? 1 : 8) tc_epilogue_ker
     s_recv[(c / TCE_GROUPS) * RB_ROWS + j] = v;
   }
   __syncthreads();
-  gemm_reduce_epilogue<EPI>(p, s_ct, TCE_MAX_COLS, rb, n_cols, s_recv, own_max, s_colbuf, s_rstd, rank);
+  gemm_reduce_epilogue<EPI, 1, false>(p, s_ct, TCE_MAX_COLS, rb, n_cols, s_recv, own_max, s_colbuf, s_rstd, rank);
 }
 
 }  // namespace ls
