@@ -211,7 +211,9 @@ int loopspec_launches_per_step(loopspec_ctx*, int32_t* out);
  * token columns);
  * *attention_path = 0 a short context capacity (up to 2560 positions; up to 512 when the context holds several
  * sequences), 1 a long one; contexts of one sequence and short capacity run the attention with one CTA per 64-position
- * chunk, all others with one warp per run of chunks.  Either pointer may be null. */
+ * chunk, all others with one warp per run of chunks.  The pipelined passes of the former change to warps where the committed
+ * sequence has grown so long that the chunks of R / d1 rows crowd the device (16 heads, R / d1 = 4: beyond 832 positions), whatever
+ * the capacity.  Either pointer may be null. */
 int loopspec_decode_paths(loopspec_ctx*, int32_t* gemm_path, int32_t* attention_path);
 
 /* Time `iters` back-to-back launches of one kernel of the pass in the decode launch configuration, cycling

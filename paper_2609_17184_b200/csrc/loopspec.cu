@@ -34,8 +34,18 @@ namespace {
 #ifndef LS_CTAS
 #define LS_CTAS 2
 #endif
-constexpr int ATT_LONE_CTX = 1000;  // context capacity up to which a lone sequence's passes of several rows run attn_kernel
 constexpr int kCtasPerSm = LS_CTAS;  // GEMM CTAs that fit one SM (shared memory and registers)
+constexpr int kSms = 148;            // SMs of the device (B200) where a rule has to know them without asking
+
+// A lone sequence of a capacity of up to ATT_MAX_RUNS chunks: committed positions up to which its pipelined passes run attn_kernel (a CTA
+// per chunk); beyond, attn_warp_kernel.  The former is the shorter chain as long as the SMs hold (nearly) all of a pass's chunks at once, the
+// latter wins once they queue: `levels` rows (pipeline levels of a sequence), kv_heads chunks each per 64 positions, against six chunks
+// per SM - ten where four query heads share a chunk's keys, which attn_kernel reads once for all four.  A function of the shape and of
+// the committed length alone, so neither the capacity of the context nor how calls cut a job changes a row's arithmetic.
+// [decode time by attn_kernel over that by attn_warp_kernel at 64, 512, 1024, 1536, 2400 positions: 16 heads, R / d1 = 4 (line 832): 0.90, 0.98,
+// 1.04, 1.13, 1.19; 2 levels (line 1728): 0.90, 0.94, 0.96, 1.03, 1.12; 6 heads, 4 levels (line 2368): 0.85, 0.87, 0.91, 0.94, 1.01; 32 query
+// on 8 kv heads, 4 levels (no line): 0.92, 0.95, 0.95, 0.99, 0.97; the same, 8 levels (line 1472): 0.96, 0.99, 1.02, 1.02, 1.02]
+int att_line(int levels, int kv_heads, int group) { return (group == 1 ? 6 : 10) * kSms / (levels * kv_heads) * ATT_CHUNK; }
 
 struct GemmPlan {
   int n_rb, kpr, cs, n_clusters, grid;
@@ -254,8 +264,8 @@ struct Layout {  // byte offsets into the workspace
 struct Derived {
   int att_mode;   // how attention work items are cut (see att_run_len)
   int att_long;   // what loopspec_decode_paths reports of the context capacity
-  int att_warps;  // decode attention by one warp per item (attn_warp_kernel)
-  int att_warps_one;  // ... of passes with one row per sequence
+  int att_warps;  // every decode pass's attention by one warp per item (attn_warp_kernel)
+  int att_line;   // ... otherwise: by attn_kernel up to this many committed positions (vanilla passes: always)
   int S, NB, B, max_rows_dec, max_rows_pf, max_rows, slots, ids_cap, n_hid, n_logit_vecs, p_logit_base, n_sq, sq_stride, max_chunks,
       trace_cap, Hq, Hkv, d1, d2;
   // Raven-style layout (P and C hold transformer blocks): all layers in one list - prelude, recurrent, coda
@@ -360,13 +370,12 @@ bool resolve_sched(const loopspec_model* m, const loopspec_sched* s, Derived* d,
   d->max_chunks = (s->max_ctx + ATT_CHUNK - 1) / ATT_CHUNK;
   d->att_mode = std::min(d->S, ATT_BATCH_SEQS);
   d->att_long = d->max_chunks > (d->S > 1 ? 8 : ATT_MAX_RUNS) ? 1 : 0;
-  // One CTA per item only where the work of an item is its latency: the few items of a lone sequence of short capacity, and - up to
-  // one chunk per item - every pass of one row (vanilla decoding) [us, attn_kernel / attn_warp_kernel, 536 positions: 1 row 6.5 / 9.5,
-  // 4 rows 8.2 / 10.5, 7 rows 14.2 / 11.5; 3000 positions, against the best of runs of chunks by one CTA: 4 rows 24 / 22, 7 rows 47 / 36;
-  // jobs of 64 greedy tokens of the 1.4B shape, prefill included, ms: 560 positions 100 / 107, 1000 130 / 127, 1600 166 / 157, 2200
-  // 215 / 200; 24 vanilla tokens: 1000 positions 115 / 126, 2200 178 / 184; batches: attn_warp_kernel's comment]
-  d->att_warps_one = d->S > 1 || d->att_long ? 1 : 0;
-  d->att_warps = d->att_warps_one || s->max_ctx > ATT_LONE_CTX ? 1 : 0;
+  // One CTA per item only for the few items of a lone sequence of short capacity, where the work of an item is its latency - every pass
+  // of one row (vanilla decoding), pipelined ones up to att_line positions [us, attn_kernel / attn_warp_kernel, 536 positions: 1 row
+  // 6.5 / 9.5, 4 rows 8.2 / 10.5, 7 rows 14.2 / 11.5; 3000 positions, against the best of runs of chunks by one CTA: 4 rows 24 / 22,
+  // 7 rows 47 / 36; 24 vanilla tokens with their prompt, ms: 1000 positions 115 / 126, 2200 178 / 184; batches: attn_warp_kernel's comment]
+  d->att_warps = d->S > 1 || d->att_long ? 1 : 0;
+  d->att_line = att_line((m->R + d1 - 1) / d1, m->n_kv_heads, m->n_q_heads / m->n_kv_heads);
   d->trace_cap = m->R * s->max_ctx + 64;  // a token can take R passes (restart)
   d->Hq = m->n_q_heads * m->head_dim;
   d->Hkv = m->n_kv_heads * m->head_dim;
@@ -509,7 +518,9 @@ struct loopspec_ctx {
   int* host_flags_dev = nullptr;
   int* pin_ids = nullptr;              // pinned staging for prompt / ids
   size_t pin_ids_cap = 0;
-  cudaGraphExec_t g_step = nullptr, g_vanilla = nullptr;
+  cudaGraphExec_t g_step[2] = {nullptr, nullptr}, g_vanilla = nullptr;  // (the step's attention by attn_kernel, by attn_warp_kernel)
+  bool cur_warps = false;  // which of the two the next launch_attention of decode rows takes
+  int armed_ids = 0;       // committed ids of sequence 0 when the decode rows were last built from outside a graph
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   std::vector<char> prefilled;
   bool pending_verify = false, sticky = false, vanilla_mode = false, use_pdl = true;
@@ -852,11 +863,13 @@ int col_groups(loopspec_ctx* c, const RowTable* tab) {
   return (c->d.max_rows_dec + GROUP_ROWS - 1) / GROUP_ROWS;
 }
 
-// a pass of vanilla decoding: one row per sequence
-bool is_vanilla_table(loopspec_ctx* c, const RowTable* tab) {
-  const RowTable* const first = c->at<RowTable>(c->L.tab_van);
-  return (tab >= first && tab < first + c->m.R) || tab == c->at<RowTable>(c->L.tab_vanc);
-}
+// whether pipelined passes of this context run attn_warp_kernel when `ids` ids are committed, and a scope in which launches do
+bool step_on_warps(loopspec_ctx* c, int ids) { return c->d.att_warps || ids > c->d.att_line; }
+struct WarpsGuard {
+  loopspec_ctx* c;
+  WarpsGuard(loopspec_ctx* c_, bool warps) : c(c_) { c->cur_warps = warps; }
+  ~WarpsGuard() { c->cur_warps = c->d.att_warps != 0; }
+};
 
 // decode attention of block `l` on the rows of `tab`
 cudaError_t launch_attention(loopspec_ctx* c, const RowTable* tab, int l, unsigned long long* tl, int tl_id, bool prefill_rows = false) {
@@ -884,7 +897,7 @@ cudaError_t launch_attention(loopspec_ctx* c, const RowTable* tab, int l, unsign
       return e;
     return launch_k(attn_prefill_fold_kernel<64>, fold_grid, dim3(16), 0, c->stream, a, c->use_pdl);
   }
-  const AttnLaunch k = attn_launch(m.head_dim, G, c->n_sm, (is_vanilla_table(c, tab) ? d.att_warps_one : d.att_warps) != 0);
+  const AttnLaunch k = attn_launch(m.head_dim, G, c->n_sm, c->cur_warps);
   return launch_k(k.fn, dim3(k.grid), dim3(k.block), k.smem, c->stream, a, c->use_pdl);
 }
 
@@ -1258,7 +1271,8 @@ cudaError_t launch_pf_prompt(loopspec_ctx* c, int seq, int n) {
   return launch_k(pf_readout_kernel, dim3(1), dim3(256), 0, c->stream, q, c->use_pdl);
 }
 
-int capture(loopspec_ctx* c, cudaGraphExec_t* out, bool vanilla) {
+int capture(loopspec_ctx* c, cudaGraphExec_t* out, bool vanilla, bool warps) {
+  WarpsGuard warps_guard(c, warps);
   cudaGraph_t g = nullptr;
   CU(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t e;
@@ -1370,7 +1384,7 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
   if (workspace_bytes < L.total) return LOOPSPEC_ECAPACITY;
 
   loopspec_ctx* c = new loopspec_ctx();
-  c->m = *m, c->s = *s, c->d = d, c->L = L, c->n_sm = n_sm;
+  c->m = *m, c->s = *s, c->d = d, c->L = L, c->n_sm = n_sm, c->cur_warps = d.att_warps != 0;
   c->s.d1 = d.d1, c->s.d2 = d.d2;
   if (c->s.top_p <= 0.f || c->s.top_p > 1.f) c->s.top_p = 1.f;  // 0 and anything above 1: no nucleus cut
   // (A kernel's shared-memory limit is the process's, not the context's: every context asks for the same ceiling, so that none
@@ -1423,8 +1437,8 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
   // Every kernel of the chain asks for the same (largest) shared-memory carve-out: the GEMM CTAs need it, and an SM
   // whose partition was set by a small-shared-memory kernel would have to drain before it can host one.
   {
-    const void* small_fns[] = {(const void*)attn_launch(m->head_dim, m->n_q_heads / m->n_kv_heads, c->n_sm, d.att_warps != 0).fn,
-                               (const void*)attn_launch(m->head_dim, m->n_q_heads / m->n_kv_heads, c->n_sm, d.att_warps_one != 0).fn, (const void*)prep_planes_kernel,
+    const void* small_fns[] = {(const void*)attn_launch(m->head_dim, m->n_q_heads / m->n_kv_heads, c->n_sm, false).fn,
+                               (const void*)attn_launch(m->head_dim, m->n_q_heads / m->n_kv_heads, c->n_sm, true).fn, (const void*)prep_planes_kernel,
                                (const void*)select_kernel, (const void*)control_kernel, (const void*)vanilla_control_kernel,
                                (const void*)kv_commit_kernel};
     for (const void* f : small_fns)
@@ -1432,7 +1446,7 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
         (void)cudaGetLastError();
   }
   {
-    const AttnLaunch k = attn_launch(m->head_dim, m->n_q_heads / m->n_kv_heads, c->n_sm, d.att_warps != 0);
+    const AttnLaunch k = attn_launch(m->head_dim, m->n_q_heads / m->n_kv_heads, c->n_sm, true);
     if (k.smem && cudaFuncSetAttribute((const void*)k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem) != cudaSuccess) {
       delete c;
       return LOOPSPEC_ECUDA;
@@ -1639,7 +1653,8 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
 
 int loopspec_destroy(loopspec_ctx* c) {
   if (!c) return LOOPSPEC_OK;
-  if (c->g_step) cudaGraphExecDestroy(c->g_step);
+  for (cudaGraphExec_t g : c->g_step)
+    if (g) cudaGraphExecDestroy(g);
   if (c->g_vanilla) cudaGraphExecDestroy(c->g_vanilla);
   if (c->ev0) cudaEventDestroy(c->ev0);
   if (c->ev1) cudaEventDestroy(c->ev1);
@@ -1736,6 +1751,7 @@ static int arm_decode(loopspec_ctx* c, int n_tokens, bool unlimited = false) {
                   want, spec_depth, c->s.max_ctx);
     tgt[s] = unlimited ? c->d.ids_cap : ndec[s] + n_tokens;
   }
+  c->armed_ids = nids[0];
   memcpy(c->pin_ids, tgt.data(), MAX_SEQS * 4);
   CU(c, cudaMemcpyAsync(c->seqs().n_target, c->pin_ids, MAX_SEQS * 4, cudaMemcpyHostToDevice, c->stream));
   if (c->vanilla_mode) {  // drop back from vanilla decoding: the root restarts at depth 0
@@ -1758,7 +1774,10 @@ int loopspec_step(loopspec_ctx* c, int32_t* n_rows_out, int32_t* n_need_verify_o
   int rc = arm_decode(c, 0, true);
   if (rc) return rc;
   int rows = c->host_flags[HF_N_ROWS];
-  CU(c, launch_step(c, (1 << RO_D1) | (1 << RO_D2), PH_ADVANCE | PH_BUILD, false, nullptr));
+  {
+    WarpsGuard warps_guard(c, step_on_warps(c, c->armed_ids));
+    CU(c, launch_step(c, (1 << RO_D1) | (1 << RO_D2), PH_ADVANCE | PH_BUILD, false, nullptr));
+  }
   CU(c, cudaStreamSynchronize(c->stream));
   int need = c->host_flags[HF_NEED_VERIFY];
   c->pending_verify = need > 0;
@@ -1819,7 +1838,6 @@ int loopspec_decode(loopspec_ctx* c, int32_t n_tokens, int32_t* ids_out) {
   CU(c, cudaMemcpyAsync(start.data(), c->seqs().n_dec, MAX_SEQS * 4, cudaMemcpyDeviceToHost, c->stream));
   int rc = arm_decode(c, n_tokens);
   if (rc) return rc;
-  if (!c->g_step && (rc = capture(c, &c->g_step, false))) return rc;
   // every commit needs at least d1 more passes, so `remaining * d1` replays can never overshoot
   std::vector<int> ndec(MAX_SEQS);
   for (;;) {
@@ -1830,12 +1848,19 @@ int loopspec_decode(loopspec_ctx* c, int32_t n_tokens, int32_t* ids_out) {
     for (int s = 0; s < c->d.S; ++s)
       if (c->prefilled[s]) remaining = std::max(remaining, start[s] + n_tokens - ndec[s]);
     if (remaining <= 0) break;
+    const int ids = c->armed_ids + (ndec[0] - start[0]);
+    const bool warps = step_on_warps(c, ids);
+    cudaGraphExec_t& graph = c->g_step[warps];
+    if (!graph && (rc = capture(c, &graph, false, warps))) return rc;
     if (kTune && getenv("LOOPSPEC_DBG_REPLAYS")) {  // tuning aid: a fixed number of replays, whatever they commit
-      for (int i = 0; i < atoi(getenv("LOOPSPEC_DBG_REPLAYS")); ++i) CU(c, cudaGraphLaunch(c->g_step, c->stream));
+      for (int i = 0; i < atoi(getenv("LOOPSPEC_DBG_REPLAYS")); ++i) CU(c, cudaGraphLaunch(graph, c->stream));
       CU(c, cudaStreamSynchronize(c->stream));
       return LOOPSPEC_OK;
     }
-    for (int i = 0; i < remaining * c->d.d1; ++i) CU(c, cudaGraphLaunch(c->g_step, c->stream));
+    int replays = remaining * c->d.d1;
+    // below the line: up to the first pass that can commit the id beyond it, so that the passes after that commit are the other graph's
+    if (!warps) replays = (int)std::min<long long>(replays, (long long)(c->d.att_line - ids) * c->d.d1 + 1);
+    for (int i = 0; i < replays; ++i) CU(c, cudaGraphLaunch(graph, c->stream));
   }
   return copy_ids_out(c, start, n_tokens, ids_out);
 }
@@ -1858,7 +1883,7 @@ int loopspec_vanilla_decode(loopspec_ctx* c, int32_t n_tokens, int32_t* ids_out)
   CU(c, cudaGetLastError());
   c->vanilla_mode = true;
   int rc;
-  if (!c->g_vanilla && (rc = capture(c, &c->g_vanilla, true))) return rc;
+  if (!c->g_vanilla && (rc = capture(c, &c->g_vanilla, true, c->d.att_warps != 0))) return rc;
   for (int i = 0; i < n_tokens; ++i) CU(c, cudaGraphLaunch(c->g_vanilla, c->stream));
   CU(c, cudaStreamSynchronize(c->stream));
   if ((rc = check_device_error(c))) return rc;
@@ -1933,7 +1958,8 @@ int loopspec_debug_drop_tile(loopspec_ctx* c, int32_t unit, int32_t wait_us) {
   if (!c->dg) return fail(c, LOOPSPEC_EUNSUPPORTED, "no tcgen05 readout kernel in this context (fp32 weights)");
   c->dg_drop_unit = unit;
   c->dg_wait_cycles = (unit >= 0 && wait_us > 0) ? (long long)wait_us * 2000 : TC_WAIT_CYCLES;
-  if (c->g_step) cudaGraphExecDestroy(c->g_step), c->g_step = nullptr;  // captured launches carry the old setting
+  for (cudaGraphExec_t& g : c->g_step)  // captured launches carry the old setting
+    if (g) cudaGraphExecDestroy(g), g = nullptr;
   if (c->g_vanilla) cudaGraphExecDestroy(c->g_vanilla), c->g_vanilla = nullptr;
   return LOOPSPEC_OK;
 }
@@ -1999,6 +2025,7 @@ int loopspec_time_kernel(loopspec_ctx* c, int32_t which, int32_t rows, int32_t i
     }
     t.chunk_start[rows] = items, t.attn_items = items;
   }
+  WarpsGuard warps_guard(c, which == 5 ? step_on_warps(c, t.n_canon[0]) : c->d.att_warps != 0);  // (5: as a pipelined pass at that length)
   CU(c, cudaMemcpyAsync(c->ws + c->L.tab_pf, &t, sizeof t, cudaMemcpyHostToDevice, c->stream));
   CU(c, cudaMemsetAsync(c->ws + c->L.hid + (size_t)c->d.S * c->d.NB * c->m.hidden * 4, 0, (size_t)rows * c->m.hidden * 4, c->stream));
   const RowTable* tab = c->at<RowTable>(c->L.tab_pf);
