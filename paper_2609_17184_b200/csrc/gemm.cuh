@@ -911,9 +911,10 @@ struct TcEpiParams {
   int Hq;              // query width (rows of the query buffer)
 };
 
-// (eight CTAs per SM: at 40 registers instead of 32 the QKV epilogue of 24 to 48 rows made eight sequences' passes 3 % longer)
+// Eight CTAs per SM in every variant [32 registers; at 48 to 56 passes of more than 64 rows are longer: 10 sequences of the 1.4B shape
+// 111.7 / 106.1 ms, 12 117.3 / 109.4, R = 32 with (2, 8) 578 / 555.  Left to the compiler: 32 too, but two sequences 66.0 / 66.6 ms]
 template <int EPI, bool GROUPED>
-__global__ void __launch_bounds__(GEMM_THREADS, GROUPED ? 1 : 8) tc_epilogue_kernel(const __grid_constant__ TcEpiParams q) {
+__global__ void __launch_bounds__(GEMM_THREADS, 8) tc_epilogue_kernel(const __grid_constant__ TcEpiParams q) {
   __shared__ float s_recv[(TCE_MAX_COLS / TCE_GROUPS) * RB_ROWS];
   __shared__ float s_colbuf[2 * RB_ROWS];
   __shared__ float s_rstd[TCE_MAX_COLS];
