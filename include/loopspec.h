@@ -192,14 +192,17 @@ int loopspec_get_row_trace(loopspec_ctx*, int32_t* out, int32_t max_out, int32_t
 int loopspec_debug_logits(loopspec_ctx*, int32_t seq, int32_t which, float* out_V);
 
 /* Failure injection on the host side of the bounded device waits (App. B describes no failure handling; this serves the
- * library's own tests).  Every wait inside the tcgen05 kernels (an mbarrier a TMA copy completes, a stage the tensor
- * core releases, a cluster partner's partial sums) is bounded by the clock; when one runs out the kernel raises a flag,
+ * library's own tests).  Every wait on an mbarrier (a TMA copy completes it, the tensor core releases a stage, a cluster
+ * partner hands its partial sums over) is bounded by the clock; when one runs out the kernel raises a flag,
  * carries on with whatever data it has so that every barrier still receives its arrivals, and ends; the call that
  * launched it returns LOOPSPEC_ETIMEOUT, the results of that pass are void, the context stays usable (prefill the
  * sequence again).  This call makes such a wait run out: from now on CTA 0 of the readout GEMM never requests ring unit
  * `unit` (unit >= 0) - and, where a decode pass runs its layers on the tcgen05 path (loopspec_decode_paths), those GEMMs
  * request no unit from this one on - so the wait for it gives up after about wait_us microseconds.  unit = -1 restores normal operation
- * (and the normal bound of ~0.2 s).  Nothing faults or hangs: the skipped copy is simply never issued. */
+ * (and the normal bound of ~0.2 s).  Nothing faults or hangs: the skipped copy is simply never issued.
+ * fp32 weights: the CTAs of a cluster wait, bounded, for each other's partial sums in every GEMM, the prompt's included; one that has
+ * waited in vain does so once more, sixteen times as long, when all of them have been sent.  unit 0: those waits count on four bytes that
+ * nobody sends (ETIMEOUT); unit >= 1 only sets the bound. */
 int loopspec_debug_drop_tile(loopspec_ctx*, int32_t unit, int32_t wait_us);
 
 /* Number of kernels one decode step (one graph replay of loopspec_decode) launches. */
@@ -231,7 +234,8 @@ int loopspec_time_kernel(loopspec_ctx*, int32_t which, int32_t rows, int32_t ite
  * activations split into three bf16 terms, fp32 accumulation; fp32 weights use the CUDA-core path).
  * All pointers device; x, y fp32; scratch: device, 16-byte aligned, loopspec_linear_scratch_bytes(M, N, K)
  * bytes (it receives the bf16 planes of x where x is split by a launch of its own - more than 16 rows, fp32 weights, an x
- * that is not 16-byte aligned; W is read in place; contents on entry are irrelevant).  M <= 64, N % 16 == 0, K % 8 == 0, W 16-byte aligned, else LOOPSPEC_EINVAL. */
+ * that is not 16-byte aligned; W is read in place; contents on entry are irrelevant).  fp32 weights: should a CTA's partial sums
+ * be lost on their way to another one of its cluster (a bounded wait, then a second one), the affected values of y are NaN.  M <= 64, N % 16 == 0, K % 8 == 0, W 16-byte aligned, else LOOPSPEC_EINVAL. */
 size_t loopspec_linear_scratch_bytes(int32_t M, int32_t N, int32_t K);
 int loopspec_op_linear(const void* W, int32_t weight_dtype, const float* x, float* y, int32_t M, int32_t N,
                        int32_t K, void* scratch, size_t scratch_bytes, void* cuda_stream);

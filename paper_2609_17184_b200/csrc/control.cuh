@@ -12,7 +12,7 @@ constexpr int MAX_NODES = 512;   // max_seqs * nodes-per-sequence
 enum { PH_ADVANCE = 1, PH_VERIFY = 2, PH_BUILD = 4 };
 enum { HF_ERROR = 0, HF_N_ROWS = 2, HF_NEED_VERIFY = 3, HF_FIRST_TOKEN = 4, HF_COUNT = 8 };
 enum { ERR_NODES = 1, ERR_CTX = 2, ERR_SPEC = 3, ERR_WAIT = 4 /* bounded wait, readout GEMM */, ERR_WAIT_PF = 5 /* GEMM of a prompt or of a wide decode pass */,
-       ERR_WAIT_DEC = 6 /* cluster GEMM */ };
+       ERR_WAIT_F32 = 6 /* GEMM of fp32 weights */ };
 
 struct ControlParams {
   int att_mode;     // how attention work items are cut (att_run_len)

@@ -90,7 +90,9 @@ struct GemmParams {
   float2* argpart;        // LOGITS: [column][row block] (largest logit of the block, its vocabulary index as int bits)
   int F;                  // SWIGLU: ffn width
   int perm, perm_a, perm_d;  // order of the row tiles in the packed weights (see packed_tile)
-  volatile int* err;      // host-visible error flag (a bounded wait in a tcgen05 kernel ran out)
+  volatile int* err;      // host-visible error flag (a bounded wait ran out); null: a stand-alone call
+  long long wait_cycles;  // fp32 kernel: bound of the wait for a cluster's partial columns
+  int owed;               // ... test hook: bytes that wait counts on beyond those that are sent (0 in production)
   long long* dbg;         // tuning aid: cycle stamps of CTA 0 / thread 0 (null in production)
   unsigned long long* tl; // tuning aid: kernel timeline (null in production)
   int tl_id;
@@ -306,8 +308,8 @@ __device__ __forceinline__ void gemm_load_cols(const GemmParams& p, int n_cols, 
 }
 
 // ---- hand-over of the partial columns inside a cluster without a cluster barrier (fp32 kernel): every rank that finishes columns has an
-// mbarrier in its shared memory, and the contributors' stores count their bytes on it (st.async).  [A job of the 256-wide model, passes
-// of 2 to 4 rows: 4 % shorter.  The bf16 kernels keep plain stores and the barrier: there the jobs with several rows per pass got 4 %
+// mbarrier in its shared memory, and the contributors' stores count their bytes on it (st.async).  [Decode of 64 tokens of the 256-wide
+// model, passes of 2 to 4 rows: 3.65 ms, 3.78 with plain stores and the barrier.  The bf16 kernels keep plain stores and the barrier: there the jobs with several rows per pass got 4 %
 // longer, those with one row no shorter.]
 __device__ __forceinline__ unsigned gemm_mapa(unsigned addr, unsigned rank) {
   unsigned r;
@@ -322,21 +324,25 @@ __device__ __forceinline__ int gemm_owned(int n_cols, int cs, int rank, unsigned
 __device__ __forceinline__ void gemm_arm(unsigned bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-constexpr int GEMM_ERR_WAIT = 6;  // what the host's flag shows of a wait that ran out (ERR_WAIT_DEC)
-constexpr long long GEMM_WAIT_CYCLES = 400000000LL;  // ~0.2 s
-__device__ __forceinline__ bool gemm_recv_wait(unsigned bar, unsigned parity) {
+constexpr int GEMM_ERR_WAIT = 6;  // what the host's flag shows of a wait that ran out (ERR_WAIT_F32)
+__device__ __forceinline__ bool gemm_recv_wait(unsigned bar, long long limit) {
   const long long t0 = clock64();
   for (;;) {
+    const bool last = clock64() - t0 > limit;  // (read first: a process suspended here tries again after it)
     unsigned ok;
     asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(bar), "r"(parity)
+        : "r"(bar)
         : "memory");
-    if (ok) return true;
-    if (clock64() - t0 > GEMM_WAIT_CYCLES) return false;
+    if (ok || last) return ok;
   }
 }
+// Beside it every thread of the cluster arrives at the cluster barrier once its stores are issued and passes it before it leaves (or
+// before it tries again), so that no store finds the shared memory of a CTA that has left, and a rank that is merely slow - its
+// process was suspended - costs time and not the result [without the barrier: 3.66 ms].
+__device__ __forceinline__ void gemm_cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+__device__ __forceinline__ void gemm_cluster_wait() { asm volatile("barrier.cluster.wait;" ::: "memory"); }
 
 // push this thread's accumulator fragments (rows warp*16+g / +8, columns n*8+2t / +1) into the receive buffers of
 // the ranks that own the columns: stores to distributed shared memory, made visible by the cluster barrier or (ASYNC) counted on the
@@ -641,7 +647,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_f32_kernel(const __grid_con
   int kb_lo, kb_hi;
   gemm_krange(kpr, cs, rank, kb_lo, kb_hi);
   const int upt = kb_hi - kb_lo;
-  const int n_tasks = (p.n_rb - cid + p.n_clusters - 1) / p.n_clusters;
+  const int n_tasks = (p.n_rb - cid + p.n_clusters - 1) / p.n_clusters;  // (one where cs > 1: plan_gemm_f32)
   const int own_max = (NTOK + cs - 1) / cs;
   __shared__ __align__(8) unsigned long long s_recv_bar;
   const unsigned recv_bar = (unsigned)__cvta_generic_to_shared(&s_recv_bar);
@@ -675,7 +681,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_f32_kernel(const __grid_con
   if (cs > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (n_cols <= 0) return;
   const int owned = gemm_owned(n_cols, cs, rank, p.inv_cs);
-  const unsigned recv_bytes = (unsigned)(cs * owned * RB_ROWS * 4);
+  const unsigned recv_bytes = (unsigned)(cs * owned * RB_ROWS * 4 + p.owed);
   if (tid == 0 && owned > 0) gemm_arm(recv_bar, recv_bytes);
   __syncthreads();
 
@@ -762,17 +768,23 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_f32_kernel(const __grid_con
           if (c == 2 * t + 1) tot[n][2 * h + 1] = v;
         }
     gemm_push_tile<NG, true>(tot, recv, own_max, n_cols, cs, p.inv_cs, rank, recv_bar, cluster);
+    bool joined = cs == 1;  // this thread has passed the cluster barrier
     if (cs == 1) {
       __syncthreads();
-    } else if (owned > 0) {
-      if (!gemm_recv_wait(recv_bar, task & 1) && p.err) *p.err = GEMM_ERR_WAIT;
-      if (task + 1 < n_tasks) {
-        __syncthreads();
-        if (tid == 0) gemm_arm(recv_bar, recv_bytes);
+    } else {
+      gemm_cluster_arrive();
+      if (owned > 0 && !gemm_recv_wait(recv_bar, p.wait_cycles)) {
+        gemm_cluster_wait();  // from here on every store has been issued
+        joined = true;
+        if (!gemm_recv_wait(recv_bar, 16 * p.wait_cycles)) {  // no sums: no number for a caller without a flag, a tame one otherwise
+          for (int s = 0; s < cs * own_max; ++s) recv[s * RB_ROWS + (tid & (RB_ROWS - 1))] = p.err ? 0.f : NAN;
+          if (p.err) *p.err = GEMM_ERR_WAIT;
+        }
       }
     }
     gemm_reduce_epilogue<EPI>(p, s_ct, NTOK, rb, n_cols, recv, own_max, colbuf, s_rstd, rank);
-    if (task + 1 < n_tasks) cluster.sync();
+    if (!joined) gemm_cluster_wait();
+    if (task + 1 < n_tasks) __syncthreads();
   }
 }
 __host__ __device__ constexpr int gemm_f32_smem_bytes(int NG) {

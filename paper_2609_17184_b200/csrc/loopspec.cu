@@ -144,7 +144,7 @@ DgPlan plan_dg(int n_rb, int K, int MP, const int* max_clusters /* [9], by clust
 }
 int ng_for_rows(int rows) { return rows <= 8 ? 1 : rows <= 16 ? 2 : rows <= 32 ? 4 : 8; }
 
-static_assert(GEMM_ERR_WAIT == ERR_WAIT_DEC, "the flag a cluster GEMM raises");
+static_assert(GEMM_ERR_WAIT == ERR_WAIT_F32, "the flag a cluster GEMM of fp32 weights raises");
 static_assert(SEL_ARG_BLOCK == RB_ROWS, "the selection reads one argmax partial per lm_head row block");
 
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -687,7 +687,8 @@ GemmParams gemm_params(loopspec_ctx* c, int which, int layer, const RowTable* ta
   const GemmPlan& g = c->cur_plan[which];
   p.n_rb = g.n_rb, p.kb_per_rb = g.kpr, p.cluster_size = g.cs, p.n_clusters = g.n_clusters, p.inv_cs = inv_of(g.cs);
   p.hid = c->at<float>(c->L.hid), p.H = m.hidden, p.eps = m.rms_eps, p.tab = tab;
-  p.err = c->host_flags_dev + HF_ERROR;
+  p.err = c->host_flags_dev + HF_ERROR, p.wait_cycles = c->dg_wait_cycles;
+  p.owed = c->dg_drop_unit == 0 ? 4 : 0;
   const void* const* lp = (which == G_LM || which == G_ADAPT) ? nullptr : &c->layers[6 * layer];
   __nv_bfloat16* xpl = c->at<__nv_bfloat16>(c->L.xplanes);
   switch (which) {
@@ -1091,9 +1092,9 @@ int check_device_error(loopspec_ctx* c) {
   int e = c->host_flags[HF_ERROR];
   if (!e) return LOOPSPEC_OK;
   c->host_flags[HF_ERROR] = 0;
-  if (e == ERR_WAIT_DEC) return fail(c, LOOPSPEC_ETIMEOUT, "a bounded device-side wait ran out (GEMM of a decode pass's block)");
-  if (e == ERR_WAIT || e == ERR_WAIT_PF)  // a bounded wait inside a kernel ran out: the pass's results are void, the context is not
-    return fail(c, LOOPSPEC_ETIMEOUT, "a bounded device-side wait ran out (%s)", e == ERR_WAIT ? "readout GEMM" : "GEMM of a prompt or of a wide decode pass");
+  if (e == ERR_WAIT || e == ERR_WAIT_PF || e == ERR_WAIT_F32)  // a bounded wait inside a kernel ran out: the pass's results are void, the context is not
+    return fail(c, LOOPSPEC_ETIMEOUT, "a bounded device-side wait ran out (%s)",
+                e == ERR_WAIT ? "readout GEMM" : e == ERR_WAIT_PF ? "GEMM of a prompt or of a wide decode pass" : "GEMM of fp32 weights");
   return fail(c, LOOPSPEC_ECAPACITY, "device scheduler reported %s",
               e == ERR_NODES ? "node/row table overflow" : e == ERR_CTX ? "max_ctx exceeded" : "speculative chain too deep");
 }
@@ -1422,7 +1423,7 @@ int loopspec_init(const loopspec_model* m, const loopspec_sched* s, const loopsp
   const int cs_cap = c->ng_dec == 1 ? 11 : 8;
   for (int i = 0; i < 6; ++i) c->plan[i] = m->weight_dtype ? plan_gemm(n_rbs[i], Ks[i], slots, false, 1, cs_cap) : plan_gemm_f32(n_rbs[i], Ks[i], slots);
   for (int i = 0; i < 6; ++i) c->plan_pf[i] = m->weight_dtype ? plan_gemm(n_rbs[i], Ks[i], slots, false) : c->plan[i];
-  if (kTune) {  // tuning aid: cluster size of GEMM i from LOOPSPEC_CS_i
+  if (kTune && m->weight_dtype) {  // tuning aid: cluster size of GEMM i from LOOPSPEC_CS_i (fp32: a cluster takes one row block)
     for (int i = 0; i < 6; ++i) {
       char name[32];
       snprintf(name, sizeof name, "LOOPSPEC_CS_%d", i);
@@ -1955,7 +1956,7 @@ int loopspec_debug_logits(loopspec_ctx* c, int32_t seq, int32_t which, float* ou
 
 int loopspec_debug_drop_tile(loopspec_ctx* c, int32_t unit, int32_t wait_us) {
   if (!c || unit < -1 || wait_us < 0) return LOOPSPEC_EINVAL;
-  if (!c->dg) return fail(c, LOOPSPEC_EUNSUPPORTED, "no tcgen05 readout kernel in this context (fp32 weights)");
+  if (!c->dg && c->m.weight_dtype == 1) return fail(c, LOOPSPEC_EUNSUPPORTED, "no tcgen05 readout kernel in this context");
   c->dg_drop_unit = unit;
   c->dg_wait_cycles = (unit >= 0 && wait_us > 0) ? (long long)wait_us * 2000 : TC_WAIT_CYCLES;
   for (cudaGraphExec_t& g : c->g_step)  // captured launches carry the old setting
@@ -2102,7 +2103,7 @@ int loopspec_op_linear(const void* W, int32_t weight_dtype, const float* x, floa
   memset(&p, 0, sizeof p);
   p.W = W, p.N = N, p.K = K, p.n_rb = g.n_rb, p.kb_per_rb = g.kpr, p.cluster_size = g.cs, p.n_clusters = g.n_clusters, p.inv_cs = inv_of(g.cs);
   p.xplanes = q.planes, p.x_ld = K, p.m_fixed = M;
-  p.out = y, p.out_ld = N;
+  p.out = y, p.out_ld = N, p.wait_cycles = TC_WAIT_CYCLES;
   GemmFn fn = gemm_fn(weight_dtype, ng, EPI_PLAIN);
   if (gemm_smem(weight_dtype, ng) > 48 * 1024 &&
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(weight_dtype, ng)) != cudaSuccess)

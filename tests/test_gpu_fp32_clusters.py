@@ -5,6 +5,8 @@ import numpy as np
 import pytest
 import torch
 
+from tests import gpu_util as U
+
 pytestmark = pytest.mark.gpu
 
 
@@ -22,3 +24,45 @@ def test_fp32_linear_inside_clusters(M, N, K):
     for _ in range(3):  # bit for bit, and whatever shares the call
         assert np.array_equal(ls.linear(wt, xt).cpu().numpy().view(np.uint32), y.view(np.uint32))
     assert np.array_equal(ls.linear(wt, xt[:1].contiguous()).cpu().numpy()[0].view(np.uint32), y[0].view(np.uint32))
+
+
+def test_a_hand_over_that_never_comes_is_reported_and_survived():
+    """The waits for a cluster's partial sums count on four bytes that nobody sends: they run out, twice, the kernel raises its flag and
+    ends, the call returns ETIMEOUT; afterwards the context works like before."""
+    import time
+    import paper_2609_17184_b200 as ls
+    ref = U.oracle_run("tiny", 16, 12, 1, 2)
+    ctx = U.make_ctx("tiny", 1, 2, max_ctx=64)
+    assert ctx.prefill(ref["prompt"]) == ref["first"]
+    for call in (ctx.step, lambda: ctx.prefill(ref["prompt"]), lambda: ctx.decode(4), lambda: ctx.vanilla_decode(4)):
+        ctx.debug_drop_tile(-1)
+        ctx.prefill(ref["prompt"])
+        ctx.debug_drop_tile(0, wait_us=20)
+        t0 = time.time()
+        with pytest.raises(ls.LoopSpecError) as e:
+            call()
+        assert e.value.status == "ETIMEOUT", e.value
+        assert time.time() - t0 < 5.0
+    ctx.debug_drop_tile(-1)
+    assert ctx.prefill(ref["prompt"]) == ref["first"]
+    ctx.decode(12)
+    U.assert_same_run(ctx, ref, 12)
+    ctx.close()
+
+
+@pytest.mark.parametrize("name", ["tiny", "tiny_gqa_f32"])
+def test_a_bound_shorter_than_a_hand_over_costs_time_and_nothing_else(name):
+    """Whoever has waited for a microsecond in vain stays until every sum has been sent and finishes with them."""
+    ref = U.oracle_run(name, 16, 12, 1, 2)
+    ctx = U.make_ctx(name, 1, 2, max_ctx=64)
+    want = None
+    for short in (False, True):
+        if short:
+            ctx.debug_drop_tile(1, wait_us=1)
+        assert ctx.prefill(ref["prompt"]) == ref["first"]
+        ctx.decode(12)
+        U.assert_same_run(ctx, ref, 12)
+        z = ctx.debug_logits(0, 0).view(np.uint32)
+        assert want is None or np.array_equal(z, want)
+        want = z
+    ctx.close()
