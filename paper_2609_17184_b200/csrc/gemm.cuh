@@ -57,7 +57,7 @@ struct GemmParams {
   int N, K;
   int n_rb, kb_per_rb;    // row blocks; 32-wide k-blocks per row
   int cluster_size, n_clusters;
-  unsigned inv_cs;        // ceil(2^32 / cluster_size)
+  unsigned inv_cs;        // cluster kernels: ceil(2^32 / cluster_size)
   // activations: bf16 planes [col][3][x_ld]
   const __nv_bfloat16* xplanes;
   int x_ld;
@@ -162,8 +162,10 @@ __device__ __forceinline__ void gemm_krange(int kpr, int cs, int rank, int& lo, 
 // ---- every rank has pushed its partial columns into the owners' receive buffers: sum them in rank order and
 // finish this CTA's columns.  Column c of row block rb is finished by rank (c mod cluster size); threads 0..127
 // take one column, threads 128..255 the next one of this rank, one output row each.
-// SMALL: the cluster kernels' divisions as multiplications and shifts (their code runs cold); the epilogue kernel of the wide passes keeps
-// the divisions [eight sequences: 268 ms with, 271 without; one row per pass on the cluster kernels: 139.4 / 138.3 ms].
+// SMALL: divisions as multiplications and shifts.  The cluster kernels run their code cold and want it short; the epilogue kernel of the wide
+// passes keeps the divisions [decode times with / without, medians of four or five processes that differ by 0.2 %: cluster kernels, 1.4B
+// shape, one row per pass 130.7 / 131.1 ms, 100 positions 118.5 / 119.4, 768-wide model 18.94 / 19.14, 256-wide 3.65 / 3.69; epilogue kernel,
+// eight sequences 106.8 / 105.3, ten 105.8 / 106.2, two 65.9 / 66.2].
 template <int EPI, int KH = 1, bool SMALL = true>
 __device__ __forceinline__ void gemm_reduce_epilogue(const GemmParams& p, const int* ct, int ntok, int rb, int n_cols, const float* recv,
                                                      int own_max, float* colbuf, const float* s_rstd, int rank, float pre_h = 0.f,

@@ -105,7 +105,7 @@ GemmPlan plan_gemm_f32(int n_rb, int K, int slots) {
   return g;
 }
 
-unsigned inv_of(int cs) { return (unsigned)(((1ull << 32) + cs - 1) / cs); }  // GemmParams.inv_cs
+unsigned inv_of(int cs) { return (unsigned)(((1ull << 32) + cs - 1) / cs); }  // GemmParams.inv_cs of the cluster kernels
 
 size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 
@@ -791,7 +791,7 @@ cudaError_t launch_tc_gemm(loopspec_ctx* c, int which, int layer, const RowTable
   // one grid plane per group of 64 token columns (a plane whose group holds no row returns at once)
   const int groups = cfg_i == 1 ? col_groups(c, tab) : 1;
   q.g = gemm_params(c, which, layer, tab);
-  q.g.cluster_size = TCE_GROUPS, q.g.inv_cs = inv_of(TCE_GROUPS), q.g.recv_ranks = 1, q.Hq = c->d.Hq;
+  q.g.cluster_size = TCE_GROUPS, q.g.recv_ranks = 1, q.Hq = c->d.Hq;
   q.part = c->at<float>(c->L.tcpart), q.n_split = t.n_split, q.cols_ld = tc.cols;
   LinearTcParams p;
   memset(&p, 0, sizeof p);
@@ -847,7 +847,7 @@ cudaError_t launch_dg_lm(loopspec_ctx* c, const RowTable* tab, bool one_sum = fa
   DgParams q;
   memset(&q, 0, sizeof q);
   q.g = gemm_params(c, G_LM, 0, tab);
-  q.g.cluster_size = g.cs, q.g.inv_cs = inv_of(g.cs), q.g.n_clusters = g.n_clusters, q.g.n_rb = g.n_rb;
+  q.g.cluster_size = g.cs, q.g.n_clusters = g.n_clusters, q.g.n_rb = g.n_rb;
   if (one_sum) q.g.n_sq = 1;
   q.g.err = c->host_flags_dev + HF_ERROR, q.g.tl_id = 120;
   q.MP = c->dg_mp, q.stages = g.stages, q.acc_bufs = g.acc_bufs, q.recv_bufs = g.recv_bufs, q.err_code = ERR_WAIT;
