@@ -15,6 +15,9 @@ def test_decode_paths_follow_the_row_and_context_capacity():
     fp32 weights never leave the CUDA cores."""
     cases = [(dict(name="tiny_bf16", max_seqs=1, max_ctx=256), (0, 0)),
              (dict(name="tiny_bf16", max_seqs=4, max_ctx=256), (1, 0)),
+             (dict(name="tiny_bf16", max_seqs=1, max_ctx=1001), (0, 0)),
+             (dict(name="tiny_bf16", max_seqs=1, max_ctx=2560), (0, 0)),
+             (dict(name="tiny_bf16", max_seqs=1, max_ctx=2561), (0, 1)),
              (dict(name="tiny_bf16", max_seqs=1, max_ctx=3000), (0, 1)),
              (dict(name="tiny_bf16", max_seqs=4, max_ctx=1024), (1, 1)),
              (dict(name="tiny_bf16", max_seqs=4, max_ctx=512), (1, 0)),
