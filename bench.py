@@ -421,7 +421,8 @@ def run_ours(args):
         result["gemm_roofline"] = result["roofline"]
         att_bytes = att["rows"] * shape.n_kv_heads * att["context"] * shape.head_dim * 4
         result["roofline"] = {"bound": "hbm", "kernel": ("attn_warp_kernel (decode attention over the cached context: one warp per run of chunks on the "
-                              "tensor cores)") if att.get("path") or batch > 1 else "attn_kernel (decode attention, one work item per 64-position chunk)", "achieved": att["GBps"], "peak": peak, "unit": "GB/s",
+                              "tensor cores)") if att.get("path") or batch > 1 else "attn_kernel / attn_warp_kernel (decode attention of a lone sequence, one work item per "
+                              "64-position chunk; which of the two: by the context's length)", "achieved": att["GBps"], "peak": peak, "unit": "GB/s",
                               "frac": round(att["GBps"] / peak, 4), "peak_kind": f"of {peak_kind}",
                               "frac_of_nominal_8TBs": round(att["GBps"] / NOMINAL_HBM_GBS, 4),
                               "traffic": int(att_bytes * ATTN_TRAFFIC[0]) if att.get("path") else None,
