@@ -311,8 +311,8 @@ __device__ __forceinline__ void gemm_load_cols(const GemmParams& p, int n_cols, 
 
 // ---- hand-over of the partial columns inside a cluster without a cluster barrier (fp32 kernel): every rank that finishes columns has an
 // mbarrier in its shared memory, and the contributors' stores count their bytes on it (st.async).  [Decode of 64 tokens of the 256-wide
-// model, passes of 2 to 4 rows: 3.65 ms, 3.78 with plain stores and the barrier.  The bf16 kernels keep plain stores and the barrier: there the jobs with several rows per pass got 4 %
-// longer, those with one row no shorter.]
+// model, passes of 2 to 4 rows: 3.65 ms, 3.78 with plain stores and the barrier.  The bf16 kernels keep plain stores and the barrier: whole
+// jobs with several rows per pass were 4 % longer without, which is also what such jobs differ by, those with one row no shorter.]
 __device__ __forceinline__ unsigned gemm_mapa(unsigned addr, unsigned rank) {
   unsigned r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
